@@ -562,8 +562,7 @@ gs_status gs_compare(const float* dev_a, const float* dev_b, int H, int W, int K
     CmpAcc* acc = nullptr;
     GS_CUDA(cudaMallocAsync((void**)&acc, sizeof(CmpAcc) * K, st));
     gs_status rs = launch_zero_acc(acc, K, st);
-    size_t img = (size_t)H * W * 3;
-    for (int k = 0; k < K && rs == GS_OK; k++) rs = launch_compare(dev_a + k * img, dev_b + k * img, H, W, acc + k, st);
+    if (rs == GS_OK) rs = launch_compare(dev_a, dev_b, H, W, K, acc, st);
     if (rs == GS_OK) rs = launch_finalize(acc, K, dev_out, st);
     cudaFreeAsync(acc, st);
     return rs;

@@ -325,7 +325,7 @@ gs_status launch_blend_image(const BlendRec* recs, const uint32_t* ids, const ui
                              float* img, cudaStream_t st);
 gs_status launch_blend_compare(const BlendRec* recs, const uint32_t* ids, const uint2* ranges, const DevCamera& cam,
                                const float* clean, CmpAcc* acc, unsigned long long* work, cudaStream_t st);
-gs_status launch_compare(const float* a, const float* b, int H, int W, CmpAcc* acc, cudaStream_t st);
+gs_status launch_compare(const float* a, const float* b, int H, int W, int K, CmpAcc* acc, cudaStream_t st);
 gs_status launch_finalize(const CmpAcc* acc, int count, gs_result* out, cudaStream_t st);
 gs_status launch_records_to_blend(const gs_record* in, uint64_t n, BlendRec* out, cudaStream_t st);
 
