@@ -261,21 +261,19 @@ GS_API gs_status gs_inject_and_render_ex(gs_scene* scene, const gs_flip* dev_fli
 /* Enable (default) or disable CUDA-graph replay of the batched dirty-tile step. */
 GS_API gs_status gs_set_graphs(gs_scene* scene, int enable);
 /* Work counters for measurement: while enabled, the dirty-tile kernels add
- * up, per batch: [0] pixel-primitive evaluations, [1] tiles blended, [2] list
- * entries staged, [3] dirty tiles dropped by the plan (every pixel keeps its
- * clean value), of which [4] by the stop-key test, [5] by the tile reach
- * test, [6] because no pixel is reached, [7] because every reached pixel
- * stopped before the change, [8] list entries walked by a warp of the
- * dirty-tile blend (survivors of its box cull), [9] of them blended by at
- * least one of its pixels, [10] 8x8 pixel blocks re-blended, and the SM
- * cycles the dirty-tile blend's warps spend per phase: [11] setting up a block
- * (work queue, plan item, checkpoint, sublist searches), [12] the walk over
- * its entries, [13] the comparison with the clean image and the reductions,
- * then [14] the pixels the plan left active in the re-blended blocks and [15]
- * the same weighted by the entries each block's warp walked (so [15] / [8] is
- * the mean number of a walk step's 64 pixel slots that hold an active pixel)
- * (graphs are bypassed while counting).  gs_read_work copies those 16 counts
- * into host_counts[16] and resets them (synchronises). */
+ * up, per batch: [0] list entries blended at a pixel, [1] candidate tiles (some
+ * 8x8 block can be reached), [2] as [0], [3] dirty tiles and blocks dropped
+ * (every pixel keeps its clean value), of which [4] tiles by the stop test, [5]
+ * tiles by the reach tests, [6] blocks because no pixel is reached, [7] blocks
+ * because every reached pixel stopped before the change, [8] list entries
+ * stepped over by the dirty-tile blend's warps (the longest of 32 pixels counts),
+ * [9] as [8], [10] 8x8 pixel blocks re-blended, and the SM cycles its warps spend
+ * per phase: [11] finding the active pixels, [12] the walk over their lists, [13]
+ * the comparison with the clean image and the sums, then [14] the pixels
+ * re-blended and [15] the same weighted by the entries each one's warp stepped
+ * over (so [0] / [15] is the share of a walk step's lanes that blend) (graphs are
+ * bypassed while counting).  gs_read_work copies those 16 counts into
+ * host_counts[16] and resets them (synchronises). */
 GS_API gs_status gs_count_work(gs_scene* scene, int enable);
 GS_API gs_status gs_read_work(gs_scene* scene, uint64_t* host_counts);
 /* Kernel timing for measurement: while enabled, CUDA events bracket the two
@@ -296,11 +294,17 @@ GS_API gs_status gs_read_kernel_ms(gs_scene* scene, float* ms);
  * pairs' tile keys (4 uint64).  GS_ERR_STATE while timing is off or before the
  * first gs_render after it was switched on. */
 GS_API gs_status gs_read_render_ms(gs_scene* scene, float* ms, uint64_t* counts);
-/* Variants per dirty-tile launch (0 = largest allowed, min(2048, 8192 / K)). */
+/* Most variants per dirty-tile batch (0 = largest allowed: 65536 / K, as far as
+ * the batch's worst case of candidate tiles, variants * K * tiles, fits 2^28, and
+ * at least min(2048, 8192 / K)).  Larger values are cut to that.  The buffers grow
+ * to the largest batch a call has needed so far (20 B per variant, view and tile),
+ * or to what the device has room for.  With SSIM on a batch has at most min(2048,
+ * 8192 / K) variants. */
 GS_API gs_status gs_set_batch(gs_scene* scene, int batch);
 /* Autotuner: times the campaign over dev_flips[0, count) at batch sizes
- * 8, 16, 32, 64, 128, 256, 512, 1024, 2048 (those <= min(2048, 8192 / K)), keeps the fastest for this scene and
- * returns it (and its time per variant in microseconds, may be NULL).
+ * 8, 16, 32, ... (powers of two up to the largest allowed and up to the first
+ * that takes the whole list), keeps the fastest for this scene and returns it (and
+ * its time per variant in microseconds, may be NULL).
  * Synchronises the stream. */
 GS_API gs_status gs_autotune(gs_scene* scene, const gs_flip* dev_flips, int count, int guard_mode, uint64_t word_mask,
                              int* best_batch, float* best_us_per_variant, void* stream);

@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
+#include <initializer_list>
 #include <mutex>
 #include <string>
 
@@ -18,37 +19,27 @@ gs_status launch_apply_flips(void* planes, int fmt, uint64_t n, int nwords, cons
 gs_status launch_preprocess(const gs_scene* s, const DevCamera& cam, BlendRec* recs, uint2* rects, uint32_t* keys,
                             uint32_t* vals, gs_record* dbg, cudaStream_t st);
 gs_status launch_inject_prep(const gs_scene* s, const DevCamera* dev_cams, int K, const gs_flip* flips, int B,
-                             int guard_mode, uint64_t mask, const uint2* const* dev_clean_rects,
-                             const BlendRec* const* dev_clean_recs, DirtyDesc* desc, uint32_t* item_off, CmpAcc* acc,
-                             unsigned int* queue, cudaStream_t st);
+                             int guard_mode, uint64_t mask, const void* dev_views, DirtyDesc* desc, uint2* rows,
+                             CmpAcc* acc, unsigned int* queue, cudaStream_t st);
 gs_status build_tile_lists(RenderWork& w, uint64_t n, int tiles_x, int tiles_y, uint32_t** ids_out, cudaStream_t st);
 gs_status launch_ranges_to_offsets(const uint2* ranges, int ntiles, uint32_t* offsets, const unsigned long long* total,
                                    cudaStream_t st);
 gs_status launch_zero_acc(CmpAcc* acc, int count, cudaStream_t st);
-gs_status launch_dirty_blend(const void* dev_views, const DirtyDesc* desc, const uint32_t* item_off, int BK, int K,
-                             void* plan, uint2* cand, uint32_t* groups, uint32_t gcap, CmpAcc* acc,
-                             unsigned int* queue, unsigned long long* work, cudaEvent_t ev_mid, const SsimBufs& sb,
-                             cudaStream_t st);
+gs_status launch_dirty_blend(gs_scene* s, int BK, bool regions, const SsimBufs& sb, cudaStream_t st);
 gs_status launch_ssim_out(const CmpAcc* acc, int count, const void* dev_views, int K, double* out, cudaStream_t st);
 gs_status launch_regions_out(const CmpAcc* acc, int count, unsigned long long* out, cudaStream_t st);
 gs_status launch_finalize_dirty(const CmpAcc* acc, int count, gs_result* out, const unsigned int* clean_nonfin, int K,
-                                cudaStream_t st);
-size_t plan_item_size();
+                                unsigned int* queue, cudaStream_t st);
 size_t view_ptrs_size();
-gs_status launch_stop_keys(const uint2* ranges, const uint32_t* tile_stop, const uint32_t* dk, const uint32_t* ids,
-                           int ntiles, unsigned long long* out, cudaStream_t st);
-void fill_view_ptrs(void* host_dst, const ViewState& vs);
-gs_status launch_blists(const BlendRec* recs, const uint32_t* ids, const uint2* ranges, const DevCamera& cam,
-                        uint32_t* counts, const uint32_t* off, uint32_t* pos, BlendRec* brec, cudaStream_t st);
+void fill_view_ptrs(void* host_dst, const ViewState& vs, uint32_t bin0);
 gs_status launch_exclusive_scan(const uint32_t* in, uint64_t n, uint32_t* out, unsigned long long* scratch,
                                 unsigned long long* total, cudaStream_t st);
 uint64_t scan_scratch_len(uint64_t n);
-gs_status launch_blend_image_stop(const BlendRec* recs, const uint32_t* ids, const uint2* ranges, const DevCamera& cam,
-                                  float* img, uint32_t* stop, uint32_t* tile_stop, float4* ck, const uint32_t* ck_off,
-                                  const uint32_t* ck_cnt, unsigned int* clean_nonfin, cudaStream_t st);
-int ck_stride_value();
-int ck_max_per_tile();
-gs_status launch_gather_depth(const BlendRec* recs, const uint32_t* ids, uint64_t n, uint32_t* dk, cudaStream_t st);
+gs_status launch_blend_clean(const ViewState& v, uint32_t* counts, unsigned int* clean_nonfin, cudaStream_t st);
+gs_status launch_ranks(const uint32_t* key, const uint32_t* id, uint64_t n, const ViewState& v, cudaStream_t st);
+gs_status launch_row_counts(const ViewState& v, uint32_t* rows, cudaStream_t st);
+gs_status launch_list_lens(const uint32_t* counts, uint64_t n, uint32_t cap, uint32_t* lens, cudaStream_t st);
+gs_status launch_fill_lists(const ViewState& v, const uint32_t* off, uint32_t cap, cudaStream_t st);
 gs_status launch_offsets_to_ranges(const uint32_t* offsets, int ntiles, uint2* ranges, cudaStream_t st);
 uint32_t key_to_bits(uint32_t key, int fmt);
 int dirty_grid();
@@ -89,6 +80,21 @@ gs_status dmalloc(void** p, size_t bytes) {
         *p = nullptr;
         return set_error(GS_ERR_OOM, std::string("cudaMalloc(") + std::to_string(bytes) + "): " + cudaGetErrorString(e));
     }
+    return GS_OK;
+}
+
+void release(Buf& b) {
+    cudaFree(b.p);
+    b = Buf{};
+}
+
+// At least `bytes` in b; what it holds stays unless it is too small, or far too
+// large (twice the size and 64 MB).
+gs_status reserve(Buf& b, size_t bytes) {
+    if (b.p && b.cap >= bytes && b.cap <= 2 * bytes + (64ull << 20)) return GS_OK;
+    release(b);
+    GS_TRY(dmalloc(&b.p, bytes));
+    b.cap = bytes;
     return GS_OK;
 }
 
@@ -143,62 +149,56 @@ void free_ssim_buffers(gs_scene* s);
 void free_views(gs_scene* s) {
     destroy_graphs(s);
     free_ssim_buffers(s);
-    for (auto& v : s->views) {
-        cudaFree(v.recs);
-        cudaFree(v.rects);
-        cudaFree(v.ids);
-        cudaFree(v.dk);
-        cudaFree(v.ranges);
-        cudaFree(v.clean);
-        cudaFree(v.stop);
-        cudaFree(v.tile_stop);
-        cudaFree(v.stop_key);
-        cudaFree(v.bl_off);
-        cudaFree(v.bl_pos);
-        cudaFree(v.bl_rec);
-        cudaFree(v.ck);
-        cudaFree(v.ck_off);
-        cudaFree(v.ck_cnt);
-    }
     s->views.clear();
     s->K = 0;
     cudaFree(s->dev_cams);
     cudaFree(s->dev_views);
-    cudaFree(s->dev_clean_rects);
-    cudaFree(s->dev_clean_recs);
     cudaFree(s->clean_nonfin);
     s->clean_nonfin = nullptr;
     s->dev_cams = nullptr;
     s->dev_views = nullptr;
-    s->dev_clean_rects = nullptr;
-    s->dev_clean_recs = nullptr;
+}
+
+// the views' memory as well
+void free_view_memory(gs_scene* s) {
+    free_views(s);
+    for (auto& b : s->view_bufs) release(b);
+    s->view_bufs.clear();
+    release(s->list_tmp);
 }
 
 void free_ssim_buffers(gs_scene* s) {
+    cudaFree(s->ssim.plan);
     cudaFree(s->ssim.slot_group);
     cudaFree(s->ssim.slot_flags);
     cudaFree(s->ssim.deltas);
     cudaFree(s->ssim.tile_map);
     cudaFree(s->ssim.ssim_map);
     cudaFree(s->ssim.overflow);
+    cudaFree(s->ssim.claims);
     s->ssim = SsimBufs{};
 }
 
-// SSIM buffers sized for the current batch capacity (zeroed: generation 0 is never current)
+// Variants per batch with SSIM on: its buffers are sized for them.
+int ssim_batch(int K) { return std::max(1, std::min(kSmallBatch, kSmallPairs / K)); }
+
+// SSIM buffers (zeroed: generation 0 is never current)
 static gs_status alloc_ssim_buffers(gs_scene* s) {
-    const int K = std::max(s->K, 1);
+    const int K = std::max(s->K, 1), B = std::min(s->cap_B, ssim_batch(K));
     SsimBufs b{};
-    b.slot_cap = (uint32_t)std::min<uint64_t>(s->plan_cap, 1ull << 18);
-    b.delta_cap = (uint32_t)std::min<uint64_t>((kTilePix / 32) * s->plan_cap, 1ull << 19);
     b.max_tiles = (uint32_t)std::max(s->max_tiles, 1);
-    const size_t maps = (size_t)s->cap_B * K * b.max_tiles;
+    const size_t maps = (size_t)B * K * b.max_tiles;
+    b.slot_cap = (uint32_t)std::min<uint64_t>(maps, 3ull << 17);
+    b.delta_cap = (uint32_t)std::min<uint64_t>((kTilePix / 32) * maps, 1ull << 19);
     s->ssim = b;   // caps now; pointers below
+    GS_TRY(dmalloc((void**)&s->ssim.plan, sizeof(PlanItem) * b.slot_cap));
     GS_TRY(dmalloc((void**)&s->ssim.slot_group, sizeof(uint32_t) * 8 * b.slot_cap));
     GS_TRY(dmalloc((void**)&s->ssim.slot_flags, sizeof(uint32_t) * b.slot_cap));
     GS_TRY(dmalloc((void**)&s->ssim.deltas, sizeof(float4) * 32 * (size_t)b.delta_cap));
     GS_TRY(dmalloc((void**)&s->ssim.tile_map, sizeof(unsigned long long) * maps));
     GS_TRY(dmalloc((void**)&s->ssim.ssim_map, sizeof(unsigned long long) * maps));
     GS_TRY(dmalloc((void**)&s->ssim.overflow, sizeof(unsigned int)));
+    GS_TRY(dmalloc((void**)&s->ssim.claims, sizeof(uint32_t) * 9 * (size_t)b.slot_cap));
     GS_CUDA(cudaMemset(s->ssim.tile_map, 0, sizeof(unsigned long long) * maps));
     GS_CUDA(cudaMemset(s->ssim.ssim_map, 0, sizeof(unsigned long long) * maps));
     GS_CUDA(cudaMemset(s->ssim.overflow, 0, sizeof(unsigned int)));
@@ -213,61 +213,97 @@ gs_status ensure_ssim_buffers(gs_scene* s) {
     return rs;
 }
 
-gs_status ensure_batch_buffers(gs_scene* s, int B, int fpv) {
-    int K = std::max(s->K, 1);
-    if (B <= s->cap_B && fpv * B <= s->cap_flips) return GS_OK;
-    destroy_graphs(s);
-    free_ssim_buffers(s);
+void free_batch_buffers(gs_scene* s) {
     cudaFree(s->flip_stage);
     cudaFree(s->desc);
-    cudaFree(s->item_off);
     cudaFree(s->acc);
     cudaFree(s->res_stage);
     cudaFree(s->queue);
     cudaFree(s->saved);
-    cudaFree(s->plan);
+    cudaFree(s->rows);
     cudaFree(s->cand);
-    cudaFree(s->groups);
+    cudaFree(s->cand_at);
+    cudaFree(s->cand_sorted);
+    cudaFree(s->bins);
     s->flip_stage = nullptr;
     s->desc = nullptr;
-    s->item_off = nullptr;
     s->acc = nullptr;
     s->res_stage = nullptr;
     s->queue = nullptr;
     s->saved = nullptr;
-    s->plan = nullptr;
-    s->cand = nullptr;
-    s->groups = nullptr;
-    const int cb = std::max(B, s->cap_B);
-    const int cf = std::max(fpv * B, s->cap_flips);
-    // no capacity until every buffer below is allocated: a failure part way (out
-    // of memory) leaves nothing that a later call could take for usable
+    s->rows = s->cand = s->cand_sorted = nullptr;
+    s->cand_at = s->bins = nullptr;
     s->cap_B = 0;
     s->cap_flips = 0;
-    s->plan_cap = 0;
-    GS_TRY(dmalloc((void**)&s->flip_stage, sizeof(gs_flip) * cf));
-    GS_TRY(dmalloc((void**)&s->desc, sizeof(DirtyDesc) * cb * K));
-    GS_TRY(dmalloc((void**)&s->item_off, sizeof(uint32_t) * (2 * cb * K + 1)));   // offsets + per-pair counts
-    GS_TRY(dmalloc((void**)&s->acc, sizeof(CmpAcc) * cb * K));
-    GS_TRY(dmalloc((void**)&s->res_stage, sizeof(gs_result) * cb * K));
-    GS_TRY(dmalloc((void**)&s->queue, sizeof(unsigned int) * 8));
-    GS_CUDA(cudaMemset(s->queue, 0, sizeof(unsigned int) * 8));   // queue[6]: batch generation
-    GS_TRY(dmalloc((void**)&s->saved, sizeof(uint32_t) * cf));
+    s->cap_flip_mem = s->cap_pairs = s->cap_cands = s->cap_rows = s->cap_bins = 0;
+}
+
+gs_status ensure_batch_buffers(gs_scene* s, int B, int fpv) {
+    int K = std::max(s->K, 1);
+    if (B <= s->cap_B && fpv * B <= s->cap_flips) return GS_OK;
+    const int cb = std::max(B, s->cap_B);
+    const int cf = std::max(fpv * B, s->cap_flips);
     // every (variant, view) can dirty at most every tile of its view
-    s->plan_cap = (uint64_t)cb * K * (uint64_t)std::max(s->max_tiles, 1);
-    // groups are coded (plan slot << 3) | block in 32 bits
-    if (s->plan_cap >= (1ull << 29)) return set_error(GS_ERR_CAPACITY, "too many dirty tiles per batch for this view size");
-    GS_TRY(dmalloc(&s->plan, plan_item_size() * s->plan_cap));
-    GS_TRY(dmalloc((void**)&s->cand, sizeof(uint2) * s->plan_cap));
-    GS_TRY(dmalloc((void**)&s->groups, sizeof(uint32_t) * kDirtyBlocks * s->plan_cap));
+    const uint64_t pairs = (uint64_t)cb * K, cands = pairs * (uint64_t)std::max(s->max_tiles, 1);
+    const uint64_t rows = pairs * (uint64_t)std::max(s->max_tiles_y, 1), bins = std::max(s->all_tiles, 1u);
+    if (cands >= (1ull << 29)) return set_error(GS_ERR_CAPACITY, "too many dirty tiles per batch for this view size");
+    destroy_graphs(s);
+    free_ssim_buffers(s);
+    // new views (which reset cap_B) fit the memory of the last ones as often as not
+    if ((uint64_t)cf > s->cap_flip_mem || pairs > s->cap_pairs || cands > s->cap_cands || rows > s->cap_rows ||
+        bins > s->cap_bins) {
+        // no capacity until every buffer below is allocated: a failure part way (out
+        // of memory) leaves nothing that a later call could take for usable
+        free_batch_buffers(s);
+        GS_TRY(dmalloc((void**)&s->flip_stage, sizeof(gs_flip) * cf));
+        GS_TRY(dmalloc((void**)&s->desc, sizeof(DirtyDesc) * pairs));
+        GS_TRY(dmalloc((void**)&s->acc, sizeof(CmpAcc) * pairs));
+        GS_TRY(dmalloc((void**)&s->res_stage, sizeof(gs_result) * pairs));
+        GS_TRY(dmalloc((void**)&s->queue, sizeof(unsigned int) * 8));
+        const unsigned int q0[8] = {0u, 0u, 0u, 0u, 0u, 0u, 1u, 0u};   // [6]: batch generation
+        GS_CUDA(cudaMemcpy(s->queue, q0, sizeof(q0), cudaMemcpyHostToDevice));
+        GS_TRY(dmalloc((void**)&s->saved, sizeof(uint32_t) * cf));
+        GS_TRY(dmalloc((void**)&s->rows, sizeof(uint2) * rows));
+        GS_TRY(dmalloc((void**)&s->cand, sizeof(uint2) * cands));
+        GS_TRY(dmalloc((void**)&s->cand_at, sizeof(uint32_t) * cands));
+        GS_TRY(dmalloc((void**)&s->cand_sorted, sizeof(uint2) * cands));
+        GS_TRY(dmalloc((void**)&s->bins, sizeof(uint32_t) * bins));
+        GS_CUDA(cudaMemset(s->bins, 0, sizeof(uint32_t) * bins));
+        s->cap_flip_mem = (uint64_t)cf;
+        s->cap_pairs = pairs;
+        s->cap_cands = cands;
+        s->cap_rows = rows;
+        s->cap_bins = bins;
+    }
     s->cap_B = cb;
     s->cap_flips = cf;
     return GS_OK;
 }
 
-// Variants per dirty-tile launch: the injector's scan covers at most 1024
-// (variant, view) pairs in one block.
-int max_batch(int K) { return std::max(1, std::min(kMaxBatch, kMaxPairs / K)); }
+// Most variants per dirty-tile batch: kMaxPairs (variant, view) pairs and
+// kMaxCands candidate tiles, or a small batch whatever its tiles.  A large batch
+// amortises the launches and the tail of the longest walks, and lets the variants
+// that re-blend a tile share its blend lists in the L2: 50,000 upsets of a 134,826-
+// primitive scene took 2.07 ms in 25 batches, 0.55 ms in one.
+int max_batch(const gs_scene* s) {
+    const uint64_t K = (uint64_t)std::max(s->K, 1), tiles = (uint64_t)std::max(s->max_tiles, 1);
+    const uint64_t small = std::min<uint64_t>(kSmallBatch, kSmallPairs / K);
+    return (int)std::max<uint64_t>(1, std::max(small, std::min<uint64_t>(kMaxPairs / K, kMaxCands / (K * tiles))));
+}
+
+// Buffers for a call of B variants (at most `chunk` a batch): grown in powers of
+// two, so that small calls hold little; out of memory falls back to a smaller
+// batch.  Returns the variants a batch can have in *chunk.
+gs_status size_batch(gs_scene* s, int B, int* chunk) {
+    while (true) {
+        int cap = 64;
+        while (cap < B && cap < *chunk) cap *= 2;
+        cap = std::min(cap, *chunk);
+        const gs_status rs = ensure_batch_buffers(s, cap, 1);
+        if (rs != GS_ERR_OOM || cap <= 64) return rs;
+        *chunk = cap / 2;
+    }
+}
 
 gs_status check_flip_args(gs_scene* s, const gs_flip* flips, int B, int fpv, int guard_mode, uint64_t mask) {
     if (!s || (!flips && B > 0) || B < 0 || fpv < 1) return set_error(GS_ERR_ARG, "bad campaign arguments");
@@ -282,27 +318,24 @@ gs_status check_flip_args(gs_scene* s, const gs_flip* flips, int B, int fpv, int
 }
 
 // enqueue one dirty-tile batch (B <= cap_B, flips already in flip_stage)
-gs_status enqueue_dirty(gs_scene* s, int B, int guard_mode, uint64_t mask, bool ssim, cudaStream_t st) {
+gs_status enqueue_dirty(gs_scene* s, int B, int guard_mode, uint64_t mask, bool ssim, bool regions, cudaStream_t st) {
     int K = s->K;
-    GS_TRY(launch_inject_prep(s, s->dev_cams, K, s->flip_stage, B, guard_mode, mask,
-                              (const uint2* const*)s->dev_clean_rects, (const BlendRec* const*)s->dev_clean_recs,
-                              s->desc, s->item_off, s->acc, s->queue, st));
+    GS_TRY(launch_inject_prep(s, s->dev_cams, K, s->flip_stage, B, guard_mode, mask, s->dev_views, s->desc, s->rows,
+                              s->acc, s->queue, st));
     // external records: inside a stream capture they become event-record nodes of the graph
     if (s->ev_k0) GS_CUDA(cudaEventRecordWithFlags(s->ev_k0, st, cudaEventRecordExternal));
-    const SsimBufs sb = ssim ? s->ssim : SsimBufs{};
-    GS_TRY(launch_dirty_blend(s->dev_views, s->desc, s->item_off, B * K, K, s->plan, s->cand, s->groups,
-                              (uint32_t)(kDirtyBlocks * s->plan_cap), s->acc, s->queue, s->work_ctr, s->ev_kp, sb,
-                              st));
+    GS_TRY(launch_dirty_blend(s, B * K, regions, ssim ? s->ssim : SsimBufs{}, st));
     if (s->ev_k1) GS_CUDA(cudaEventRecordWithFlags(s->ev_k1, st, cudaEventRecordExternal));
-    GS_TRY(launch_finalize_dirty(s->acc, B * K, s->res_stage, s->clean_nonfin, K, st));
+    GS_TRY(launch_finalize_dirty(s->acc, B * K, s->res_stage, s->clean_nonfin, K, s->queue, st));
     return GS_OK;
 }
 
-gs_status run_dirty_batch(gs_scene* s, int B, int guard_mode, uint64_t mask, bool ssim, cudaStream_t st) {
-    if (!s->use_graphs || s->work_ctr) return enqueue_dirty(s, B, guard_mode, mask, ssim, st);
+gs_status run_dirty_batch(gs_scene* s, int B, int guard_mode, uint64_t mask, bool ssim, bool regions,
+                          cudaStream_t st) {
+    if (!s->use_graphs || s->work_ctr) return enqueue_dirty(s, B, guard_mode, mask, ssim, regions, st);
     GraphEntry* ge = nullptr;
     for (auto& g : s->graphs)
-        if (g.B == B && g.guard == guard_mode && g.mask == mask && g.ssim == ssim) ge = &g;
+        if (g.B == B && g.guard == guard_mode && g.mask == mask && g.ssim == ssim && g.regions == regions) ge = &g;
     if (!ge) {
         dirty_grid();   // occupancy query outside the capture
         cudaStream_t cs;
@@ -312,12 +345,13 @@ gs_status run_dirty_batch(gs_scene* s, int B, int guard_mode, uint64_t mask, boo
         g.guard = guard_mode;
         g.mask = mask;
         g.ssim = ssim;
+        g.regions = regions;
         cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) {
             cudaStreamDestroy(cs);
             return cuda_error(e, "cudaStreamBeginCapture");
         }
-        gs_status qs = enqueue_dirty(s, B, guard_mode, mask, ssim, cs);
+        gs_status qs = enqueue_dirty(s, B, guard_mode, mask, ssim, regions, cs);
         e = cudaStreamEndCapture(cs, &g.graph);
         cudaStreamDestroy(cs);
         if (qs != GS_OK) {
@@ -417,7 +451,7 @@ gs_status gs_load_scene(const void* planes, int src_on_device, uint64_t n, int s
 
 gs_status gs_free_scene(gs_scene* s) {
     if (!s) return GS_OK;
-    free_views(s);
+    free_view_memory(s);
     free_render_work(s->work);
     cudaFree(s->planes);
     cudaFree(s->pbox_lo);
@@ -425,18 +459,9 @@ gs_status gs_free_scene(gs_scene* s) {
     cudaFree(s->dev_box);
     cudaFree(s->dev_err);
     cudaFree(s->dev_clamps);
-    cudaFree(s->flip_stage);
     cudaFree(s->host_io_flips);
     cudaFree(s->host_io_out);
-    cudaFree(s->desc);
-    cudaFree(s->item_off);
-    cudaFree(s->acc);
-    cudaFree(s->res_stage);
-    cudaFree(s->queue);
-    cudaFree(s->saved);
-    cudaFree(s->plan);
-    cudaFree(s->cand);
-    cudaFree(s->groups);
+    free_batch_buffers(s);
     free_ssim_buffers(s);
     cudaFree(s->clean_nonfin);
     cudaFree(s->work_ctr);
@@ -568,119 +593,130 @@ gs_status gs_compare(const float* dev_a, const float* dev_b, int H, int W, int K
     return rs;
 }
 
+// Several arrays in one device allocation, each on a 256-byte boundary.
+struct Part {
+    void** p;
+    size_t bytes;
+};
+static gs_status place(Buf& buf, std::initializer_list<Part> parts) {
+    size_t total = 0;
+    for (const Part& q : parts) total += (q.bytes + 255) & ~(size_t)255;
+    GS_TRY(reserve(buf, total));
+    char* at = (char*)buf.p;
+    for (const Part& q : parts) {
+        *q.p = at;
+        at += (q.bytes + 255) & ~(size_t)255;
+    }
+    return GS_OK;
+}
+
+// Entries of a view's blend lists (22 B each) that are kept: views with more
+// (hundreds of barely visible primitives over every pixel) keep the front of
+// each pixel's list and read the rest from the tile's list.
+constexpr uint64_t kMaxListEntries = 1ull << 29;
+
+// The blend lists and rows of view v (its first pass is done): sizes on
+// the device, one read-back of the totals, then the second pass.
+static gs_status build_lists(gs_scene* s, ViewState& v, Buf& buf, uint32_t* counts, cudaStream_t st) {
+    const uint64_t ntiles = (uint64_t)v.cam.tiles_x * v.cam.tiles_y;
+    const uint64_t P = (uint64_t)v.cam.tile_w * v.cam.tile_h, npix = ntiles * P;
+    uint32_t *rows = nullptr, *lens = nullptr, *off = nullptr;
+    unsigned long long *scratch = nullptr, *total = nullptr;
+    GS_TRY(place(s->list_tmp, {{(void**)&rows, 4 * ntiles},
+                               {(void**)&lens, 4 * npix},
+                               {(void**)&off, 4 * npix},
+                               {(void**)&scratch, 8 * scan_scratch_len(npix)},
+                               {(void**)&total, 8 * 6}}));
+    GS_TRY(launch_row_counts(v, rows, st));
+    GS_TRY(launch_exclusive_scan(rows, ntiles, v.row_off, scratch, total, st));
+    uint32_t cap = 0xfffffffdu;
+    unsigned long long tot[6];
+    while (true) {
+        GS_TRY(launch_list_lens(counts, npix, cap, lens, st));
+        GS_TRY(launch_exclusive_scan(lens, npix, off, scratch, total + 3, st));
+        GS_CUDA(cudaMemcpyAsync(tot, total, sizeof(tot), cudaMemcpyDeviceToHost, st));
+        GS_CUDA(cudaStreamSynchronize(st));
+        if (tot[2] >= 0xffffffffull) return set_error(GS_ERR_CAPACITY, "too many blend-list rows");
+        if (tot[5] > std::max<uint64_t>(kMaxListEntries, kWalk * npix)) {
+            cap = (uint32_t)std::min<uint64_t>(cap / 2, std::max<uint64_t>(kMaxListEntries / npix, kWalk) - kWalk);
+            continue;
+        }
+        const gs_status rs = place(buf, {{(void**)&v.row_idx, 4 * P * tot[2]},
+                                         {(void**)&v.ent, sizeof(float4) * tot[5]},
+                                         {(void**)&v.rk, 4 * tot[5]},
+                                         {(void**)&v.state, sizeof(float4) * (tot[5] / kWalk)}});
+        if (rs == GS_OK) break;
+        if (rs != GS_ERR_OOM || cap == 0) return rs;
+        // keep less of the lists (a quarter of the mean length at a time)
+        cap = (uint32_t)std::min<uint64_t>(cap / 4, tot[5] / npix / 4);
+    }
+    v.ck_total = tot[2] - ntiles;
+    return launch_fill_lists(v, off, cap, st);
+}
+
 // The clean per-view state of gs_set_views, for validated arguments.
 static gs_status build_views(gs_scene* s, const gs_camera* host_cams, int K, cudaStream_t st) {
     free_views(s);
+    for (size_t i = 2 * (size_t)K; i < s->view_bufs.size(); i++) release(s->view_bufs[i]);
+    s->view_bufs.resize(2 * (size_t)K);
     s->views.resize(K);
     s->K = K;
     std::vector<DevCamera> dcams(K);
     std::vector<char> vptrs(view_ptrs_size() * K);
-    std::vector<const uint2*> crects(K);
-    std::vector<const BlendRec*> crecs(K);
     GS_TRY(dmalloc((void**)&s->clean_nonfin, sizeof(unsigned int) * K));
     GS_CUDA(cudaMemsetAsync(s->clean_nonfin, 0, sizeof(unsigned int) * K, st));
     uint64_t max_pairs = 0;
-    int max_tiles = 0;
+    int max_tiles = 0, max_tiles_y = 0;
+    uint32_t all_tiles = 0;
     for (int k = 0; k < K; k++) {
         ViewState& v = s->views[k];
         v.cam = make_dev_camera(host_cams[k], s->tile_w, s->tile_h);
         dcams[k] = v.cam;
         int ntiles = v.cam.tiles_x * v.cam.tiles_y;
+        const size_t pix = (size_t)v.cam.W * v.cam.H, tpix = (size_t)ntiles * v.cam.tile_w * v.cam.tile_h;
         uint32_t* ids = nullptr;
         uint64_t np = 0;
         GS_TRY(render_lists_sized(s, s->work, v.cam, &ids, &np, st));
-        GS_TRY(dmalloc((void**)&v.recs, sizeof(BlendRec) * std::max<uint64_t>(s->n, 1)));
-        GS_TRY(dmalloc((void**)&v.rects, sizeof(uint2) * std::max<uint64_t>(s->n, 1)));
-        GS_TRY(dmalloc((void**)&v.ids, sizeof(uint32_t) * std::max<uint64_t>(np, 1)));
-        GS_TRY(dmalloc((void**)&v.dk, sizeof(uint32_t) * std::max<uint64_t>(np, 1)));
-        GS_TRY(dmalloc((void**)&v.ranges, sizeof(uint2) * ntiles));
-        GS_TRY(dmalloc((void**)&v.clean, sizeof(float) * (size_t)v.cam.W * v.cam.H * 3));
-        GS_TRY(dmalloc((void**)&v.stop, sizeof(uint32_t) * (size_t)v.cam.W * v.cam.H));
-        GS_TRY(dmalloc((void**)&v.tile_stop, sizeof(uint32_t) * ntiles));
-        GS_TRY(dmalloc((void**)&v.stop_key, sizeof(unsigned long long) * ntiles));
+        uint32_t* counts = nullptr;   // scratch of this build
+        GS_TRY(place(s->view_bufs[2 * k], {{(void**)&v.recs, sizeof(BlendRec) * s->n},
+                                           {(void**)&v.rects, sizeof(uint2) * s->n},
+                                           {(void**)&v.rank, 4 * s->n},
+                                           {(void**)&v.sdk, 4 * s->n},
+                                           {(void**)&v.sid, 4 * s->n},
+                                           {(void**)&v.ids, 4 * np},
+                                           {(void**)&v.ranges, sizeof(uint2) * ntiles},
+                                           {(void**)&v.clean, 12 * pix},
+                                           {(void**)&v.stop, 4 * tpix},
+                                           {(void**)&v.tile_stop, (size_t)4 * ntiles},
+                                           {(void**)&v.tile_last, (size_t)4 * ntiles},
+                                           {(void**)&v.row_key, (size_t)4 * ntiles * kRowsPerTile},
+                                           {(void**)&v.row_off, (size_t)4 * ntiles},
+                                           {(void**)&v.row_cnt, (size_t)4 * ntiles},
+                                           {(void**)&counts, 4 * tpix}}));
         GS_CUDA(cudaMemcpyAsync(v.recs, s->work.recs, sizeof(BlendRec) * s->n, cudaMemcpyDeviceToDevice, st));
         GS_CUDA(cudaMemcpyAsync(v.rects, s->work.rects, sizeof(uint2) * s->n, cudaMemcpyDeviceToDevice, st));
         GS_CUDA(cudaMemcpyAsync(v.ids, ids, sizeof(uint32_t) * np, cudaMemcpyDeviceToDevice, st));
         GS_CUDA(cudaMemcpyAsync(v.ranges, s->work.ranges, sizeof(uint2) * ntiles, cudaMemcpyDeviceToDevice, st));
-        GS_TRY(launch_blend_image_stop(v.recs, v.ids, v.ranges, v.cam, v.clean, v.stop, v.tile_stop, nullptr, nullptr,
-                                       nullptr, s->clean_nonfin + k, st));
-        GS_TRY(launch_gather_depth(v.recs, v.ids, np, v.dk, st));
-        // checkpoints of the clean blend: per tile, every ck_stride list entries up to
-        // (before) the tile's last stop index, at most ck_max_per_tile
-        {
-            std::vector<uint32_t> tstop(ntiles), cnt(ntiles), off(ntiles);
-            std::vector<uint2> rg(ntiles);
-            GS_CUDA(cudaMemcpyAsync(tstop.data(), v.tile_stop, 4 * ntiles, cudaMemcpyDeviceToHost, st));
-            GS_CUDA(cudaMemcpyAsync(rg.data(), v.ranges, sizeof(uint2) * ntiles, cudaMemcpyDeviceToHost, st));
-            GS_CUDA(cudaStreamSynchronize(st));
-            uint64_t total = 0;
-            const uint32_t G = (uint32_t)ck_stride_value();
-            for (int t = 0; t < ntiles; t++) {
-                const uint32_t L = rg[t].y - rg[t].x;
-                const uint32_t last = L > 0 ? std::min(tstop[t], L - 1) : 0u;
-                cnt[t] = std::min(last / G, (uint32_t)ck_max_per_tile());
-                off[t] = (uint32_t)total;
-                total += cnt[t];
-            }
-            if (total >= 0xffffffffull) return set_error(GS_ERR_CAPACITY, "too many blend checkpoints");
-            v.ck_total = total;
-            GS_TRY(dmalloc((void**)&v.ck, sizeof(float4) * (size_t)(v.cam.tile_w * v.cam.tile_h) *
-                                              std::max<uint64_t>(total, 1)));
-            GS_TRY(dmalloc((void**)&v.ck_off, 4 * ntiles));
-            GS_TRY(dmalloc((void**)&v.ck_cnt, 4 * ntiles));
-            GS_CUDA(cudaMemcpyAsync(v.ck_off, off.data(), 4 * ntiles, cudaMemcpyHostToDevice, st));
-            GS_CUDA(cudaMemcpyAsync(v.ck_cnt, cnt.data(), 4 * ntiles, cudaMemcpyHostToDevice, st));
-            GS_TRY(launch_blend_image_stop(v.recs, v.ids, v.ranges, v.cam, v.clean, v.stop, v.tile_stop, v.ck,
-                                           v.ck_off, v.ck_cnt, nullptr, st));
-            GS_CUDA(cudaStreamSynchronize(st));
-        }
-        GS_TRY(launch_stop_keys(v.ranges, v.tile_stop, v.dk, v.ids, ntiles, v.stop_key, st));
+        GS_TRY(launch_ranks(s->work.dkey[s->work.cur], s->work.dval[s->work.cur], s->n, v, st));
+        GS_TRY(launch_blend_clean(v, counts, s->clean_nonfin + k, st));
+        GS_TRY(build_lists(s, v, s->view_bufs[2 * k + 1], counts, st));
         v.npairs = np;
-        // per (tile, 8x8 block) sublists of the clean lists
-        {
-            const uint64_t nb = (uint64_t)ntiles * (uint64_t)((v.cam.tile_w * v.cam.tile_h) / 64);
-            uint32_t* counts = nullptr;
-            unsigned long long* scratch = nullptr;
-            GS_TRY(dmalloc((void**)&v.bl_off, sizeof(uint32_t) * (nb + 1)));
-            GS_TRY(dmalloc((void**)&counts, sizeof(uint32_t) * nb));
-            GS_TRY(dmalloc((void**)&scratch, sizeof(unsigned long long) * (scan_scratch_len(nb) + 3)));
-            unsigned long long* total = scratch + scan_scratch_len(nb);
-            gs_status bs =
-                launch_blists(v.recs, v.ids, v.ranges, v.cam, counts, nullptr, nullptr, nullptr, st);
-            if (bs == GS_OK) bs = launch_exclusive_scan(counts, nb, v.bl_off, scratch, total, st);
-            unsigned long long tot = 0;
-            if (bs == GS_OK && cudaMemcpyAsync(&tot, total, sizeof(tot), cudaMemcpyDeviceToHost, st) != cudaSuccess)
-                bs = set_error(GS_ERR_CUDA, "sublist total");
-            if (bs == GS_OK && cudaStreamSynchronize(st) != cudaSuccess) bs = set_error(GS_ERR_CUDA, "sublist sync");
-            cudaFree(counts);
-            cudaFree(scratch);
-            GS_TRY(bs);
-            if (tot >= 0xffffffffull) return set_error(GS_ERR_CAPACITY, "block sublists exceed 2^32 entries");
-            const uint32_t tot32 = (uint32_t)tot;
-            GS_CUDA(cudaMemcpyAsync(v.bl_off + nb, &tot32, sizeof(tot32), cudaMemcpyHostToDevice, st));
-            GS_TRY(dmalloc((void**)&v.bl_pos, sizeof(uint32_t) * std::max<uint64_t>(tot, 1)));
-            GS_TRY(dmalloc((void**)&v.bl_rec, sizeof(BlendRec) * std::max<uint64_t>(tot, 1)));
-            GS_TRY(launch_blists(v.recs, v.ids, v.ranges, v.cam, nullptr, v.bl_off, v.bl_pos, v.bl_rec, st));
-            GS_CUDA(cudaStreamSynchronize(st));
-        }
-        fill_view_ptrs(vptrs.data() + view_ptrs_size() * k, v);
-        crects[k] = v.rects;
-        crecs[k] = v.recs;
+        fill_view_ptrs(vptrs.data() + view_ptrs_size() * k, v, all_tiles);
+        all_tiles += (uint32_t)ntiles;
         max_pairs = std::max(max_pairs, np);
         max_tiles = std::max(max_tiles, ntiles);
+        max_tiles_y = std::max(max_tiles_y, v.cam.tiles_y);
     }
     GS_TRY(dmalloc((void**)&s->dev_cams, sizeof(DevCamera) * K));
     GS_TRY(dmalloc(&s->dev_views, vptrs.size()));
-    GS_TRY(dmalloc((void**)&s->dev_clean_rects, sizeof(uint2*) * K));
-    GS_TRY(dmalloc((void**)&s->dev_clean_recs, sizeof(BlendRec*) * K));
     GS_CUDA(cudaMemcpyAsync(s->dev_cams, dcams.data(), sizeof(DevCamera) * K, cudaMemcpyHostToDevice, st));
     GS_CUDA(cudaMemcpyAsync(s->dev_views, vptrs.data(), vptrs.size(), cudaMemcpyHostToDevice, st));
-    GS_CUDA(cudaMemcpyAsync(s->dev_clean_rects, crects.data(), sizeof(uint2*) * K, cudaMemcpyHostToDevice, st));
-    GS_CUDA(cudaMemcpyAsync(s->dev_clean_recs, crecs.data(), sizeof(BlendRec*) * K, cudaMemcpyHostToDevice, st));
     // the plain loop re-renders a single-flip variant: at most one primitive
     // changes, adding at most one grid's worth of pairs
     s->full_cap_pairs = max_pairs + (uint64_t)max_tiles + 1024;
     s->max_tiles = max_tiles;
+    s->max_tiles_y = max_tiles_y;
+    s->all_tiles = all_tiles;
     // buffers for the dirty engine
     s->cap_B = 0;
     s->cap_flips = 0;
@@ -697,7 +733,7 @@ gs_status gs_set_views(gs_scene* s, const gs_camera* host_cams, int K, void* str
     // a failure part way (out of memory, a capacity limit) leaves no half-built
     // views behind: campaign calls then report GS_ERR_STATE instead of reading them
     if (rs != GS_OK) {
-        free_views(s);
+        free_view_memory(s);
         s->host_cams.clear();
         return rs;
     }
@@ -765,17 +801,18 @@ gs_status inject_and_render(gs_scene* s, const gs_flip* dev_flips, int B, int gu
                             gs_result* dev_out, uint64_t* dev_regions, double* dev_ssim, void* stream) {
     cudaStream_t st = (cudaStream_t)stream;
     const int K = s->K;
-    const int max_chunk = max_batch(K);
-    const int chunk = s->batch > 0 ? std::min(s->batch, max_chunk) : max_chunk;
+    const int max_chunk = max_batch(s);
+    int chunk = s->batch > 0 ? std::min(s->batch, max_chunk) : max_chunk;
     const bool ssim = dev_ssim != nullptr;
+    if (ssim) chunk = std::min(chunk, ssim_batch(K));
     if (ssim && (s->tile_w != kTile || s->tile_h != kTile))
         return set_error(GS_ERR_STATE, "the dirty-tile SSIM needs 16 x 16 render tiles (gs_set_tile)");
-    GS_TRY(ensure_batch_buffers(s, chunk, 1));
+    GS_TRY(size_batch(s, B, &chunk));
     if (ssim) GS_TRY(ensure_ssim_buffers(s));
     for (int b0 = 0; b0 < B; b0 += chunk) {
         int nb = std::min(chunk, B - b0);
         GS_CUDA(cudaMemcpyAsync(s->flip_stage, dev_flips + b0, sizeof(gs_flip) * nb, cudaMemcpyDeviceToDevice, st));
-        GS_TRY(run_dirty_batch(s, nb, guard_mode, word_mask, ssim, st));
+        GS_TRY(run_dirty_batch(s, nb, guard_mode, word_mask, ssim, dev_regions != nullptr, st));
         GS_CUDA(cudaMemcpyAsync(dev_out + (size_t)b0 * K, s->res_stage, sizeof(gs_result) * nb * K,
                                 cudaMemcpyDeviceToDevice, st));
         if (dev_regions)
@@ -936,8 +973,7 @@ gs_status gs_autotune(gs_scene* s, const gs_flip* dev_flips, int count, int guar
     if (count < 1 || !best_batch) return set_error(GS_ERR_ARG, "bad gs_autotune arguments");
     cudaStream_t st = (cudaStream_t)stream;
     const int K = s->K;
-    const int max_chunk = max_batch(K);
-    const int cands[9] = {8, 16, 32, 64, 128, 256, 512, 1024, 2048};
+    const int max_chunk = max_batch(s);
     gs_result* out = nullptr;
     GS_CUDA(cudaMallocAsync((void**)&out, sizeof(gs_result) * (size_t)count * K, st));
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -948,11 +984,11 @@ gs_status gs_autotune(gs_scene* s, const gs_flip* dev_flips, int count, int guar
         return set_error(GS_ERR_CUDA, "gs_autotune: event creation failed");
     }
     const int prev_batch = s->batch;
-    int best = max_chunk;
+    int best = std::min(8, max_chunk);
     float best_t = 1e30f;
     gs_status rs = GS_OK;
-    for (int c : cands) {
-        if (c > max_chunk) break;
+    // powers of two up to the largest allowed, and up to the first that takes the list whole
+    for (int c = 8; c <= max_chunk && (c == 8 || c / 2 < count); c *= 2) {
         s->batch = c;
         // warm (graph capture), then time the whole list at this batch size
         int warm = std::min(count, c);

@@ -30,8 +30,11 @@ __host__ __device__ inline bool tile_shape_ok(int tw, int th) {
 // log2 of the 8x4 blocks per tile row (tw / 8 = 1, 2, 4)
 __host__ __device__ inline int tile_lgx(int tw) { return tw == 8 ? 0 : (tw == 16 ? 1 : 2); }
 constexpr int kMaxWords = 59;
-constexpr int kMaxPairs = 8192;       // (variant, view) pairs per dirty-tile launch (one scan block)
-constexpr int kMaxBatch = 2048;       // variants per dirty-tile launch (also <= kMaxPairs / views)
+constexpr int kMaxPairs = 65536;      // (variant, view) pairs per dirty-tile batch
+constexpr uint64_t kMaxCands = 1ull << 28;   // candidate tiles a batch has room for, unless it is small (20 B each)
+constexpr int kSmallPairs = 8192, kSmallBatch = 2048;   // such a batch; also the largest with SSIM on
+constexpr int kRowsPerTile = 64;      // rows of a tile after row 0
+constexpr int kWalk = 4;              // blend-list entries taken at a time: 64 bytes
 // first bit of the sign and exponent bits a sign+exponent code protects
 __host__ __device__ inline int ecc_first_bit(int fmt) { return fmt == GS_FP32 ? 23 : (fmt == GS_FP16 ? 10 : 7); }
 constexpr int kSseFracBits = 39;      // fixed-point scale of per-pixel squared errors (3 * 2^39 * 5.1e6 px < 2^64)
@@ -119,86 +122,123 @@ __host__ __device__ inline unsigned long long rect_cells(uint2 rect, int W, int 
 struct ViewPtrs {
     const BlendRec* recs;
     const uint32_t* ids;
-    const uint32_t* dk;      // depth bits of ids[j] (list-aligned)
+    const uint32_t* rank;    // place of each primitive in the view's (depth, index) order
+    const uint32_t* sdk;     // that order: depth keys
+    const uint32_t* sid;     // and primitives
+    const uint2* rects;
     const uint2* ranges;
     const float* clean;
-    const uint32_t* stop;    // clean stop index of every pixel
-    const uint32_t* tile_stop;   // largest stop index of each tile
-    const unsigned long long* stop_key;   // (depth bits, id) of the list entry at tile_stop; ~0 if none
-    const uint32_t* bl_off;      // per (tile, 8x8 block): start of its sublist in bl_pos (ntiles * kDirtyBlocks + 1)
-    const uint32_t* bl_pos;      // positions (in the tile's list) of the entries whose box meets the block
-    const BlendRec* bl_rec;      // their records, same order
-    const float4* ck;            // clean-blend checkpoints (T, C) of every pixel
-    const uint32_t* ck_off;      // first checkpoint of each tile
-    const uint32_t* ck_cnt;      // checkpoints of each tile (after kCkStride, 2 kCkStride, ... entries)
-    int W, H, tiles_x, tile_w, tile_h, pad[3];
+    const uint32_t* stop;        // rank of the entry that stopped each clean pixel (tile, natural order)
+    const uint32_t* tile_stop;   // the largest of them in each tile
+    const uint32_t* row_idx;     // rows of every pixel of a tile, tile order: where its blend list continues (into ent / rk)
+    const uint32_t* row_off;     // first row of each tile (row 0: the lists' starts)
+    const uint32_t* row_key;     // [tile][kRowsPerTile] rank of the last entry before row 1, 2, ... (0xffffffff: no row)
+    const float4* ent;           // pixel blend lists: (alpha, colour) of the entries a pixel blends, front to back
+    const uint32_t* rk;          // their ranks
+    const float4* state;         // clean blend (T, C) in front of every kWalk-th entry of the lists
+    int W, H, tiles_x, tile_w, tile_h;
+    uint32_t bin0;               // tiles of the views before this one
+    uint32_t pad[2];
 };
 
-// One dirty tile that needs re-blending (112 B).  ins is the insertion position
-// in the clean list without the primitive's old entry; cut is the first changed
-// position of the clean list; rec is the corrupted record (when flags bit 1);
-// mask marks the tile's active pixels (natural order, 8 x 32 bits).
+constexpr uint32_t kNoRank = 0xfffffffeu;   // above every primitive's rank, below a list's end (0xffffffff)
+
+// Candidate tile of a batch: x = (variant, view) | 8x8 blocks to look at << 20 |
+// view << 24, y = tile x | tile y << 16.
+constexpr int kUnitVars = 16;   // candidates a block of the dirty blend takes at a time
+constexpr uint32_t kCandPair = (1u << 20) - 1u;
+static_assert(kMaxPairs <= (1 << 20), "a candidate packs its pair into 20 bits");
+
+// One dirty tile that is re-blended, kept for the dirty-tile SSIM (48 B): mask
+// marks the tile's active pixels (natural order, 8 x 32 bits).
 struct __align__(16) PlanItem {
-    BlendRec rec;
     uint32_t mask[kTilePix / 32];
     uint32_t bk;      // (variant, view) = variant * K + view
     uint32_t tile;
-    uint32_t s, e;    // clean list range
-    uint32_t pp, ins, cut;
-    uint32_t flags;   // bit 0: old entry in this tile, bit 1: corrupted entry in this tile
+    uint32_t pad[2];
 };
-static_assert(sizeof(PlanItem) == 112 && offsetof(PlanItem, mask) == 48 && offsetof(PlanItem, bk) == 80 &&
-                  offsetof(PlanItem, pp) == 96,
-              "k_plan writes PlanItem as 7 16-byte parts");
+static_assert(sizeof(PlanItem) == 48, "k_plan writes PlanItem as 3 16-byte parts");
 
 // Buffers of the dirty-tile SSIM (all NULL when it is off): per plan slot the
 // delta index of each of its 8x4 blocks (0xffffffff: none), per delta index the
 // new values of the block's 32 pixels, per (variant, view) and tile the plan
 // slot (generation << 32 | slot) and the SSIM claim (generation << 32).
 struct SsimBufs {
+    PlanItem* plan;                    // [slot_cap] the re-blended tiles
     uint32_t* slot_group;              // [slot_cap * 8]
     uint32_t* slot_flags;              // [slot_cap] changed pixels: bit 4 any, 0-3 within 5 of the left/right/top/bottom edge
     float4* deltas;                    // [delta_cap * 32]
     unsigned long long* tile_map;      // [B*K * max_tiles]
     unsigned long long* ssim_map;      // [B*K * max_tiles]
     unsigned int* overflow;            // set when a capacity is exceeded
+    uint32_t* claims;                  // [slot_cap * 9] claimed tiles: plan slot * 9 + neighbour
     uint32_t slot_cap, delta_cap, max_tiles, pad;
 };
 
-// Dirty-tile work descriptor of one (variant, view).
-struct DirtyDesc {
+// Dirty-tile work descriptor of one (variant, view).  An empty rect: the record
+// is not there (not binned, or alpha < 1/255 everywhere).
+struct __align__(16) DirtyDesc {
     BlendRec rec;          // corrupted primitive's record
-    uint32_t prim;
-    int32_t new_vis;       // corrupted primitive binned?
-    int32_t old_vis;       // clean primitive binned?
-    uint32_t n_items;      // dirty tiles
+    BlendRec old;          // clean primitive's record
     uint16_t nx0, ny0, nx1, ny1;   // corrupted rect
     uint16_t ox0, oy0, ox1, oy1;   // clean rect
-    float old_depth;       // clean primitive's depth (when old_vis)
-    uint32_t pad[3];
+    uint32_t new_rank;     // clean entries of lower rank lie in front of the corrupted one (kNoRank: not there)
+    uint32_t old_rank;     // the clean entry's rank (kNoRank: not there)
+    uint32_t prim, pad;
+};
+
+// The union of the half-open intervals [n0, n1) and [o0, o1) as a list: first
+// [n0, n1), then what [o0, o1) has outside it.
+struct Union1 {
+    int n0, nlen, o0, left, right0, len;
+    __host__ __device__ Union1(int a0, int a1, int b0, int b1) {
+        const bool none = a1 <= a0;
+        n0 = none ? b0 : a0;
+        nlen = none ? 0 : a1 - a0;
+        o0 = b0;
+        const int n1 = n0 + nlen;
+        left = max(0, min(b1, n0) - b0);
+        right0 = max(b0, n1);
+        len = nlen + left + max(0, b1 - right0);
+    }
+    __host__ __device__ int at(int j) const {
+        if (j < nlen) return n0 + j;
+        const int r = j - nlen;
+        return r < left ? o0 + r : right0 + (r - left);
+    }
 };
 
 // ----------------------------------------------------------------------------
 // per-view clean state and scratch
 // ----------------------------------------------------------------------------
+// A device allocation that its owner keeps and reuses (reserve / release in
+// gs_api.cu).
+struct Buf {
+    void* p = nullptr;
+    size_t cap = 0;
+};
+
 struct ViewState {
     DevCamera cam{};
     BlendRec* recs = nullptr;        // [n]
     uint2* rects = nullptr;          // [n] (x0 | y0 << 16, x1 | y1 << 16)
+    uint32_t* rank = nullptr;        // [n] place in the view's (depth, index) order
+    uint32_t* sdk = nullptr;         // [n] depth keys in that order
+    uint32_t* sid = nullptr;         // [n] primitives in that order
     uint32_t* ids = nullptr;         // [npairs] sorted tile lists
-    uint32_t* dk = nullptr;          // [npairs] depth bits of ids[j]
     uint2* ranges = nullptr;         // [ntiles] (start, end)
     float* clean = nullptr;          // [H*W*3]
-    uint32_t* stop = nullptr;        // [H*W] list index that stopped each clean pixel
-    uint32_t* tile_stop = nullptr;   // [ntiles] largest stop index in each tile
-    unsigned long long* stop_key = nullptr;   // [ntiles] (depth bits << 32 | id) of the entry at tile_stop (~0: none)
-    uint32_t* bl_off = nullptr;      // [ntiles * kDirtyBlocks + 1] start of each (tile, 8x8 block) sublist in bl_pos
-    uint32_t* bl_pos = nullptr;      // list positions whose box meets the block, ascending per sublist
-    BlendRec* bl_rec = nullptr;      // the records of those entries, in the same order (streamed by the blend)
-    float4* ck = nullptr;            // clean-blend checkpoints [total][pixels of a tile]
-    uint32_t* ck_off = nullptr;      // [ntiles]
-    uint32_t* ck_cnt = nullptr;      // [ntiles]
-    uint64_t ck_total = 0;
+    uint32_t* stop = nullptr;        // [ntiles][pixels of a tile] rank of the entry that stopped the clean pixel
+    uint32_t* tile_stop = nullptr;   // [ntiles] the largest of them
+    uint32_t* tile_last = nullptr;   // [ntiles] largest list position that stopped a pixel (build only)
+    uint32_t* row_idx = nullptr;     // [rows][pixels of a tile] where each pixel's blend list continues
+    uint32_t* row_off = nullptr;     // [ntiles] first row
+    uint32_t* row_cnt = nullptr;     // [ntiles] rows after row 0 (build only)
+    uint32_t* row_key = nullptr;     // [ntiles][kRowsPerTile] rank of the last entry before each row after row 0
+    float4* ent = nullptr;           // pixel blend lists (alpha, r, g, b)
+    uint32_t* rk = nullptr;          // their ranks
+    float4* state = nullptr;         // clean blend in front of every kWalk-th entry of the lists
+    uint64_t ck_total = 0;           // rows after the tiles' row 0 (the server's size estimate)
     uint64_t npairs = 0;
     uint64_t cap_pairs = 0;
 };
@@ -223,6 +263,7 @@ struct RenderWork {
     unsigned long long* total = nullptr;        // [0] pair count, [1] overflow flag
     unsigned long long* host_total = nullptr;   // pinned mirror
     int passes[2] = {0, 0};                     // radix passes of the last build: depth keys, pair tile keys
+    int cur = 0;                                // dkey / dval buffer that holds the last build's depth order
 };
 
 struct GraphEntry {
@@ -230,6 +271,7 @@ struct GraphEntry {
     int guard = -2;
     uint64_t mask = 0;
     bool ssim = false;
+    bool regions = false;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
 };
@@ -254,12 +296,14 @@ struct gs_scene {
     // clean per-view state of the campaign
     int K = 0;
     std::vector<gs::ViewState> views;
+    std::vector<gs::Buf> view_bufs;         // two per view: they hold all of its state; kept from one gs_set_views to the next
+    gs::Buf list_tmp;                       // scratch of a view's build
     gs::DevCamera* dev_cams = nullptr;
     void* dev_views = nullptr;              // ViewPtrs[K]
-    void* dev_clean_rects = nullptr;        // const uint2*[K]
-    void* dev_clean_recs = nullptr;         // const BlendRec*[K]
     uint64_t full_cap_pairs = 0;
     int max_tiles = 0;
+    int max_tiles_y = 0;
+    uint32_t all_tiles = 0;                 // tiles of all views
     gs::RenderWork work;                    // scratch of the full render pipeline
     int tile_w = gs::kTile, tile_h = gs::kTile;   // render tile shape (gs_set_tile)
     std::vector<gs_camera> host_cams;       // the cameras of gs_set_views (rebuilt on a tile change)
@@ -267,20 +311,21 @@ struct gs_scene {
     // batch buffers (dirty engine and plain loop)
     int cap_B = 0;
     int cap_flips = 0;
+    uint64_t cap_flip_mem = 0, cap_pairs = 0, cap_cands = 0, cap_rows = 0, cap_bins = 0;   // elements the buffers below hold
     gs_flip* flip_stage = nullptr;
     gs_flip* host_io_flips = nullptr;       // device copies of gs_inject_and_render_host's inputs / outputs
     gs_result* host_io_out = nullptr;
     size_t host_io_flips_cap = 0, host_io_out_cap = 0;
     gs::DirtyDesc* desc = nullptr;
-    uint32_t* item_off = nullptr;
     gs::CmpAcc* acc = nullptr;
     gs_result* res_stage = nullptr;
-    unsigned int* queue = nullptr;
-    void* plan = nullptr;                   // dirty tiles to re-blend (PlanItem[plan_cap])
-    uint2* cand = nullptr;                  // candidate tiles of the plan's first pass [plan_cap]
-    uint32_t* groups = nullptr;             // 8x8 pixel blocks to re-blend, (item << 3) | block [kDirtyBlocks * plan_cap]
+    unsigned int* queue = nullptr;          // batch counters (see k_plan)
+    uint2* rows = nullptr;                  // tile rows to look at: (pair, tile y | view << 16) [pairs * max_tiles_y]
+    uint2* cand = nullptr;                  // candidate tiles [pairs * max_tiles]
+    uint32_t* cand_at = nullptr;            // their places inside their tile's bin (large batches)
+    uint2* cand_sorted = nullptr;           // the same by tile (large batches)
+    uint32_t* bins = nullptr;               // candidates per tile, then bin starts [all_tiles] (zero between batches)
     gs::SsimBufs ssim{};                    // dirty-tile SSIM buffers (allocated on first use, else NULL)
-    uint64_t plan_cap = 0;
     unsigned int* clean_nonfin = nullptr;   // [K] non-finite pixels of each clean view
     uint32_t* saved = nullptr;
     bool use_graphs = true;

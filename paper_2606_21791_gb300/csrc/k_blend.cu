@@ -16,10 +16,11 @@
 // depend on which tiles ran or in what order: a dirty-tile re-blend and a full
 // re-render give identical records.
 //
-// Dirty-tile engine: a persistent kernel takes (variant, view, dirty tile) work
-// items from an atomic queue.  A dirty tile is re-blended from the clean sorted
-// list with the flipped primitive's clean entry removed and its corrupted record
-// merged in at its (depth, index) position, and compared on the fly.
+// Dirty-tile engine: the plan lists the (variant, view, tile) candidates that the
+// flipped primitive's clean or corrupted record can reach; the dirty blend decides
+// per pixel, re-blends the pixels that can change from their own blend lists
+// (kept with the clean view), with the clean entry left out and the corrupted
+// record at its (depth, index) place, and compares them on the fly.
 #include <mutex>
 
 #include "gs_internal.h"
@@ -70,24 +71,7 @@ __device__ __forceinline__ BlendRec load_rec(const BlendRec* recs, uint32_t id) 
 struct Pix {
     float T, c0, c1, c2;
     bool done;
-    uint32_t stop;   // list index of the entry that stopped the pixel (T would drop below 1e-4)
 };
-
-// Pixel geometry of thread `tid` in a tw x th tile: warp w covers the 8x4 block w
-// of the natural order.
-struct PixGeo {
-    int px, py;
-    float pxc, pyc;
-    float wx0, wx1, wy0, wy1;   // pixel-centre bounds of the warp's block
-    bool inside;
-};
-
-// Natural pixel of index u in a tw x th tile.
-__device__ __forceinline__ void pix_of(int tile_x, int tile_y, int tw, int th, int u, int& px, int& py) {
-    const int w = u >> 5, l = u & 31, lg = tile_lgx(tw);
-    px = tile_x * tw + (w & ((1 << lg) - 1)) * 8 + (l & 7);
-    py = tile_y * th + (w >> lg) * 4 + (l >> 3);
-}
 
 // 8x8 block b of a tile with 8x4 blocks per row nbx = 1 << lg: its upper 8x4
 // block in the natural order (the lower one is that + nbx) and its offset in the tile.
@@ -126,23 +110,13 @@ __device__ __forceinline__ bool blend_alpha(float mx, float my, float ca, float 
     return !(alpha < 1.0f / 255.0f);
 }
 
-// Work counters (measurement builds of the kernels only): [0] pixel-primitive
-// evaluations, [1] tiles blended, [2] list entries staged.
-//
 // Each warp tests 32 staged entries at a time against its pixel block (one box
 // load per lane, a ballot), then walks only the survivors in list order.  An
 // entry culled here cannot reach alpha >= 1/255 at any of the warp's pixels, so
 // skipping it changes no pixel; a NaN box never culls.
-// Checkpoints of the clean blend: the state (T, C) of every pixel of a tile after
-// each kCkStride list entries, kept for the first `count` positions of the tile.
-constexpr int kCkStride = 64;
-constexpr int kCkMaxPerTile = 64;
-struct CkWrite {
-    float4* ck;      // NULL: no checkpoints
-    uint32_t off;    // first checkpoint of this tile
-    uint32_t count;  // checkpoints of this tile
-    uint32_t pix;    // pixels of a tile (one checkpoint holds one state per pixel)
-};
+// List entries per row of a tile: where each pixel's blend list stands is kept for
+// every kRowStride-th entry of the tile's list, up to its last stop.
+constexpr int kRowStride = 64;
 
 // Survivors a warp takes at a time: their alphas do not depend on the pixel
 // state, so they are computed as independent chains, then applied in list order.
@@ -181,25 +155,37 @@ __device__ __forceinline__ bool apply_entry(Pix& p, bool live, bool ok, float a,
     return stop_here;
 }
 
+// alpha of an entry at this lane's two pixels, which share a column (centres
+// (pxc, pyA) and (pxc, pyB), npy = (-pyA, -pyB)): the x offset and the exponent's
+// terms that depend on it alone (ca dx dx, -cb dx) are computed once for both,
+// the rest of gauss_power's order as packed fp32x2 operations over the two
+// pixels, so every pixel gets the bits of a one-pixel evaluation (blend_alpha).
+__device__ __forceinline__ float2 alpha_pair(const EntryQ& q, float pxc, float2 npy, bool& okA, bool& okB) {
+    const float dx = __fsub_rn(q.q0.x, pxc);
+    const float t1 = __fmul_rn(__fmul_rn(q.q0.z, dx), dx);
+    const float bdxn = __fmul_rn(-q.q0.w, dx);
+    const float2 dy = __fadd2_rn(make_float2(q.q0.y, q.q0.y), npy);   // my - py, one rounding each
+    const float2 sq = __ffma2_rn(__fmul2_rn(make_float2(q.cc, q.cc), dy), dy, make_float2(t1, t1));
+    const float2 pw = __ffma2_rn(make_float2(bdxn, bdxn), dy, __fmul2_rn(make_float2(-0.5f, -0.5f), sq));
+    const float2 pl = __fmul2_rn(pw, make_float2(kLog2e, kLog2e));
+    const float2 a = __fmul2_rn(make_float2(q.opac, q.opac), make_float2(ex2_approx(pl.x), ex2_approx(pl.y)));
+    okA = !(pw.x > 0.0f) && !(a.x < 1.0f / 255.0f);
+    okB = !(pw.y > 0.0f) && !(a.y < 1.0f / 255.0f);
+    return a;
+}
+
 // Walk the survivors m (bit i: entry c + i) in list order for this lane's two
-// pixels, which share a column (centres (pxc, pyA) and (pxc, pyB)): the x
-// offset and the exponent's terms that depend on it alone (ca dx dx, -cb dx) are
-// computed once for both, the rest of gauss_power's order as packed fp32x2
-// operations over the two pixels, so every pixel gets the bits of a one-pixel
-// evaluation of the same entries.
-// TRACK: record, per pixel, the list index (base + entry) where it stopped.
-// steps (measurement builds only): [0] entries walked by the warp, [1] of them
-// blended by at least one lane.
-template <bool COUNT, bool TRACK, class Fetch>
+// pixels: apply(entry index, live, ok flags, alphas, colour) takes them one by
+// one, kAlphaGroup at a time; after() follows each such group.
+template <class Fetch, class Apply, class After>
 __device__ __forceinline__ void walk_survivors2(unsigned m, int c, const Fetch& fetch, float pxc, float pyA,
-                                                float pyB, Pix& pA, Pix& pB, unsigned int& nev, uint32_t base,
-                                                unsigned* steps) {
-    if (COUNT && steps) steps[0] += __popc(m);
+                                                float pyB, const Apply& apply, const After& after) {
     const float2 npy = make_float2(-pyA, -pyB);
     while (m) {
         int e[kAlphaGroup];
         bool v[kAlphaGroup], okA[kAlphaGroup], okB[kAlphaGroup];
-        float aA[kAlphaGroup], aB[kAlphaGroup], cr[kAlphaGroup], cg[kAlphaGroup], cb[kAlphaGroup];
+        float2 a[kAlphaGroup];
+        float cr[kAlphaGroup], cg[kAlphaGroup], cb[kAlphaGroup];
 #pragma unroll
         for (int k = 0; k < kAlphaGroup; k++) {
             v[k] = m != 0u;
@@ -209,37 +195,15 @@ __device__ __forceinline__ void walk_survivors2(unsigned m, int c, const Fetch& 
 #pragma unroll
         for (int k = 0; k < kAlphaGroup; k++) {
             const EntryQ q = fetch(e[k]);
-            const float dx = __fsub_rn(q.q0.x, pxc);
-            const float t1 = __fmul_rn(__fmul_rn(q.q0.z, dx), dx);
-            const float bdxn = __fmul_rn(-q.q0.w, dx);
-            const float2 dy = __fadd2_rn(make_float2(q.q0.y, q.q0.y), npy);   // my - py, one rounding each
-            const float2 sq = __ffma2_rn(__fmul2_rn(make_float2(q.cc, q.cc), dy), dy, make_float2(t1, t1));
-            const float2 pw = __ffma2_rn(make_float2(bdxn, bdxn), dy, __fmul2_rn(make_float2(-0.5f, -0.5f), sq));
-            const float2 pl = __fmul2_rn(pw, make_float2(kLog2e, kLog2e));
-            const float2 a = __fmul2_rn(make_float2(q.opac, q.opac), make_float2(ex2_approx(pl.x), ex2_approx(pl.y)));
-            aA[k] = a.x;
-            aB[k] = a.y;
-            okA[k] = !(pw.x > 0.0f) && !(a.x < 1.0f / 255.0f);
-            okB[k] = !(pw.y > 0.0f) && !(a.y < 1.0f / 255.0f);
+            a[k] = alpha_pair(q, pxc, npy, okA[k], okB[k]);
             cr[k] = q.r;
             cg[k] = q.g;
             cb[k] = q.b;
         }
         // apply in list order with selects (no divergent branch per entry)
 #pragma unroll
-        for (int k = 0; k < kAlphaGroup; k++) {
-            const bool liveA = v[k] && !pA.done, liveB = v[k] && !pB.done;
-            if (COUNT) {
-                nev += (liveA ? 1u : 0u) + (liveB ? 1u : 0u);
-                if (steps) steps[1] += __any_sync(0xffffffffu, (liveA && okA[k]) || (liveB && okB[k])) ? 1u : 0u;
-            }
-            const bool sA = apply_entry(pA, liveA, okA[k], aA[k], cr[k], cg[k], cb[k]);
-            const bool sB = apply_entry(pB, liveB, okB[k], aB[k], cr[k], cg[k], cb[k]);
-            if (TRACK) {
-                pA.stop = sA ? base + (uint32_t)e[k] : pA.stop;
-                pB.stop = sB ? base + (uint32_t)e[k] : pB.stop;
-            }
-        }
+        for (int k = 0; k < kAlphaGroup; k++) apply(e[k], v[k], okA[k], okB[k], a[k], cr[k], cg[k], cb[k]);
+        after();
     }
 }
 
@@ -276,9 +240,9 @@ __device__ __forceinline__ Pix2Geo pix2_geo(int tile_x, int tile_y, int tw, int 
 
 // Entries [c, c + 32) of a staged batch for one warp: cull 32 boxes against the
 // warp's 8x8 pixel block with one ballot, then walk the survivors in list order.
-template <bool COUNT, bool TRACK>
-__device__ __forceinline__ void blend_chunk2(const Stage& s, int c, int cnt, uint32_t base, const Pix2Geo& g, Pix& pA,
-                                             Pix& pB, unsigned int& nev) {
+template <class Apply, class After>
+__device__ __forceinline__ void blend_chunk2(const Stage& s, int c, int cnt, const Pix2Geo& g, const Apply& apply,
+                                             const After& after) {
     const int lane = threadIdx.x & 31;
     const int j = c + lane;
     bool pass = false;
@@ -291,25 +255,7 @@ __device__ __forceinline__ void blend_chunk2(const Stage& s, int c, int cnt, uin
         const float4 q1 = s.q1[e];
         return EntryQ{s.q0[e], q1.x, q1.y, q1.z, q1.w, s.qb[e]};
     };
-    walk_survivors2<COUNT, TRACK>(m, c, fetch, g.pxc, g.pycA, g.pycB, pA, pB, nev, base, nullptr);
-}
-
-template <bool COUNT, bool TRACK>
-__device__ __forceinline__ void blend_batch2(const Stage& s, int cnt, uint32_t base, const Pix2Geo& g, Pix& pA,
-                                             Pix& pB, unsigned int& nev, const CkWrite& ckw) {
-    for (int c = 0; c < cnt; c += 32) {
-        if (__all_sync(0xffffffffu, pA.done && pB.done)) return;
-        if (ckw.ck && base + (uint32_t)c > 0 && ((base + (uint32_t)c) % kCkStride) == 0) {
-            // the state after entries [0, base + c) of the list
-            const uint32_t j = (base + (uint32_t)c) / kCkStride;
-            if (j <= ckw.count) {
-                float4* row = ckw.ck + (size_t)(ckw.off + j - 1) * ckw.pix;
-                row[g.u0] = make_float4(pA.T, pA.c0, pA.c1, pA.c2);
-                row[g.u1] = make_float4(pB.T, pB.c0, pB.c1, pB.c2);
-            }
-        }
-        blend_chunk2<COUNT, TRACK>(s, c, cnt, base, g, pA, pB, nev);
-    }
+    walk_survivors2(m, c, fetch, g.pxc, g.pycA, g.pycB, apply, after);
 }
 
 __device__ __forceinline__ float clamp01(float v) { return v > 0.0f ? (v < 1.0f ? v : 1.0f) : 0.0f; }
@@ -388,78 +334,326 @@ __device__ __forceinline__ void compare_tile2(const Pix2Geo& g, float a0, float 
     }
 }
 
-// MODE 0: write the image; 1: compare with the clean image; 2: write the image
-// and each pixel's stop index (0xffffffff if it never stopped), which the
-// dirty-tile kernel uses to leave pixels that stopped before a change untouched.
+// MODE 0: write the image; 1: compare with the clean image.
 // One block of tw * th / 2 threads per tw x th tile: warp b blends the tile's
-// 8x8 block b, two pixels per lane (the dirty-tile kernel's walk).
+// 8x8 block b, two pixels per lane.
 template <int MODE, bool COUNT>
 __global__ __launch_bounds__(kBT / 2) void k_blend_full(const BlendRec* __restrict__ recs,
                                                        const uint32_t* __restrict__ ids,
                                                        const uint2* __restrict__ ranges, int W, int H, int tiles_x,
                                                        int tw, int th, float* __restrict__ img,
                                                        const float* __restrict__ clean, CmpAcc* acc,
-                                                       unsigned long long* work, uint32_t* __restrict__ stop,
-                                                       uint32_t* __restrict__ tile_stop, float4* __restrict__ ck,
-                                                       const uint32_t* __restrict__ ck_off,
-                                                       const uint32_t* __restrict__ ck_cnt,
-                                                       unsigned int* __restrict__ clean_nonfin) {
+                                                       unsigned long long* work) {
     __shared__ Stage s;
     const int tile = blockIdx.x;
     const uint32_t P = (uint32_t)(tw * th);   // pixels of a tile = records staged per batch
-    const CkWrite ckw{ck, ck ? ck_off[tile] : 0u, ck ? ck_cnt[tile] : 0u, P};
     const Pix2Geo g = pix2_geo(tile % tiles_x, tile / tiles_x, tw, th, W, H);
-    Pix pA{1.0f, 0.0f, 0.0f, 0.0f, !g.inA, 0xffffffffu}, pB{1.0f, 0.0f, 0.0f, 0.0f, !g.inB, 0xffffffffu};
+    Pix pA{1.0f, 0.0f, 0.0f, 0.0f, !g.inA}, pB{1.0f, 0.0f, 0.0f, 0.0f, !g.inB};
     const uint2 rg = ranges[tile];
     unsigned int nev = 0, staged = 0;
+    auto apply = [&](int, bool v, bool okA, bool okB, float2 a, float cr, float cg, float cb) {
+        const bool liveA = v && !pA.done, liveB = v && !pB.done;
+        if (COUNT) nev += (liveA ? 1u : 0u) + (liveB ? 1u : 0u);
+        apply_entry(pA, liveA, okA, a.x, cr, cg, cb);
+        apply_entry(pB, liveB, okB, a.y, cr, cg, cb);
+    };
     for (uint32_t base = rg.x; base < rg.y; base += P) {
         const int cnt = (int)min(P, rg.y - base);
         for (int j = threadIdx.x; j < cnt; j += blockDim.x) stage_put(s, j, load_rec(recs, ids[base + j]));
         __syncthreads();
         staged += cnt;
-        blend_batch2<COUNT, MODE == 2>(s, cnt, base - rg.x, g, pA, pB, nev, ckw);
+        for (int c = 0; c < cnt && !__all_sync(0xffffffffu, pA.done && pB.done); c += 32)
+            blend_chunk2(s, c, cnt, g, apply, [] {});
         // also the barrier that lets the next batch overwrite the stage
         if (__syncthreads_count(pA.done && pB.done) == (int)blockDim.x) break;
     }
     if (COUNT) add_work(work, nev, staged);
     const float a0 = __fadd_rn(pA.c0, pA.T), a1 = __fadd_rn(pA.c1, pA.T), a2 = __fadd_rn(pA.c2, pA.T);   // over white
     const float b0 = __fadd_rn(pB.c0, pB.T), b1 = __fadd_rn(pB.c1, pB.T), b2 = __fadd_rn(pB.c2, pB.T);
-    if (MODE != 1) {
+    if (MODE == 0) {
         if (g.inA) {
             const size_t px = (size_t)g.pyA * W + g.px;
             img[px * 3] = a0;
             img[px * 3 + 1] = a1;
             img[px * 3 + 2] = a2;
-            if (MODE == 2) stop[px] = pA.stop;
         }
         if (g.inB) {
             const size_t px = (size_t)g.pyB * W + g.px;
             img[px * 3] = b0;
             img[px * 3 + 1] = b1;
             img[px * 3 + 2] = b2;
-            if (MODE == 2) stop[px] = pB.stop;
-        }
-        if (MODE == 2 && clean_nonfin) {
-            const int bad = (g.inA && !(isfinite(a0) && isfinite(a1) && isfinite(a2)) ? 1 : 0) +
-                            (g.inB && !(isfinite(b0) && isfinite(b1) && isfinite(b2)) ? 1 : 0);
-            const unsigned wb = __reduce_add_sync(0xffffffffu, (unsigned)bad);
-            if ((threadIdx.x & 31) == 0 && wb) atomicAdd(clean_nonfin, wb);
-        }
-        if (MODE == 2) {
-            // the tile's largest stop index: a change at or after it leaves every pixel as it is
-            __shared__ uint32_t wmax[kBT / 32];
-            const uint32_t m = __reduce_max_sync(0xffffffffu, max(g.inA ? pA.stop : 0u, g.inB ? pB.stop : 0u));
-            if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                uint32_t t = 0;
-                for (int w = 0; w < (int)(blockDim.x >> 5); w++) t = max(t, wmax[w]);
-                tile_stop[tile] = t;
-            }
         }
     } else {
         compare_tile2(g, a0, a1, a2, b0, b1, b2, clean, W, acc);
     }
+}
+
+// ---------------------------------------------------------------------------
+// Clean views: the blend of k_blend_full, and what the dirty-tile engine keeps
+// of it.  Two passes of the same blend:
+//   FILL = false: the image, the rank of the entry that stopped each pixel
+//     (0xffffffff if none), each tile's largest stop and the length of each
+//     pixel's blend list;
+//   FILL = true: the pixels' blend lists, the blend's state in front of every
+//     kWalk-th of their entries, and the rows that say where each list stands at
+//     every kRowStride-th entry of the tile's list.
+//
+// A pixel's blend list holds the entries its blend takes (power <= 0 and alpha >=
+// 1/255), front to back, as (capped alpha, colour) and rank in the view's order.
+// Only the flipped primitive's entry differs between a variant and the clean
+// scene, so a dirty pixel is re-blended from its list: no exponent, and no entry
+// that the pixel skips (2M primitives at 1600x1040 leave 20-35 entries a pixel of
+// tile lists of 1,885).  The list goes on past the clean stop, because a variant
+// that lacks an entry stops later: it ends where the product of (1 - alpha) over
+// its entries has fallen below kListEndT.  A variant lacks at most one entry,
+// whose alpha is at most 0.99, so its own T there is below 100 kListEndT (1 +
+// rounding) < 1e-4: it has stopped.  (A NaN alpha makes the product NaN, which
+// ends no list; a NaN corrupted alpha makes every channel NaN for good, wherever
+// the walk ends.)  The end is marked by an alpha so large that T (1 - alpha) <
+// 1e-4 for any T, kListEnd at rank 0xffffffff; a list cut at `cap` entries (views
+// whose lists would not fit) is marked by kListCut at the rank from which the
+// tile's list has to be read.
+// ---------------------------------------------------------------------------
+constexpr float kListEndT = 0.9e-6f;
+constexpr float kListEnd = 1e30f, kListCut = 2e30f;
+
+struct CleanPix {
+    float T, c0, c1, c2;   // the clean blend (frozen where it stopped)
+    float Tv;              // product of (1 - alpha) over every entry taken, stopped or not
+    bool stopped, done;    // done: the list ends here
+    uint32_t stop, last;   // rank and list position of the entry that stopped it
+    uint32_t n;            // entries taken
+    uint32_t off, flushed; // FILL: start of the list, entries written out
+};
+
+struct ListOut {
+    float4* ent;
+    uint32_t* rk;
+    const uint32_t* off;   // [tiles * pixels of a tile] start of each pixel's list
+    uint32_t cap;          // most entries kept per pixel
+    float4* state;
+    uint32_t* row_idx;
+    const uint32_t* row_off;
+    const uint32_t* row_cnt;
+};
+
+// Entries of a pixel on their way to its list: a lane takes an entry here and
+// there, so writing each by itself would cost two partial stores per entry (0.72
+// ms per pass of a 1600x1040 view of 300k primitives, 0.44 ms this way); four at a
+// time they leave as whole 64-byte pieces.  Ring of 8 per pixel: a walk group adds at most
+// kAlphaGroup.
+struct ListRing {
+    float4 e[8][64];    // [entry % 8][pixel of the 8x8 block]
+    uint32_t r[8][64];
+};
+
+// two entries to a 32-byte aligned place, one 256-bit store
+__device__ __forceinline__ void store_pair(float4* p, const float4& a, const float4& b) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(a.x), "f"(a.y), "f"(a.z),
+                 "f"(a.w), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w)
+                 : "memory");
+}
+
+// four entries [p.flushed, p.flushed + 4) of ring column `col` to the list
+__device__ __forceinline__ void flush4(CleanPix& p, const ListRing& ring, int col, const ListOut& lo) {
+    const int k = (int)(p.flushed & 4u);
+    const size_t at = (size_t)p.off + p.flushed;
+    store_pair(lo.ent + at, ring.e[k][col], ring.e[k + 1][col]);
+    store_pair(lo.ent + at + 2, ring.e[k + 2][col], ring.e[k + 3][col]);
+    *reinterpret_cast<uint4*>(lo.rk + at) =
+        make_uint4(ring.r[k][col], ring.r[k + 1][col], ring.r[k + 2][col], ring.r[k + 3][col]);
+    p.flushed += 4u;
+}
+
+template <bool FILL>
+__device__ __forceinline__ void clean_entry(CleanPix& p, bool live, bool ok, float a, float cr, float cg, float cb,
+                                            uint32_t rank, uint32_t li, const ListOut& lo, ListRing* ring, int col) {
+    const bool act = live && ok;
+    const float al = a > 0.99f ? 0.99f : a;   // keeps NaN
+    const float Tn = __fmul_rn(p.Tv, __fsub_rn(1.0f, al));
+    const bool run = act && !p.stopped;       // then Tv is the blend's T
+    const bool upd = run && !(Tn < 1e-4f);
+    const float w = __fmul_rn(al, p.Tv);
+    const float4 before = make_float4(p.T, p.c0, p.c1, p.c2);
+    p.c0 = upd ? __fmaf_rn(cr, w, p.c0) : p.c0;
+    p.c1 = upd ? __fmaf_rn(cg, w, p.c1) : p.c1;
+    p.c2 = upd ? __fmaf_rn(cb, w, p.c2) : p.c2;
+    p.T = upd ? Tn : p.T;
+    if (!FILL) {
+        p.stop = (run && !upd) ? rank : p.stop;
+        p.last = (run && !upd) ? li : p.last;
+    }
+    p.stopped = p.stopped || (run && !upd);
+    p.Tv = act ? Tn : p.Tv;
+    if (FILL && act && p.n <= lo.cap) {
+        const bool cut = p.n == lo.cap;
+        ring->e[p.n & 7u][col] = cut ? make_float4(kListCut, 0.0f, 0.0f, 0.0f) : make_float4(al, cr, cg, cb);
+        ring->r[p.n & 7u][col] = rank;
+    }
+    if (FILL && act && p.n <= lo.cap && (p.n & (kWalk - 1u)) == 0u)   // the state in front of this entry
+        lo.state[(p.off + p.n) / kWalk] = before;
+    p.n += act ? 1u : 0u;
+    p.done = p.done || (act && Tn < kListEndT);
+}
+
+template <bool FILL>
+__global__ __launch_bounds__(kBT / 2) void k_blend_clean(const BlendRec* __restrict__ recs,
+                                                        const uint32_t* __restrict__ ids,
+                                                        const uint32_t* __restrict__ rank,
+                                                        const uint2* __restrict__ ranges, int W, int H, int tiles_x,
+                                                        int tw, int th, float* __restrict__ img,
+                                                        uint32_t* __restrict__ stop, uint32_t* __restrict__ tile_stop,
+                                                        uint32_t* __restrict__ tile_last, uint32_t* __restrict__ counts,
+                                                        unsigned int* __restrict__ clean_nonfin, ListOut lo) {
+    extern __shared__ __align__(16) unsigned char ring_mem[];   // FILL: one ListRing per warp
+    __shared__ Stage s;
+    __shared__ uint32_t rk[kBT];   // ranks of the staged entries
+    const int tile = blockIdx.x, lane = threadIdx.x & 31;
+    ListRing* ring = FILL ? reinterpret_cast<ListRing*>(ring_mem) + (threadIdx.x >> 5) : nullptr;
+    const uint32_t P = (uint32_t)(tw * th);
+    const Pix2Geo g = pix2_geo(tile % tiles_x, tile / tiles_x, tw, th, W, H);
+    CleanPix pA{1.0f, 0.0f, 0.0f, 0.0f, 1.0f, !g.inA, !g.inA, 0xffffffffu, 0xffffffffu, 0u, 0u, 0u};
+    CleanPix pB{1.0f, 0.0f, 0.0f, 0.0f, 1.0f, !g.inB, !g.inB, 0xffffffffu, 0xffffffffu, 0u, 0u, 0u};
+    const uint2 rg = ranges[tile];
+    const uint32_t row0 = FILL ? lo.row_off[tile] : 0u, rows = FILL ? lo.row_cnt[tile] : 0u;
+    if (FILL) {
+        pA.off = lo.off[(size_t)tile * P + g.u0];
+        pB.off = lo.off[(size_t)tile * P + g.u1];
+    }
+    auto put_row = [&](uint32_t j) {   // after the first j kRowStride entries of the tile's list
+        const size_t r = (size_t)(row0 + j) * P;
+        lo.row_idx[r + g.u0] = pA.off + min(pA.n, lo.cap);
+        lo.row_idx[r + g.u1] = pB.off + min(pB.n, lo.cap);
+    };
+    if (FILL) put_row(0u);
+    uint32_t at = 0;   // list index of entry 0 of the staged batch
+    auto apply = [&](int e, bool v, bool okA, bool okB, float2 a, float cr, float cg, float cb) {
+        clean_entry<FILL>(pA, v && !pA.done, okA, a.x, cr, cg, cb, rk[e], at + (uint32_t)e, lo, ring, lane);
+        clean_entry<FILL>(pB, v && !pB.done, okB, a.y, cr, cg, cb, rk[e], at + (uint32_t)e, lo, ring, lane + 32);
+    };
+    // entries of the ring not yet written out (a cut list takes one past cap: its mark)
+    auto pending = [&](const CleanPix& p) { return (int)(min(p.n, lo.cap + 1u) - p.flushed); };
+    auto drain = [&]() {   // after each walk group: make room for the next
+        if (!FILL) return;
+        if (!__any_sync(0xffffffffu, max(pending(pA), pending(pB)) > 8 - kAlphaGroup)) return;
+        if (pending(pA) >= 4) flush4(pA, *ring, lane, lo);
+        if (pending(pB) >= 4) flush4(pB, *ring, lane + 32, lo);
+    };
+    for (uint32_t base = rg.x; base < rg.y; base += P) {
+        const int cnt = (int)min(P, rg.y - base);
+        for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
+            const uint32_t id = ids[base + j];
+            stage_put(s, j, load_rec(recs, id));
+            rk[j] = rank[id];
+        }
+        __syncthreads();
+        at = base - rg.x;
+        for (int c = 0; c < cnt && !__all_sync(0xffffffffu, pA.done && pB.done); c += 32) {
+            const uint32_t li = at + (uint32_t)c;
+            if (FILL && li > 0 && li % kRowStride == 0 && li / kRowStride <= rows) put_row(li / kRowStride);
+            blend_chunk2(s, c, cnt, g, apply, drain);
+        }
+        // also the barrier that lets the next batch overwrite the stage
+        if (__syncthreads_count(pA.done && pB.done) == (int)blockDim.x) break;
+    }
+    if (FILL) {
+        auto finish = [&](CleanPix& p, int col) {
+            if (p.n <= lo.cap) {
+                ring->e[p.n & 7u][col] = make_float4(kListEnd, 0.0f, 0.0f, 0.0f);
+                ring->r[p.n & 7u][col] = 0xffffffffu;
+                if ((p.n & (kWalk - 1u)) == 0u)   // a walk may resume at the mark itself
+                    lo.state[(p.off + p.n) / kWalk] = make_float4(p.T, p.c0, p.c1, p.c2);
+            }
+            // the list's space is a multiple of eight entries: whole pieces, up to the mark
+            while (p.flushed <= min(p.n, lo.cap)) flush4(p, *ring, col, lo);
+        };
+        finish(pA, lane);
+        finish(pB, lane + 32);
+        return;
+    }
+    const size_t t0 = (size_t)tile * P;
+    counts[t0 + g.u0] = pA.n;
+    counts[t0 + g.u1] = pB.n;
+    stop[t0 + g.u0] = pA.stop;
+    stop[t0 + g.u1] = pB.stop;
+    const float a0 = __fadd_rn(pA.c0, pA.T), a1 = __fadd_rn(pA.c1, pA.T), a2 = __fadd_rn(pA.c2, pA.T);   // over white
+    const float b0 = __fadd_rn(pB.c0, pB.T), b1 = __fadd_rn(pB.c1, pB.T), b2 = __fadd_rn(pB.c2, pB.T);
+    if (g.inA) {
+        const size_t px = (size_t)g.pyA * W + g.px;
+        img[px * 3] = a0;
+        img[px * 3 + 1] = a1;
+        img[px * 3 + 2] = a2;
+    }
+    if (g.inB) {
+        const size_t px = (size_t)g.pyB * W + g.px;
+        img[px * 3] = b0;
+        img[px * 3 + 1] = b1;
+        img[px * 3 + 2] = b2;
+    }
+    const unsigned bad = (g.inA && !(isfinite(a0) && isfinite(a1) && isfinite(a2)) ? 1u : 0u) +
+                         (g.inB && !(isfinite(b0) && isfinite(b1) && isfinite(b2)) ? 1u : 0u);
+    const unsigned wb = __reduce_add_sync(0xffffffffu, bad);
+    if ((threadIdx.x & 31) == 0 && wb) atomicAdd(clean_nonfin, wb);
+    // the tile's largest stop: a change at or after it leaves every pixel as it is
+    __shared__ uint32_t wmax[2][kBT / 32];
+    const uint32_t m = __reduce_max_sync(0xffffffffu, max(g.inA ? pA.stop : 0u, g.inB ? pB.stop : 0u));
+    const uint32_t ml = __reduce_max_sync(0xffffffffu, max(g.inA ? pA.last : 0u, g.inB ? pB.last : 0u));
+    if (lane == 0) {
+        wmax[0][threadIdx.x >> 5] = m;
+        wmax[1][threadIdx.x >> 5] = ml;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t t = 0, l = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); w++) {
+            t = max(t, wmax[0][w]);
+            l = max(l, wmax[1][w]);
+        }
+        tile_stop[tile] = t;
+        tile_last[tile] = l;
+    }
+}
+
+// The view's order: rank of every primitive, and the order's own keys (kept for
+// the corrupted entries' places).
+__global__ void k_ranks(const uint32_t* __restrict__ key, const uint32_t* __restrict__ id, uint64_t n,
+                        uint32_t* __restrict__ rank, uint32_t* __restrict__ sdk, uint32_t* __restrict__ sid) {
+    const uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    const uint32_t p = id[j];
+    rank[p] = (uint32_t)j;
+    sdk[j] = key[j];
+    sid[j] = p;
+}
+
+// Rows of each tile: row 0 and one every kRowStride list entries up to the tile's
+// last stop, at most kRowsPerTile.
+__global__ void k_row_counts(const uint2* __restrict__ ranges, const uint32_t* __restrict__ tile_last, int ntiles,
+                             uint32_t* __restrict__ row_cnt, uint32_t* __restrict__ rows) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= ntiles) return;
+    const uint32_t L = ranges[t].y - ranges[t].x;
+    const uint32_t last = L > 0 ? min(tile_last[t], L - 1u) : 0u;
+    const uint32_t c = min(last / (uint32_t)kRowStride, (uint32_t)kRowsPerTile);
+    row_cnt[t] = c;
+    rows[t] = c + 1u;
+}
+
+// Rank of the last entry before each row after row 0 (0xffffffff: no such row).
+__global__ void k_row_keys(const uint2* __restrict__ ranges, const uint32_t* __restrict__ ids,
+                           const uint32_t* __restrict__ rank, const uint32_t* __restrict__ row_cnt, int ntiles,
+                           uint32_t* __restrict__ row_key) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int t = i / kRowsPerTile, r = i % kRowsPerTile + 1;
+    if (t >= ntiles) return;
+    row_key[i] = (uint32_t)r <= row_cnt[t] ? rank[ids[ranges[t].x + (uint32_t)(r * kRowStride) - 1u]] : 0xffffffffu;
+}
+
+// Space of each pixel's blend list: its entries (at most cap) and the end mark,
+// in whole groups of kWalk.
+__global__ void k_list_lens(const uint32_t* __restrict__ counts, uint64_t n, uint32_t cap, uint32_t* __restrict__ lens) {
+    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) lens[i] = (min(counts[i], cap) + (uint32_t)kWalk) & ~(uint32_t)(kWalk - 1);
 }
 
 // Image pairs (blockIdx.y): a stream over both images, four pixels (three 16-byte
@@ -528,8 +722,11 @@ __global__ __launch_bounds__(kBT) void k_compare(const float* __restrict__ a, co
 
 // clean_nonfin (dirty engine only): per view, the clean image's non-finite
 // pixels, which count for every variant except where a pixel was re-blended.
-__global__ void k_finalize(const CmpAcc* acc, int count, gs_result* out, const unsigned int* clean_nonfin, int K) {
+// queue (dirty engine only): the batch's counters, cleared for the next one.
+__global__ void k_finalize(const CmpAcc* acc, int count, gs_result* out, const unsigned int* clean_nonfin, int K,
+                           unsigned int* queue) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (queue && i < 8) queue[i] = i == 6 ? queue[6] + 1u : 0u;   // [6]: batch generation (tags of the SSIM maps)
     if (i >= count) return;
     CmpAcc a = acc[i];
     gs_result r;
@@ -549,37 +746,6 @@ __global__ void k_zero_acc(CmpAcc* acc, int count) {
 // ---------------------------------------------------------------------------
 // dirty-tile persistent kernel
 // ---------------------------------------------------------------------------
-
-
-// First index in [lo, hi) whose (depth bits, id) is not below (dkey, p); the
-// lists are sorted by (depth, id).  Called by a whole warp: each round probes 31
-// splitters and keeps the 1/32 of the interval that holds the answer.
-__device__ __forceinline__ uint32_t warp_lower_bound(const uint32_t* __restrict__ dk, const uint32_t* __restrict__ ids,
-                                                     uint32_t lo, uint32_t hi, uint32_t dkey, uint32_t p) {
-    const int lane = threadIdx.x & 31;
-    while (hi - lo > 32) {
-        const uint32_t len = hi - lo;
-        bool less = false;
-        if (lane < 31) {
-            const uint32_t pos = lo + (uint32_t)(((uint64_t)len * (uint32_t)(lane + 1)) >> 5);
-            const uint32_t k = dk[pos], id = ids[pos];
-            less = k < dkey || (k == dkey && id < p);
-        }
-        const int c = __popc(__ballot_sync(0xffffffffu, less));
-        const uint32_t nlo = c == 0 ? lo : lo + (uint32_t)(((uint64_t)len * (uint32_t)c) >> 5) + 1;
-        const uint32_t nhi = c == 31 ? hi : lo + (uint32_t)(((uint64_t)len * (uint32_t)(c + 1)) >> 5);
-        lo = nlo;
-        hi = nhi;
-    }
-    bool less = false;
-    const uint32_t pos = lo + lane;
-    if (pos < hi) {
-        const uint32_t k = dk[pos], id = ids[pos];
-        less = k < dkey || (k == dkey && id < p);
-    }
-    return lo + __popc(__ballot_sync(0xffffffffu, less));
-}
-
 
 
 // A pixel of a dirty tile keeps its clean value, bit for bit, when its clean
@@ -626,120 +792,223 @@ __device__ __forceinline__ bool rect_reachable(float mx, float my, float ca, flo
     return !(qmin > 2.0f * L + 2.0e-5f * M);
 }
 
-__device__ __forceinline__ bool tile_reachable(const BlendRec& q, float x0, float x1, float y0, float y1) {
-    return rect_reachable(q.mx, q.my, q.ca, q.cb, q.cc, q.opac, x0, x1, y0, y1);
-}
-
-__device__ __forceinline__ bool affects(const BlendRec& q, float x, float y) {
-    float alpha;
-    return blend_alpha(q.mx, q.my, q.ca, q.cb, q.cc, q.opac, x, y, alpha);
-}
-
-// (variant, view) of a work item: the last bk with off[bk] <= item.
-__device__ __forceinline__ int item_owner(const uint32_t* off, int BK, uint32_t item) {
-    int lo = 0, hi = BK - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (off[mid] <= item) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
-// Tile of the j-th dirty tile of a (variant, view): the corrupted rect row-major,
-// then the tiles of the clean rect outside it, row-major.  The clean rect minus
-// the corrupted one is three bands: the rows above their overlap (full width),
-// the overlapping rows (minus the overlap's columns) and the rows below.
-__device__ __forceinline__ void item_tile(const DirtyDesc& d, uint32_t j, int& tx, int& ty) {
-    const uint32_t wn = (uint32_t)d.nx1 - d.nx0;
-    const uint32_t an = d.new_vis ? wn * ((uint32_t)d.ny1 - d.ny0) : 0u;
-    if (j < an) {
-        tx = d.nx0 + (int)(j % wn);
-        ty = d.ny0 + (int)(j / wn);
+// Tiles [t0, t1) of tile columns [c0, c1) whose pixel centres record q can reach
+// with alpha >= 1/255 somewhere in the rows of pixel centres [y0, y1]:
+// conservative, by the extent of the record's conic over the band.  The blend's
+// power is within g M of -q(d)/2, M = ((|ca| + |cb|) dx^2 + (|cc| + |cb|) dy^2)/2
+// and g = 1e-6 (several ulps), so with margins of 4e-5 on the diagonal the
+// candidates satisfy d^T Q'' d <= R, Q'' = [[ca - 4e-5 (|ca| + |cb|), cb], [cb, cc
+// - 4e-5 (|cc| + |cb|)]], R = 2 ln(255 opacity) + 2e-3 (the margin covers the
+// fast log and exp2).  At a fixed dy they lie between -cb dy / q_xx +- sqrt(q_xx R -
+// det dy^2) / q_xx, whatever the sign of the determinant: of an ellipse (det > 0)
+// the right end is concave in dy, with its maximum at dy* = -(cb / q_yy) sqrt(R
+// q_yy / det), and the left end mirrors it; with det <= 0 (needles, whose
+// determinant is lost in the margins) the right end is convex and the left one
+// concave, so the band's ends bound both.  The determinant is lowered by its own
+// rounding error (the region only grows); the rounding of the ends is covered by a
+// slack of one pixel, 2e-3 of the half width at dy = 0 (the root of a cancelling
+// difference) and 1e-4 of the largest half width.  No bound (all columns): opacity
+// NaN, a first diagonal term that the margin makes negative, or terms near overflow.
+__device__ __forceinline__ void band_tiles(const BlendRec& q, float y0, float y1, int c0, int c1, int tw, int& t0,
+                                           int& t1) {
+    t0 = c0;
+    t1 = c1;
+    const float L = __logf(255.0f * q.opac) + 1e-3f;
+    if (L < 0.0f) {   // alpha <= opacity < 1/255 everywhere (with margin); NaN falls through
+        t1 = c0;
         return;
     }
-    uint32_t r = j - an;
-    const uint32_t w0 = (uint32_t)d.ox1 - d.ox0;
-    const int lx = max((int)d.ox0, (int)d.nx0), hx = min((int)d.ox1, (int)d.nx1);
-    const int ly = max((int)d.oy0, (int)d.ny0), hy = min((int)d.oy1, (int)d.ny1);
-    if (d.new_vis && hx > lx && hy > ly) {
-        const uint32_t above = (uint32_t)(ly - d.oy0) * w0;
-        if (r >= above) {
-            r -= above;
-            const uint32_t wb = w0 - (uint32_t)(hx - lx), left = (uint32_t)(lx - d.ox0);
-            const uint32_t band = (uint32_t)(hy - ly) * wb;
-            if (r < band) {
-                const uint32_t q = r % wb;
-                ty = ly + (int)(r / wb);
-                tx = q < left ? d.ox0 + (int)q : hx + (int)(q - left);
-                return;
-            }
-            r -= band;
-            ty = hy + (int)(r / w0);
-            tx = d.ox0 + (int)(r % w0);
+    const float acb = fabsf(q.cb);
+    const float qxx = q.ca - 4e-5f * (fabsf(q.ca) + acb), qyy = q.cc - 4e-5f * (fabsf(q.cc) + acb);
+    const float pxy = qxx * qyy, pcb = q.cb * q.cb;
+    const float det = (pxy - pcb) - 4.8e-7f * (fabsf(pxy) + pcb);
+    if (!(qxx > 1e-30f) || !(fabsf(det) < 1e20f) || !(pcb < 1e20f) || !(L < 3.0e38f) || !(fabsf(q.mx) < 4e6f) ||
+        !(fabsf(q.my) < 4e6f))
+        return;
+    const float R = 2.0f * L + 2e-3f, rq = 1.0f / qxx, h0 = sqrtf(R * rq);
+    float da = q.my - y1, db = q.my - y0, dp0, dp1, dm0, dm1, hx;   // where the right / left end is furthest out
+    if (det > 0.0f && qyy > 1e-30f) {
+        const float rdet = R / det;
+        const float hy = sqrtf(rdet * qxx) * (1.0f + 1e-4f) + 1.0f;
+        hx = sqrtf(rdet * qyy);
+        if (!(hy < 1e12f) || !(hx < 1e12f)) return;
+        da = fmaxf(da, -hy);
+        db = fminf(db, hy);
+        if (da > db) {   // the band misses the ellipse
+            t1 = c0;
             return;
         }
+        const float dys = -q.cb / qyy * hx;
+        dp0 = dp1 = fminf(fmaxf(dys, da), db);
+        dm0 = dm1 = fminf(fmaxf(-dys, da), db);
+    } else {
+        dp0 = dm0 = da;
+        dp1 = dm1 = db;
+        const float far = fmaxf(fabsf(da), fabsf(db));
+        hx = sqrtf(fmaxf(qxx * R - det * far * far, 0.0f)) * rq;
     }
-    ty = d.oy0 + (int)(r / w0);
-    tx = d.ox0 + (int)(r % w0);
+    auto half = [&](float dy) { return sqrtf(fmaxf(qxx * R - det * dy * dy, 0.0f)); };
+    const float xp = fmaxf(-q.cb * dp0 + half(dp0), -q.cb * dp1 + half(dp1)) * rq;
+    const float xm = fminf(-q.cb * dm0 - half(dm0), -q.cb * dm1 - half(dm1)) * rq;
+    const float slack = 1.0f + 2e-3f * h0 + 1e-4f * hx + 1e-5f * (fabsf(xp) + fabsf(xm));
+    const float inv = 1.0f / (float)tw;   // tile edges are powers of two: exact
+    const float f0 = floorf((q.mx - xp - slack) * inv), f1 = floorf((q.mx - xm + slack) * inv) + 1.0f;
+    if (!isfinite(f0) || !isfinite(f1)) return;
+    t0 = (int)fminf(fmaxf(f0, (float)c0), (float)c1);
+    t1 = (int)fminf(fmaxf(f1, (float)t0), (float)c1);
 }
 
-// Plan, first pass: one (variant, view, dirty tile) work item per thread.
-// Decodes the tile and drops it when every pixel's clean blend stopped before
-// the first changed list position (stop-key test, exact) or when neither
-// changed record can reach it (conservative tile test); the others are
-// appended to cand as (bk, tx | ty << 16), counted in counts[2].
-template <bool COUNT>
-__global__ __launch_bounds__(256) void k_plan_filter(const ViewPtrs* __restrict__ views,
-                                                    const DirtyDesc* __restrict__ desc,
-                                                    const uint32_t* __restrict__ item_off, int BK, int K,
-                                                    uint2* __restrict__ cand, unsigned int* __restrict__ counts,
-                                                    unsigned long long* work) {
-    const int lane = threadIdx.x & 31;
-    __shared__ uint32_t s_off[kMaxPairs + 1];   // item_off[0, BK], BK <= kMaxPairs
-    for (int i = threadIdx.x; i <= BK; i += blockDim.x) s_off[i] = item_off[i];
-    __syncthreads();
-    const uint32_t total = s_off[BK];
-    const uint32_t stride = gridDim.x * blockDim.x;
+// Plan: the candidate tiles of a batch.  Lane = tile row of a pair (the
+// injector's list): the columns that either record reaches in that row
+// (band_tiles), then the warp's 32 rows' tiles are taken 32 at a time.  A tile is
+// dropped when every pixel's clean blend stopped in front of both changed entries
+// (tile_stop, exact) or when neither record can reach any of its 8x8 blocks
+// (rect_reachable, conservative); the others become candidates with the blocks to
+// look at.
+// Issue-bound; the row step is what keeps it small: an exploded primitive's rect
+// spans the frame, but its ellipse crosses a few columns of each row (20,000 upsets
+// of a 2M-primitive scene, 4 views: 28.5M tiles by rects, 1.4M by rows; 0.16 ms,
+// and 0.82 ms where needles kept their whole rows).
+// counts[1] rows, [2] candidates, [3] SSIM plan slots.
+// BIN: also count the candidates of each tile (bins) and keep each one's place.
+template <bool COUNT, bool BIN>
+__global__ __launch_bounds__(256) void k_plan(const ViewPtrs* __restrict__ views, const DirtyDesc* __restrict__ desc,
+                                              const uint2* __restrict__ rows, uint2* __restrict__ cand,
+                                              uint32_t* __restrict__ cand_at, uint32_t* __restrict__ bins,
+                                              unsigned int* __restrict__ counts, unsigned long long* work,
+                                              SsimBufs sb) {
+    // tiles that some pixel's clean blend reached behind the change, waiting for the
+    // block tests: x = pair | 1 << 20 (corrupted record there) | 1 << 21 (clean record
+    // there) | view << 24, y = tile x | tile y << 16
+    __shared__ uint2 wait[256 / 32][64];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t nrows = counts[1], nwarps = (gridDim.x * blockDim.x) >> 5;
+    // rows a warp takes at a time: all lanes when there is enough work for every warp
+    const uint32_t per = min(32u, (nrows + nwarps - 1u) / nwarps);
     unsigned int drop_key = 0, drop_box = 0;
-    // warp-uniform trip count (the ballot below needs the whole warp)
-    for (uint32_t base = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < total; base += stride) {
-        const uint32_t item = base + (uint32_t)lane;
-        bool keep = false;
-        int bk = 0, tx = 0, ty = 0;
-        if (item < total) {
-            bk = item_owner(s_off, BK, item);
-            const DirtyDesc& d = desc[bk];
-            item_tile(d, item - s_off[bk], tx, ty);
-            const ViewPtrs& v = views[bk % K];
-            const int tile = ty * v.tiles_x + tx;
-            const bool has_old = d.old_vis && tx >= d.ox0 && tx < d.ox1 && ty >= d.oy0 && ty < d.oy1;
-            const bool has_new = d.new_vis && tx >= d.nx0 && tx < d.nx1 && ty >= d.ny0 && ty < d.ny1;
-            // every pixel of the tile stopped before the first changed list position
-            // (tile_stop < cut) exactly when the entry at tile_stop sorts below the
-            // keys of both changed entries
-            unsigned long long kmin = ~0ull;
-            if (has_old) kmin = ((unsigned long long)__float_as_uint(d.old_depth) << 32) | d.prim;
-            if (has_new) kmin = min(kmin, ((unsigned long long)__float_as_uint(d.rec.depth) << 32) | d.prim);
-            const bool stopped = v.stop_key[tile] < kmin;
-            if (!stopped) {
-                const float rx0 = (float)(tx * v.tile_w) + 0.5f, ry0 = (float)(ty * v.tile_h) + 0.5f;
-                const float rx1 = fminf((float)(tx * v.tile_w + v.tile_w - 1), (float)(v.W - 1)) + 0.5f;
-                const float ry1 = fminf((float)(ty * v.tile_h + v.tile_h - 1), (float)(v.H - 1)) + 0.5f;
-                keep = (has_new && tile_reachable(d.rec, rx0, rx1, ry0, ry1)) ||
-                       (has_old && tile_reachable(v.recs[d.prim], rx0, rx1, ry0, ry1));
+    int nwait = 0;
+    // the block tests of the first (at most 32) waiting tiles, one per lane
+    auto test_blocks = [&](int n) {
+        uint32_t blocks = 0u, bin = 0u, tile = 0u;
+        const uint2 w = lane < n ? wait[warp][lane] : make_uint2(0u, 0u);
+        if (lane < n) {
+            const DirtyDesc& d = desc[w.x & kCandPair];
+            const ViewPtrs& v = views[w.x >> 24];
+            const bool has_new = (w.x >> 20) & 1u, has_old = (w.x >> 21) & 1u;
+            const int tx = (int)(w.y & 0xffffu), ty = (int)(w.y >> 16);
+            tile = (uint32_t)ty * (uint32_t)v.tiles_x + (uint32_t)tx;
+            bin = v.bin0 + tile;
+            const int lg = tile_lgx(v.tile_w), nb = (v.tile_w * v.tile_h) >> 6;
+            for (int b = 0; b < nb; b++) {
+                const int bx = tx * v.tile_w + block_x0(b, lg), by = ty * v.tile_h + block_y0(b, lg);
+                const float x0 = (float)bx + 0.5f, x1 = fminf((float)(bx + 7), (float)(v.W - 1)) + 0.5f;
+                const float y0 = (float)by + 0.5f, y1 = fminf((float)(by + 7), (float)(v.H - 1)) + 0.5f;
+                if (bx >= v.W || by >= v.H) continue;
+                const bool r = (has_new && rect_reachable(d.rec.mx, d.rec.my, d.rec.ca, d.rec.cb, d.rec.cc,
+                                                          d.rec.opac, x0, x1, y0, y1)) ||
+                               (has_old && rect_reachable(d.old.mx, d.old.my, d.old.ca, d.old.cb, d.old.cc,
+                                                          d.old.opac, x0, x1, y0, y1));
+                blocks |= r ? 1u << b : 0u;
             }
-            if (COUNT && !keep) (stopped ? drop_key : drop_box)++;
+            if (COUNT && !blocks) drop_box++;
+            if (COUNT && blocks) atomicAdd(&work[1], 1ull);
         }
-        const unsigned m = __ballot_sync(0xffffffffu, keep);
-        if (m) {
-            uint32_t b0 = 0;
-            if (lane == 0) b0 = atomicAdd(&counts[2], (unsigned)__popc(m));
-            b0 = __shfl_sync(0xffffffffu, b0, 0);
-            if (keep)
-                cand[b0 + __popc(m & ((1u << lane) - 1u))] =
-                    make_uint2((uint32_t)bk, (uint32_t)tx | ((uint32_t)ty << 16));
+        const unsigned m = __ballot_sync(0xffffffffu, blocks != 0u);
+        if (!m) return;
+        uint32_t c0 = 0, s0 = 0;
+        if (lane == 0) {
+            c0 = atomicAdd(&counts[2], (unsigned)__popc(m));
+            if (sb.plan) s0 = atomicAdd(&counts[3], (unsigned)__popc(m));
+        }
+        c0 = __shfl_sync(0xffffffffu, c0, 0) + __popc(m & ((1u << lane) - 1u));
+        s0 = __shfl_sync(0xffffffffu, s0, 0) + __popc(m & ((1u << lane) - 1u));
+        if (!blocks) return;
+        const uint32_t bk = w.x & kCandPair;
+        cand[c0] = make_uint2(bk | (blocks << 20) | (w.x & 0xff000000u), w.y);
+        if (BIN) cand_at[c0] = atomicAdd(&bins[bin], 1u);
+        if (sb.plan) {   // dirty-tile SSIM: tile -> slot of this batch, nothing re-blended yet
+            if (s0 < sb.slot_cap) {
+                const uint4 none = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
+                uint4* sg = reinterpret_cast<uint4*>(sb.slot_group + (size_t)s0 * 8);
+                sg[0] = none;
+                sg[1] = none;
+                uint4* item = reinterpret_cast<uint4*>(&sb.plan[s0]);
+                item[0] = make_uint4(0u, 0u, 0u, 0u);
+                item[1] = make_uint4(0u, 0u, 0u, 0u);
+                item[2] = make_uint4(bk, tile, 0u, 0u);
+                sb.slot_flags[s0] = 0u;
+                sb.tile_map[(size_t)bk * sb.max_tiles + tile] = ((unsigned long long)counts[6] << 32) | s0;
+            } else {
+                atomicOr(sb.overflow, 1u);
+            }
+        }
+    };
+    for (uint32_t base = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per; base < nrows; base += nwarps * per) {
+        const bool have = (uint32_t)lane < per && base + (uint32_t)lane < nrows;
+        uint2 row = make_uint2(0u, 0u);
+        int n0 = 0, n1 = 0, o0 = 0, o1 = 0;   // columns either record reaches
+        if (have) {
+            row = rows[base + (uint32_t)lane];
+            const DirtyDesc& d = desc[row.x];
+            const ViewPtrs& v = views[row.y >> 16];
+            const int ty = (int)(row.y & 0xffffu), th = v.tile_h, tw = v.tile_w;
+            const float y0 = (float)(ty * th) + 0.5f, y1 = fminf((float)(ty * th + th - 1), (float)(v.H - 1)) + 0.5f;
+            const bool rn = ty >= d.ny0 && ty < d.ny1, ro = ty >= d.oy0 && ty < d.oy1;
+            if (rn) band_tiles(d.rec, y0, y1, d.nx0, d.nx1, tw, n0, n1);
+            if (ro) band_tiles(d.old, y0, y1, d.ox0, d.ox1, tw, o0, o1);
+            if (COUNT)
+                drop_box += (unsigned)(Union1(rn ? d.nx0 : 0, rn ? d.nx1 : 0, ro ? d.ox0 : 0, ro ? d.ox1 : 0).len -
+                                       Union1(n0, n1, o0, o1).len);
+        }
+        const uint32_t cnt = (uint32_t)Union1(n0, n1, o0, o1).len;
+        uint32_t incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const uint32_t excl = incl - cnt, total = __shfl_sync(0xffffffffu, incl, 31);
+        for (uint32_t q0 = 0; q0 < total; q0 += 32) {
+            const uint32_t q = q0 + (uint32_t)lane;
+            int s = 0;   // the row this tile belongs to: the last lane whose offset is <= q
+#pragma unroll
+            for (int step = 16; step > 0; step >>= 1) {
+                const int m = s + step;
+                if (__shfl_sync(0xffffffffu, excl, m) <= q) s = m;
+            }
+            const int j = (int)(q - __shfl_sync(0xffffffffu, excl, s));
+            const uint32_t bk = __shfl_sync(0xffffffffu, row.x, s), yv = __shfl_sync(0xffffffffu, row.y, s);
+            const int a0 = __shfl_sync(0xffffffffu, n0, s), a1 = __shfl_sync(0xffffffffu, n1, s);
+            const int b0 = __shfl_sync(0xffffffffu, o0, s), b1 = __shfl_sync(0xffffffffu, o1, s);
+            bool keep = false;
+            uint2 w = make_uint2(0u, 0u);
+            if (q < total) {
+                const int tx = Union1(a0, a1, b0, b1).at(j), ty = (int)(yv & 0xffffu);
+                const DirtyDesc& d = desc[bk];
+                const ViewPtrs& v = views[yv >> 16];
+                const bool has_new = tx >= a0 && tx < a1, has_old = tx >= b0 && tx < b1;
+                const uint32_t cut = min(has_new ? d.new_rank : kNoRank, has_old ? d.old_rank : kNoRank);
+                keep = v.tile_stop[(uint32_t)ty * (uint32_t)v.tiles_x + (uint32_t)tx] >= cut;
+                w = make_uint2(bk | (has_new ? 1u << 20 : 0u) | (has_old ? 1u << 21 : 0u) | ((yv >> 16) << 24),
+                               (uint32_t)tx | ((uint32_t)ty << 16));
+                if (COUNT && !keep) drop_key++;
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, keep);
+            if (keep) wait[warp][nwait + __popc(m & ((1u << lane) - 1u))] = w;
+            nwait += __popc(m);
+            __syncwarp();
+            if (nwait >= 32) {
+                test_blocks(32);
+                __syncwarp();
+                const uint2 rest = wait[warp][32 + lane];
+                __syncwarp();
+                wait[warp][lane] = rest;
+                nwait -= 32;
+                __syncwarp();
+            }
         }
     }
+    if (nwait) test_blocks(nwait);
     if (COUNT) {
         const unsigned k = __reduce_add_sync(0xffffffffu, drop_key), x = __reduce_add_sync(0xffffffffu, drop_box);
         if (lane == 0 && (k + x)) {
@@ -750,455 +1019,485 @@ __global__ __launch_bounds__(256) void k_plan_filter(const ViewPtrs* __restrict_
     }
 }
 
-// Plan, second pass: one warp per candidate tile (grid-strided, so the
-// expensive tiles spread over all warps).  The exact per-pixel reach test, the
-// removal and insertion positions (warp searches) and the per-pixel stop test;
-// a tile with an active pixel is appended to the plan (counts[1]) with its
-// groups (counts[3] heavy, counts[4] light), any other keeps its clean values
-// (Delta = 0).
-constexpr int kHeavyWalk = 1024;   // list entries
-template <bool COUNT>
-__global__ __launch_bounds__(256, 4) void k_plan_exact(const ViewPtrs* __restrict__ views,
-                                                      const DirtyDesc* __restrict__ desc, int K,
-                                                      const uint2* __restrict__ cand, PlanItem* __restrict__ plan,
-                                                      uint32_t* __restrict__ groups, uint32_t gcap,
-                                                      unsigned int* __restrict__ counts, unsigned long long* work,
-                                                      SsimBufs sb) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+// Candidates by tile, so that the warps that run side by side re-blend the same
+// pixels for different variants and find their blend lists in the L2: the bins'
+// starts (each block scans 1024 bins and draws its place from counts[4]; the
+// order of the blocks does not matter) and the candidates' copy into them.
+__global__ __launch_bounds__(1024) void k_bin_starts(uint32_t* __restrict__ bins, uint32_t nbins,
+                                                    unsigned int* __restrict__ counts) {
+    __shared__ uint32_t wsum[32];
+    __shared__ uint32_t start;
+    const uint32_t i = blockIdx.x * 1024u + threadIdx.x;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t c = i < nbins ? bins[i] : 0u;
+    uint32_t x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[wid] = x;
+    __syncthreads();
+    if (wid == 0) {
+        uint32_t t = wsum[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, t, o);
+            if (lane >= o) t += y;
+        }
+        wsum[lane] = t;
+        if (lane == 31) start = t ? atomicAdd(&counts[4], t) : 0u;
+    }
+    __syncthreads();
+    if (i < nbins) bins[i] = start + x - c + (wid > 0 ? wsum[wid - 1] : 0u);
+}
+
+__global__ __launch_bounds__(256) void k_bin_cands(const ViewPtrs* __restrict__ views,
+                                                   const uint2* __restrict__ cand, const uint32_t* __restrict__ cand_at,
+                                                   const uint32_t* __restrict__ bins,
+                                                   const unsigned int* __restrict__ counts, uint2* __restrict__ out) {
     const uint32_t n = counts[2];
-    unsigned int drop_reach = 0, drop_stop = 0;
-    for (uint32_t i = warp; i < n; i += nwarps) {
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const uint2 c = cand[i];
-        const int ibk = (int)c.x, itx = (int)(c.y & 0xffffu), ity = (int)(c.y >> 16);
-        const DirtyDesc& d = desc[ibk];
-        const ViewPtrs& v = views[ibk % K];
-        const int tile = ity * v.tiles_x + itx;
-        const bool has_old = d.old_vis && itx >= d.ox0 && itx < d.ox1 && ity >= d.oy0 && ity < d.oy1;
-        const bool has_new = d.new_vis && itx >= d.nx0 && itx < d.nx1 && ity >= d.ny0 && ity < d.ny1;
-        const BlendRec nrec = d.rec;
-        const BlendRec orec = has_old ? v.recs[d.prim] : nrec;
-        const uint32_t prim = d.prim;
-        const int nw = (v.tile_w * v.tile_h) >> 5;   // 8x4 blocks of the tile
-        unsigned reach[kBT / 32];
-        bool any = false;
-#pragma unroll
-        for (int q = 0; q < kBT / 32; q++) {
-            int px, py;
-            pix_of(itx, ity, v.tile_w, v.tile_h, q * 32 + lane, px, py);
-            const float x = (float)px + 0.5f, y = (float)py + 0.5f;
-            const bool r = q < nw && px < v.W && py < v.H &&
-                           ((has_old && affects(orec, x, y)) || (has_new && affects(nrec, x, y)));
-            reach[q] = __ballot_sync(0xffffffffu, r);
-            any |= reach[q] != 0u;
-        }
-        uint32_t pp = 0, ins = 0, cut = 0xffffffffu;
-        uint2 rg = make_uint2(0u, 0u);
-        if (any) {
-            rg = v.ranges[tile];
-            if (has_old) {
-                pp = warp_lower_bound(v.dk, v.ids, rg.x, rg.y, __float_as_uint(orec.depth), prim) - rg.x;
-                cut = pp;
-            }
-            if (has_new) {
-                ins = warp_lower_bound(v.dk, v.ids, rg.x, rg.y, __float_as_uint(nrec.depth), prim) - rg.x;
-                cut = min(cut, ins);   // clean-list position of the insertion
-                if (has_old && pp < ins) ins -= 1;
-            }
-            // then the reached pixels whose clean blend had not stopped before the change
-            any = false;
-#pragma unroll
-            for (int q = 0; q < kBT / 32; q++) {
-                int px, py;
-                pix_of(itx, ity, v.tile_w, v.tile_h, q * 32 + lane, px, py);
-                bool a = false;
-                if ((reach[q] >> lane) & 1u) a = v.stop[(size_t)py * v.W + px] >= cut;
-                reach[q] = __ballot_sync(0xffffffffu, a);   // now: active pixels
-                any |= reach[q] != 0u;
-            }
-        }
-        if (!any) {   // every pixel keeps its clean value
-            if (COUNT) (cut == 0xffffffffu ? drop_reach : drop_stop)++;
-            continue;
-        }
-        // the item's 7 16-byte parts, one per lane; one group per 8x8 block with an
-        // active pixel, (slot << 3) | block.  Groups of tiles with a long walk
-        // ahead (from the checkpoint the blend resumes at) go to the front of the
-        // group array and are blended first, the others to the back.
-        const int lg = tile_lgx(v.tile_w), nb = nw >> 1;
-        uint32_t word = 0;
-#pragma unroll
-        for (int b = 0; b < kDirtyBlocks; b++) {
-            const int wa = block_upper(b, lg), wb = wa + (1 << lg);
-            uint32_t bw = 0;
-#pragma unroll
-            for (int q = 0; q < kBT / 32; q++) bw |= (q == wa || q == wb) ? reach[q] : 0u;
-            word = lane == b ? bw : word;
-        }
-        const unsigned gm = __ballot_sync(0xffffffffu, lane < nb && word != 0u);
-        const uint32_t Lm = (rg.y - rg.x) - (has_old ? 1u : 0u) + (has_new ? 1u : 0u);
-        const uint32_t walk = Lm - min(cut / (uint32_t)kCkStride, v.ck_cnt[tile]) * (uint32_t)kCkStride;
-        const bool heavy = walk >= (uint32_t)kHeavyWalk;
-        uint32_t slot = 0, gbase = 0;
-        if (lane == 0) {
-            slot = atomicAdd(&counts[1], 1u);
-            gbase = atomicAdd(&counts[heavy ? 3 : 4], (unsigned)__popc(gm));
-        }
-        slot = __shfl_sync(0xffffffffu, slot, 0);
-        gbase = __shfl_sync(0xffffffffu, gbase, 0);
-        if ((gm >> lane) & 1u) {
-            const uint32_t gi = gbase + __popc(gm & ((1u << lane) - 1u));
-            groups[heavy ? gi : gcap - 1u - gi] = (slot << 3) | (uint32_t)lane;
-        }
-        if (sb.tile_map) {   // dirty-tile SSIM: tile -> slot of this batch, no block delta yet
-            if (slot < sb.slot_cap) {
-                if (lane < kTilePix / 32) sb.slot_group[(size_t)slot * 8 + lane] = 0xffffffffu;
-                if (lane == 0) sb.slot_flags[slot] = 0u;
-                if (lane == 0)
-                    sb.tile_map[(size_t)ibk * sb.max_tiles + (size_t)tile] =
-                        ((unsigned long long)counts[6] << 32) | slot;
-            } else if (lane == 0) {
-                atomicOr(sb.overflow, 1u);
-            }
-        }
-        uint4* dst = reinterpret_cast<uint4*>(&plan[slot]);
-        if (lane < 3) {
-            dst[lane] = reinterpret_cast<const uint4*>(&d.rec)[lane];
-        } else if (lane == 3) {
-            dst[3] = make_uint4(reach[0], reach[1], reach[2], reach[3]);
-        } else if (lane == 4) {
-            dst[4] = make_uint4(reach[4], reach[5], reach[6], reach[7]);
-        } else if (lane == 5) {
-            dst[5] = make_uint4((uint32_t)ibk, (uint32_t)tile, rg.x, rg.y);
-        } else if (lane == 6) {
-            dst[6] = make_uint4(pp, ins, cut, (has_old ? 1u : 0u) | (has_new ? 2u : 0u));
-        }
-    }
-    if (COUNT && lane == 0 && (drop_reach + drop_stop)) {   // warp-uniform counts
-        atomicAdd(&work[3], (unsigned long long)(drop_reach + drop_stop));
-        atomicAdd(&work[6], (unsigned long long)drop_reach);
-        atomicAdd(&work[7], (unsigned long long)drop_stop);
+        const ViewPtrs& v = views[c.x >> 24];
+        const uint32_t tile = (c.y >> 16) * (uint32_t)v.tiles_x + (c.y & 0xffffu);
+        out[bins[v.bin0 + tile] + cand_at[i]] = c;
     }
 }
 
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    const unsigned saddr = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(saddr), "l"(gmem) : "memory");
-}
-
-// Dirty-tile blend, one warp per work unit: an 8x8 pixel block of a planned
-// tile that holds an active pixel (the plan's groups, (item << 3) | block), two
-// pixels per lane (one column, four rows apart, so the exponent's x terms are
-// shared).
-// The warp streams the tile's merged list -- the clean list with the old entry
-// removed and the corrupted record inserted -- through a ring of kWarpRing
-// chunks of 32 entries in shared memory, filled by cp.async gathers issued
-// kWarpRing - 1 chunks ahead, so the gathers overlap the blend.  Each chunk is
-// culled against the box of the block's pixels that are still blending (active
-// and not stopped; recomputed per chunk) with one ballot and the survivors are
-// walked in list order (the same arithmetic as the full-frame blend).  Active pixels resume from the clean blend's last checkpoint at or
-// before the first changed position; the result is compared with the clean
-// image on the fly.  Warps are independent: no block barrier.
-constexpr int kWarpRing = 2;
-constexpr int kDirtyWarps = 4;   // warps per block
-struct WarpRing {
-    float4 q[kWarpRing][3][32];   // [chunk slot][16-byte part of the record][entry]
+// One pixel's part of a unit's comparison, in words that add up without overflow
+// over the 256 pixels of a tile: the fixed-point squared error (< 2^41) in a low
+// part of 20 bits and a high one, the peak difference, and the footprint /
+// non-finite / clean-non-finite counts 10 bits apart.
+struct DirtySum {
+    uint32_t fx_lo, fx_hi, maxbits, counts;
+    bool foot;
 };
 
-// First index in [lo, hi) of the ascending array a whose value is not below key
-// (whole warp: each round probes 31 splitters and keeps 1/32 of the interval).
-__device__ __forceinline__ uint32_t warp_lower_bound_u32(const uint32_t* __restrict__ a, uint32_t lo, uint32_t hi,
-                                                         uint32_t key) {
-    const int lane = threadIdx.x & 31;
-    while (hi - lo > 32) {
-        const uint32_t len = hi - lo;
-        bool less = false;
-        if (lane < 31) less = a[lo + (uint32_t)(((uint64_t)len * (uint32_t)(lane + 1)) >> 5)] < key;
-        const int c = __popc(__ballot_sync(0xffffffffu, less));
-        const uint32_t nlo = c == 0 ? lo : lo + (uint32_t)(((uint64_t)len * (uint32_t)c) >> 5) + 1;
-        const uint32_t nhi = c == 31 ? hi : lo + (uint32_t)(((uint64_t)len * (uint32_t)(c + 1)) >> 5);
-        lo = nlo;
-        hi = nhi;
-    }
-    const uint32_t pos = lo + (uint32_t)lane;
-    const bool less = pos < hi && a[pos] < key;
-    return lo + __popc(__ballot_sync(0xffffffffu, less));
-}
-
-// Entry m of the merged list: the inserted record (returns true) or the clean
-// list entry ci (relative to the tile's range).
-__device__ __forceinline__ bool merged_entry(uint32_t m, bool has_old, bool has_new, uint32_t pp, uint32_t ins,
-                                             uint32_t& ci) {
-    if (has_new && m == ins) return true;
-    const uint32_t j = (has_new && m > ins) ? m - 1u : m;
-    ci = (has_old && j >= pp) ? j + 1u : j;
-    return false;
-}
-
-__device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait_group() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-// One pixel's part of a block's comparison: fixed-point squared error, peak
-// difference, footprint / non-finite / clean-non-finite flags and screen cell.
-struct BlockCmp {
-    unsigned long long fx = 0ull, cells = 0ull;
-    float m = 0.0f;
-    unsigned foot = 0u, bad = 0u, clean_bad = 0u;
-};
-
-__device__ __forceinline__ void block_cmp_add(BlockCmp& b, bool active, float v0, float v1, float v2, const float* c,
-                                              int px, int py, int W, int H) {
-    if (!active) return;
+__device__ __forceinline__ DirtySum dirty_sum(float v0, float v1, float v2, float k0, float k1, float k2) {
+    const float c[3] = {k0, k1, k2};
     const PixCmp r = pixel_compare(v0, v1, v2, c);
-    b.fx += r.fx;
-    b.m = fmaxf(b.m, r.m);
-    b.foot += r.foot ? 1u : 0u;
-    b.bad += r.nonfin ? 1u : 0u;
-    b.clean_bad += !(isfinite(c[0]) && isfinite(c[1]) && isfinite(c[2])) ? 1u : 0u;
-    if (r.foot) b.cells |= cell_bit(px, py, W, H);
+    DirtySum s;
+    s.fx_lo = (uint32_t)r.fx & 0xfffffu;
+    s.fx_hi = (uint32_t)(r.fx >> 20);
+    s.maxbits = __float_as_uint(r.m);   // r.m >= 0
+    s.foot = r.foot;
+    s.counts = (r.foot ? 1u : 0u) | (r.nonfin ? 1u << 10 : 0u) |
+               (!(isfinite(k0) && isfinite(k1) && isfinite(k2)) ? 1u << 20 : 0u);
+    return s;
 }
+
+// Two neighbouring entries of a blend list (32-byte aligned), one 256-bit load.
+__device__ __forceinline__ void load_pair(const float4* p, float4& a, float4& b) {
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+        : "l"(p));
+}
+
+// The state of one dirty pixel's walk.
+struct DirtyPix {
+    float T, c0, c1, c2;
+    // Takes an entry of capped alpha al; true when the walk ends there: the pixel
+    // stops before it (T would drop below 1e-4), an end mark, or T became NaN, after
+    // which every channel is NaN whatever follows (poison()).
+    __device__ __forceinline__ bool take(float al, float r, float g, float b) {
+        const float Tn = __fmul_rn(T, __fsub_rn(1.0f, al));
+        if (!(Tn >= 1e-4f)) return true;
+        const float w = __fmul_rn(al, T);
+        c0 = __fmaf_rn(r, w, c0);
+        c1 = __fmaf_rn(g, w, c1);
+        c2 = __fmaf_rn(b, w, c2);
+        T = Tn;
+        return false;
+    }
+    __device__ __forceinline__ void poison(float al) {   // al: the alpha that ended the walk
+        if (isnan(al)) T = c0 = c1 = c2 = NAN;
+    }
+};
+
+// Dirty-tile blend.  A block of kDirtyWarps warps takes up to kUnitVars consecutive
+// candidate tiles (in a large batch, mostly variants of a few tiles) in two steps.
+//
+// (1) Per candidate and 8x8 pixel block, by a warp: which pixels are active.  A
+// pixel keeps its clean value, bit for bit, when its clean blend stopped in front of
+// both changed entries, or when its blend skips the removed (clean) and the inserted
+// (corrupted) record (power > 0 or alpha < 1/255, by the blend's own arithmetic):
+// its state changes are then those of the clean blend.
+//
+// (2) The active (pixel, candidate) pairs, ordered by pixel, 32 at a time, one per
+// lane: the pair resumes from the clean blend's state kept at or in front of the
+// first change and walks the pixel's blend list from there -- without the removed
+// entry and with the corrupted one at its place -- by the same operations in the
+// same order as the full-frame blend, and compares the result with the clean pixel.
+//
+// Why by pixel: a lane's gather of its list costs one L1 lookup per load and list,
+// and pairs of one pixel of one tile read the same lines.  With one variant's
+// pixels over the lanes (32 lists per warp) the walk took 150 SM cycles per group of
+// 8 entries whatever the occupancy.  Why 16 candidates: a tile of a 2M-primitive
+// view holds three of a batch's, which would leave most of a block's warps idle.
+// Bound by issue and the gathers' latency together (43% of issue slots, 18% of the
+// DRAM rate at 24 warps per SM; 40 warps of 48 registers and 4 entries at a time
+// took it from 4.6 to 3.6 ms).  20,000 upsets of a 2M-primitive scene in four
+// 1600x1040 views: 3.55 ms, where the walk over block sublists with every alpha
+// evaluated took 6.0 ms.
+constexpr int kDirtyWarps = 8;   // warps per block
+constexpr int kDirtyThreads = kDirtyWarps * 32;
+static_assert(kDirtyThreads >= kTilePix, "a thread per pixel of the tile");
+struct __align__(16) DirtyVar {   // one candidate
+    const uint32_t* row_idx;      // the tile's row to resume from
+    const float* clean;           // the clean image's pixel at the tile's corner
+    const float4* ent;            // blend lists, their ranks and states
+    const uint32_t* rk;
+    const float4* state;
+    int W3;                       // floats per image row
+    uint32_t bk, ins, pp;         // pair; ranks of the changed entries
+    float r, g, b;                // the corrupted record's colour
+    uint32_t cx, cy, tile;        // the candidate
+    uint32_t fx_lo, fx_hi, maxbits, counts;   // sums over its pixels (see DirtySum)
+    uint32_t cells_lo, cells_hi, edge, pad;
+    uint32_t unit[kDirtyBlocks];              // SSIM: delta units of the blocks (0xffffffff: none)
+    unsigned long long mask[kDirtyBlocks];    // active pixels of each 8x8 block
+};
 
 template <bool COUNT>
-__global__ __launch_bounds__(kDirtyWarps * 32, 6) void k_dirty(const ViewPtrs* __restrict__ views, int K,
-                                                              const PlanItem* __restrict__ plan,
-                                                              const uint32_t* __restrict__ groups, uint32_t gcap,
-                                                              const unsigned int* __restrict__ counts,
-                                                              CmpAcc* __restrict__ acc,
-                                                              unsigned int* __restrict__ queue,
-                                                              unsigned long long* work, SsimBufs sb) {
-    __shared__ WarpRing rings[kDirtyWarps];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    WarpRing& R = rings[warp];
-    const uint32_t nheavy = counts[3], ngroups = counts[3] + counts[4];
-    // measurement builds: SM cycles each warp spends per phase (set-up of a group,
-    // the walk, the comparison and reductions)
+__global__ __launch_bounds__(kDirtyThreads, 5) void k_dirty(const ViewPtrs* __restrict__ views,
+                                                           const DirtyDesc* __restrict__ desc,
+                                                           const uint2* __restrict__ cand, int tw, int th,
+                                                           unsigned int* __restrict__ counts,
+                                                           uint32_t* __restrict__ bins, uint32_t nbins,
+                                                           CmpAcc* __restrict__ acc, bool regions,
+                                                           unsigned long long* work, SsimBufs sb) {
+    __shared__ DirtyVar var[kUnitVars];
+    __shared__ float alpha[kUnitVars][kTilePix];   // the corrupted entry's capped alpha at each pixel, -1: not taken
+    __shared__ uint16_t pairs[kUnitVars * kTilePix];   // candidate << 8 | 8x8 block << 6 | pixel of the block
+    __shared__ uint32_t wsum[kDirtyWarps];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int lg = tile_lgx(tw), nb = (tw * th) >> 6;
+    const uint32_t P = (uint32_t)(tw * th), ncand = counts[2];
+    // candidates a block takes at a time: all kUnitVars when there are enough for every block
+    const uint32_t per = min((uint32_t)kUnitVars, (ncand + gridDim.x - 1u) / gridDim.x);
+    // the bins are free again: clear them for the next batch
+    for (uint32_t i = blockIdx.x * kDirtyThreads + (uint32_t)tid; i < nbins; i += gridDim.x * kDirtyThreads) bins[i] = 0u;
+    // measurement builds: SM cycles each warp spends per phase (the activity of the
+    // candidates' pixels, the walk, the comparison and reductions)
     long long t_pro = 0, t_walk = 0, t_epi = 0;
-    while (true) {
-        long long c0 = COUNT ? clock64() : 0;
-        uint32_t gi = 0;
-        if (lane == 0) gi = atomicAdd(&queue[0], 1u);
-        gi = __shfl_sync(0xffffffffu, gi, 0);
-        if (gi >= ngroups) break;
-        // heavy groups first (front of the array), then the light ones (from the back)
-        const uint32_t code = groups[gi < nheavy ? gi : gcap - 1u - (gi - nheavy)];
-        const PlanItem* it = &plan[code >> 3];
-        const int b = (int)(code & 7u);            // 8x8 block of the tile
-        const uint4 f5 = reinterpret_cast<const uint4*>(it)[5];   // bk, tile, s, e
-        const uint4 f6 = reinterpret_cast<const uint4*>(it)[6];   // pp, ins, cut, flags
-        const int bk = (int)f5.x;
-        const uint32_t tile = f5.y, pp = f6.x, ins = f6.y, cut = f6.z;
-        const bool has_old = f6.w & 1u, has_new = f6.w & 2u;
-        const ViewPtrs& v = views[bk % K];
-        const int tw = v.tile_w, th = v.tile_h, lg = tile_lgx(tw), nb = (tw * th) >> 6;
-        const int wA = block_upper(b, lg), wB = wA + (1 << lg);   // the block's upper and lower 8x4 halves
-        const uint32_t amA = it->mask[wA], amB = it->mask[wB];
-        const int tx = (int)(tile % (uint32_t)v.tiles_x), ty = (int)(tile / (uint32_t)v.tiles_x);
-        // lane: pixel A of the upper half, pixel B four rows below it
-        const int px = tx * tw + block_x0(b, lg) + (lane & 7);
-        const int pyA = ty * th + block_y0(b, lg) + (lane >> 3);
-        const int pyB = pyA + 4;
-        const bool inA = (amA >> lane) & 1u, inB = (amB >> lane) & 1u;   // decided by the plan (inside the image)
-        const bool act = inA || inB;
-        PixGeo g;   // the box of the block's active pixel centres
-        g.wx0 = (float)__reduce_min_sync(0xffffffffu, act ? px : 0x7fffffff) + 0.5f;
-        g.wx1 = (float)__reduce_max_sync(0xffffffffu, act ? px : -1) + 0.5f;
-        g.wy0 = (float)__reduce_min_sync(0xffffffffu, inA ? pyA : (inB ? pyB : 0x7fffffff)) + 0.5f;
-        g.wy1 = (float)__reduce_max_sync(0xffffffffu, inB ? pyB : (inA ? pyA : -1)) + 0.5f;
-        // this lane's pixels: A in the upper half, B four rows below it
-        const int x0 = px, y0 = pyA, u0 = wA * 32 + lane, y1 = pyB, u1 = wB * 32 + lane;
-        const bool actA = inA, actB = inB;
-        const float pxc = (float)x0 + 0.5f, pycA = (float)y0 + 0.5f, pycB = (float)y1 + 0.5f;
-        Pix pA{1.0f, 0.0f, 0.0f, 0.0f, !actA, 0u}, pB{1.0f, 0.0f, 0.0f, 0.0f, !actB, 0u};
-        // The merged list equals the clean list before `cut`, so an active pixel
-        // (not stopped before `cut`) can resume from the clean blend's state at the
-        // last checkpoint at or before `cut`.
-        const uint32_t cstar = min(cut / (uint32_t)kCkStride, v.ck_cnt[tile]);
-        const uint32_t start = cstar * (uint32_t)kCkStride;
-        if (cstar > 0) {
-            const float4* ckt = v.ck + (size_t)(v.ck_off[tile] + cstar - 1) * (uint32_t)(tw * th);
-            if (actA) {
-                const float4 st = ckt[u0];
-                pA.T = st.x;
-                pA.c0 = st.y;
-                pA.c1 = st.z;
-                pA.c2 = st.w;
-            }
-            if (actB) {
-                const float4 st = ckt[u1];
-                pB.T = st.x;
-                pB.c0 = st.y;
-                pB.c1 = st.z;
-                pB.c2 = st.w;
-            }
-        }
-        // This block's sublist of the clean list (the entries whose box meets the
-        // block, positions ascending) from `start`, without the old entry and with the
-        // corrupted record at its place: every entry outside the sublist fails the
-        // cull below anyway.
-        const uint32_t boff = v.bl_off[(size_t)tile * nb + b];
-        const uint32_t blen = v.bl_off[(size_t)tile * nb + b + 1] - boff;
-        const uint32_t* B = v.bl_pos + boff;
-        const uint32_t k0 = warp_lower_bound_u32(B, 0, blen, start);
-        bool has_kpp = false;
-        uint32_t kpp = 0, lins = 0;
-        if (has_old) {
-            kpp = warp_lower_bound_u32(B, 0, blen, pp);
-            has_kpp = kpp < blen && B[kpp] == pp;
-        }
-        if (has_new) {
-            // clean-list position before which the corrupted record goes (ins counts
-            // the list without the old entry; at ins == pp both readings coincide)
-            const uint32_t ins_c = (has_old && ins >= pp) ? ins + 1u : ins;
-            const uint32_t tins = warp_lower_bound_u32(B, 0, blen, ins_c);
-            lins = tins - k0 - ((has_kpp && kpp < tins) ? 1u : 0u);
-        }
-        const uint32_t Lb = (blen - k0) - (has_kpp ? 1u : 0u) + (has_new ? 1u : 0u);
-        const uint32_t nch = (Lb + 31u) / 32u;
-        // source of this lane's entry in chunk c (NULL past the end)
-        auto src_of = [&](uint32_t c) -> const BlendRec* {
-            const uint32_t m = c * 32u + (uint32_t)lane;
-            if (c >= nch || m >= Lb) return nullptr;
-            uint32_t ci = 0;
-            if (merged_entry(m, has_kpp, has_new, kpp - k0, lins, ci)) return &it->rec;
-            return v.bl_rec + boff + k0 + ci;   // the sublist's records are stored in order
-        };
-        auto issue = [&](uint32_t c, const BlendRec* src) {
-            if (src) {
-                const int slot = (int)(c % (uint32_t)kWarpRing);
-#pragma unroll
-                for (int part = 0; part < 3; part++)
-                    cp_async16(&R.q[slot][part][lane], reinterpret_cast<const float4*>(src) + part);
-            }
-            cp_async_commit_group();
-        };
-        // the previous unit's copies may still be landing in the ring
-        cp_async_wait_all();
-        __syncwarp();
-#pragma unroll
-        for (int c = 0; c < kWarpRing - 1; c++) issue((uint32_t)c, src_of((uint32_t)c));
-        const BlendRec* next_src = src_of(kWarpRing - 1);
-        unsigned int nev = 0, staged = 0;
-        unsigned steps[2] = {0u, 0u};
-        long long c1 = COUNT ? clock64() : 0;
-        for (uint32_t c = 0; c < nch; c++) {
-            __syncwarp();   // every lane is done with the slot the next issue overwrites
-            issue(c + kWarpRing - 1, next_src);
-            next_src = src_of(c + kWarpRing);
-            cp_async_wait_group<kWarpRing - 1>();   // this lane's copies of chunk c have landed
-            __syncwarp();                            // and every other lane's
-            const int slot = (int)(c % (uint32_t)kWarpRing);
-            const uint32_t base = c * 32u;
-            const int cnt = (int)min(32u, Lb - base);
-            staged += (uint32_t)cnt;
-            if (c > 0) {   // the box of the pixel centres still blending: a stopped pixel takes no entry
-                const bool la = !pA.done, lb = !pB.done;
-                g.wx0 = (float)__reduce_min_sync(0xffffffffu, (la || lb) ? px : 0x7fffffff) + 0.5f;
-                g.wx1 = (float)__reduce_max_sync(0xffffffffu, (la || lb) ? px : -1) + 0.5f;
-                g.wy0 = (float)__reduce_min_sync(0xffffffffu, la ? pyA : (lb ? pyB : 0x7fffffff)) + 0.5f;
-                g.wy1 = (float)__reduce_max_sync(0xffffffffu, lb ? pyB : (la ? pyA : -1)) + 0.5f;
-            }
-            bool pass = false;
-            if (lane < cnt) {
-                const float4 a = R.q[slot][0][lane], bb = R.q[slot][1][lane];
-                // the entry's box [mx - ex, mx + ex] x [my - ey, my + ey] against the block's,
-                // then the conservative conic test over the block's pixel centres
-                pass = !(a.x + bb.z < g.wx0 || a.x - bb.z > g.wx1 || a.y + bb.w < g.wy0 || a.y - bb.w > g.wy1) &&
-                       rect_reachable(a.x, a.y, a.z, a.w, bb.x, bb.y, g.wx0, g.wx1, g.wy0, g.wy1);
-            }
-            const unsigned m = __ballot_sync(0xffffffffu, pass);
-            auto fetch = [&](int e) {
-                const float4 q1 = R.q[slot][1][e], q2 = R.q[slot][2][e];
-                return EntryQ{R.q[slot][0][e], q1.x, q1.y, q2.x, q2.y, q2.z};
+    for (uint32_t c0 = blockIdx.x * per; c0 < ncand; c0 += gridDim.x * per) {
+        const long long t0 = COUNT ? clock64() : 0;
+        const int nv = (int)min(per, ncand - c0);
+        __syncthreads();   // the previous candidates are done with the shared arrays
+        for (int task = warp; task < nv * nb; task += kDirtyWarps) {
+            const int vi = task / nb, b = task % nb;
+            const uint2 c = cand[c0 + (uint32_t)vi];
+            const uint32_t bk = c.x & kCandPair;
+            const int tx = (int)(c.y & 0xffffu), ty = (int)(c.y >> 16);
+            const ViewPtrs& v = views[c.x >> 24];
+            const uint32_t tile = (uint32_t)ty * (uint32_t)v.tiles_x + (uint32_t)tx;
+            const DirtyDesc& d = desc[bk];
+            const uint4 rects = *reinterpret_cast<const uint4*>(&d.nx0);   // corrupted x0 | y0 << 16, x1 | y1 << 16, clean
+            auto in_rect = [&](uint32_t q0, uint32_t q1) {
+                return tx >= (int)(q0 & 0xffffu) && tx < (int)(q1 & 0xffffu) && ty >= (int)(q0 >> 16) &&
+                       ty < (int)(q1 >> 16);
             };
-            walk_survivors2<COUNT, false>(m, 0, fetch, pxc, pycA, pycB, pA, pB, nev, base, steps);
-            if (__all_sync(0xffffffffu, pA.done && pB.done)) break;
-        }
-        long long c2 = COUNT ? clock64() : 0;
-        // compare the active pixels with the clean image; every other pixel keeps
-        // its clean value (Delta = 0), and the clean image's non-finite pixels are
-        // counted once per view at finalize
-        const float a0 = __fadd_rn(pA.c0, pA.T), a1 = __fadd_rn(pA.c1, pA.T), a2 = __fadd_rn(pA.c2, pA.T);
-        const float b0 = __fadd_rn(pB.c0, pB.T), b1 = __fadd_rn(pB.c1, pB.T), b2 = __fadd_rn(pB.c2, pB.T);
-        const float* cA = v.clean + ((size_t)y0 * v.W + x0) * 3;
-        const float* cB = v.clean + ((size_t)y1 * v.W + px) * 3;
-        if (sb.deltas) {   // dirty-tile SSIM: keep the block's new values, two 32-pixel delta units per group
-            const uint32_t slot = code >> 3;
-            if (2u * gi + 1u < sb.delta_cap && slot < sb.slot_cap) {
-                // delta unit 2 gi: upper half, 2 gi + 1: lower half; one entry per pixel of the half
-                if (actA) sb.deltas[(size_t)(2u * gi) * 32 + lane] = make_float4(a0, a1, a2, 0.0f);
-                if (actB) sb.deltas[(size_t)(2u * gi + 1u) * 32 + lane] = make_float4(b0, b1, b2, 0.0f);
-                if (lane == 0) {
-                    sb.slot_group[(size_t)slot * 8 + wA] = 2u * gi;
-                    sb.slot_group[(size_t)slot * 8 + wB] = 2u * gi + 1u;
+            const bool has_new = in_rect(rects.x, rects.y), has_old = in_rect(rects.z, rects.w);
+            const uint32_t ins = has_new ? d.new_rank : kNoRank, pp = has_old ? d.old_rank : kNoRank;
+            const uint32_t cut = min(ins, pp);
+            unsigned mA = 0u, mB = 0u;
+            if ((c.x >> (20 + b)) & 1u) {
+                const int wA = block_upper(b, lg), wB = wA + (1 << lg);
+                // this lane's two pixels of the block: (lane % 8, lane / 8) and four rows below
+                const uint32_t* stop = v.stop + (size_t)tile * P + lane;
+                const uint32_t stA = stop[wA * 32], stB = stop[wB * 32];
+                const int px = tx * tw + block_x0(b, lg) + (lane & 7), pyA = ty * th + block_y0(b, lg) + (lane >> 3);
+                const float pxc = (float)px + 0.5f, pycA = (float)pyA + 0.5f;
+                const float2 npy = make_float2(-pycA, -(pycA + 4.0f));
+                bool okA = false, okB = false;
+                if (has_old) {
+                    const BlendRec& q = d.old;
+                    alpha_pair(EntryQ{make_float4(q.mx, q.my, q.ca, q.cb), q.cc, q.opac, 0.0f, 0.0f, 0.0f}, pxc, npy,
+                               okA, okB);
                 }
-                // where the changed pixels are: which neighbouring tiles their SSIM windows reach
-                auto edge = [&](bool a, int x, int y, float n0, float n1, float n2, const float* c) -> unsigned {
-                    const bool ch = a && (__float_as_uint(n0) != __float_as_uint(c[0]) ||
-                                          __float_as_uint(n1) != __float_as_uint(c[1]) ||
-                                          __float_as_uint(n2) != __float_as_uint(c[2]));
-                    const int lx = x - tx * tw, ly = y - ty * th;
-                    return ch ? (16u | (lx < 5 ? 1u : 0u) | (lx > tw - 6 ? 2u : 0u) | (ly < 5 ? 4u : 0u) |
-                                 (ly > th - 6 ? 8u : 0u))
-                              : 0u;
-                };
-                const unsigned f = edge(actA, x0, y0, a0, a1, a2, cA) | edge(actB, px, y1, b0, b1, b2, cB);
-                const unsigned fo = __reduce_or_sync(0xffffffffu, f);
-                if (lane == 0 && fo) atomicOr(&sb.slot_flags[slot], fo);
-            } else if (lane == 0) {
-                atomicOr(sb.overflow, 1u);
+                float aA = -1.0f, aB = -1.0f;
+                if (has_new) {
+                    const BlendRec& q = d.rec;
+                    bool nA, nB;
+                    const float2 a = alpha_pair(
+                        EntryQ{make_float4(q.mx, q.my, q.ca, q.cb), q.cc, q.opac, 0.0f, 0.0f, 0.0f}, pxc, npy, nA, nB);
+                    aA = nA ? (a.x > 0.99f ? 0.99f : a.x) : -1.0f;   // keeps NaN
+                    aB = nB ? (a.y > 0.99f ? 0.99f : a.y) : -1.0f;
+                    okA |= nA;
+                    okB |= nB;
+                }
+                alpha[vi][b * 64 + lane] = aA;
+                alpha[vi][b * 64 + 32 + lane] = aB;
+                okA = okA && px < v.W && pyA < v.H;
+                okB = okB && px < v.W && pyA + 4 < v.H;
+                mA = __ballot_sync(0xffffffffu, okA && stA >= cut);
+                mB = __ballot_sync(0xffffffffu, okB && stB >= cut);
+                if (COUNT) {
+                    const bool any = __any_sync(0xffffffffu, okA || okB);
+                    if (lane == 0 && (mA | mB)) atomicAdd(&work[10], 1ull);
+                    if (lane == 0 && !(mA | mB)) {
+                        atomicAdd(&work[3], 1ull);
+                        atomicAdd(&work[any ? 7 : 6], 1ull);
+                    }
+                }
+            }
+            if (lane == 0) var[vi].mask[b] = (unsigned long long)mA | ((unsigned long long)mB << 32);
+            if (b == 0) {
+                // the rows in front of the first change (the keys ascend)
+                const uint32_t* key = v.row_key + (size_t)tile * kRowsPerTile + lane;
+                const uint32_t key0 = key[0], key1 = key[32];
+                const uint32_t row = v.row_off[tile] + (uint32_t)(__popc(__ballot_sync(0xffffffffu, key0 < cut)) +
+                                                                  __popc(__ballot_sync(0xffffffffu, key1 < cut)));
+                if (lane == 0) {
+                    DirtyVar& q = var[vi];
+                    q.row_idx = v.row_idx + (size_t)row * P;
+                    q.W3 = 3 * v.W;
+                    q.clean = v.clean + ((size_t)(ty * th) * v.W + tx * tw) * 3;
+                    q.ent = v.ent;
+                    q.rk = v.rk;
+                    q.state = v.state;
+                    q.bk = bk;
+                    q.ins = ins;
+                    q.pp = pp;
+                    q.r = d.rec.r;
+                    q.g = d.rec.g;
+                    q.b = d.rec.b;
+                    q.cx = c.x;
+                    q.cy = c.y;
+                    q.tile = tile;
+                    q.fx_lo = q.fx_hi = q.maxbits = q.counts = 0u;
+                    q.cells_lo = q.cells_hi = q.edge = 0u;
+                }
             }
         }
-        BlockCmp r;
-        block_cmp_add(r, actA, a0, a1, a2, cA, x0, y0, v.W, v.H);
-        block_cmp_add(r, actB, b0, b1, b2, cB, px, y1, v.W, v.H);
-        unsigned long long fx = r.fx;
-        float mx = r.m;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            fx += __shfl_xor_sync(0xffffffffu, fx, o);
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        __syncthreads();
+        if (sb.plan && warp < (kUnitVars * kDirtyBlocks) / 32) {   // dirty-tile SSIM: two 32-pixel delta units per block
+            const int vi = tid / nb, b = tid % nb;
+            const unsigned long long mask = vi < nv ? var[vi].mask[b] : 0ull;
+            const unsigned am = __ballot_sync(0xffffffffu, mask != 0ull);
+            uint32_t unit = 0;
+            if (lane == 0 && am) unit = atomicAdd(&counts[5], (unsigned)__popc(am));
+            unit = __shfl_sync(0xffffffffu, unit, 0) + (uint32_t)__popc(am & ((1u << lane) - 1u));
+            if (mask) {
+                const unsigned long long e = sb.tile_map[(size_t)var[vi].bk * sb.max_tiles + var[vi].tile];
+                const uint32_t slot = (uint32_t)e;
+                const int wA = block_upper(b, lg), wB = wA + (1 << lg);
+                if ((uint32_t)(e >> 32) == counts[6] && 2u * unit + 1u < sb.delta_cap) {
+                    sb.plan[slot].mask[wA] = (uint32_t)mask;
+                    sb.plan[slot].mask[wB] = (uint32_t)(mask >> 32);
+                    sb.slot_group[(size_t)slot * 8 + wA] = 2u * unit;
+                    sb.slot_group[(size_t)slot * 8 + wB] = 2u * unit + 1u;
+                    var[vi].unit[b] = unit;
+                } else {
+                    var[vi].unit[b] = 0xffffffffu;
+                    atomicOr(sb.overflow, 1u);
+                }
+            }
         }
-        const unsigned nfoot = __reduce_add_sync(0xffffffffu, r.foot);
-        const unsigned nbad = __reduce_add_sync(0xffffffffu, r.bad);
-        const unsigned ncb = __reduce_add_sync(0xffffffffu, r.clean_bad);
-        // screen cells holding a footprint pixel (contamination of a sort-first partition)
-        const unsigned long long cells =
-            (unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned)r.cells) |
-            ((unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned)(r.cells >> 32)) << 32);
-        if (lane == 0) {
-            CmpAcc* A = &acc[bk];
+        // the pairs by pixel: thread t lists the candidates of pixel t
+        uint32_t m = 0u;
+        if (tid < nb * 64)
+            for (int vi = 0; vi < nv; vi++) m |= ((unsigned)(var[vi].mask[tid >> 6] >> (tid & 63)) & 1u) << vi;
+        const uint32_t cnt = (uint32_t)__popc(m);
+        uint32_t incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) wsum[warp] = incl;
+        __syncthreads();
+        uint32_t at = incl - cnt, npairs = 0;
+#pragma unroll
+        for (int w = 0; w < kDirtyWarps; w++) {
+            at += w < warp ? wsum[w] : 0u;
+            npairs += wsum[w];
+        }
+        for (; m; m &= m - 1u) pairs[at++] = (uint16_t)((__ffs(m) - 1) << 8 | tid);
+        __syncthreads();
+        if (COUNT) t_pro += clock64() - t0;
+        unsigned int nev = 0, nst = 0;
+        for (uint32_t r0 = (uint32_t)warp * 32u; r0 < npairs; r0 += kDirtyThreads) {
+            const long long t1 = COUNT ? clock64() : 0;
+            const bool act = r0 + (uint32_t)lane < npairs;
+            const int code = pairs[act ? r0 + (uint32_t)lane : r0];
+            const int vi = code >> 8, u8 = code & 255, b = u8 >> 6, u6 = u8 & 63;
+            DirtyVar& q = var[vi];
+            const int lx = block_x0(b, lg) + (u6 & 7), ly = block_y0(b, lg) + (u6 >> 3);   // in the tile
+            const int u = (block_upper(b, lg) + ((u6 >> 5) << lg)) * 32 + (u6 & 31);
+            DirtyPix p{1.0f, 0.0f, 0.0f, 0.0f};
+            float k0 = 0.0f, k1 = 0.0f, k2 = 0.0f;   // the clean pixel
+            if (act) {
+                const float4* ent = q.ent;
+                uint32_t i = q.row_idx[u] & ~(uint32_t)(kWalk - 1);
+                const float* kp = q.clean + (ly * q.W3 + lx * 3);
+                k0 = kp[0];
+                k1 = kp[1];
+                k2 = kp[2];
+                const float4 st = q.state[i / kWalk];
+                p.T = st.x;
+                p.c0 = st.y;
+                p.c1 = st.z;
+                p.c2 = st.w;
+                const uint32_t ins = q.ins, pp = q.pp;
+                const float na = alpha[vi][u8];   // the corrupted entry at this pixel, when its blend takes it
+                bool pend = !(na < 0.0f);         // still to be inserted (a NaN alpha too)
+                bool old = pp != kNoRank;         // the removed entry may still lie ahead
+                float4 e[kWalk];
+                float last = 0.0f;                // the alpha that ended the walk
+                bool end = false;
+                do {
+#pragma unroll
+                    for (int k = 0; k < kWalk; k += 2) load_pair(ent + i + k, e[k], e[k + 1]);
+                    if (COUNT) nst++;
+                    if (pend || old) {   // ranks matter until both changes are behind
+                        // the first entry of this group behind the corrupted one (the end's rank is
+                        // above every other) and the removed entry
+                        int at_new = 0, at_old = kWalk;
+                        uint32_t q_last = 0u;
+#pragma unroll
+                        for (int k = 0; k < kWalk; k += 4) {
+                            const uint4 x = __ldg(reinterpret_cast<const uint4*>(q.rk + i + k));
+                            const int first = x.x >= ins ? 0 : (x.y >= ins ? 1 : (x.z >= ins ? 2 : (x.w >= ins ? 3 : 4)));
+                            at_new = at_new == k ? k + first : at_new;
+                            at_old = x.x == pp ? k : (x.y == pp ? k + 1 : (x.z == pp ? k + 2 : (x.w == pp ? k + 3 : at_old)));
+                            q_last = x.w;
+                        }
+                        at_new = pend ? at_new : kWalk;
+#pragma unroll
+                        for (int k = 0; k < kWalk; k++) {
+                            // a cut list's rest, and an entry that belongs there, come from the tile's list
+                            if (k == at_new && !end && e[k].x != kListCut) {
+                                pend = false;
+                                if (COUNT) nev++;
+                                last = na;
+                                end = p.take(na, q.r, q.g, q.b);
+                            }
+                            if (!end && (k != at_old || e[k].x == kListCut)) {
+                                if (COUNT) nev++;
+                                last = e[k].x;
+                                end = p.take(e[k].x, e[k].y, e[k].z, e[k].w);
+                            }
+                        }
+                        old = old && q_last < pp;
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < kWalk; k++) {
+                            if (end) continue;
+                            if (COUNT) nev++;
+                            last = e[k].x;
+                            end = p.take(e[k].x, e[k].y, e[k].z, e[k].w);
+                        }
+                    }
+                    i += kWalk;
+                } while (!end);
+                p.poison(last);
+                if (last == kListCut) {
+                    // a list cut short: the rest comes from the tile's list, from the mark's rank on
+                    const ViewPtrs& v = views[q.cx >> 24];
+                    const float x = (float)((int)(q.cy & 0xffffu) * tw + lx) + 0.5f;
+                    const float y = (float)((int)(q.cy >> 16) * th + ly) + 0.5f;
+                    uint32_t from = 0xffffffffu;
+                    for (int k = 0; k < kWalk; k++) {
+                        const uint32_t j = i - kWalk + (uint32_t)k;
+                        if (ent[j].x == kListCut && from == 0xffffffffu) from = q.rk[j];
+                    }
+                    const uint2 rg = v.ranges[q.tile];
+                    const uint32_t L = rg.y - rg.x;
+                    bool stopped = false;
+                    for (uint32_t j = 0; j <= L && !stopped; j++) {   // j == L: the list's end
+                        const uint32_t id = j < L ? v.ids[rg.x + j] : 0u, rank = j < L ? v.rank[id] : 0xffffffffu;
+                        if (rank < from) continue;
+                        if (pend && rank >= ins) {
+                            pend = false;
+                            stopped = p.take(na, q.r, q.g, q.b);
+                            p.poison(na);
+                        }
+                        if (rank == pp || j == L || stopped) continue;
+                        const BlendRec z = load_rec(v.recs, id);
+                        float al;
+                        if (COUNT) nev++;
+                        if (blend_alpha(z.mx, z.my, z.ca, z.cb, z.cc, z.opac, x, y, al)) {
+                            al = al > 0.99f ? 0.99f : al;
+                            stopped = p.take(al, z.r, z.g, z.b);
+                            p.poison(al);
+                        }
+                    }
+                }
+            }
+            __syncwarp();
+            const long long t2 = COUNT ? clock64() : 0;
+            // compare with the clean image; every inactive pixel keeps its clean value
+            // (Delta = 0), and the clean image's non-finite pixels are counted once per
+            // view at finalize
+            const float a0 = __fadd_rn(p.c0, p.T), a1 = __fadd_rn(p.c1, p.T), a2 = __fadd_rn(p.c2, p.T);
+            DirtySum s{};
+            if (act) s = dirty_sum(a0, a1, a2, k0, k1, k2);
+            const bool one = nv == 1;   // block-uniform
+            if (one) {
+                s.fx_lo = __reduce_add_sync(0xffffffffu, s.fx_lo);
+                s.fx_hi = __reduce_add_sync(0xffffffffu, s.fx_hi);
+                s.counts = __reduce_add_sync(0xffffffffu, s.counts);
+                s.maxbits = __reduce_max_sync(0xffffffffu, s.maxbits);
+            }
+            if (one ? lane == 0 : act) {
+                if (s.fx_lo) atomicAdd(&q.fx_lo, s.fx_lo);
+                if (s.fx_hi) atomicAdd(&q.fx_hi, s.fx_hi);
+                if (s.counts) atomicAdd(&q.counts, s.counts);
+                if (s.maxbits) atomicMax(&q.maxbits, s.maxbits);
+            }
+            if (regions && act && s.foot) {   // screen cells holding a footprint pixel
+                const ViewPtrs& v = views[q.cx >> 24];
+                const unsigned long long cell = cell_bit((int)(q.cy & 0xffffu) * tw + lx, (int)(q.cy >> 16) * th + ly, v.W, v.H);
+                if ((unsigned)cell) atomicOr(&q.cells_lo, (unsigned)cell);
+                if ((unsigned)(cell >> 32)) atomicOr(&q.cells_hi, (unsigned)(cell >> 32));
+            }
+            if (sb.plan && act && q.unit[b] != 0xffffffffu) {   // dirty-tile SSIM: the new values
+                sb.deltas[(size_t)(2u * q.unit[b] + (uint32_t)(u6 >> 5)) * 32 + (u6 & 31)] = make_float4(a0, a1, a2, 0.0f);
+                // where the changed pixels are: which neighbouring tiles their SSIM windows reach
+                const bool ch = __float_as_uint(a0) != __float_as_uint(k0) || __float_as_uint(a1) != __float_as_uint(k1) ||
+                                __float_as_uint(a2) != __float_as_uint(k2);
+                if (ch)
+                    atomicOr(&q.edge, 16u | (lx < 5 ? 1u : 0u) | (lx > tw - 6 ? 2u : 0u) | (ly < 5 ? 4u : 0u) |
+                                          (ly > th - 6 ? 8u : 0u));
+            }
+            if (COUNT) {
+                const unsigned steps = __reduce_max_sync(0xffffffffu, nst);
+                nst = 0;
+                t_walk += t2 - t1;
+                t_epi += clock64() - t2;
+                if (lane == 0) {
+                    const unsigned npix = min(32u, npairs - r0);
+                    atomicAdd(&work[8], (unsigned long long)(steps * kWalk));
+                    atomicAdd(&work[9], (unsigned long long)(steps * kWalk));
+                    atomicAdd(&work[14], (unsigned long long)npix);
+                    atomicAdd(&work[15], (unsigned long long)steps * kWalk * npix);
+                }
+            }
+        }
+        __syncthreads();
+        if (tid < nv) {
+            const DirtyVar& q = var[tid];
+            CmpAcc* A = &acc[q.bk];
+            const unsigned long long fx = (unsigned long long)q.fx_lo + ((unsigned long long)q.fx_hi << 20);
+            const unsigned long long cells = (unsigned long long)q.cells_lo | ((unsigned long long)q.cells_hi << 32);
+            const unsigned foot = q.counts & 1023u, bad = (q.counts >> 10) & 1023u, clean_bad = q.counts >> 20;
             if (cells) atomicOr(&A->reg_actual, cells);
             if (fx) atomicAdd(&A->sse_fx, fx);
-            if (mx > 0.0f) atomicMax(&A->maxabs_bits, __float_as_uint(mx));
-            if (nfoot) atomicAdd(&A->footprint, nfoot);
-            if (nbad) atomicAdd(&A->nonfinite, nbad);
-            if (ncb) atomicAdd(&A->clean_nonfinite_replaced, ncb);
+            if (q.maxbits) atomicMax(&A->maxabs_bits, q.maxbits);
+            if (foot) atomicAdd(&A->footprint, foot);
+            if (bad) atomicAdd(&A->nonfinite, bad);
+            if (clean_bad) atomicAdd(&A->clean_nonfinite_replaced, clean_bad);
+            if (q.edge)   // set only where the tile has a slot
+                atomicOr(&sb.slot_flags[(uint32_t)sb.tile_map[(size_t)q.bk * sb.max_tiles + q.tile]], q.edge);
         }
         if (COUNT) {
             const unsigned wn = __reduce_add_sync(0xffffffffu, nev);
-            // a tile counts once, on its first group (lowest block with an active pixel)
-            const bool first =
-                __ballot_sync(0xffffffffu, lane < b && (it->mask[block_upper(lane & 3, lg)] |
-                                                        it->mask[block_upper(lane & 3, lg) + (1 << lg)]) != 0u) == 0u;
-            if (lane == 0) {
-                if (wn) atomicAdd(&work[0], (unsigned long long)wn);
-                if (first) atomicAdd(&work[1], 1ull);
-                atomicAdd(&work[2], (unsigned long long)staged);
-                atomicAdd(&work[8], (unsigned long long)steps[0]);
-                atomicAdd(&work[9], (unsigned long long)steps[1]);
-                atomicAdd(&work[10], 1ull);
-                const unsigned npix = (unsigned)(__popc(amA) + __popc(amB));
-                atomicAdd(&work[14], (unsigned long long)npix);
-                atomicAdd(&work[15], (unsigned long long)npix * steps[0]);
+            if (lane == 0 && wn) {
+                atomicAdd(&work[0], (unsigned long long)wn);
+                atomicAdd(&work[2], (unsigned long long)wn);
             }
-            t_pro += c1 - c0;
-            t_walk += c2 - c1;
-            t_epi += clock64() - c2;
         }
     }
     if (COUNT && lane == 0) {
@@ -1206,7 +1505,6 @@ __global__ __launch_bounds__(kDirtyWarps * 32, 6) void k_dirty(const ViewPtrs* _
         atomicAdd(&work[12], (unsigned long long)t_walk);
         atomicAdd(&work[13], (unsigned long long)t_epi);
     }
-    cp_async_wait_all();   // leave no copy in flight
 }
 
 __global__ void k_records_to_blend(const gs_record* in, uint64_t n, BlendRec* out) {
@@ -1230,11 +1528,6 @@ __global__ void k_records_to_blend(const gs_record* in, uint64_t n, BlendRec* ou
     out[i] = q;
 }
 
-__global__ void k_gather_depth(const BlendRec* recs, const uint32_t* ids, uint64_t n, uint32_t* dk) {
-    uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) dk[i] = __float_as_uint(recs[ids[i]].depth);
-}
-
 __global__ void k_offsets_to_ranges(const uint32_t* offsets, int ntiles, uint2* ranges) {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < ntiles) ranges[t] = make_uint2(offsets[t], offsets[t + 1]);
@@ -1247,8 +1540,7 @@ gs_status launch_blend_image(const BlendRec* recs, const uint32_t* ids, const ui
     const int tx = cam.tiles_x, ty = cam.tiles_y, P = cam.tile_w * cam.tile_h / 2;   // threads: two pixels each
     if (tx * ty == 0) return GS_OK;
     k_blend_full<0, false><<<tx * ty, P, 0, st>>>(recs, ids, ranges, cam.W, cam.H, tx, cam.tile_w, cam.tile_h, img,
-                                                   nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
-                                                   nullptr, nullptr);
+                                                   nullptr, nullptr, nullptr);
     GS_CUDA(cudaGetLastError());
     return GS_OK;
 }
@@ -1259,24 +1551,57 @@ gs_status launch_blend_compare(const BlendRec* recs, const uint32_t* ids, const 
     if (tx * ty == 0) return GS_OK;
     if (work)
         k_blend_full<1, true><<<tx * ty, P, 0, st>>>(recs, ids, ranges, cam.W, cam.H, tx, cam.tile_w, cam.tile_h,
-                                                     nullptr, clean, acc, work, nullptr, nullptr, nullptr, nullptr,
-                                                     nullptr, nullptr);
+                                                     nullptr, clean, acc, work);
     else
         k_blend_full<1, false><<<tx * ty, P, 0, st>>>(recs, ids, ranges, cam.W, cam.H, tx, cam.tile_w, cam.tile_h,
-                                                      nullptr, clean, acc, nullptr, nullptr, nullptr, nullptr,
-                                                      nullptr, nullptr, nullptr);
+                                                      nullptr, clean, acc, nullptr);
     GS_CUDA(cudaGetLastError());
     return GS_OK;
 }
 
-gs_status launch_blend_image_stop(const BlendRec* recs, const uint32_t* ids, const uint2* ranges, const DevCamera& cam,
-                                  float* img, uint32_t* stop, uint32_t* tile_stop, float4* ck, const uint32_t* ck_off,
-                                  const uint32_t* ck_cnt, unsigned int* clean_nonfin, cudaStream_t st) {
-    const int tx = cam.tiles_x, ty = cam.tiles_y, P = cam.tile_w * cam.tile_h / 2;   // threads: two pixels each
+// First pass over a clean view: image, stops, list lengths.
+gs_status launch_blend_clean(const ViewState& v, uint32_t* counts, unsigned int* clean_nonfin, cudaStream_t st) {
+    const DevCamera& cam = v.cam;
+    const int tx = cam.tiles_x, ty = cam.tiles_y, P = cam.tile_w * cam.tile_h / 2;
     if (tx * ty == 0) return GS_OK;
-    k_blend_full<2, false><<<tx * ty, P, 0, st>>>(recs, ids, ranges, cam.W, cam.H, tx, cam.tile_w, cam.tile_h, img,
-                                                   nullptr, nullptr, nullptr, stop, tile_stop, ck, ck_off, ck_cnt,
-                                                   clean_nonfin);
+    k_blend_clean<false><<<tx * ty, P, 0, st>>>(v.recs, v.ids, v.rank, v.ranges, cam.W, cam.H, tx, cam.tile_w,
+                                                cam.tile_h, v.clean, v.stop, v.tile_stop, v.tile_last, counts,
+                                                clean_nonfin, ListOut{});
+    GS_CUDA(cudaGetLastError());
+    return GS_OK;
+}
+
+// Second pass: blend lists (off: their starts, at most cap entries each) and checkpoint rows.
+gs_status launch_fill_lists(const ViewState& v, const uint32_t* off, uint32_t cap, cudaStream_t st) {
+    const DevCamera& cam = v.cam;
+    const int tx = cam.tiles_x, ty = cam.tiles_y, P = cam.tile_w * cam.tile_h / 2;
+    if (tx * ty == 0) return GS_OK;
+    const int smem = (int)sizeof(ListRing) * (P / 32);
+    GS_CUDA(cudaFuncSetAttribute(k_blend_clean<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    k_blend_clean<true><<<tx * ty, P, smem, st>>>(v.recs, v.ids, v.rank, v.ranges, cam.W, cam.H, tx, cam.tile_w,
+                                                  cam.tile_h, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
+                                                  ListOut{v.ent, v.rk, off, cap, v.state, v.row_idx, v.row_off, v.row_cnt});
+    k_row_keys<<<(tx * ty * kRowsPerTile + 255) / 256, 256, 0, st>>>(v.ranges, v.ids, v.rank, v.row_cnt, tx * ty,
+                                                                       v.row_key);
+    GS_CUDA(cudaGetLastError());
+    return GS_OK;
+}
+
+gs_status launch_ranks(const uint32_t* key, const uint32_t* id, uint64_t n, const ViewState& v, cudaStream_t st) {
+    if (n > 0) k_ranks<<<(unsigned)div_up(n, 256), 256, 0, st>>>(key, id, n, v.rank, v.sdk, v.sid);
+    GS_CUDA(cudaGetLastError());
+    return GS_OK;
+}
+
+gs_status launch_row_counts(const ViewState& v, uint32_t* rows, cudaStream_t st) {
+    const int ntiles = v.cam.tiles_x * v.cam.tiles_y;
+    if (ntiles > 0) k_row_counts<<<(ntiles + 255) / 256, 256, 0, st>>>(v.ranges, v.tile_last, ntiles, v.row_cnt, rows);
+    GS_CUDA(cudaGetLastError());
+    return GS_OK;
+}
+
+gs_status launch_list_lens(const uint32_t* counts, uint64_t n, uint32_t cap, uint32_t* lens, cudaStream_t st) {
+    if (n > 0) k_list_lens<<<(unsigned)div_up(n, 256), 256, 0, st>>>(counts, n, cap, lens);
     GS_CUDA(cudaGetLastError());
     return GS_OK;
 }
@@ -1301,7 +1626,7 @@ gs_status launch_zero_acc(CmpAcc* acc, int count, cudaStream_t st) {
 
 gs_status launch_finalize(const CmpAcc* acc, int count, gs_result* out, cudaStream_t st) {
     if (count <= 0) return GS_OK;
-    k_finalize<<<(count + 255) / 256, 256, 0, st>>>(acc, count, out, nullptr, 1);
+    k_finalize<<<(count + 255) / 256, 256, 0, st>>>(acc, count, out, nullptr, 1, nullptr);
     GS_CUDA(cudaGetLastError());
     return GS_OK;
 }
@@ -1320,9 +1645,9 @@ gs_status launch_regions_out(const CmpAcc* acc, int count, unsigned long long* o
 }
 
 gs_status launch_finalize_dirty(const CmpAcc* acc, int count, gs_result* out, const unsigned int* clean_nonfin, int K,
-                                cudaStream_t st) {
+                                unsigned int* queue, cudaStream_t st) {
     if (count <= 0) return GS_OK;
-    k_finalize<<<(count + 255) / 256, 256, 0, st>>>(acc, count, out, clean_nonfin, K);
+    k_finalize<<<(count + 255) / 256, 256, 0, st>>>(acc, count, out, clean_nonfin, K, queue);
     GS_CUDA(cudaGetLastError());
     return GS_OK;
 }
@@ -1331,182 +1656,78 @@ int dirty_grid() {
     static int blocks = 0;
     if (!blocks) {
         int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dirty<false>, kDirtyWarps * 32, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dirty<false>, kDirtyThreads, 0);
         if (per_sm < 1) per_sm = 1;
         blocks = per_sm * num_sms();
     }
     return blocks;
 }
 
-size_t plan_item_size() { return sizeof(PlanItem); }
+gs_status launch_dirty_ssim(const void* dev_views, int K, unsigned int* queue, const SsimBufs& sb, CmpAcc* acc,
+                            cudaStream_t st);
 
-// ev_mid (optional): recorded between the plan kernels and the blend kernel.
-// queue[0]: blend work queue, queue[1]: plan items, queue[2]: candidate tiles,
-// queue[3] / queue[4]: heavy / light groups (all zeroed by the injector); cand
-// holds as many entries as plan, groups gcap = 8 per plan entry.
-gs_status launch_dirty_ssim(const void* dev_views, int K, const void* plan, const unsigned int* queue,
-                            const SsimBufs& sb, CmpAcc* acc, cudaStream_t st);
+// Candidates are put in tile order from this many (variant, view) pairs on: with
+// fewer, hardly two variants meet in a tile, and the two launches cost 10 us (1,024
+// pairs of a 300k-primitive scene: 1.14 ms in order, 1.18 ms as planned; 200 pairs
+// of a 5k-primitive one: no difference).
+constexpr int kSortPairs = 512;
 
-gs_status launch_dirty_blend(const void* dev_views, const DirtyDesc* desc, const uint32_t* item_off, int BK, int K,
-                             void* plan, uint2* cand, uint32_t* groups, uint32_t gcap, CmpAcc* acc,
-                             unsigned int* queue, unsigned long long* work, cudaEvent_t ev_mid, const SsimBufs& sb,
-                             cudaStream_t st) {
-    const ViewPtrs* views = (const ViewPtrs*)dev_views;
-    PlanItem* pl = (PlanItem*)plan;
+// One batch after the injector.  ev_mid (optional): recorded between the plan and
+// the blend kernel.  s->queue: [1] tile rows, [2] candidates, [3] SSIM plan
+// slots, [4] bin places, [5] SSIM delta units, cleared by the finaliser; [6] batch
+// generation; [7] tiles the SSIM visits.
+gs_status launch_dirty_blend(gs_scene* s, int BK, bool regions, const SsimBufs& sb, cudaStream_t st) {
+    const ViewPtrs* views = (const ViewPtrs*)s->dev_views;
     const int plan_blocks = num_sms() * 8;
-    if (work) {
-        k_plan_filter<true><<<plan_blocks, 256, 0, st>>>(views, desc, item_off, BK, K, cand, queue, work);
-        k_plan_exact<true><<<plan_blocks, 256, 0, st>>>(views, desc, K, cand, pl, groups, gcap, queue, work, sb);
-    } else {
-        k_plan_filter<false><<<plan_blocks, 256, 0, st>>>(views, desc, item_off, BK, K, cand, queue, nullptr);
-        k_plan_exact<false><<<plan_blocks, 256, 0, st>>>(views, desc, K, cand, pl, groups, gcap, queue, nullptr, sb);
+    const uint32_t nbins = s->all_tiles;
+    const bool bin = BK >= kSortPairs;
+    unsigned long long* work = s->work_ctr;
+    auto plan = work ? (bin ? k_plan<true, true> : k_plan<true, false>) : (bin ? k_plan<false, true> : k_plan<false, false>);
+    plan<<<plan_blocks, 256, 0, st>>>(views, s->desc, s->rows, s->cand, s->cand_at, s->bins, s->queue, work, sb);
+    if (bin) {
+        k_bin_starts<<<(nbins + 1023) / 1024, 1024, 0, st>>>(s->bins, nbins, s->queue);
+        k_bin_cands<<<plan_blocks, 256, 0, st>>>(views, s->cand, s->cand_at, s->bins, s->queue, s->cand_sorted);
     }
-    if (ev_mid) {
-        cudaError_t e = cudaEventRecordWithFlags(ev_mid, st, cudaEventRecordExternal);
+    if (s->ev_kp) {
+        cudaError_t e = cudaEventRecordWithFlags(s->ev_kp, st, cudaEventRecordExternal);
         if (e != cudaSuccess) return set_error(GS_ERR_CUDA, cudaGetErrorString(e));
     }
-    if (work)
-        k_dirty<true><<<dirty_grid(), kDirtyWarps * 32, 0, st>>>(views, K, pl, groups, gcap, queue, acc, queue, work,
-                                                                sb);
-    else
-        k_dirty<false><<<dirty_grid(), kDirtyWarps * 32, 0, st>>>(views, K, pl, groups, gcap, queue, acc, queue,
-                                                                 nullptr, sb);
-    if (sb.tile_map) GS_TRY(launch_dirty_ssim(dev_views, K, plan, queue, sb, acc, st));
+    auto dirty = work ? k_dirty<true> : k_dirty<false>;
+    dirty<<<dirty_grid(), kDirtyThreads, 0, st>>>(views, s->desc, bin ? s->cand_sorted : s->cand,
+                                                  s->tile_w, s->tile_h, s->queue, s->bins, bin ? nbins : 0u, s->acc,
+                                                  regions, work, sb);
+    if (sb.plan) GS_TRY(launch_dirty_ssim(s->dev_views, s->K, s->queue, sb, s->acc, st));
     GS_CUDA(cudaGetLastError());
     return GS_OK;
 }
 
 size_t view_ptrs_size() { return sizeof(ViewPtrs); }
 
-gs_status launch_gather_depth(const BlendRec* recs, const uint32_t* ids, uint64_t n, uint32_t* dk, cudaStream_t st) {
-    if (n == 0) return GS_OK;
-    k_gather_depth<<<(unsigned)div_up(n, 256), 256, 0, st>>>(recs, ids, n, dk);
-    GS_CUDA(cudaGetLastError());
-    return GS_OK;
-}
-
-int ck_stride_value() { return kCkStride; }
-int ck_max_per_tile() { return kCkMaxPerTile; }
-
-// Per tile: the sort key (depth bits << 32 | id) of the list entry at which the
-// last of its pixels stopped; ~0 when some pixel never stopped.  Every pixel of
-// the tile stopped before a change whose key is above it.
-__global__ void k_stop_keys(const uint2* __restrict__ ranges, const uint32_t* __restrict__ tile_stop,
-                            const uint32_t* __restrict__ dk, const uint32_t* __restrict__ ids, int ntiles,
-                            unsigned long long* __restrict__ out) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= ntiles) return;
-    const uint2 rg = ranges[t];
-    const uint32_t ts = tile_stop[t];
-    unsigned long long key = ~0ull;
-    if (ts != 0xffffffffu && ts < rg.y - rg.x)
-        key = ((unsigned long long)dk[rg.x + ts] << 32) | (unsigned long long)ids[rg.x + ts];
-    out[t] = key;
-}
-
-gs_status launch_stop_keys(const uint2* ranges, const uint32_t* tile_stop, const uint32_t* dk, const uint32_t* ids,
-                           int ntiles, unsigned long long* out, cudaStream_t st) {
-    if (ntiles > 0) k_stop_keys<<<(ntiles + 255) / 256, 256, 0, st>>>(ranges, tile_stop, dk, ids, ntiles, out);
-    GS_CUDA(cudaGetLastError());
-    return GS_OK;
-}
-
-void fill_view_ptrs(void* host_dst, const ViewState& vs) {
-    ViewPtrs v;
+void fill_view_ptrs(void* host_dst, const ViewState& vs, uint32_t bin0) {
+    ViewPtrs v{};
     v.recs = vs.recs;
     v.ids = vs.ids;
-    v.dk = vs.dk;
+    v.rank = vs.rank;
+    v.sdk = vs.sdk;
+    v.sid = vs.sid;
+    v.rects = vs.rects;
     v.ranges = vs.ranges;
     v.clean = vs.clean;
     v.stop = vs.stop;
     v.tile_stop = vs.tile_stop;
-    v.stop_key = vs.stop_key;
-    v.bl_off = vs.bl_off;
-    v.bl_pos = vs.bl_pos;
-    v.bl_rec = vs.bl_rec;
-    v.ck = vs.ck;
-    v.ck_off = vs.ck_off;
-    v.ck_cnt = vs.ck_cnt;
+    v.row_idx = vs.row_idx;
+    v.row_off = vs.row_off;
+    v.row_key = vs.row_key;
+    v.ent = vs.ent;
+    v.rk = vs.rk;
+    v.state = vs.state;
     v.W = vs.cam.W;
     v.H = vs.cam.H;
     v.tiles_x = vs.cam.tiles_x;
     v.tile_w = vs.cam.tile_w;
     v.tile_h = vs.cam.tile_h;
-    v.pad[0] = v.pad[1] = v.pad[2] = 0;
+    v.bin0 = bin0;
     memcpy(host_dst, &v, sizeof(v));
-}
-
-// ---------------------------------------------------------------------------
-// Per (tile, 8x8 block) sublists of the clean tile lists: the positions of the
-// entries whose box [mx - ex, mx + ex] x [my - ey, my + ey] meets the block's
-// pixel-centre box (the same comparisons as the dirty-tile cull, on a box that
-// contains every active-pixel box of the block, so an entry left out would be
-// culled there anyway).  One warp per tile; positions ascend in each sublist.
-// ---------------------------------------------------------------------------
-template <bool FILL>
-__global__ void k_blists(const BlendRec* __restrict__ recs, const uint32_t* __restrict__ ids,
-                         const uint2* __restrict__ ranges, int ntiles, int tiles_x, int tw, int th,
-                         uint32_t* __restrict__ counts, const uint32_t* __restrict__ off, uint32_t* __restrict__ pos,
-                         BlendRec* __restrict__ brec) {
-    const int lane = threadIdx.x & 31;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
-    const int lg = tile_lgx(tw), nb = (tw * th) >> 6;   // 8x8 blocks per tile
-    for (int t = warp; t < ntiles; t += nwarps) {
-        const uint2 rg = ranges[t];
-        const int tx = t % tiles_x, ty = t / tiles_x;
-        uint32_t base[kDirtyBlocks];
-#pragma unroll
-        for (int b = 0; b < kDirtyBlocks; b++) base[b] = (FILL && b < nb) ? off[(size_t)t * nb + b] : 0u;
-        for (uint32_t j0 = 0; j0 < rg.y - rg.x; j0 += 32) {
-            const uint32_t j = j0 + (uint32_t)lane;
-            unsigned mb = 0u;
-            uint32_t id = 0;
-            if (j < rg.y - rg.x) {
-                id = ids[rg.x + j];
-                const float4* r = reinterpret_cast<const float4*>(recs + id);
-                const float4 a = __ldg(r), b = __ldg(r + 1);   // (mx, my, ca, cb), (cc, opac, ex, ey)
-#pragma unroll
-                for (int k = 0; k < kDirtyBlocks; k++) {
-                    const float wx0 = (float)(tx * tw + block_x0(k, lg)) + 0.5f, wx1 = wx0 + 7.0f;
-                    const float wy0 = (float)(ty * th + block_y0(k, lg)) + 0.5f, wy1 = wy0 + 7.0f;
-                    const bool pass =
-                        k < nb && !(a.x + b.z < wx0 || a.x - b.z > wx1 || a.y + b.w < wy0 || a.y - b.w > wy1);
-                    mb |= pass ? (1u << k) : 0u;
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < kDirtyBlocks; k++) {
-                const unsigned bw = __ballot_sync(0xffffffffu, (mb >> k) & 1u);
-                if (FILL && ((mb >> k) & 1u)) {
-                    const uint32_t q = base[k] + __popc(bw & ((1u << lane) - 1u));
-                    pos[q] = j;
-                    brec[q] = recs[id];
-                }
-                base[k] += (uint32_t)__popc(bw);
-            }
-        }
-        if (!FILL && lane < nb) {
-            uint32_t c = 0;
-#pragma unroll
-            for (int k = 0; k < kDirtyBlocks; k++) c = lane == k ? base[k] : c;
-            counts[(size_t)t * nb + lane] = c;
-        }
-    }
-}
-
-gs_status launch_blists(const BlendRec* recs, const uint32_t* ids, const uint2* ranges, const DevCamera& cam,
-                        uint32_t* counts, const uint32_t* off, uint32_t* pos, BlendRec* brec, cudaStream_t st) {
-    const int ntiles = cam.tiles_x * cam.tiles_y;
-    if (ntiles <= 0) return GS_OK;
-    const int blocks = std::max(1, std::min((ntiles + 7) / 8, num_sms() * 16));
-    if (pos)
-        k_blists<true><<<blocks, 256, 0, st>>>(recs, ids, ranges, ntiles, cam.tiles_x, cam.tile_w, cam.tile_h, nullptr,
-                                               off, pos, brec);
-    else
-        k_blists<false><<<blocks, 256, 0, st>>>(recs, ids, ranges, ntiles, cam.tiles_x, cam.tile_w, cam.tile_h, counts,
-                                                nullptr, nullptr, nullptr);
-    GS_CUDA(cudaGetLastError());
-    return GS_OK;
 }
 
 gs_status launch_records_to_blend(const gs_record* in, uint64_t n, BlendRec* out, cudaStream_t st) {

@@ -516,12 +516,27 @@ __device__ __forceinline__ uint2 alpha_tiles(uint2 rect, const BlendRec& r, int 
     return make_uint2((uint32_t)fx0 | ((uint32_t)fy0 << 16), (uint32_t)fx1 | ((uint32_t)fy1 << 16));
 }
 
+// Clean entries in front of an entry with key (dkey, p) in the view's (depth,
+// index) order.
+__device__ __forceinline__ uint32_t order_lower_bound(const uint32_t* __restrict__ sdk, const uint32_t* __restrict__ sid,
+                                                      uint32_t n, uint32_t dkey, uint32_t p) {
+    uint32_t lo = 0, hi = n;
+    while (lo < hi) {
+        const uint32_t mid = lo + ((hi - lo) >> 1);
+        const uint32_t k = sdk[mid];
+        if (k < dkey || (k == dkey && sid[mid] < p))
+            lo = mid + 1;
+        else
+            hi = mid;
+    }
+    return lo;
+}
+
 template <int FMT>
 __global__ __launch_bounds__(kPrepWarps * 32) void k_inject_prep(
     const void* planes, uint64_t n, int nwords, int sh_degree, const DevCamera* cams, int K, const gs_flip* flips,
     int B, int guard_mode, uint64_t mask, const uint32_t* box, const void* pblo, const void* pbhi, int nbox,
-    const uint2* const* clean_rects, const BlendRec* const* clean_recs, DirtyDesc* desc, uint32_t* n_items,
-    CmpAcc* acc) {
+    const ViewPtrs* views, DirtyDesc* desc, uint2* rows, unsigned int* queue, CmpAcc* acc) {
     __shared__ float sv[kPrepWarps][kMaxWords];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int b = blockIdx.x * kPrepWarps + wib;
@@ -561,116 +576,93 @@ __global__ __launch_bounds__(kPrepWarps * 32) void k_inject_prep(
     clamps = __reduce_add_sync(0xffffffffu, clamps);
     changed = ok && __any_sync(0xffffffffu, changed);
     __syncwarp();
-    if (lane >= K) return;
-    const int k = lane, bk = b * K + k;
-    DirtyDesc d;
-    d.prim = p;
-    uint2 rect = make_uint2(0, 0);
-    float rad = 0.0f;
-    const bool nvb = ok && preprocess_core(SharedSrc{sv[wib]}, sh_degree, cams[k], d.rec, rect, rad);
-    const uint2 orect_b = ok ? clean_rects[k][p] : make_uint2(0, 0);   // binned rects (contamination cells)
-    const uint2 rect_b = nvb ? rect : make_uint2(0, 0);
-    // dirty tiles: the binned rects cut to the records' alpha boxes
-    if (nvb) rect = alpha_tiles(rect, d.rec, cams[k].tile_w, cams[k].tile_h);
-    const uint2 orect = orect_b.y != 0u ? alpha_tiles(orect_b, clean_recs[k][p], cams[k].tile_w, cams[k].tile_h)
-                                        : orect_b;
-    const bool nv = nvb && (rect.x & 0xffff) < (rect.y & 0xffff) && (rect.x >> 16) < (rect.y >> 16);
-    const uint32_t ox0 = orect.x & 0xffff, oy0 = orect.x >> 16, ox1 = orect.y & 0xffff, oy1 = orect.y >> 16;
-    const bool ov = ox1 > ox0 && oy1 > oy0;
-    uint32_t nx0 = rect.x & 0xffff, ny0 = rect.x >> 16, nx1 = rect.y & 0xffff, ny1 = rect.y >> 16;
-    if (!nv) nx0 = ny0 = nx1 = ny1 = 0;
-    const uint32_t an = nv ? (nx1 - nx0) * (ny1 - ny0) : 0u;
-    const uint32_t ao = ov ? (ox1 - ox0) * (oy1 - oy0) : 0u;
-    uint32_t ix = 0, iy = 0;
-    if (nv && ov) {
-        const int lx = max((int)nx0, (int)ox0), hx = min((int)nx1, (int)ox1);
-        const int ly = max((int)ny0, (int)oy0), hy = min((int)ny1, (int)oy1);
-        ix = hx > lx ? (uint32_t)(hx - lx) : 0u;
-        iy = hy > ly ? (uint32_t)(hy - ly) : 0u;
-    }
-    const uint32_t items = an + ao - ix * iy;
-    d.new_vis = nv;
-    d.old_vis = ov;
-    d.old_depth = ov ? clean_recs[k][p].depth : 0.0f;
-    d.pad[0] = d.pad[1] = d.pad[2] = 0u;
-    d.n_items = items;
-    d.nx0 = (uint16_t)nx0;
-    d.ny0 = (uint16_t)ny0;
-    d.nx1 = (uint16_t)nx1;
-    d.ny1 = (uint16_t)ny1;
-    d.ox0 = (uint16_t)ox0;
-    d.oy0 = (uint16_t)oy0;
-    d.ox1 = (uint16_t)ox1;
-    d.oy1 = (uint16_t)oy1;
-    if (!nv) d.rec = BlendRec{0, 0, 0, 0, 0, 0, -INFINITY, -INFINITY, 0, 0, 0, 0};
-    desc[bk] = d;
-    n_items[bk] = items;
-    CmpAcc z;
-    z.sse_fx = 0ull;
-    z.maxabs_bits = 0u;
-    z.footprint = 0u;
-    z.nonfinite = 0u;
-    z.clamps = (k == 0) ? clamps : 0u;   // clamps reported once per variant, on view 0
-    z.clean_nonfinite_replaced = 0u;
-    z.pad = 0u;
-    z.reg_actual = 0ull;
-    z.ssim_fx = 0ull;
-    // contamination prediction: the cells the primitive's tile rects meet, before
-    // and after the upset, when its stored words changed
-    const int tw = cams[k].tile_w, th = cams[k].tile_h;
-    z.reg_pred = changed ? rect_cells(orect_b, cams[k].W, cams[k].H, tw, th) |
-                               rect_cells(rect_b, cams[k].W, cams[k].H, tw, th)
-                         : 0ull;
-    acc[bk] = z;
-}
-
-// Exclusive scan of the dirty-tile counts of the B*K <= kMaxPairs (variant,
-// view) pairs (single block of 1024 threads, kPairsPerThread consecutive pairs
-// each); resets the work-queue counters.
-constexpr int kPairsPerThread = kMaxPairs / 1024;
-__global__ __launch_bounds__(1024) void k_items_scan(const uint32_t* n_items, int total, uint32_t* item_off,
-                                                     unsigned int* queue) {
-    __shared__ uint32_t wsum[32];
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    uint32_t a[kPairsPerThread];
-    uint32_t items = 0;
-#pragma unroll
-    for (int j = 0; j < kPairsPerThread; j++) {
-        const int p = tid * kPairsPerThread + j;
-        a[j] = p < total ? n_items[p] : 0u;
-        items += a[j];
-    }
-    uint32_t x = items;
-    for (int o = 1; o < 32; o <<= 1) {
-        uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) wsum[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        uint32_t s = wsum[lane];
-        for (int o = 1; o < 32; o <<= 1) {
-            uint32_t y = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += y;
+    int ny0 = 0, ny1 = 0, oy0 = 0, oy1 = 0;   // lane k: the tile rows of view k
+    if (lane < K) {
+        const int k = lane, bk = b * K + k;
+        const ViewPtrs& v = views[k];
+        const int tw = v.tile_w, th = v.tile_h;
+        DirtyDesc d;
+        uint2 rect = make_uint2(0, 0);
+        float rad = 0.0f;
+        const bool nvb = ok && preprocess_core(SharedSrc{sv[wib]}, sh_degree, cams[k], d.rec, rect, rad);
+        const uint2 orect_b = ok ? v.rects[p] : make_uint2(0, 0);   // binned rects (contamination cells)
+        const uint2 rect_b = nvb ? rect : make_uint2(0, 0);
+        // dirty tiles: the binned rects cut to the records' alpha boxes
+        if (nvb) rect = alpha_tiles(rect, d.rec, tw, th);
+        const bool binned = orect_b.y != 0u;
+        d.old = ok ? v.recs[p] : BlendRec{0, 0, 0, 0, 0, 0, -INFINITY, -INFINITY, 0, 0, 0, 0};
+        const uint2 orect = binned ? alpha_tiles(orect_b, d.old, tw, th) : make_uint2(0, 0);
+        const bool nv = nvb && (rect.x & 0xffff) < (rect.y & 0xffff) && (rect.x >> 16) < (rect.y >> 16);
+        const bool ov = (orect.x & 0xffff) < (orect.y & 0xffff) && (orect.x >> 16) < (orect.y >> 16);
+        if (!nv) {
+            rect = make_uint2(0, 0);
+            d.rec = BlendRec{0, 0, 0, 0, 0, 0, -INFINITY, -INFINITY, 0, 0, 0, 0};
         }
-        wsum[lane] = s;
+        const uint2 oc = ov ? orect : make_uint2(0, 0);
+        d.nx0 = (uint16_t)(rect.x & 0xffff);
+        d.ny0 = (uint16_t)(rect.x >> 16);
+        d.nx1 = (uint16_t)(rect.y & 0xffff);
+        d.ny1 = (uint16_t)(rect.y >> 16);
+        d.ox0 = (uint16_t)(oc.x & 0xffff);
+        d.oy0 = (uint16_t)(oc.x >> 16);
+        d.ox1 = (uint16_t)(oc.y & 0xffff);
+        d.oy1 = (uint16_t)(oc.y >> 16);
+        ny0 = d.ny0;
+        ny1 = d.ny1;
+        oy0 = d.oy0;
+        oy1 = d.oy1;
+        // the place of both entries in the view's order: an upset that leaves the depth
+        // alone leaves the place alone
+        const uint32_t orank = binned ? v.rank[p] : kNoRank;
+        d.old_rank = ov ? orank : kNoRank;
+        d.new_rank = kNoRank;
+        if (nv)
+            d.new_rank = binned && __float_as_uint(d.old.depth) == __float_as_uint(d.rec.depth)
+                             ? orank
+                             : order_lower_bound(v.sdk, v.sid, (uint32_t)n, __float_as_uint(d.rec.depth), p);
+        d.prim = p;
+        d.pad = 0u;
+        desc[bk] = d;
+        CmpAcc z;
+        z.sse_fx = 0ull;
+        z.maxabs_bits = 0u;
+        z.footprint = 0u;
+        z.nonfinite = 0u;
+        z.clamps = (k == 0) ? clamps : 0u;   // clamps reported once per variant, on view 0
+        z.clean_nonfinite_replaced = 0u;
+        z.pad = 0u;
+        z.reg_actual = 0ull;
+        z.ssim_fx = 0ull;
+        // contamination prediction: the cells the primitive's tile rects meet, before
+        // and after the upset, when its stored words changed
+        z.reg_pred = changed ? rect_cells(orect_b, v.W, v.H, tw, th) | rect_cells(rect_b, v.W, v.H, tw, th) : 0ull;
+        acc[bk] = z;
     }
-    __syncthreads();
-    uint32_t run = x - items + (wid > 0 ? wsum[wid - 1] : 0u);   // exclusive offset of this thread's first pair
+    // the variant's tile rows, in any order among the variants: one per lane, whole
+    // warps writing consecutive items
+    const uint32_t cnt = (uint32_t)Union1(ny0, ny1, oy0, oy1).len;
+    uint32_t incl = cnt;
 #pragma unroll
-    for (int j = 0; j < kPairsPerThread; j++) {
-        const int p = tid * kPairsPerThread + j;
-        if (p < total) item_off[p] = run;
-        run += a[j];
-        if (p == total - 1) item_off[total] = run;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
     }
-    if (tid == 0) {
-        queue[0] = 0u;
-        queue[1] = 0u;
-        queue[2] = 0u;
-        queue[3] = 0u;
-        queue[4] = 0u;
-        queue[6] += 1u;   // batch generation (tags of the dirty-tile SSIM maps)
+    const uint32_t excl = incl - cnt, total = __shfl_sync(0xffffffffu, incl, 31);
+    uint32_t base = 0;
+    if (lane == 0 && total) base = atomicAdd(&queue[1], total);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    for (uint32_t q0 = 0; q0 < total; q0 += 32) {
+        const uint32_t q = q0 + (uint32_t)lane;
+        int s = 0;   // the last lane whose offset is <= q
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1) {
+            const int m = s + step;
+            if (__shfl_sync(0xffffffffu, excl, m) <= q) s = m;
+        }
+        const int j = (int)(q - __shfl_sync(0xffffffffu, excl, s));
+        const int a0 = __shfl_sync(0xffffffffu, ny0, s), a1 = __shfl_sync(0xffffffffu, ny1, s);
+        const int b0 = __shfl_sync(0xffffffffu, oy0, s), b1 = __shfl_sync(0xffffffffu, oy1, s);
+        if (q < total) rows[base + q] = make_uint2((uint32_t)(b * K + s), (uint32_t)Union1(a0, a1, b0, b1).at(j) | ((uint32_t)s << 16));
     }
 }
 
@@ -725,18 +717,15 @@ gs_status launch_preprocess(const gs_scene* s, const DevCamera& cam, BlendRec* r
 }
 
 gs_status launch_inject_prep(const gs_scene* s, const DevCamera* dev_cams, int K, const gs_flip* flips, int B,
-                             int guard_mode, uint64_t mask, const uint2* const* dev_clean_rects,
-                             const BlendRec* const* dev_clean_recs, DirtyDesc* desc, uint32_t* item_off, CmpAcc* acc,
-                             unsigned int* queue, cudaStream_t st) {
-    if (B * K > kMaxPairs || K > 32) return set_error(GS_ERR_ARG, "B * K must be <= 8192 and K <= 32");
-    // the per-(variant, view) item counts go to the tail of item_off, past the B*K+1 offsets
-    uint32_t* n_items = item_off + (B * K + 1);
+                             int guard_mode, uint64_t mask, const void* dev_views, DirtyDesc* desc, uint2* rows,
+                             CmpAcc* acc, unsigned int* queue, cudaStream_t st) {
+    if (B * K > kMaxPairs || K > 32) return set_error(GS_ERR_ARG, "B * K must be <= 65536 and K <= 32");
     const int blocks = (B + kPrepWarps - 1) / kPrepWarps;
 #define GS_PREP(F)                                                                                            \
     k_inject_prep<F><<<blocks, kPrepWarps * 32, 0, st>>>(s->planes, s->n, s->nwords, s->sh_degree, dev_cams, K, \
                                                          flips, B, guard_mode, mask, s->dev_box, s->pbox_lo,    \
-                                                         s->pbox_hi, s->nbox_words, dev_clean_rects,            \
-                                                         dev_clean_recs, desc, n_items, acc)
+                                                         s->pbox_hi, s->nbox_words, (const ViewPtrs*)dev_views, \
+                                                         desc, rows, queue, acc)
     if (s->fmt == GS_FP32)
         GS_PREP(GS_FP32);
     else if (s->fmt == GS_FP16)
@@ -744,7 +733,6 @@ gs_status launch_inject_prep(const gs_scene* s, const DevCamera* dev_cams, int K
     else
         GS_PREP(GS_BF16);
 #undef GS_PREP
-    k_items_scan<<<1, 1024, 0, st>>>(n_items, B * K, item_off, queue);
     GS_CUDA(cudaGetLastError());
     return GS_OK;
 }

@@ -584,6 +584,7 @@ gs_status build_tile_lists(RenderWork& w, uint64_t n, int tiles_x, int tiles_y, 
     // depth order of the primitives
     GS_TRY(radix_sort(w.dkey, w.dval, nullptr, n, 32, w.hist, w.hpart, cur, st));
     const uint32_t* sorted_ids = w.dval[cur];
+    w.cur = cur;
     w.passes[0] = 4;   // 32-bit depth keys, 8 bits a pass
     // tiles per primitive in depth order, exclusive scan, pair count
     unsigned blocks = (unsigned)div_up(std::max<uint64_t>(n, 1), 256);

@@ -214,41 +214,59 @@ SsimW ssim_weights() {
 // value (deltas written by the blend kernel, found through the per-(variant,
 // view) tile -> plan slot map and the slot's block -> delta index table).
 // Each tile within one tile of a planned tile is claimed once (atomicMax of a
-// per-batch generation tag) and processed by one block.
+// per-batch generation tag) by the claim kernel, which lists it (queue[7] counts);
+// the tiles listed are then processed by one block each.
 // ---------------------------------------------------------------------------
+
+// Thread per (plan slot, one of the 3x3 tiles around it): claims the tile if a
+// changed pixel's window reaches it -- the tile itself if any pixel changed, a
+// neighbour if one changed within 5 pixels of the shared edge.  (Claimed by the
+// processing blocks, one pair after another, the 9 tests of each slot cost more
+// than the tiles.)
+__global__ __launch_bounds__(256) void k_ssim_claim(const ViewPtrs* __restrict__ views, int K,
+                                                    unsigned int* __restrict__ queue, SsimBufs sb) {
+    const uint32_t n_items = min(queue[3], sb.slot_cap);   // beyond it the batch reports an overflow
+    const unsigned long long gen = (unsigned long long)queue[6] << 32;
+    const int lane = threadIdx.x & 31;
+    for (uint32_t base = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < n_items * 9u;
+         base += gridDim.x * blockDim.x) {
+        const uint32_t pair = base + (uint32_t)lane;
+        bool claim = false;
+        if (pair < n_items * 9u) {
+            const uint32_t slot = pair / 9u, nb = pair % 9u;
+            const unsigned f = sb.slot_flags[slot];
+            const int dx = (int)(nb % 3u) - 1, dy = (int)(nb / 3u) - 1;
+            if ((f & 16u) && (dx == 0 || (f & (dx < 0 ? 1u : 2u))) && (dy == 0 || (f & (dy < 0 ? 4u : 8u)))) {
+                const uint32_t bk = sb.plan[slot].bk, tile = sb.plan[slot].tile;
+                const ViewPtrs& v = views[bk % (uint32_t)K];
+                const int tiles_y = (v.H + kTile - 1) / kTile;
+                const int tx = (int)(tile % (uint32_t)v.tiles_x) + dx, ty = (int)(tile / (uint32_t)v.tiles_x) + dy;
+                if (tx >= 0 && ty >= 0 && tx < v.tiles_x && ty < tiles_y)
+                    claim = atomicMax(&sb.ssim_map[(size_t)bk * sb.max_tiles + (size_t)(ty * v.tiles_x + tx)], gen) < gen;
+            }
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, claim);
+        uint32_t at = 0;
+        if (lane == 0 && m) at = atomicAdd(&queue[7], (unsigned)__popc(m));
+        at = __shfl_sync(0xffffffffu, at, 0) + (uint32_t)__popc(m & ((1u << lane) - 1u));
+        if (claim) sb.claims[at] = pair;
+    }
+}
+
 __global__ __launch_bounds__(kSsimThreads) void k_dirty_ssim(const ViewPtrs* __restrict__ views, int K,
-                                                        const PlanItem* __restrict__ plan,
                                                         const unsigned int* __restrict__ queue, SsimBufs sb,
                                                         SsimW w11, CmpAcc* __restrict__ acc) {
     __shared__ SsimStage s;
-    __shared__ int claim;
-    const uint32_t n_items = queue[1];
+    const PlanItem* __restrict__ plan = sb.plan;
     const unsigned long long gen = (unsigned long long)queue[6] << 32;
-    for (uint32_t pair = blockIdx.x; pair < n_items * 9u; pair += gridDim.x) {
-        const uint32_t slot = pair / 9u, nb = pair % 9u;
-        const PlanItem& it = plan[slot];
+    const uint32_t n_tiles = queue[7];
+    for (uint32_t k = blockIdx.x; k < n_tiles; k += gridDim.x) {
+        const uint32_t pair = sb.claims[k], nb = pair % 9u;
+        const PlanItem& it = plan[pair / 9u];
         const ViewPtrs& v = views[it.bk % (uint32_t)K];
         const int tiles_y = (v.H + kTile - 1) / kTile;
         const int tx = (int)(it.tile % (uint32_t)v.tiles_x) + (int)(nb % 3u) - 1;
         const int ty = (int)(it.tile / (uint32_t)v.tiles_x) + (int)(nb / 3u) - 1;
-        if (threadIdx.x == 0) {
-            claim = 0;
-            // only where a changed pixel's window reaches: the tile itself if any pixel
-            // changed, a neighbour if one changed within 5 pixels of the shared edge
-            const unsigned f = slot < sb.slot_cap ? sb.slot_flags[slot] : 31u;
-            const int dx = (int)(nb % 3u) - 1, dy = (int)(nb / 3u) - 1;
-            const bool reach = (f & 16u) && (dx == 0 || (f & (dx < 0 ? 1u : 2u))) &&
-                               (dy == 0 || (f & (dy < 0 ? 4u : 8u)));
-            if (reach && tx >= 0 && ty >= 0 && tx < v.tiles_x && ty < tiles_y) {
-                const unsigned long long old =
-                    atomicMax(&sb.ssim_map[(size_t)it.bk * sb.max_tiles + (size_t)(ty * v.tiles_x + tx)], gen);
-                claim = old < gen;
-            }
-        }
-        __syncthreads();
-        const int claimed = claim;
-        __syncthreads();   // every thread has read the flag before thread 0 rewrites it
-        if (!claimed) continue;   // block-uniform
         // the 3x3 tiles around (tx, ty): delta index and active mask of each 8x4 block
         // (0xffffffff / 0: no delta), resolved once for the staging below
         __shared__ uint32_t nb_gi[9][8], nb_mask[9][8];
@@ -319,10 +337,10 @@ gs_status launch_ssim_finalize(const unsigned long long* acc, int count, int W, 
     return GS_OK;
 }
 
-gs_status launch_dirty_ssim(const void* dev_views, int K, const void* plan, const unsigned int* queue,
-                            const SsimBufs& sb, CmpAcc* acc, cudaStream_t st) {
-    k_dirty_ssim<<<num_sms() * 4, kSsimThreads, 0, st>>>((const ViewPtrs*)dev_views, K, (const PlanItem*)plan, queue, sb,
-                                                     ssim_weights(), acc);
+gs_status launch_dirty_ssim(const void* dev_views, int K, unsigned int* queue, const SsimBufs& sb, CmpAcc* acc,
+                            cudaStream_t st) {
+    k_ssim_claim<<<num_sms() * 4, 256, 0, st>>>((const ViewPtrs*)dev_views, K, queue, sb);
+    k_dirty_ssim<<<num_sms() * 4, kSsimThreads, 0, st>>>((const ViewPtrs*)dev_views, K, queue, sb, ssim_weights(), acc);
     GS_CUDA(cudaGetLastError());
     return GS_OK;
 }
