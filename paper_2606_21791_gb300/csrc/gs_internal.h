@@ -254,15 +254,20 @@ struct RenderWork {
     uint32_t* dval[2] = {nullptr, nullptr};    // primitive ids (ping-pong)
     uint32_t* cnt = nullptr;                    // tiles per primitive, in depth order
     uint32_t* off = nullptr;                    // exclusive scan of cnt
+    uint2* srect = nullptr;                     // tile rects, in depth order
+    uint32_t* tab = nullptr;                    // counting tables of the tile lists [tab_words]
+    size_t tab_words = 0;
     uint32_t* pkey[2] = {nullptr, nullptr};    // pair tile keys
-    uint32_t* pval[2] = {nullptr, nullptr};    // pair primitive ids
+    uint32_t* pval[2] = {nullptr, nullptr};    // pair primitive ids ([0]: the lists when made by counting)
+    uint64_t radix_pairs = 0;                   // pairs that pkey and pval[1] hold (large grids only)
+    uint64_t hist_items = 0;                    // items that hist and hpart serve
     uint32_t* hist = nullptr;                   // radix histograms
     unsigned long long* hpart = nullptr;        // block partials of the histogram scan
     uint32_t* scan_tmp = nullptr;               // block sums for scans
     uint2* ranges = nullptr;
     unsigned long long* total = nullptr;        // [0] pair count, [1] overflow flag
     unsigned long long* host_total = nullptr;   // pinned mirror
-    int passes[2] = {0, 0};                     // radix passes of the last build: depth keys, pair tile keys
+    int passes[2] = {0, 0};                     // 8-bit digits of the last build's keys: depths, tile ids
     int cur = 0;                                // dkey / dval buffer that holds the last build's depth order
 };
 
