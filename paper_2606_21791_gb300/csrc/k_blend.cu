@@ -238,9 +238,112 @@ __device__ __forceinline__ Pix2Geo pix2_geo(int tile_x, int tile_y, int tw, int 
     return g;
 }
 
+// Conservative test of a rectangle, all in fp32: false only if the blend cannot reach
+// alpha >= 1/255 for record q at any pixel centre of the rectangle
+// [x0, x1] x [y0, y1].  The blend's offsets d = mean - pixel are fp32
+// differences, and rounding is monotone, so every pixel's d lies in the box
+// spanned by the rounded corner offsets.  Its power is -q(d)/2 for
+// q(d) = ca dx^2 + 2 cb dx dy + cc dy^2 up to a few ulps of
+// M = ((|ca| + |cb|) max dx^2 + (|cc| + |cb|) max dy^2)/2 >= the sum of |terms|;
+// g = 1e-5 covers that and the rounding of this test's own q (both about
+// 1e-6 M).  alpha >= 1/255 needs -q/2 + g M >= -L with L = ln(255 opacity)
+// + 1e-3 (the margin covers the fast log and exp2), so the rectangle is
+// unreachable when the minimum of q over it exceeds 2 L + 2 g M.  With ca, cc > 0
+// the minimum over each edge is that of a convex 1-D quadratic; it is 0 if the
+// mean lies inside (then: reachable).  NaN opacity, or terms near overflow
+// (where the blend's own power can be NaN, which it blends): reachable.
+__device__ __forceinline__ bool rect_reachable(float mx, float my, float ca, float cb, float cc, float opac, float x0,
+                                               float x1, float y0, float y1) {
+    const float L = __logf(255.0f * opac) + 1e-3f;
+    if (!(ca > 1e-30f) || !(cc > 1e-30f) || !(L < 3.0e38f)) return true;
+    const float dx0 = mx - x1, dx1 = mx - x0;
+    const float dy0 = my - y1, dy1 = my - y0;
+    const float mdx = fmaxf(dx0 * dx0, dx1 * dx1), mdy = fmaxf(dy0 * dy0, dy1 * dy1);
+    const float M = 0.5f * ((ca + fabsf(cb)) * mdx + (cc + fabsf(cb)) * mdy);
+    if (!(M < 1.0e37f)) return true;   // terms near overflow: the blend's power may be NaN
+    if (L < 0.0f) return false;        // alpha <= opacity < 1/255 everywhere (with margin)
+    if (dx0 <= 0.0f && dx1 >= 0.0f && dy0 <= 0.0f && dy1 >= 0.0f) return true;
+    auto qf = [&](float dx, float dy) { return ca * dx * dx + 2.0f * cb * dx * dy + cc * dy * dy; };
+    // approximate reciprocals: they only place the nearest point of an edge, and
+    // a relative error e there raises q by about e^2 M, far inside the margin
+    const float rca = __fdividef(1.0f, ca), rcc = __fdividef(1.0f, cc);
+    // the nearest point of each edge (dx fixed: dy = -cb dx / cc; dy fixed: dx = -cb dy / ca), clamped to it
+    const float e0 = qf(dx0, fminf(fmaxf(-cb * dx0 * rcc, dy0), dy1));
+    const float e1 = qf(dx1, fminf(fmaxf(-cb * dx1 * rcc, dy0), dy1));
+    const float e2 = qf(fminf(fmaxf(-cb * dy0 * rca, dx0), dx1), dy0);
+    const float e3 = qf(fminf(fmaxf(-cb * dy1 * rca, dx0), dx1), dy1);
+    const float qmin = fminf(fminf(e0, e1), fminf(e2, e3));
+    return !(qmin > 2.0f * L + 2.0e-5f * M);
+}
+
+// The clean views' stages: records as they are, one entry per thread and batch.
+constexpr int kStageMax = kBT / 2;
+struct RawStage {
+    float4 q0[kStageMax];   // mx, my, ca, cb
+    float4 q1[kStageMax];   // cc, opacity, ex, ey
+    float4 q2[kStageMax];   // r, g, b, depth
+};
+
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+    const unsigned saddr = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(saddr), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
+    const unsigned saddr = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(saddr), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// Streams a tile's list [rg.x, rg.y) through two stages, one entry per thread and
+// batch: while a batch is blended, the records of the next one are copied into the
+// other stage and the indices of the one after are loaded, so a batch costs one
+// barrier and no memory latency.  copy(stage, id) may bring more of this thread's
+// entry; blend(stage, its number, entries, list index of entry 0); done: this
+// thread's pixels need no more entries (the block leaves when all do).  For the
+// clean views' two passes, which have few warps per SM to hide a batch's loads
+// behind (registers, list rings): with the ellipse test, 0.44 + 0.90 ms for two
+// 1600x1040 views of 300k primitives against 0.44 + 0.97 staged in turn, and 0.48 +
+// 1.01 staged without the test.  The plain renders have warps enough: 208 us
+// streamed, 207 staged.
+template <class Copy, class Blend, class Done>
+__device__ __forceinline__ void stream_list(RawStage (&st)[2], const BlendRec* __restrict__ recs,
+                                            const uint32_t* __restrict__ ids, uint2 rg, const Copy& copy,
+                                            const Blend& blend, const Done& done) {
+    const uint32_t nb = blockDim.x, t = threadIdx.x;
+    auto fetch = [&](int k, uint32_t id) {
+        const float4* src = reinterpret_cast<const float4*>(recs + id);
+        cp_async16(&st[k].q0[t], src);
+        cp_async16(&st[k].q1[t], src + 1);
+        cp_async16(&st[k].q2[t], src + 2);
+        copy(k, id);
+    };
+    if (rg.x + t < rg.y) fetch(0, ids[rg.x + t]);
+    uint32_t next = rg.x + nb + t < rg.y ? ids[rg.x + nb + t] : 0u;
+    int k = 0;
+    for (uint32_t base = rg.x; base < rg.y; base += nb, k ^= 1) {
+        cp_async_wait_all();
+        // the batch has landed for every thread, and every thread is done with the other stage
+        if (__syncthreads_count(done()) == (int)nb) break;
+        if (base + nb + t < rg.y) fetch(k ^ 1, next);
+        next = base + 2 * nb + t < rg.y ? ids[base + 2 * nb + t] : 0u;
+        blend(st[k], k, (int)min(nb, rg.y - base), base - rg.x);
+    }
+    cp_async_wait_all();   // leave no copy in flight
+}
+
 // Entries [c, c + 32) of a staged batch for one warp: cull 32 boxes against the
 // warp's 8x8 pixel block with one ballot, then walk the survivors in list order.
-template <class Apply, class After>
+// CONIC: survivors whose ellipse misses the block (rect_reachable: no pixel of it
+// would take them) are dropped as well, 32 tests side by side, when at least
+// kConicMin are left to gain from it: a box keeps the blocks at the corners of a
+// slanted ellipse.  One 1600x1040 view of 2M primitives: 206 us without, 195 at 5,
+// 197 at 8, 201 at 2 (189 to 195 over boxes of the same kind).  Not for the compared
+// renders of corrupted scenes: there most of a deep list is exploded primitives whose
+// ellipse does cover the block (four renders with 1000 upsets each: 558 us without,
+// 630 with).
+constexpr int kConicMin = 5;
+
+template <bool CONIC, class Apply, class After>
 __device__ __forceinline__ void blend_chunk2(const Stage& s, int c, int cnt, const Pix2Geo& g, const Apply& apply,
                                              const After& after) {
     const int lane = threadIdx.x & 31;
@@ -250,10 +353,40 @@ __device__ __forceinline__ void blend_chunk2(const Stage& s, int c, int cnt, con
         const float4 bx = s.box[j];
         pass = !(bx.y < g.wx0 || bx.x > g.wx1 || bx.w < g.wy0 || bx.z > g.wy1);
     }
-    const unsigned m = __ballot_sync(0xffffffffu, pass);
+    unsigned m = __ballot_sync(0xffffffffu, pass);
+    if (CONIC && __popc(m) >= kConicMin) {
+        if (pass) {
+            const float4 q0 = s.q0[j], q1 = s.q1[j];
+            pass = rect_reachable(q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, g.wx0, g.wx1, g.wy0, g.wy1);
+        }
+        m = __ballot_sync(0xffffffffu, pass);
+    }
     auto fetch = [&](int e) {
         const float4 q1 = s.q1[e];
         return EntryQ{s.q0[e], q1.x, q1.y, q1.z, q1.w, s.qb[e]};
+    };
+    walk_survivors2(m, c, fetch, g.pxc, g.pycA, g.pycB, apply, after);
+}
+
+template <bool CONIC, class Apply, class After>
+__device__ __forceinline__ void blend_chunk2(const RawStage& s, int c, int cnt, const Pix2Geo& g, const Apply& apply,
+                                             const After& after) {
+    const int j = c + (threadIdx.x & 31);
+    bool pass = false;
+    float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
+    if (j < cnt) {
+        a = s.q0[j];
+        b = s.q1[j];
+        pass = !(a.x + b.z < g.wx0 || a.x - b.z > g.wx1 || a.y + b.w < g.wy0 || a.y - b.w > g.wy1);
+    }
+    unsigned m = __ballot_sync(0xffffffffu, pass);
+    if (CONIC && __popc(m) >= kConicMin) {
+        pass = pass && rect_reachable(a.x, a.y, a.z, a.w, b.x, b.y, g.wx0, g.wx1, g.wy0, g.wy1);
+        m = __ballot_sync(0xffffffffu, pass);
+    }
+    auto fetch = [&](int e) {
+        const float4 q1 = s.q1[e], q2 = s.q2[e];
+        return EntryQ{s.q0[e], q1.x, q1.y, q2.x, q2.y, q2.z};
     };
     walk_survivors2(m, c, fetch, g.pxc, g.pycA, g.pycB, apply, after);
 }
@@ -363,7 +496,7 @@ __global__ __launch_bounds__(kBT / 2) void k_blend_full(const BlendRec* __restri
         __syncthreads();
         staged += cnt;
         for (int c = 0; c < cnt && !__all_sync(0xffffffffu, pA.done && pB.done); c += 32)
-            blend_chunk2(s, c, cnt, g, apply, [] {});
+            blend_chunk2<MODE == 0>(s, c, cnt, g, apply, [] {});
         // also the barrier that lets the next batch overwrite the stage
         if (__syncthreads_count(pA.done && pB.done) == (int)blockDim.x) break;
     }
@@ -506,8 +639,8 @@ __global__ __launch_bounds__(kBT / 2) void k_blend_clean(const BlendRec* __restr
                                                         uint32_t* __restrict__ tile_last, uint32_t* __restrict__ counts,
                                                         unsigned int* __restrict__ clean_nonfin, ListOut lo) {
     extern __shared__ __align__(16) unsigned char ring_mem[];   // FILL: one ListRing per warp
-    __shared__ Stage s;
-    __shared__ uint32_t rk[kBT];   // ranks of the staged entries
+    __shared__ RawStage st[2];
+    __shared__ uint32_t rks[2][kStageMax];   // ranks of the staged entries
     const int tile = blockIdx.x, lane = threadIdx.x & 31;
     ListRing* ring = FILL ? reinterpret_cast<ListRing*>(ring_mem) + (threadIdx.x >> 5) : nullptr;
     const uint32_t P = (uint32_t)(tw * th);
@@ -527,6 +660,7 @@ __global__ __launch_bounds__(kBT / 2) void k_blend_clean(const BlendRec* __restr
     };
     if (FILL) put_row(0u);
     uint32_t at = 0;   // list index of entry 0 of the staged batch
+    const uint32_t* rk = rks[0];
     auto apply = [&](int e, bool v, bool okA, bool okB, float2 a, float cr, float cg, float cb) {
         clean_entry<FILL>(pA, v && !pA.done, okA, a.x, cr, cg, cb, rk[e], at + (uint32_t)e, lo, ring, lane);
         clean_entry<FILL>(pB, v && !pB.done, okB, a.y, cr, cg, cb, rk[e], at + (uint32_t)e, lo, ring, lane + 32);
@@ -539,23 +673,18 @@ __global__ __launch_bounds__(kBT / 2) void k_blend_clean(const BlendRec* __restr
         if (pending(pA) >= 4) flush4(pA, *ring, lane, lo);
         if (pending(pB) >= 4) flush4(pB, *ring, lane + 32, lo);
     };
-    for (uint32_t base = rg.x; base < rg.y; base += P) {
-        const int cnt = (int)min(P, rg.y - base);
-        for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
-            const uint32_t id = ids[base + j];
-            stage_put(s, j, load_rec(recs, id));
-            rk[j] = rank[id];
-        }
-        __syncthreads();
-        at = base - rg.x;
-        for (int c = 0; c < cnt && !__all_sync(0xffffffffu, pA.done && pB.done); c += 32) {
-            const uint32_t li = at + (uint32_t)c;
-            if (FILL && li > 0 && li % kRowStride == 0 && li / kRowStride <= rows) put_row(li / kRowStride);
-            blend_chunk2(s, c, cnt, g, apply, drain);
-        }
-        // also the barrier that lets the next batch overwrite the stage
-        if (__syncthreads_count(pA.done && pB.done) == (int)blockDim.x) break;
-    }
+    stream_list(
+        st, recs, ids, rg, [&](int k, uint32_t id) { cp_async4(&rks[k][threadIdx.x], rank + id); },
+        [&](const RawStage& s, int k, int cnt, uint32_t li0) {
+            at = li0;
+            rk = rks[k];
+            for (int c = 0; c < cnt && !__all_sync(0xffffffffu, pA.done && pB.done); c += 32) {
+                const uint32_t li = at + (uint32_t)c;
+                if (FILL && li > 0 && li % kRowStride == 0 && li / kRowStride <= rows) put_row(li / kRowStride);
+                blend_chunk2<true>(s, c, cnt, g, apply, drain);
+            }
+        },
+        [&] { return pA.done && pB.done; });
     if (FILL) {
         auto finish = [&](CleanPix& p, int col) {
             if (p.n <= lo.cap) {
@@ -748,50 +877,6 @@ __global__ void k_zero_acc(CmpAcc* acc, int count) {
 // ---------------------------------------------------------------------------
 
 
-// A pixel of a dirty tile keeps its clean value, bit for bit, when its clean
-// blend stopped before the first changed list position, or when its blend skips
-// both the removed (clean) and the inserted (corrupted) record (power > 0 or
-// alpha < 1/255, decided by the blend's own arithmetic): the state changes of
-// its blend are then those of the clean blend.  Every other pixel is "active"
-// and must be re-blended.
-// Conservative tile test, all in fp32: false only if the blend cannot reach
-// alpha >= 1/255 for record q at any pixel centre of the rectangle
-// [x0, x1] x [y0, y1].  The blend's offsets d = mean - pixel are fp32
-// differences, and rounding is monotone, so every pixel's d lies in the box
-// spanned by the rounded corner offsets.  Its power is -q(d)/2 for
-// q(d) = ca dx^2 + 2 cb dx dy + cc dy^2 up to a few ulps of
-// M = ((|ca| + |cb|) max dx^2 + (|cc| + |cb|) max dy^2)/2 >= the sum of |terms|;
-// g = 1e-5 covers that and the rounding of this test's own q (both about
-// 1e-6 M).  alpha >= 1/255 needs -q/2 + g M >= -L with L = ln(255 opacity)
-// + 1e-3 (the margin covers the fast log and exp2), so the rectangle is
-// unreachable when the minimum of q over it exceeds 2 L + 2 g M.  With ca, cc > 0
-// the minimum over each edge is that of a convex 1-D quadratic; it is 0 if the
-// mean lies inside (then: reachable).  NaN opacity, or terms near overflow
-// (where the blend's own power can be NaN, which it blends): reachable.
-__device__ __forceinline__ bool rect_reachable(float mx, float my, float ca, float cb, float cc, float opac, float x0,
-                                               float x1, float y0, float y1) {
-    const float L = __logf(255.0f * opac) + 1e-3f;
-    if (L < 0.0f) return false;   // alpha <= opacity < 1/255 everywhere (with margin); NaN falls through
-    if (!(ca > 1e-30f) || !(cc > 1e-30f) || !(L < 3.0e38f)) return true;
-    const float dx0 = mx - x1, dx1 = mx - x0;
-    const float dy0 = my - y1, dy1 = my - y0;
-    if (dx0 <= 0.0f && dx1 >= 0.0f && dy0 <= 0.0f && dy1 >= 0.0f) return true;
-    const float mdx = fmaxf(dx0 * dx0, dx1 * dx1), mdy = fmaxf(dy0 * dy0, dy1 * dy1);
-    const float M = 0.5f * ((ca + fabsf(cb)) * mdx + (cc + fabsf(cb)) * mdy);
-    if (!(M < 1.0e37f)) return true;   // terms near overflow: the blend's power may be NaN
-    auto qf = [&](float dx, float dy) { return ca * dx * dx + 2.0f * cb * dx * dy + cc * dy * dy; };
-    // approximate reciprocals: they only place the nearest point of an edge, and
-    // a relative error e there raises q by about e^2 M, far inside the margin
-    const float rca = __fdividef(1.0f, ca), rcc = __fdividef(1.0f, cc);
-    // the nearest point of each edge (dx fixed: dy = -cb dx / cc; dy fixed: dx = -cb dy / ca), clamped to it
-    const float e0 = qf(dx0, fminf(fmaxf(-cb * dx0 * rcc, dy0), dy1));
-    const float e1 = qf(dx1, fminf(fmaxf(-cb * dx1 * rcc, dy0), dy1));
-    const float e2 = qf(fminf(fmaxf(-cb * dy0 * rca, dx0), dx1), dy0);
-    const float e3 = qf(fminf(fmaxf(-cb * dy1 * rca, dx0), dx1), dy1);
-    const float qmin = fminf(fminf(e0, e1), fminf(e2, e3));
-    return !(qmin > 2.0f * L + 2.0e-5f * M);
-}
-
 // Tiles [t0, t1) of tile columns [c0, c1) whose pixel centres record q can reach
 // with alpha >= 1/255 somewhere in the rows of pixel centres [y0, y1]:
 // conservative, by the extent of the record's conic over the band.  The blend's
@@ -857,6 +942,13 @@ __device__ __forceinline__ void band_tiles(const BlendRec& q, float y0, float y1
     t0 = (int)fminf(fmaxf(f0, (float)c0), (float)c1);
     t1 = (int)fminf(fmaxf(f1, (float)t0), (float)c1);
 }
+
+// A pixel of a dirty tile keeps its clean value, bit for bit, when its clean
+// blend stopped before the first changed list position, or when its blend skips
+// both the removed (clean) and the inserted (corrupted) record (power > 0 or
+// alpha < 1/255, decided by the blend's own arithmetic): the state changes of
+// its blend are then those of the clean blend.  Every other pixel is "active"
+// and must be re-blended.
 
 // Plan: the candidate tiles of a batch.  Lane = tile row of a pair (the
 // injector's list): the columns that either record reaches in that row
