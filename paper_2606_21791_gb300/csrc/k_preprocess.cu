@@ -371,19 +371,28 @@ __global__ __launch_bounds__(kPrepThreads) void k_preprocess(const void* planes,
 // Full preprocess with the parameter planes staged by bulk copies (TMA)
 // ---------------------------------------------------------------------------
 // Persistent blocks of 128 threads walk tiles of 128 consecutive primitives.
-// For each tile one thread issues one bulk copy per parameter plane
-// (cp.async.bulk: the tile's 128 words of that plane) into one of two
-// shared-memory stages, completing on the stage's mbarrier, one tile ahead of
-// the tile being computed: a block keeps a whole tile's words (30 KB in fp32)
-// in flight while it computes the previous tile, where the per-thread kernel
-// above keeps eight loads.  A bulk copy needs 16-byte aligned addresses and a
+// For each tile the lanes of one warp issue one bulk copy per parameter plane
+// (cp.async.bulk: the tile's 128 words of that plane) into a shared-memory stage,
+// completing on the stage's mbarrier: a block has a whole tile's words (30 KB in
+// fp32 at SH degree 3) in flight, where the per-thread kernel above keeps eight
+// loads.  With two stages a tile is copied while the one before it is computed;
+// that is worth it only where the second stage costs no resident block (the
+// launch compares both occupancies: 16-bit scenes, and fp32 up to degree 1).
+// Otherwise one stage each, and the other blocks of the SM compute meanwhile: 2M
+// primitives in fp32 at degree 3, 600 MB, took 164 us with two stages (12 warps
+// per SM, a sixth of its slots, 42% of its issue cycles, one thread issuing the
+// copies) and take 115 us with one (28 warps; 0.77 of measured copy bandwidth).
+// The same in fp16, 364 MB: 99 us, 71% of the issue cycles, 1,370 instructions a
+// primitive; more warps or larger tiles do not change it (97 to 103 us).
+// A bulk copy needs 16-byte aligned addresses and a
 // size that is a multiple of 16 bytes; plane w of tile t starts at word
 // w n + 128 t, so this kernel runs when n is a multiple of 4 (fp32) or 8
 // (fp16/bf16) and the per-thread kernel otherwise.  Every wait is bounded: a
 // block whose wait gives up sets bit 1 of the scene's device error word, waits
 // (bounded again) for its copies in flight and returns.
-constexpr int kTmaStages = 2;
 constexpr unsigned kWaitLimit = 1u << 20;   // mbarrier polls before a wait gives up
+template <int DEG>
+constexpr int kShWords = 11 + 3 * (DEG + 1) * (DEG + 1);   // planes of a scene
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -415,32 +424,35 @@ struct StageSrc {
     }
 };
 
-template <int FMT>
-__global__ __launch_bounds__(kPrepThreads) void k_preprocess_tma(const void* planes, uint64_t n, int nwords,
-                                                                 int sh_degree, DevCamera cam, BlendRec* recs,
-                                                                 uint2* rects, uint32_t* keys, uint32_t* vals,
-                                                                 gs_record* dbg, unsigned int* err) {
+template <int FMT, int DEG>
+__global__ __launch_bounds__(kPrepThreads) void k_preprocess_tma(const void* planes, uint64_t n, int stages,
+                                                                 DevCamera cam, BlendRec* recs, uint2* rects,
+                                                                 uint32_t* keys, uint32_t* vals, gs_record* dbg,
+                                                                 unsigned int* err) {
     extern __shared__ __align__(128) unsigned char stage_mem[];
-    __shared__ __align__(8) uint64_t bar[kTmaStages];
+    __shared__ __align__(8) uint64_t bar[2];
+    constexpr int nwords = kShWords<DEG>;
     constexpr unsigned esz = FMT == GS_FP32 ? 4u : 2u;
     const int t = threadIdx.x;
-    const size_t stage_bytes = (size_t)nwords * kPrepThreads * esz;
+    constexpr size_t stage_bytes = (size_t)nwords * kPrepThreads * esz;
     const uint64_t ntile = (n + kPrepThreads - 1) / kPrepThreads;
     if (t == 0) {
-        for (int s = 0; s < kTmaStages; s++)
+        for (int s = 0; s < 2; s++)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&bar[s])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    // thread 0: the tile's planes into stage s, completing on bar[s]
+    // warp 0: the tile's planes into stage s, completing on bar[s]
     auto issue = [&](uint64_t tile, int s) {
         const uint64_t p0 = tile * kPrepThreads;
         const unsigned bytes = (unsigned)min((uint64_t)kPrepThreads, n - p0) * esz;
         unsigned char* dst = stage_mem + (size_t)s * stage_bytes;
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&bar[s])),
-                     "r"(bytes * (unsigned)nwords)
-                     : "memory");
-        for (int w = 0; w < nwords; w++) {
+        if (t == 0)
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&bar[s])),
+                         "r"(bytes * (unsigned)nwords)
+                         : "memory");
+        __syncwarp();
+        for (int w = t; w < nwords; w += 32) {
             const unsigned char* src = static_cast<const unsigned char*>(planes) + ((uint64_t)w * n + p0) * esz;
             asm volatile(
                 "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
@@ -449,20 +461,22 @@ __global__ __launch_bounds__(kPrepThreads) void k_preprocess_tma(const void* pla
                 : "memory");
         }
     };
+    const bool two = stages == 2;
     uint64_t tile = blockIdx.x;
-    if (t == 0 && tile < ntile) issue(tile, 0);
-    // tile k of this block uses stage k & 1 for the (k >> 1)-th time: mbarrier phase parity (k >> 1) & 1
+    if (t < 32 && tile < ntile) issue(tile, 0);
+    // one stage: tile k of this block is its k-th use (mbarrier phase parity k & 1); two:
+    // tile k uses stage k & 1 for the (k >> 1)-th time, and tile k + 1 is copied meanwhile
     for (int k = 0; tile < ntile; tile += gridDim.x, k++) {
-        const int s = k & 1;
-        const unsigned parity = (unsigned)(k >> 1) & 1u;
+        const int s = two ? k & 1 : 0;
+        const unsigned parity = (unsigned)(two ? k >> 1 : k) & 1u;
         const uint64_t next = tile + gridDim.x;
         // stage s ^ 1 was released by the barrier that ended the previous tile
-        if (t == 0 && next < ntile) issue(next, s ^ 1);
+        if (two && t < 32 && next < ntile) issue(next, s ^ 1);
         const bool ok = mbar_wait_bounded(&bar[s], parity);
         if (__syncthreads_or(!ok)) {
             if (t == 0) atomicOr(err, 2u);
             mbar_wait_bounded(&bar[s], parity);   // the block's copies in flight land first
-            if (next < ntile) mbar_wait_bounded(&bar[s ^ 1], (unsigned)((k + 1) >> 1) & 1u);
+            if (two && next < ntile) mbar_wait_bounded(&bar[s ^ 1], (unsigned)((k + 1) >> 1) & 1u);
             return;
         }
         const uint64_t i = tile * kPrepThreads + (uint64_t)t;
@@ -470,11 +484,12 @@ __global__ __launch_bounds__(kPrepThreads) void k_preprocess_tma(const void* pla
             BlendRec rec;
             uint2 rect = make_uint2(0, 0);
             float rad = 0.0f;
-            const bool vis = preprocess_core(StageSrc<FMT>{stage_mem + (size_t)s * stage_bytes, t}, sh_degree, cam,
-                                             rec, rect, rad);
+            const bool vis =
+                preprocess_core(StageSrc<FMT>{stage_mem + (size_t)s * stage_bytes, t}, DEG, cam, rec, rect, rad);
             write_prep(i, vis, rec, rect, rad, recs, rects, keys, vals, dbg);
         }
         __syncthreads();   // every thread is done with stage s before it is refilled
+        if (!two && t < 32 && next < ntile) issue(next, 0);
     }
 }
 
@@ -687,23 +702,38 @@ DevCamera make_dev_camera(const gs_camera& c, int tile_w, int tile_h) {
     return d;
 }
 
+template <int FMT, int DEG>
+gs_status launch_preprocess_tma(const gs_scene* s, const DevCamera& cam, BlendRec* recs, uint2* rects, uint32_t* keys,
+                                uint32_t* vals, gs_record* dbg, cudaStream_t st) {
+    const auto kernel = k_preprocess_tma<FMT, DEG>;
+    constexpr int stage = kShWords<DEG> * kPrepThreads * (FMT == GS_FP32 ? 4 : 2);
+    int one = 0, two = 0;
+    GS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * stage));
+    GS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&one, kernel, kPrepThreads, stage));
+    GS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&two, kernel, kPrepThreads, 2 * stage));
+    const int stages = two >= one ? 2 : 1;
+    const unsigned blocks = (unsigned)std::min<uint64_t>(div_up(s->n, kPrepThreads),
+                                                         (uint64_t)std::max(one, 1) * num_sms());
+    kernel<<<blocks, kPrepThreads, stages * stage, st>>>(s->planes, s->n, stages, cam, recs, rects, keys, vals, dbg,
+                                                         s->dev_err);
+    GS_CUDA(cudaGetLastError());
+    return GS_OK;
+}
+
 template <int FMT>
 gs_status launch_preprocess_fmt(const gs_scene* s, const DevCamera& cam, BlendRec* recs, uint2* rects,
                                 uint32_t* keys, uint32_t* vals, gs_record* dbg, cudaStream_t st) {
     constexpr uint64_t esz = FMT == GS_FP32 ? 4 : 2;
     if ((s->n * esz) % 16 == 0) {   // every plane of every tile starts on a 16-byte boundary
-        const int smem = (int)(kTmaStages * (uint64_t)s->nwords * kPrepThreads * esz);
-        GS_CUDA(cudaFuncSetAttribute(k_preprocess_tma<FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        int per_sm = 0;
-        GS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_preprocess_tma<FMT>, kPrepThreads, smem));
-        const uint64_t ntile = div_up(s->n, kPrepThreads);
-        const unsigned blocks = (unsigned)std::min<uint64_t>(ntile, (uint64_t)std::max(per_sm, 1) * num_sms());
-        k_preprocess_tma<FMT><<<blocks, kPrepThreads, smem, st>>>(s->planes, s->n, s->nwords, s->sh_degree, cam,
-                                                                   recs, rects, keys, vals, dbg, s->dev_err);
-    } else {
-        k_preprocess<FMT><<<(unsigned)div_up(s->n, kPrepThreads), kPrepThreads, 0, st>>>(
-            s->planes, s->n, s->nwords, s->sh_degree, cam, recs, rects, keys, vals, dbg);
+        switch (s->sh_degree) {
+            case 0: return launch_preprocess_tma<FMT, 0>(s, cam, recs, rects, keys, vals, dbg, st);
+            case 1: return launch_preprocess_tma<FMT, 1>(s, cam, recs, rects, keys, vals, dbg, st);
+            case 2: return launch_preprocess_tma<FMT, 2>(s, cam, recs, rects, keys, vals, dbg, st);
+            default: return launch_preprocess_tma<FMT, 3>(s, cam, recs, rects, keys, vals, dbg, st);
+        }
     }
+    k_preprocess<FMT><<<(unsigned)div_up(s->n, kPrepThreads), kPrepThreads, 0, st>>>(
+        s->planes, s->n, s->nwords, s->sh_degree, cam, recs, rects, keys, vals, dbg);
     GS_CUDA(cudaGetLastError());
     return GS_OK;
 }
