@@ -494,14 +494,14 @@ __global__ __launch_bounds__(kPrepThreads) void k_preprocess_tma(const void* pla
 }
 
 // ---------------------------------------------------------------------------
-// Dirty-tile injector: one warp per variant.  The lanes gather the flipped
-// primitive's words, XOR the upset in the storage format and optionally guard
-// them (Algorithm 1 applied to the only primitive that can leave its box); then
-// lane k preprocesses the corrupted primitive for view k and describes the
-// dirty tiles: the union of its clean and corrupted tile rects, each cut to the
-// tiles its record's alpha >= 1/255 box reaches.  A record changes no pixel of
-// a tile outside its box, so there it may stay in (clean record) or out of
-// (corrupted record) the tile's merged list without changing a bit.  The
+// Dirty-tile injector: one warp per `per` variants.  For each of them the lanes
+// gather the flipped primitive's words, XOR the upset in the storage format and
+// optionally guard them (Algorithm 1 applied to the only primitive that can leave
+// its box); then lane v K + k preprocesses variant v's corrupted primitive for view
+// k and describes the dirty tiles: the union of its clean and corrupted tile rects,
+// each cut to the tiles its record's alpha >= 1/255 box reaches.  A record changes
+// no pixel of a tile outside its box, so there it may stay in (clean record) or out
+// of (corrupted record) the tile's merged list without changing a bit.  The
 // per-view comparison accumulators are zeroed here (guard clamps reported on
 // view 0).
 // ---------------------------------------------------------------------------
@@ -511,6 +511,13 @@ struct SharedSrc {
 };
 
 constexpr int kPrepWarps = 8;
+constexpr int kPrepStride = kMaxWords | 1;   // odd: the lanes' words of one plane lie in different banks
+
+// Variants per warp.  The preprocess is 1,400 instructions that only `per` K lanes
+// of a warp need: 50,000 variants in one view took 116 us with a warp each (issue-
+// bound) and take 45 us with eight.  Small batches leave the chip idle, and
+// one variant per warp is then the shortest chain: kPrepMinWarps warps per SM come first.
+constexpr int kPrepMaxPer = 8, kPrepMinWarps = 16;
 
 // The tiles of a binned rect (packed x0 | y0 << 16, x1 | y1 << 16) that hold a
 // pixel centre of the record's alpha >= 1/255 box, packed the same way ((0, 0):
@@ -550,56 +557,70 @@ __device__ __forceinline__ uint32_t order_lower_bound(const uint32_t* __restrict
 template <int FMT>
 __global__ __launch_bounds__(kPrepWarps * 32) void k_inject_prep(
     const void* planes, uint64_t n, int nwords, int sh_degree, const DevCamera* cams, int K, const gs_flip* flips,
-    int B, int guard_mode, uint64_t mask, const uint32_t* box, const void* pblo, const void* pbhi, int nbox,
+    int B, int per, int guard_mode, uint64_t mask, const uint32_t* box, const void* pblo, const void* pbhi, int nbox,
     const ViewPtrs* views, DirtyDesc* desc, uint2* rows, unsigned int* queue, CmpAcc* acc) {
-    __shared__ float sv[kPrepWarps][kMaxWords];
+    extern __shared__ float sv_mem[];   // [kPrepWarps][per][kPrepStride]
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int b = blockIdx.x * kPrepWarps + wib;
-    if (b >= B) return;   // whole warps only; no block-wide barrier below
-    const gs_flip f = flips[b];
+    const int b0 = (blockIdx.x * kPrepWarps + wib) * per;
+    if (b0 >= B) return;   // whole warps only; no block-wide barrier below
+    const int nv_here = min(per, B - b0);
+    float* const sv = sv_mem + wib * per * kPrepStride;
     const int nbits = FMT == GS_FP32 ? 32 : 16;
-    // an upset the sign+exponent code corrects leaves the variant clean (zero record)
-    const bool corrected =
-        guard_mode == GS_GUARD_ECC && f.word < 64 && ((mask >> f.word) & 1ull) && f.bit >= ecc_first_bit(FMT);
-    const bool ok = f.prim < n && f.word < nwords && f.bit < nbits && !corrected;
-    const uint32_t p = ok ? f.prim : 0u;
+    const int my = lane / K;   // this lane's variant (none if >= nv_here)
+    bool ok = false, changed = false;
+    uint32_t p = 0u;
     unsigned int clamps = 0;
-    bool changed = false;   // does any stored word of the primitive end up different
-    for (int w = lane; w < nwords; w += 32) {
-        const uint32_t orig = load_bits<FMT>(planes, n, w, p);
-        uint32_t bits = orig;
-        if (ok && w == f.word) bits ^= (1u << f.bit);
-        float x = decode<FMT>(bits);
-        if ((guard_mode == GS_GUARD_FIELD || guard_mode == GS_GUARD_PRIM) && ((mask >> w) & 1ull)) {
-            uint32_t lb, hb;
-            if (guard_mode == GS_GUARD_FIELD) {
-                lb = box[w];
-                hb = box[kMaxWords + w];
-            } else {
-                lb = w < nbox ? load_bits<FMT>(pblo, n, w, p) : 0u;
-                hb = w < nbox ? load_bits<FMT>(pbhi, n, w, p) : 0u;
+    for (int v = 0; v < nv_here; v++) {
+        const gs_flip f = flips[b0 + v];
+        // an upset the sign+exponent code corrects leaves the variant clean (zero record)
+        const bool corrected =
+            guard_mode == GS_GUARD_ECC && f.word < 64 && ((mask >> f.word) & 1ull) && f.bit >= ecc_first_bit(FMT);
+        const bool vok = f.prim < n && f.word < nwords && f.bit < nbits && !corrected;
+        const uint32_t vp = vok ? f.prim : 0u;
+        unsigned int vclamps = 0;
+        bool vchanged = false;   // does any stored word of the primitive end up different
+        for (int w = lane; w < nwords; w += 32) {
+            const uint32_t orig = load_bits<FMT>(planes, n, w, vp);
+            uint32_t bits = orig;
+            if (vok && w == f.word) bits ^= (1u << f.bit);
+            float x = decode<FMT>(bits);
+            if ((guard_mode == GS_GUARD_FIELD || guard_mode == GS_GUARD_PRIM) && ((mask >> w) & 1ull)) {
+                uint32_t lb, hb;
+                if (guard_mode == GS_GUARD_FIELD) {
+                    lb = box[w];
+                    hb = box[kMaxWords + w];
+                } else {
+                    lb = w < nbox ? load_bits<FMT>(pblo, n, w, vp) : 0u;
+                    hb = w < nbox ? load_bits<FMT>(pbhi, n, w, vp) : 0u;
+                }
+                const float lo = decode<FMT>(lb), hi = decode<FMT>(hb);
+                if (!(x >= lo && x <= hi)) {
+                    vclamps++;
+                    x = (x > hi) ? hi : lo;
+                }
             }
-            const float lo = decode<FMT>(lb), hi = decode<FMT>(hb);
-            if (!(x >= lo && x <= hi)) {
-                clamps++;
-                x = (x > hi) ? hi : lo;
-            }
+            sv[v * kPrepStride + w] = x;
+            vchanged |= __float_as_uint(x) != __float_as_uint(decode<FMT>(orig));
         }
-        sv[wib][w] = x;
-        changed |= __float_as_uint(x) != __float_as_uint(decode<FMT>(orig));
+        vclamps = __reduce_add_sync(0xffffffffu, vclamps);
+        vchanged = vok && __any_sync(0xffffffffu, vchanged);
+        if (my == v) {
+            ok = vok;
+            p = vp;
+            clamps = vclamps;
+            changed = vchanged;
+        }
     }
-    clamps = __reduce_add_sync(0xffffffffu, clamps);
-    changed = ok && __any_sync(0xffffffffu, changed);
     __syncwarp();
-    int ny0 = 0, ny1 = 0, oy0 = 0, oy1 = 0;   // lane k: the tile rows of view k
-    if (lane < K) {
-        const int k = lane, bk = b * K + k;
+    int ny0 = 0, ny1 = 0, oy0 = 0, oy1 = 0;   // the tile rows of this lane's pair
+    if (my < nv_here) {
+        const int k = lane - my * K, bk = b0 * K + lane;
         const ViewPtrs& v = views[k];
         const int tw = v.tile_w, th = v.tile_h;
         DirtyDesc d;
         uint2 rect = make_uint2(0, 0);
         float rad = 0.0f;
-        const bool nvb = ok && preprocess_core(SharedSrc{sv[wib]}, sh_degree, cams[k], d.rec, rect, rad);
+        const bool nvb = ok && preprocess_core(SharedSrc{sv + my * kPrepStride}, sh_degree, cams[k], d.rec, rect, rad);
         const uint2 orect_b = ok ? v.rects[p] : make_uint2(0, 0);   // binned rects (contamination cells)
         const uint2 rect_b = nvb ? rect : make_uint2(0, 0);
         // dirty tiles: the binned rects cut to the records' alpha boxes
@@ -653,7 +674,7 @@ __global__ __launch_bounds__(kPrepWarps * 32) void k_inject_prep(
         z.reg_pred = changed ? rect_cells(orect_b, v.W, v.H, tw, th) | rect_cells(rect_b, v.W, v.H, tw, th) : 0ull;
         acc[bk] = z;
     }
-    // the variant's tile rows, in any order among the variants: one per lane, whole
+    // the variants' tile rows, in any order among the warps: one per lane, whole
     // warps writing consecutive items
     const uint32_t cnt = (uint32_t)Union1(ny0, ny1, oy0, oy1).len;
     uint32_t incl = cnt;
@@ -676,8 +697,10 @@ __global__ __launch_bounds__(kPrepWarps * 32) void k_inject_prep(
         }
         const int j = (int)(q - __shfl_sync(0xffffffffu, excl, s));
         const int a0 = __shfl_sync(0xffffffffu, ny0, s), a1 = __shfl_sync(0xffffffffu, ny1, s);
-        const int b0 = __shfl_sync(0xffffffffu, oy0, s), b1 = __shfl_sync(0xffffffffu, oy1, s);
-        if (q < total) rows[base + q] = make_uint2((uint32_t)(b * K + s), (uint32_t)Union1(a0, a1, b0, b1).at(j) | ((uint32_t)s << 16));
+        const int o0 = __shfl_sync(0xffffffffu, oy0, s), o1 = __shfl_sync(0xffffffffu, oy1, s);
+        if (q < total)
+            rows[base + q] = make_uint2((uint32_t)(b0 * K + s), (uint32_t)Union1(a0, a1, o0, o1).at(j) |
+                                                                    ((uint32_t)(s % K) << 16));
     }
 }
 
@@ -750,10 +773,12 @@ gs_status launch_inject_prep(const gs_scene* s, const DevCamera* dev_cams, int K
                              int guard_mode, uint64_t mask, const void* dev_views, DirtyDesc* desc, uint2* rows,
                              CmpAcc* acc, unsigned int* queue, cudaStream_t st) {
     if (B * K > kMaxPairs || K > 32) return set_error(GS_ERR_ARG, "B * K must be <= 65536 and K <= 32");
-    const int blocks = (B + kPrepWarps - 1) / kPrepWarps;
+    const int per = std::max(1, std::min(std::min(kPrepMaxPer, 32 / K), B / (kPrepMinWarps * num_sms())));   // K >= 1
+    const int blocks = (B + kPrepWarps * per - 1) / (kPrepWarps * per);
+    const size_t smem = sizeof(float) * kPrepWarps * per * kPrepStride;
 #define GS_PREP(F)                                                                                            \
-    k_inject_prep<F><<<blocks, kPrepWarps * 32, 0, st>>>(s->planes, s->n, s->nwords, s->sh_degree, dev_cams, K, \
-                                                         flips, B, guard_mode, mask, s->dev_box, s->pbox_lo,    \
+    k_inject_prep<F><<<blocks, kPrepWarps * 32, smem, st>>>(s->planes, s->n, s->nwords, s->sh_degree, dev_cams, K, \
+                                                         flips, B, per, guard_mode, mask, s->dev_box, s->pbox_lo,    \
                                                          s->pbox_hi, s->nbox_words, (const ViewPtrs*)dev_views, \
                                                          desc, rows, queue, acc)
     if (s->fmt == GS_FP32)
