@@ -1669,7 +1669,10 @@ gs_status launch_fill_lists(const ViewState& v, const uint32_t* off, uint32_t ca
     const int tx = cam.tiles_x, ty = cam.tiles_y, P = cam.tile_w * cam.tile_h / 2;
     if (tx * ty == 0) return GS_OK;
     const int smem = (int)sizeof(ListRing) * (P / 32);
-    GS_CUDA(cudaFuncSetAttribute(k_blend_clean<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    // the largest tile's, not this one's: the attribute is the process's, and another
+    // thread may fill lists of another tile shape between these lines
+    constexpr int most = (int)sizeof(ListRing) * (kBT / 2 / 32);
+    GS_CUDA(cudaFuncSetAttribute(k_blend_clean<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     k_blend_clean<true><<<tx * ty, P, smem, st>>>(v.recs, v.ids, v.rank, v.ranges, cam.W, cam.H, tx, cam.tile_w,
                                                   cam.tile_h, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
                                                   ListOut{v.ent, v.rk, off, cap, v.state, v.row_idx, v.row_off, v.row_cnt});

@@ -1062,10 +1062,14 @@ gs_status build_tile_lists(RenderWork& w, uint64_t n, int tiles_x, int tiles_y, 
         const int tpad = (ntiles + 7) & ~7;   // table rows: whole 16-byte pieces
         uint32_t *tab = w.tab, *tot = tab + (size_t)d.segs * tpad;
         uint16_t* wtab = reinterpret_cast<uint16_t*>(tot + tpad);
-        GS_CUDA(cudaFuncSetAttribute(k_tile_hist, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.hist_smem));
-        GS_CUDA(cudaFuncSetAttribute(k_tile_place, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.place_smem));
+        // the largest any grid needs, not this one's: the attribute is the process's, and
+        // another thread may list another grid between these lines and the launches
+        const DirectShape most = direct_shape(kDirectTiles, 1);
+        GS_CUDA(cudaFuncSetAttribute(k_tile_hist, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most.hist_smem));
+        GS_CUDA(cudaFuncSetAttribute(k_tile_place, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most.place_smem));
         k_tile_hist<<<d.segs, thr, d.hist_smem, st>>>(sorted_ids, w.srect, w.off, (uint32_t)n, tiles_x, ntiles, w.total,
                                                       wtab, tab);
+        GS_CUDA(cudaGetLastError());   // the placing walk writes where these counts say
         k_tile_colscan<<<(ntiles + 31) / 32, 1024, 0, st>>>(tab, ntiles, tpad, d.segs, w.total, tot);
         k_tile_starts<<<1, kScanT, 0, st>>>(tot, ntiles, w.total, w.ranges);
         k_tile_place<<<d.segs, thr, d.place_smem, st>>>(sorted_ids, w.srect, w.off, (uint32_t)n, tiles_x, ntiles,
