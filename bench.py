@@ -4,9 +4,9 @@ Default workload (one GPU): 2,000,000 Gaussians (4 clusters, SH degree 3, fp32
 storage), four 1600x1040 views on a ring, 20,000 single-bit upsets with 70% on
 bits 24-31 of log-scale and opacity.  A step is one launch of the batched
 dirty-tile engine over B variants (B picked by the library's autotuner from
-{8, 16, ..., 2048}), replayed as a CUDA graph: inject + guard-ready preprocess
-of the flipped primitives, the two plan kernels, dirty-tile re-blend fused with
-the comparison against the clean frames, finalisation of the per-(variant,
+powers of two up to 8192), replayed as a CUDA graph: inject + guard-ready preprocess
+of the flipped primitives, the plan (and the candidates' tile order in large
+batches), dirty-pixel re-blend from blend lists fused with the comparison against the clean frames, finalisation of the per-(variant,
 view) records.  Reported beside it: the plain one-variant-per-launch
 full-render loop on the same flips and the stage split of a full render, the
 end-to-end rate through host buffers, contamination and SSIM campaigns, the
@@ -38,7 +38,9 @@ UNIT = "injections/s"
 WORKLOAD = ("2M Gaussians (4 clusters, SH degree 3, fp32), 4 ring views 1600x1040, 20k upsets "
             "(70% on bits 24-31 of log-scale/opacity), guard off")
 ENGINE = "batched dirty-tile engine (inject, plan, re-blend + compare, finalise), replayed as a CUDA graph"
-FLOP_PER_EVAL = 20          # FP32 ops per pixel-primitive evaluation of the blend (FMA = 2)
+FLOP_PER_EVAL = 9           # FP32 ops per blend-list entry of a pixel (FMA = 2)
+BYTES_PER_EVAL = 20         # a blend-list entry: capped alpha, colour, rank
+DIRECT_TILES = 13900        # grids up to this size are listed by counting, larger ones by a radix sort
 L2_FLUSH_BYTES = 256 << 20  # > 129 MB L2
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic_k_dirty_2M_4views_batch2048.txt")
@@ -467,21 +469,21 @@ def main():
     # stage split of the full render (preprocess / binning + radix sort / blend)
     stages = render_stages(G, S, h, cams, flush, dev, pk, pk_kind)
 
-    # roofline of the dominant kernel (dirty-tile blend): FP32-pipe bound
+    # roofline of the dominant kernel (dirty-pixel blend): the blend lists of the dirty
+    # pixels are read once per variant, gathered from L2 and HBM
     clocks = clk.summary()
-    sm_mhz = clocks["sm_mhz"] or pk.get("sm_max_mhz", 2070.0)
-    nsm = torch.cuda.get_device_properties(dev).multi_processor_count
-    peak_tflops = nsm * 128 * 2 * sm_mhz * 1e6 / 1e12
     kavg = sum(k[1] for k in kern_ms) / len(kern_ms) / 1000.0
     plan_avg = sum(k[0] for k in kern_ms) / len(kern_ms) / 1000.0
     evals_per_launch = work["evaluations"] / args.steps
-    achieved = evals_per_launch * FLOP_PER_EVAL / kavg / 1e12
+    achieved = evals_per_launch * BYTES_PER_EVAL / kavg / 1e9
     tr = traffic_record()
     traffic = float(tr["k_dirty_bytes_per_launch"]) if "k_dirty_bytes_per_launch" in tr else None
-    roofline = {"kernel": "k_dirty (dirty-tile blend + compare)", "bound": "alu", "achieved": achieved,
-                "peak": peak_tflops, "unit": "TFLOP/s", "frac": achieved / peak_tflops, "traffic": traffic,
-                "peak_source": f"{nsm} SMs x 128 FP32 lanes x 2 x median SM clock {sm_mhz:.0f} MHz under load",
-                "work_per_launch": {"evaluations": evals_per_launch, "flop_per_eval": FLOP_PER_EVAL,
+    hbm_peak = pk.get("hbm_gbs", 6800.0)
+    roofline = {"kernel": "k_dirty (dirty-pixel blend + compare)", "bound": "memory", "achieved": achieved,
+                "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak, "traffic": traffic,
+                "peak_source": f"copy bandwidth, {pk_kind}",
+                "work_per_launch": {"evaluations": evals_per_launch, "bytes_per_eval": BYTES_PER_EVAL,
+                                    "flop_per_eval": FLOP_PER_EVAL,
                                     "tiles": work["tiles"] / args.steps, "entries": work["entries"] / args.steps,
                                     "tiles_dropped_by_plan": work["tiles_unchanged"] / args.steps,
                                     "blocks_blended": work["blocks_blended"] / args.steps,
@@ -506,10 +508,11 @@ def main():
         "engine": {"name": ENGINE, "batch": B, "tile": f"{tile[0]}x{tile[1]}",
                    "batch_and_tile_from": ("set" if args.batch > 0 else
                                            "tile set, batch autotuned" if args.tile else
-                                           "autotuner (tiles 16x16, 8x8, 32x8; batches 8-2048)")},
+                                           "autotuner (tiles 16x16, 8x8, 32x8; batches of powers of two up to 8192)")},
         "e2e": e2e,
-        # per step: injector, item scan, two plan kernels, dirty-tile blend, finalise
-        "gpu_launches": 6 * args.steps,
+        # per step: injector, plan, dirty-pixel blend, finalise; in large batches also the
+        # candidates' tile order (two kernels)
+        "gpu_launches": (4 if B <= min(2048, 8192 // K_views) else 6) * args.steps,
         "records_gathered_on_rank0": None if gathered is None else int(gathered.shape[0]),
         "mpix_s_effective": value * K_views * Wd * Hd / 1e6,
         "mpix_s_blended": work["blocks_blended"] * 64 * world / t_total / 1e6,   # 8x8 blocks
@@ -749,11 +752,12 @@ def render_stages(G, S, h, cams, flush, dev, pk, pk_kind, reps=10):
     binning with its radix sorts and the blend; medians over `reps` renders, L2
     flushed before each.  Algorithmic bytes: the preprocess reads every word of
     every primitive and writes its 48-B blend record, 8-B tile rect and 8-B
-    depth-sort pair; the tile lists are 8-B (tile, primitive) pairs written once
-    and read once.  The radix passes move 20 B per element (the histogram reads
-    the 4-B key, the scatter reads and writes key and value), the tile count and
-    emit read 20 B per primitive and write 8 B per pair, the range pass reads 4 B
-    per pair."""
+    depth-sort pair; the tile lists are 4-B primitive indices written once and read
+    once.  The radix passes of the depth sort move 20 B per element (the histogram
+    reads the 4-B key, the scatter reads and writes key and value); listing by
+    counting reads 40 B per primitive (ids and rects, put in order once and walked
+    twice) and writes 4 B per pair.  Larger grids sort (tile, primitive) pairs by
+    radix: 20 B per pair and pass, 8 B written and 4 B read per pair besides."""
     import torch
     cam = cams[:1]
     W, H = int(cam[0]["width"]), int(cam[0]["height"])
@@ -774,8 +778,13 @@ def render_stages(G, S, h, cams, flush, dev, pk, pk_kind, reps=10):
     _, _, fmt, nwords = G.gs_scene_info(h)
     wbytes = 4 if fmt == S.FP32 else 2
     pre_bytes = n * (nwords * wbytes + 64)
-    sort_alg = pairs * 16
-    sort_moved = 20 * (n * passes_depth + pairs * passes_pairs) + 20 * n + 12 * pairs
+    tw, th = G.gs_get_tile(h)
+    counted = ((W + tw - 1) // tw) * ((H + th - 1) // th) <= DIRECT_TILES
+    if counted:
+        passes_pairs = 0
+    sort_alg = pairs * 8
+    sort_moved = 20 * n * passes_depth + (40 * n + 4 * pairs if counted else
+                                          20 * pairs * passes_pairs + 20 * n + 12 * pairs)
     hbm = pk.get("hbm_gbs")
     gbs = lambda b, ms: b / (ms * 1e-3) / 1e9
     frame = pre_ms + sort_ms + blend_ms
