@@ -43,7 +43,7 @@ BYTES_PER_EVAL = 20         # a blend-list entry: capped alpha, colour, rank
 DIRECT_TILES = 13900        # grids up to this size are listed by counting, larger ones by a radix sort
 L2_FLUSH_BYTES = 256 << 20  # > 129 MB L2
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
-TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic_k_dirty_2M_4views_batch2048.txt")
+TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic_k_dirty_2M_4views.txt")
 
 
 def log(*a):
