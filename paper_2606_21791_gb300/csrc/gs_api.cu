@@ -870,7 +870,8 @@ gs_status gs_inject_and_render_full(gs_scene* s, const gs_flip* dev_flips, int B
     const int fpv = flips_per_variant;
     GS_TRY(ensure_batch_buffers(s, 1, fpv));
     uint64_t cap = s->full_cap_pairs + (uint64_t)(fpv - 1) * s->max_tiles;
-    GS_TRY(alloc_render_work(s->work, s->n, cap, s->max_tiles));
+    // for every view's own grid: a smaller one may be listed by counting where the largest is not
+    for (const ViewState& v : s->views) GS_TRY(alloc_render_work(s->work, s->n, cap, v.cam.tiles_x * v.cam.tiles_y));
     for (int b = 0; b < B; b++) {
         const gs_flip* f = dev_flips + (size_t)b * fpv;
         GS_TRY(launch_zero_acc(s->acc, K, st));

@@ -378,14 +378,22 @@ DirectShape direct_shape(int nt, uint64_t cap) {
     return d;
 }
 
-// Words of the counting tables that serve every grid of up to nt tiles and any pair
-// capacity up to cap: the segments' totals, the warps' 16-bit counts, the tiles'
-// totals.  A block's shared memory bounds tiles x warps per SM; beyond one wave of
-// blocks the segments grow with the capacity.
+// Words of the counting tables of such a shape: the segments' totals, the tiles'
+// totals, the warps' 16-bit counts.
+size_t direct_words(const DirectShape& d, int nt) {
+    const size_t t = ((size_t)nt + 7) & ~(size_t)7;
+    return t * d.segs + t + t * d.warps / 2 * d.segs;
+}
+
+// Words that serve every grid of up to nt tiles at a pair capacity of cap.  A block's
+// shared memory bounds tiles x warps per SM, so one wave of blocks takes the same at
+// any grid; beyond it, and in small scenes, the segments go with the capacity.
 size_t direct_tab_words(int nt, uint64_t cap) {
+    const size_t per_seg = (size_t)(nt + 8) * (4 + 1);
     const size_t wave = (size_t)num_sms() * (220 * 1024 / 4);   // tiles x (warps + 2) x blocks, two bytes each
-    const size_t more = (size_t)div_up(cap, 60000) * (size_t)(nt + 8) * (4 + 1);
-    return std::max(wave, more) + (size_t)nt + 64;
+    const size_t few = (size_t)div_up(std::max<uint64_t>(cap, 1), 6 * 256) * per_seg;
+    const size_t more = (size_t)div_up(cap, 60000) * per_seg;
+    return std::max(std::min(wave, few), more) + (size_t)nt + 64;
 }
 
 // The pairs [p0, p1) in order, 2 x 32 at a time: f(tile, primitive, active of the
@@ -1030,6 +1038,9 @@ void free_render_work(RenderWork& w) {
 // *ids_out.  total[0] = usable pair count, total[1] = overflow flag.
 gs_status build_tile_lists(RenderWork& w, uint64_t n, int tiles_x, int tiles_y, uint32_t** ids_out, cudaStream_t st) {
     int ntiles = tiles_x * tiles_y;
+    // every segment's rows are written, so the tables have to hold them all
+    if (ntiles <= kDirectTiles && direct_words(direct_shape(ntiles, w.cap_pairs), ntiles) > w.tab_words)
+        return set_error(GS_ERR_CAPACITY, "the counting tables were not sized for this tile grid");
     int cur = 0;
     unsigned blocks = (unsigned)div_up(std::max<uint64_t>(n, 1), 256);
     int nparts = (int)std::max<uint64_t>(div_up(n, kScanTile), 1);

@@ -1,0 +1,101 @@
+"""The host side of libgs without a GPU: its own objects linked against a stand-in
+for the CUDA runtime (fake_cudart.cpp), which maps device memory lazily, runs no
+kernel, and checks the arrays that some of them are given."""
+import ctypes as C
+import glob
+import os
+import subprocess
+import sys
+import textwrap
+
+import pytest
+
+from paper_2606_21791_gb300 import buildlib
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="session")
+def fake():
+    """Path of the library linked against the stand-in."""
+    buildlib.build()
+    objs = [os.path.join(buildlib.BUILD, os.path.basename(s)[:-3] + ".o") for s in buildlib._sources()]
+    if not all(os.path.exists(o) for o in objs):
+        buildlib.build(force=True)
+    include = os.path.join(os.path.dirname(os.path.dirname(buildlib.nvcc())), "include")
+    lib = os.path.join(buildlib.BUILD, "libgs_fake.so")
+    src = os.path.join(HERE, "fake_cudart.cpp")
+    cmd = ["g++", "-O1", "-std=c++17", "-fPIC", "-fvisibility=hidden", "-I", include, "-shared", "-Wl,-Bsymbolic",
+           "-Wl,--no-undefined", "-o", lib, src, *objs, "-lpthread"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return lib
+
+
+PRELUDE = """
+import ctypes as C
+import numpy as np
+from paper_2606_21791_gb300 import gs as G, synth as S
+L = G.load_library({lib!r})
+for f in ("fake_live", "fake_allocations"):
+    getattr(L, f).restype = C.c_uint64
+L.fake_report.restype = C.c_char_p
+L.fake_limit.argtypes = [C.c_uint64]
+L.fake_counts.argtypes = [C.c_uint64, C.c_uint64]
+ADDR = 1 << 20   # stands for a device buffer: no kernel runs
+
+def scene(n=20_000, degree=0, fmt=S.FP32):
+    nbytes = S.words_for_degree(degree) * n * (4 if fmt == S.FP32 else 2)
+    return G.gs_load_scene(np.zeros(nbytes, np.uint8), n, degree, fmt)
+
+def cams(*sizes):
+    return np.concatenate([S.ring_cameras(1, w, h) for w, h in sizes])
+
+def clean(h=None):
+    if h is not None:
+        G.gs_free_scene(h)
+    assert L.fake_report() == b"", L.fake_report().decode()
+"""
+
+
+def run(fake, body):
+    code = PRELUDE.format(lib=fake) + textwrap.dedent(body)
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300,
+                       cwd=os.path.dirname(HERE))
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("first,second", [((1600, 1040), (2592, 1944)), ((2592, 1944), (1600, 1040)),
+                                          ((1920, 1080), (2560, 1440)), ((320, 240), (1600, 1040))])
+@pytest.mark.parametrize("tile", [(16, 16), (8, 8)])
+def test_full_rerender_over_views_of_different_sizes(fake, first, second, tile):
+    """Every view's lists are made in tables that hold them: grids on both sides of the
+    counting lists' limit, in both orders, at pair capacities that single upsets and
+    thousands of upsets a variant ask for."""
+    run(fake, f"""
+    h = scene()
+    G.gs_set_tile(h, *{tile}, stream=0)
+    L.fake_counts(2_000_000, 20)
+    G.gs_set_views(h, cams({first}, {second}), stream=0)
+    for flips in (1, 1000, 5000):
+        G.gs_inject_and_render_full(h, ADDR, 2, flips, -1, 0, ADDR, stream=0)
+    clean(h)
+    """)
+
+
+def test_counting_tables_hold_every_grid(fake):
+    """Tile grids from one tile to past the counting lists' limit, pair capacities from
+    one to two billion; a smaller grid after a larger one in the same scratch."""
+    run(fake, """
+    from itertools import product
+    total = np.zeros(1, np.uint64)
+    for (tx, ty), cap in product([(1, 1), (7, 1), (9, 9), (50, 50), (100, 65), (69, 100), (83, 83), (139, 100), (140, 100)],
+                                 [1, 1000, 1536, 2049, 300_000, 5_000_000, 40_000_000, 2_000_000_000]):
+        L.fake_counts(min(cap, 1000), 0)
+        G.gs_bin_tiles(ADDR, ADDR, 1, tx, ty, ADDR, ADDR, cap, stream=0)
+    h = scene(n=400_000)
+    L.fake_counts(9_000_000, 0)
+    for W, H in ((2200, 1600), (640, 480), (16, 16), (1600, 1040), (100, 1600), (2592, 1944), (800, 800)):
+        G.gs_render(h, cams((W, H)), ADDR, stream=0)
+    clean(h)
+    """)
