@@ -925,88 +925,74 @@ gs_status radix_sort(uint32_t* k[2], uint32_t* v[2], const unsigned long long* d
 
 }  // namespace
 
+// Grows w to n primitives, cap_pairs pairs and a grid of ntiles tiles.  What a growth
+// frees is NULL, and its size 0, until all of it is there again: a failure part way
+// leaves nothing that a later, smaller call could take for usable.
 gs_status alloc_render_work(RenderWork& w, uint64_t n, uint64_t cap_pairs, int ntiles) {
-    bool grow_n = n > w.n || !w.recs;
-    bool grow_p = cap_pairs > w.cap_pairs || !w.pval[0];
-    // the pair sort's other buffers: only for grids that are not listed by counting
-    const bool radix = ntiles > kDirectTiles;
-    bool grow_t = ntiles > w.ntiles_cap || !w.ranges;
-    auto A = [](void** p, size_t bytes) -> gs_status {
-        cudaError_t e = cudaMalloc(p, bytes ? bytes : 16);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            *p = nullptr;
-            return set_error(GS_ERR_OOM, std::string("cudaMalloc failed for render scratch: ") + cudaGetErrorString(e));
-        }
-        return GS_OK;
+    auto A = [](auto*& p, uint64_t items) -> gs_status {   // p: room for `items`, its old content gone
+        cudaFree(p);
+        p = nullptr;
+        const cudaError_t e = cudaMalloc((void**)&p, std::max<uint64_t>(items, 1) * sizeof(*p));
+        if (e == cudaSuccess) return GS_OK;
+        cudaGetLastError();
+        p = nullptr;
+        return set_error(GS_ERR_OOM, std::string("cudaMalloc failed for render scratch: ") + cudaGetErrorString(e));
     };
-    uint64_t nn = std::max<uint64_t>(n, 1);
-    if (grow_n) {
-        cudaFree(w.recs);
-        cudaFree(w.rects);
+    if (n > w.n || !w.recs) {
+        w.n = 0;
+        GS_TRY(A(w.srect, n));
+        GS_TRY(A(w.rects, n));
         for (int i = 0; i < 2; i++) {
-            cudaFree(w.dkey[i]);
-            cudaFree(w.dval[i]);
+            GS_TRY(A(w.dkey[i], n));
+            GS_TRY(A(w.dval[i], n));
         }
-        cudaFree(w.cnt);
-        cudaFree(w.off);
-        cudaFree(w.srect);
-        cudaFree(w.scan_tmp);
-        GS_TRY(A((void**)&w.srect, sizeof(uint2) * nn));
-        GS_TRY(A((void**)&w.recs, sizeof(BlendRec) * nn));
-        GS_TRY(A((void**)&w.rects, sizeof(uint2) * nn));
-        for (int i = 0; i < 2; i++) {
-            GS_TRY(A((void**)&w.dkey[i], 4 * nn));
-            GS_TRY(A((void**)&w.dval[i], 4 * nn));
-        }
-        GS_TRY(A((void**)&w.cnt, 4 * nn));
-        GS_TRY(A((void**)&w.off, 4 * nn));
-        GS_TRY(A((void**)&w.scan_tmp, sizeof(unsigned long long) * (div_up(nn, kScanTile) + 1) + 4 * nn + 64));
+        GS_TRY(A(w.cnt, n));
+        GS_TRY(A(w.off, n));
+        // block sums of the scans (8 B each), then the large primitives' list and its length
+        GS_TRY(A(w.scan_tmp, 2 * (div_up(std::max<uint64_t>(n, 1), kScanTile) + 1) + n + 16));
+        GS_TRY(A(w.recs, n));   // last: it says that they are all there
         w.n = n;
     }
-    if (grow_p) {
-        cudaFree(w.pval[0]);
-        GS_TRY(A((void**)&w.pval[0], 4 * std::max<uint64_t>(cap_pairs, 1)));
+    if (cap_pairs > w.cap_pairs || !w.pval[0]) {
+        w.cap_pairs = 0;
+        GS_TRY(A(w.pval[0], cap_pairs));
         w.cap_pairs = cap_pairs;
     }
+    // the pair sort's other buffers: only for grids that are not listed by counting
+    const bool radix = ntiles > kDirectTiles;
     if (radix && w.cap_pairs > w.radix_pairs) {
-        uint32_t** more[3] = {&w.pkey[0], &w.pkey[1], &w.pval[1]};
-        for (uint32_t** q : more) {
-            cudaFree(*q);
-            GS_TRY(A((void**)q, 4 * w.cap_pairs));
-        }
+        w.radix_pairs = 0;
+        GS_TRY(A(w.pkey[0], w.cap_pairs));
+        GS_TRY(A(w.pkey[1], w.cap_pairs));
+        GS_TRY(A(w.pval[1], w.cap_pairs));
         w.radix_pairs = w.cap_pairs;
     }
     const uint64_t big = std::max<uint64_t>({w.radix_pairs, w.n, (uint64_t)1});
     if (big > w.hist_items) {
-        cudaFree(w.hist);
-        cudaFree(w.hpart);
         w.hist_items = 0;
         const int hb = radix_blocks_upto(big);
-        GS_TRY(A((void**)&w.hist, 4ull * 256 * hb));
-        GS_TRY(A((void**)&w.hpart, sizeof(unsigned long long) * std::max(hist_parts(hb) + 8, 136)));
+        GS_TRY(A(w.hist, 256ull * hb));
+        GS_TRY(A(w.hpart, std::max(hist_parts(hb) + 8, 136)));
         w.hist_items = big;
     }
     if (!radix) {
         const size_t need = direct_tab_words(std::max(ntiles, 1), w.cap_pairs);
         if (need > w.tab_words) {
-            cudaFree(w.tab);
             w.tab_words = 0;
-            GS_TRY(A((void**)&w.tab, 4 * need));
+            GS_TRY(A(w.tab, need));
             w.tab_words = need;
         }
     }
-    if (grow_t) {
-        cudaFree(w.ranges);
-        GS_TRY(A((void**)&w.ranges, sizeof(uint2) * std::max(ntiles, 1)));
+    if (ntiles > w.ntiles_cap || !w.ranges) {
+        w.ntiles_cap = 0;
+        GS_TRY(A(w.ranges, std::max(ntiles, 1)));
         w.ntiles_cap = ntiles;
     }
-    if (!w.total) {
-        GS_TRY(A((void**)&w.total, sizeof(unsigned long long) * 8));
-        if (cudaMallocHost((void**)&w.host_total, sizeof(unsigned long long) * 8) != cudaSuccess) {
-            cudaGetLastError();
-            return set_error(GS_ERR_OOM, "cudaMallocHost failed");
-        }
+    if (!w.total) GS_TRY(A(w.total, 8));
+    if (!w.host_total && cudaMallocHost((void**)&w.host_total, sizeof(unsigned long long) * 8) != cudaSuccess) {
+        cudaGetLastError();
+        w.host_total = nullptr;
+        return set_error(GS_ERR_OOM, "cudaMallocHost failed");
     }
     return GS_OK;
 }

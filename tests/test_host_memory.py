@@ -99,3 +99,34 @@ def test_counting_tables_hold_every_grid(fake):
         G.gs_render(h, cams((W, H)), ADDR, stream=0)
     clean(h)
     """)
+
+
+def test_scratch_after_a_failed_growth(fake):
+    """A slot's scratch fails to grow for a large scene, at any of its allocations; the
+    next request, of a small one, is given live arrays, and nothing is freed twice."""
+    run(fake, """
+    for grid in ((640, 480), (2592, 1944)):
+        for extra in [0, 1 << 20] + [m << 21 for m in range(1, 90)]:
+            small, big = scene(n=5000), scene(n=600_000)
+            srv = G.gs_server_create(1 << 40, 1)
+            ids = [G.gs_server_add_scene(srv, h) for h in (small, big)]
+
+            def render(i, size, pairs):
+                L.fake_counts(pairs, 0)
+                t = G.gs_server_submit(srv, G.make_request(G.GS_REQ_RENDER, ids[i], cams(size)[0], dev_rgb=ADDR))
+                G.gs_server_wait(srv, t)
+
+            render(0, (640, 480), 9000)
+            L.fake_limit(L.fake_live() + extra)
+            try:
+                render(1, grid, 3_000_000)
+            except G.GsError as e:
+                assert e.status == G.GS_ERR_OOM, e
+            L.fake_limit((1 << 64) - 1)
+            render(0, (640, 480), 9000)
+            render(0, (2592, 1944), 20_000)
+            G.gs_server_destroy(srv)
+            G.gs_free_scene(big)
+            clean(small)
+            assert L.fake_live() == 0
+    """)
