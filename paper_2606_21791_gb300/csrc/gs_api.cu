@@ -371,6 +371,24 @@ gs_status run_dirty_batch(gs_scene* s, int B, int guard_mode, uint64_t mask, boo
     return GS_OK;
 }
 
+void free_prim_box(gs_scene* s) {
+    cudaFree(s->pbox_lo);
+    cudaFree(s->pbox_hi);
+    s->pbox_lo = s->pbox_hi = nullptr;
+    s->nbox_words = 0;
+}
+
+gs_status load_prim_box(gs_scene* s, const void* lo, const void* hi, int src_on_device, int nbox_words) {
+    const size_t bytes = (size_t)s->n * nbox_words * word_bytes(s->fmt);
+    GS_TRY(dmalloc(&s->pbox_lo, (bytes + 15) & ~(size_t)15));
+    GS_TRY(dmalloc(&s->pbox_hi, (bytes + 15) & ~(size_t)15));
+    const cudaMemcpyKind kind = src_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+    GS_CUDA(cudaMemcpy(s->pbox_lo, lo, bytes, kind));
+    GS_CUDA(cudaMemcpy(s->pbox_hi, hi, bytes, kind));
+    s->nbox_words = nbox_words;
+    return GS_OK;
+}
+
 }  // namespace
 
 gs_status render_lists_sized_ext(gs_scene* s, RenderWork& w, const DevCamera& cam, uint32_t** ids, uint64_t* npairs,
@@ -454,8 +472,7 @@ gs_status gs_free_scene(gs_scene* s) {
     free_view_memory(s);
     free_render_work(s->work);
     cudaFree(s->planes);
-    cudaFree(s->pbox_lo);
-    cudaFree(s->pbox_hi);
+    free_prim_box(s);
     cudaFree(s->dev_box);
     cudaFree(s->dev_err);
     cudaFree(s->dev_clamps);
@@ -531,17 +548,10 @@ gs_status gs_set_prim_box(gs_scene* s, const void* lo, const void* hi, int src_o
     if (!s || !lo || !hi || nbox_words < 1 || nbox_words > s->nwords)
         return set_error(GS_ERR_ARG, "bad gs_set_prim_box arguments");
     destroy_graphs(s);
-    cudaFree(s->pbox_lo);
-    cudaFree(s->pbox_hi);
-    s->pbox_lo = s->pbox_hi = nullptr;
-    size_t bytes = (size_t)s->n * nbox_words * word_bytes(s->fmt);
-    GS_TRY(dmalloc(&s->pbox_lo, (bytes + 15) & ~(size_t)15));
-    GS_TRY(dmalloc(&s->pbox_hi, (bytes + 15) & ~(size_t)15));
-    cudaMemcpyKind kind = src_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    GS_CUDA(cudaMemcpy(s->pbox_lo, lo, bytes, kind));
-    GS_CUDA(cudaMemcpy(s->pbox_hi, hi, bytes, kind));
-    s->nbox_words = nbox_words;
-    return GS_OK;
+    free_prim_box(s);
+    const gs_status rs = load_prim_box(s, lo, hi, src_on_device, nbox_words);
+    if (rs != GS_OK) free_prim_box(s);   // both halves or none: half a box is no box
+    return rs;
 }
 
 gs_status gs_guard(gs_scene* s, int mode, uint64_t word_mask, uint64_t* dev_clamps, void* stream) {

@@ -130,3 +130,27 @@ def test_scratch_after_a_failed_growth(fake):
             clean(small)
             assert L.fake_live() == 0
     """)
+
+
+def test_boxes_after_a_failed_upload(fake):
+    """Per-primitive boxes of which only one half found room are no boxes."""
+    run(fake, """
+    h = scene()
+    box = np.zeros(14 * 20_000, np.uint32)
+    G.gs_set_prim_box(h, box, box, 14)
+    G.gs_set_views(h, cams((320, 240)), stream=0)
+    for extra in (0, box.nbytes // 2, box.nbytes):   # on top of the boxes that are replaced
+        L.fake_limit(L.fake_live() - 2 * box.nbytes + extra)
+        for call in (lambda: G.gs_set_prim_box(h, box, box, 14),
+                     lambda: G.gs_inject_and_render(h, ADDR, 8, 1, G.GS_GUARD_PRIM, 1, ADDR, stream=0),
+                     lambda: G.gs_guard(h, G.GS_GUARD_PRIM, 1, stream=0)):
+            try:
+                call()
+                raise SystemExit("accepted")
+            except G.GsError as e:
+                assert e.status in (G.GS_ERR_OOM, G.GS_ERR_STATE, G.GS_ERR_ARG), e   # as with no boxes
+        L.fake_limit((1 << 64) - 1)
+        G.gs_set_prim_box(h, box, box, 14)
+        G.gs_inject_and_render(h, ADDR, 8, 1, G.GS_GUARD_PRIM, 1, ADDR, stream=0)
+    clean(h)
+    """)
