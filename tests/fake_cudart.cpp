@@ -92,9 +92,9 @@ void check(const std::string& name, void** a) {
         inside("k_tile_place", "the tiles' starts", arg<void*>(a, 9), 4 * nt);
         inside("k_tile_place", "the lists", arg<void*>(a, 10), 4 * (size_t)arg<unsigned long long*>(a, 6)[0]);
     }
-    if (is("k_preprocess")) {
+    if (is("12k_preprocessI") || is("16k_preprocess_tmaI")) {   // the file's name is part of its other kernels' names
         const uint64_t n = arg<uint64_t>(a, 1);
-        const int at = is("k_preprocess_tma") ? 4 : 5;   // records, rects, keys, values
+        const int at = is("16k_preprocess_tmaI") ? 4 : 5;   // records, rects, keys, values
         const size_t each[4] = {48, 8, 4, 4};
         for (int i = 0; i < 4; i++)
             if (arg<void*>(a, at + i)) inside("k_preprocess", "an output", arg<void*>(a, at + i), each[i] * n);
