@@ -259,8 +259,8 @@ gs_status ensure_batch_buffers(gs_scene* s, int B, int fpv) {
         GS_TRY(dmalloc((void**)&s->desc, sizeof(DirtyDesc) * pairs));
         GS_TRY(dmalloc((void**)&s->acc, sizeof(CmpAcc) * pairs));
         GS_TRY(dmalloc((void**)&s->res_stage, sizeof(gs_result) * pairs));
-        GS_TRY(dmalloc((void**)&s->queue, sizeof(unsigned int) * 8));
-        const unsigned int q0[8] = {0u, 0u, 0u, 0u, 0u, 0u, 1u, 0u};   // [6]: batch generation
+        GS_TRY(dmalloc((void**)&s->queue, sizeof(unsigned int) * 16));
+        const unsigned int q0[16] = {0u, 0u, 0u, 0u, 0u, 0u, 1u};   // [6]: batch generation
         GS_CUDA(cudaMemcpy(s->queue, q0, sizeof(q0), cudaMemcpyHostToDevice));
         GS_TRY(dmalloc((void**)&s->saved, sizeof(uint32_t) * cf));
         GS_TRY(dmalloc((void**)&s->rows, sizeof(uint2) * rows));

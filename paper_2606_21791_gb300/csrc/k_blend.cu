@@ -855,7 +855,7 @@ __global__ __launch_bounds__(kBT) void k_compare(const float* __restrict__ a, co
 __global__ void k_finalize(const CmpAcc* acc, int count, gs_result* out, const unsigned int* clean_nonfin, int K,
                            unsigned int* queue) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (queue && i < 8) queue[i] = i == 6 ? queue[6] + 1u : 0u;   // [6]: batch generation (tags of the SSIM maps)
+    if (queue && i < 16) queue[i] = i == 6 ? queue[6] + 1u : 0u;   // [6]: batch generation (tags of the SSIM maps)
     if (i >= count) return;
     CmpAcc a = acc[i];
     gs_result r;
@@ -961,7 +961,7 @@ __device__ __forceinline__ void band_tiles(const BlendRec& q, float y0, float y1
 // spans the frame, but its ellipse crosses a few columns of each row (20,000 upsets
 // of a 2M-primitive scene, 4 views: 28.5M tiles by rects, 1.4M by rows; 0.16 ms,
 // and 0.82 ms where needles kept their whole rows).
-// counts[1] rows, [2] candidates, [3] SSIM plan slots.
+// counts[1] rows, [2] candidates, [3] their blocks to look at, [9] SSIM plan slots.
 // BIN: also count the candidates of each tile (bins) and keep each one's place.
 template <bool COUNT, bool BIN>
 __global__ __launch_bounds__(256) void k_plan(const ViewPtrs* __restrict__ views, const DirtyDesc* __restrict__ desc,
@@ -1007,10 +1007,12 @@ __global__ __launch_bounds__(256) void k_plan(const ViewPtrs* __restrict__ views
         }
         const unsigned m = __ballot_sync(0xffffffffu, blocks != 0u);
         if (!m) return;
+        const unsigned nblk = __reduce_add_sync(0xffffffffu, (unsigned)__popc(blocks));
         uint32_t c0 = 0, s0 = 0;
-        if (lane == 0) {
-            c0 = atomicAdd(&counts[2], (unsigned)__popc(m));
-            if (sb.plan) s0 = atomicAdd(&counts[3], (unsigned)__popc(m));
+        if (lane == 0) {   // both counts in one addition
+            c0 = (uint32_t)atomicAdd(reinterpret_cast<unsigned long long*>(&counts[2]),
+                                     (unsigned long long)__popc(m) | ((unsigned long long)nblk << 32));
+            if (sb.plan) s0 = atomicAdd(&counts[9], (unsigned)__popc(m));
         }
         c0 = __shfl_sync(0xffffffffu, c0, 0) + __popc(m & ((1u << lane) - 1u));
         s0 = __shfl_sync(0xffffffffu, s0, 0) + __popc(m & ((1u << lane) - 1u));
@@ -1266,14 +1268,28 @@ __global__ __launch_bounds__(kDirtyThreads, 5) void k_dirty(const ViewPtrs* __re
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int lg = tile_lgx(tw), nb = (tw * th) >> 6;
     const uint32_t P = (uint32_t)(tw * th), ncand = counts[2];
-    // candidates a block takes at a time: all kUnitVars when there are enough for every block
-    const uint32_t per = min((uint32_t)kUnitVars, (ncand + gridDim.x - 1u) / gridDim.x);
+    // Candidates of a unit, which blocks draw one after another.  A second unit costs its
+    // set-up (6 us) again, so a block's share is one unit where the candidates are light.
+    // Where most are reached in most of their blocks (the corrupted record covers them), a
+    // unit may hold many times another's pixels: an eighth of a share, of at least one
+    // candidate from 0.6 of the blocks on, two from 0.55.  300 upsets of 2M primitives, four
+    // views (0.70, share 12): 202 us in shares, 124 in eighths; 3,000 of 134,826 (0.44,
+    // share 10): 48 us in shares, 70 in eighths.
+    const uint32_t share = (ncand + gridDim.x - 1u) / gridDim.x;
+    const float covered = (float)counts[3] / ((float)max(ncand, 1u) * (float)nb);
+    const uint32_t least = nb < 4 || covered < 0.55f ? (uint32_t)kUnitVars : (covered < 0.6f ? 2u : 1u);
+    const uint32_t per = min((uint32_t)kUnitVars, share <= least + 1u ? share : max(least, (share + 7u) / 8u));
+    __shared__ uint32_t next_unit;
     // the bins are free again: clear them for the next batch
     for (uint32_t i = blockIdx.x * kDirtyThreads + (uint32_t)tid; i < nbins; i += gridDim.x * kDirtyThreads) bins[i] = 0u;
     // measurement builds: SM cycles each warp spends per phase (the activity of the
     // candidates' pixels, the walk, the comparison and reductions)
     long long t_pro = 0, t_walk = 0, t_epi = 0;
-    for (uint32_t c0 = blockIdx.x * per; c0 < ncand; c0 += gridDim.x * per) {
+    // units are drawn: the first by place, the next ones while this one is at work
+    for (uint32_t unit = blockIdx.x, drawn = 0u;; unit = next_unit) {
+        const uint32_t c0 = unit * per;
+        if (c0 >= ncand) break;   // the same for the whole block
+        if (tid == 0) drawn = gridDim.x + atomicAdd(&counts[0], 1u);
         const long long t0 = COUNT ? clock64() : 0;
         const int nv = (int)min(per, ncand - c0);
         __syncthreads();   // the previous candidates are done with the shared arrays
@@ -1568,6 +1584,7 @@ __global__ __launch_bounds__(kDirtyThreads, 5) void k_dirty(const ViewPtrs* __re
                 }
             }
         }
+        if (tid == 0) next_unit = drawn;
         __syncthreads();
         if (tid < nv) {
             const DirtyVar& q = var[tid];
@@ -1768,9 +1785,9 @@ gs_status launch_dirty_ssim(const void* dev_views, int K, unsigned int* queue, c
 constexpr int kSortPairs = 512;
 
 // One batch after the injector.  ev_mid (optional): recorded between the plan and
-// the blend kernel.  s->queue: [1] tile rows, [2] candidates, [3] SSIM plan
-// slots, [4] bin places, [5] SSIM delta units, cleared by the finaliser; [6] batch
-// generation; [7] tiles the SSIM visits.
+// the blend kernel.  s->queue, cleared by the finaliser but for [6]: [0] units drawn,
+// [1] tile rows, [2] candidates and [3] their blocks to look at, [4] bin places, [5] SSIM
+// delta units, [6] batch generation, [7] tiles the SSIM visits, [9] SSIM plan slots.
 gs_status launch_dirty_blend(gs_scene* s, int BK, bool regions, const SsimBufs& sb, cudaStream_t st) {
     const ViewPtrs* views = (const ViewPtrs*)s->dev_views;
     const int plan_blocks = num_sms() * 8;

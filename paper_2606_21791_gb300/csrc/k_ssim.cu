@@ -225,7 +225,7 @@ SsimW ssim_weights() {
 // than the tiles.)
 __global__ __launch_bounds__(256) void k_ssim_claim(const ViewPtrs* __restrict__ views, int K,
                                                     unsigned int* __restrict__ queue, SsimBufs sb) {
-    const uint32_t n_items = min(queue[3], sb.slot_cap);   // beyond it the batch reports an overflow
+    const uint32_t n_items = min(queue[9], sb.slot_cap);   // beyond it the batch reports an overflow
     const unsigned long long gen = (unsigned long long)queue[6] << 32;
     const int lane = threadIdx.x & 31;
     for (uint32_t base = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < n_items * 9u;
