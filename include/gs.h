@@ -370,8 +370,10 @@ GS_API gs_status gs_blend_lists(const gs_record* dev_recs, uint64_t n, const uin
  * renders and storm frames run alone on their scene; one campaign per scene)
  * and whose render scratch fits the budget; so requests that arrive while
  * others run are admitted as slots and memory free up, and run concurrently on
- * separate streams.  A request larger than the budget left after the resident
- * scenes is refused with GS_ERR_BUSY.  Device buffers in a request must stay
+ * separate streams.  A campaign grows its scene's batch buffers as far as the
+ * budget has room, runs in smaller batches otherwise, and gives the growth back
+ * when a request waits for memory.  A request larger than the budget left after
+ * the resident scenes is refused with GS_ERR_BUSY.  Device buffers in a request must stay
  * valid until gs_server_wait returns for it.  While a scene is registered with
  * a running server, the caller changes it only through requests: calls that
  * rebuild or free its state (gs_set_views, gs_set_tile, gs_autotune_tile,

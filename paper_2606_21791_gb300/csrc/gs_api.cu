@@ -238,20 +238,43 @@ void free_batch_buffers(gs_scene* s) {
     s->cap_flip_mem = s->cap_pairs = s->cap_cands = s->cap_rows = s->cap_bins = 0;
 }
 
+// Elements of the batch buffers for cb variants and cf upsets: every (variant, view) can
+// dirty at most every tile of its view.
+struct BatchSize {
+    uint64_t flips = 0, pairs = 0, cands = 0, rows = 0, bins = 0;
+    size_t bytes() const {
+        return flips * (sizeof(gs_flip) + 4) + pairs * (sizeof(DirtyDesc) + sizeof(CmpAcc) + sizeof(gs_result)) +
+               cands * (2 * sizeof(uint2) + 4) + rows * sizeof(uint2) + bins * 4;
+    }
+};
+BatchSize batch_size(const gs_scene* s, int cb, int cf) {
+    BatchSize b;
+    b.flips = (uint64_t)cf;
+    b.pairs = (uint64_t)cb * std::max(s->K, 1);
+    b.cands = b.pairs * (uint64_t)std::max(s->max_tiles, 1);
+    b.rows = b.pairs * (uint64_t)std::max(s->max_tiles_y, 1);
+    b.bins = std::max(s->all_tiles, 1u);
+    return b;
+}
+BatchSize batch_held(const gs_scene* s) {
+    return BatchSize{s->cap_flip_mem, s->cap_pairs, s->cap_cands, s->cap_rows, s->cap_bins};
+}
+bool batch_fits(const BatchSize& b, const BatchSize& held) {
+    return b.flips <= held.flips && b.pairs <= held.pairs && b.cands <= held.cands && b.rows <= held.rows &&
+           b.bins <= held.bins;
+}
+
 gs_status ensure_batch_buffers(gs_scene* s, int B, int fpv) {
-    int K = std::max(s->K, 1);
     if (B <= s->cap_B && fpv * B <= s->cap_flips) return GS_OK;
     const int cb = std::max(B, s->cap_B);
     const int cf = std::max(fpv * B, s->cap_flips);
-    // every (variant, view) can dirty at most every tile of its view
-    const uint64_t pairs = (uint64_t)cb * K, cands = pairs * (uint64_t)std::max(s->max_tiles, 1);
-    const uint64_t rows = pairs * (uint64_t)std::max(s->max_tiles_y, 1), bins = std::max(s->all_tiles, 1u);
+    const BatchSize need = batch_size(s, cb, cf);
+    const uint64_t pairs = need.pairs, cands = need.cands, rows = need.rows, bins = need.bins;
     if (cands >= (1ull << 29)) return set_error(GS_ERR_CAPACITY, "too many dirty tiles per batch for this view size");
     destroy_graphs(s);
     free_ssim_buffers(s);
     // new views (which reset cap_B) fit the memory of the last ones as often as not
-    if ((uint64_t)cf > s->cap_flip_mem || pairs > s->cap_pairs || cands > s->cap_cands || rows > s->cap_rows ||
-        bins > s->cap_bins) {
+    if (!batch_fits(need, batch_held(s))) {
         // no capacity until every buffer below is allocated: a failure part way (out
         // of memory) leaves nothing that a later call could take for usable
         free_batch_buffers(s);
@@ -291,14 +314,28 @@ int max_batch(const gs_scene* s) {
     return (int)std::max<uint64_t>(1, std::max(small, std::min<uint64_t>(kMaxPairs / K, kMaxCands / (K * tiles))));
 }
 
-// Buffers for a call of B variants (at most `chunk` a batch): grown in powers of
-// two, so that small calls hold little; out of memory falls back to a smaller
-// batch.  Returns the variants a batch can have in *chunk.
+// Variants per batch of a campaign: the caller's choice, or the most.
+int campaign_batch(const gs_scene* s) { return s->batch > 0 ? std::min(s->batch, max_batch(s)) : max_batch(s); }
+
+// Variants the buffers of a call of B variants, at most `chunk` a batch, are sized for:
+// powers of two, so that small calls hold little.
+int batch_cap(int B, int chunk) {
+    int cap = 64;
+    while (cap < B && cap < chunk) cap *= 2;
+    return std::min(cap, chunk);
+}
+
+// Buffers for a call of B variants (at most `chunk` a batch): a smaller batch where they
+// would take more than batch_room, or than there is memory.  Returns the variants a batch
+// can have in *chunk.
 gs_status size_batch(gs_scene* s, int B, int* chunk) {
     while (true) {
-        int cap = 64;
-        while (cap < B && cap < *chunk) cap *= 2;
-        cap = std::min(cap, *chunk);
+        const int cap = batch_cap(B, *chunk);
+        const BatchSize need = batch_size(s, std::max(cap, s->cap_B), std::max(cap, s->cap_flips)), held = batch_held(s);
+        if (cap > 64 && !batch_fits(need, held) && need.bytes() > s->batch_room) {
+            *chunk = cap / 2;
+            continue;
+        }
         const gs_status rs = ensure_batch_buffers(s, cap, 1);
         if (rs != GS_ERR_OOM || cap <= 64) return rs;
         *chunk = cap / 2;
@@ -390,6 +427,40 @@ gs_status load_prim_box(gs_scene* s, const void* lo, const void* hi, int src_on_
 }
 
 }  // namespace
+
+size_t scene_bytes(const gs_scene* s) {
+    size_t b = (size_t)s->n * (s->nwords + (s->pbox_lo ? 2 * s->nbox_words : 0)) * word_bytes(s->fmt);
+    for (const Buf& v : s->view_bufs) b += v.cap;
+    b += s->list_tmp.cap + render_work_bytes(s->work) + batch_held(s).bytes();
+    b += sizeof(gs_flip) * s->host_io_flips_cap + sizeof(gs_result) * s->host_io_out_cap;
+    if (s->ssim.tile_map) {
+        const SsimBufs& q = s->ssim;
+        const size_t pairs = (size_t)std::min(s->cap_B, ssim_batch(std::max(s->K, 1))) * std::max(s->K, 1);
+        b += (size_t)q.slot_cap * (sizeof(PlanItem) + 4 * (8 + 1 + 9)) + (size_t)q.delta_cap * 32 * sizeof(float4) +
+             2 * sizeof(unsigned long long) * pairs * q.max_tiles;
+    }
+    return b;
+}
+
+size_t allow_batch_growth(gs_scene* s, int B, size_t room) {
+    const BatchSize held = batch_held(s);
+    s->batch_room = room > ~held.bytes() ? ~(size_t)0 : held.bytes() + room;
+    if (s->K == 0 || B < 1) return 0;
+    for (int chunk = campaign_batch(s);; chunk /= 2) {   // as size_batch will settle
+        const int cap = batch_cap(B, chunk);
+        const BatchSize need = batch_size(s, std::max(cap, s->cap_B), std::max(cap, s->cap_flips));
+        if (batch_fits(need, held)) return 0;
+        if (cap <= 64 || need.bytes() <= s->batch_room) return need.bytes() - std::min(need.bytes(), held.bytes());
+        chunk = cap;
+    }
+}
+
+void trim_batch_buffers(gs_scene* s) {
+    destroy_graphs(s);
+    free_ssim_buffers(s);
+    free_batch_buffers(s);
+    if (s->K > 0) ensure_batch_buffers(s, 64, 1);   // (out of memory: the next campaign tries again)
+}
 
 gs_status render_lists_sized_ext(gs_scene* s, RenderWork& w, const DevCamera& cam, uint32_t** ids, uint64_t* npairs,
                                  cudaStream_t st) {
@@ -811,8 +882,7 @@ gs_status inject_and_render(gs_scene* s, const gs_flip* dev_flips, int B, int gu
                             gs_result* dev_out, uint64_t* dev_regions, double* dev_ssim, void* stream) {
     cudaStream_t st = (cudaStream_t)stream;
     const int K = s->K;
-    const int max_chunk = max_batch(s);
-    int chunk = s->batch > 0 ? std::min(s->batch, max_chunk) : max_chunk;
+    int chunk = campaign_batch(s);
     const bool ssim = dev_ssim != nullptr;
     if (ssim) chunk = std::min(chunk, ssim_batch(K));
     if (ssim && (s->tile_w != kTile || s->tile_h != kTile))

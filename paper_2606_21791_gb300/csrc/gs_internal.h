@@ -238,7 +238,7 @@ struct ViewState {
     float4* ent = nullptr;           // pixel blend lists (alpha, r, g, b)
     uint32_t* rk = nullptr;          // their ranks
     float4* state = nullptr;         // clean blend in front of every kWalk-th entry of the lists
-    uint64_t ck_total = 0;           // rows after the tiles' row 0 (the server's size estimate)
+    uint64_t ck_total = 0;           // rows after the tiles' row 0
     uint64_t npairs = 0;
     uint64_t cap_pairs = 0;
 };
@@ -314,6 +314,7 @@ struct gs_scene {
     std::vector<gs_camera> host_cams;       // the cameras of gs_set_views (rebuilt on a tile change)
 
     // batch buffers (dirty engine and plain loop)
+    size_t batch_room = ~(size_t)0;         // most bytes the batch buffers may take (see allow_batch_growth)
     int cap_B = 0;
     int cap_flips = 0;
     uint64_t cap_flip_mem = 0, cap_pairs = 0, cap_cands = 0, cap_rows = 0, cap_bins = 0;   // elements the buffers below hold
@@ -363,10 +364,18 @@ DevCamera make_dev_camera(const gs_camera& c, int tile_w, int tile_h);
 
 // gs_api.cu: the camera sizes and focal lengths the kernels accept
 bool valid_camera(const gs_camera& c);
+// Device bytes a scene holds: parameters, boxes, views, scratch, batch buffers.
+size_t scene_bytes(const gs_scene* s);
+// Lets a campaign of B single upsets grow the scene's batch buffers by up to `room` bytes
+// (it runs in smaller batches otherwise); returns by how much it will.
+size_t allow_batch_growth(gs_scene* s, int B, size_t room);
+void trim_batch_buffers(gs_scene* s);   // back to what gs_set_views allocates
 
 // k_sort.cu
 gs_status alloc_render_work(RenderWork& w, uint64_t n, uint64_t cap_pairs, int ntiles);
 void free_render_work(RenderWork& w);
+size_t render_work_bytes(const RenderWork& w);                                // device bytes it holds
+size_t render_work_bytes(uint64_t n, uint64_t pairs, int ntiles);             // ... and would hold for one view
 gs_status launch_rects_to_keys(const float* depth, const int32_t* rects, uint64_t n, int tiles_x, int tiles_y,
                                uint32_t* keys, uint32_t* vals, uint2* prects, cudaStream_t st);
 

@@ -997,6 +997,23 @@ gs_status alloc_render_work(RenderWork& w, uint64_t n, uint64_t cap_pairs, int n
     return GS_OK;
 }
 
+// Device bytes of a scratch of these sizes (see alloc_render_work).
+static size_t work_bytes(uint64_t n, uint64_t pairs, uint64_t radix_pairs, uint64_t hist_items, size_t tab_words,
+                         int ntiles) {
+    const int hb = radix_blocks_upto(std::max<uint64_t>(hist_items, 1));
+    const size_t prims = n * (sizeof(BlendRec) + 2 * sizeof(uint2) + 7 * 4) + 8 * (div_up(n, kScanTile) + 1) + 64;
+    const size_t radix = 12 * radix_pairs + 1024ull * hb + 8ull * std::max(hist_parts(hb) + 8, 136);
+    return prims + 4 * pairs + radix + 4 * tab_words + sizeof(uint2) * (size_t)ntiles + 64;
+}
+size_t render_work_bytes(uint64_t n, uint64_t pairs, int ntiles) {
+    const bool radix = ntiles > kDirectTiles;
+    return work_bytes(n, pairs, radix ? pairs : 0, std::max<uint64_t>(radix ? pairs : 0, n),
+                      radix ? 0 : direct_tab_words(std::max(ntiles, 1), pairs), ntiles);
+}
+size_t render_work_bytes(const RenderWork& w) {
+    return w.recs ? work_bytes(w.n, w.cap_pairs, w.radix_pairs, w.hist_items, w.tab_words, w.ntiles_cap) : 0;
+}
+
 void free_render_work(RenderWork& w) {
     cudaFree(w.recs);
     cudaFree(w.rects);

@@ -10,7 +10,9 @@
 // render or a storm frame writes the resident parameters (flips, guard
 // clamps) and runs alone on its scene; (2) the memory it would add (growth of
 // the slot's render scratch) fits the budget next to the resident scenes and
-// the scratch already held.  Requests that arrive while others run are admitted
+// the scratch already held; a campaign grows its scene's batch buffers as far as
+// the budget has room (it runs in smaller batches otherwise), and gives the growth back
+// when a request waits for memory.  Requests that arrive while others run are admitted
 // as soon as a slot and memory free up, so work from different requests
 // overlaps on the device.  A request that can never fit is refused
 // (GS_ERR_BUSY).  Latencies are taken on the host clock from submission (or the
@@ -48,7 +50,8 @@ struct Req {
 
 struct SceneEntry {
     gs_scene* s = nullptr;
-    uint64_t resident = 0;
+    uint64_t resident = 0;   // device bytes when it was added
+    uint64_t grown = 0;      // and what campaigns have grown its batch buffers by since (given back when memory is short)
     int readers = 0;
     bool campaign = false;
     bool writer = false;
@@ -61,23 +64,6 @@ struct Slot {
     unsigned long long* clamps = nullptr;
     std::thread th;
 };
-
-uint64_t render_scratch_bytes(uint64_t n, uint64_t pairs, int ntiles) {
-    // records, rects, depth keys/values (x2), counts, offsets, scan space, pairs (x2 keys and values),
-    // histograms, ranges
-    return n * (sizeof(BlendRec) + 8 + 16 + 8 + 12) + pairs * 16 + ntiles * 8 + (pairs / 2048 + 1) * 1024 + (1 << 20);
-}
-
-uint64_t scene_resident_bytes(const gs_scene* s) {
-    uint64_t b = s->n * (uint64_t)s->nwords * word_bytes(s->fmt);
-    if (s->pbox_lo) b += 2ull * s->n * s->nbox_words * word_bytes(s->fmt);
-    for (const auto& v : s->views)
-        b += s->n * (sizeof(BlendRec) + 8) + v.npairs * 8 + (uint64_t)v.cam.tiles_x * v.cam.tiles_y * 8 +
-             (uint64_t)v.cam.W * v.cam.H * 16 + v.ck_total * 16ull * (uint64_t)(v.cam.tile_w * v.cam.tile_h) +
-             (uint64_t)v.cam.tiles_x * v.cam.tiles_y * 12;
-    b += render_scratch_bytes(s->work.n, s->work.cap_pairs, s->work.ntiles_cap);
-    return b;
-}
 
 double now_ms(std::chrono::steady_clock::time_point t0) {
     return std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
@@ -114,17 +100,30 @@ bool scene_allows(const SceneEntry& e, const gs_request& r) {
 
 uint64_t request_need(gs_server* sv, const Req* q) {
     const gs_request& r = q->r;
-    if (r.kind == GS_REQ_CAMPAIGN) return 0;   // runs in the scene's own (resident) buffers
+    if (r.kind == GS_REQ_CAMPAIGN) return 0;   // runs in the scene's own buffers, which grow as far as there is room
     const gs_scene* s = sv->scenes[r.scene].s;
     DevCamera cam = make_dev_camera(r.cam, s->tile_w, s->tile_h);
     int ntiles = cam.tiles_x * cam.tiles_y;
-    return render_scratch_bytes(s->n, std::max<uint64_t>(8 * s->n, 1024), ntiles);
+    return render_work_bytes(s->n, std::max<uint64_t>(8 * s->n, 1024), ntiles);
 }
 
 uint64_t resident_total(gs_server* sv) {
     uint64_t r = 0;
     for (auto& e : sv->scenes) r += e.resident;
     return r;
+}
+
+uint64_t used_total(gs_server* sv) {
+    uint64_t r = resident_total(sv) + sv->scratch_total;
+    for (auto& e : sv->scenes) r += e.grown;
+    return r;
+}
+
+// What a scene holds now, when no campaign runs on it (under the server lock).
+void account(SceneEntry& e) {
+    const uint64_t b = scene_bytes(e.s);
+    e.resident = std::min(e.resident, b);
+    e.grown = b - e.resident;
 }
 
 // run one request on a slot's stream (scene s, taken under the server lock);
@@ -163,7 +162,7 @@ void worker(gs_server* sv, int slot_id) {
         uint64_t extra = 0;
         while (!pick) {
             if (sv->stop && sv->queue.empty()) return;
-            uint64_t base = resident_total(sv) + sv->scratch_total;
+            const uint64_t base = used_total(sv);
             bool mem_blocked = false;
             for (auto it = sv->queue.begin(); it != sv->queue.end(); ++it) {
                 Req* q = *it;
@@ -183,6 +182,20 @@ void worker(gs_server* sv, int slot_id) {
             }
             if (!pick) {
                 if (sv->stop && sv->queue.empty()) return;
+                auto idle = std::find_if(sv->scenes.begin(), sv->scenes.end(),
+                                         [](const SceneEntry& e) { return e.grown > 0 && !e.campaign && !e.writer; });
+                if (mem_blocked && idle != sv->scenes.end()) {
+                    // memory blocks the queue: a scene without a campaign gives its batch buffers' growth back
+                    SceneEntry& e = *idle;
+                    e.campaign = true;
+                    lk.unlock();
+                    trim_batch_buffers(e.s);
+                    lk.lock();
+                    e.campaign = false;
+                    account(e);
+                    sv->cv_work.notify_all();
+                    continue;
+                }
                 if (mem_blocked && sl.scratch > 0) {
                     // memory blocks the queue: give this idle slot's scratch back
                     uint64_t give = sl.scratch;
@@ -206,6 +219,10 @@ void worker(gs_server* sv, int slot_id) {
         else e.readers++;
         sl.scratch += extra;
         sv->scratch_total += extra;
+        if (pick->r.kind == GS_REQ_CAMPAIGN) {
+            const uint64_t used = used_total(sv);
+            e.grown += allow_batch_growth(e.s, pick->r.nflips, sv->budget > used ? sv->budget - used : 0);
+        }
         pick->status = -2;
         pick->slot = slot_id;
         if (pick->mem_waited) sv->mem_delayed++;
@@ -218,8 +235,16 @@ void worker(gs_server* sv, int slot_id) {
 
         lk.lock();
         if (writes) e.writer = false;
-        else if (pick->r.kind == GS_REQ_CAMPAIGN) e.campaign = false;
-        else e.readers--;
+        else if (pick->r.kind == GS_REQ_CAMPAIGN) {
+            e.campaign = false;
+            scene->batch_room = ~(size_t)0;
+            account(e);
+        } else e.readers--;
+        const uint64_t held = render_work_bytes(sl.work);   // more pairs than the request was admitted for
+        if (held > sl.scratch) {
+            sv->scratch_total += held - sl.scratch;
+            sl.scratch = held;
+        }
         pick->t_done = now_ms(sv->t0);
         pick->err = msg;
         pick->status = rs;
@@ -259,9 +284,8 @@ gs_status gs_server_create(uint64_t hbm_budget_bytes, int nslots, gs_server** ou
 gs_status gs_server_add_scene(gs_server* sv, gs_scene* s, int* scene_id) {
     if (!sv || !s || !scene_id) return set_error(GS_ERR_ARG, "bad gs_server_add_scene arguments");
     std::lock_guard<std::mutex> lk(sv->mu);
-    uint64_t res = scene_resident_bytes(s);
-    if (resident_total(sv) + sv->scratch_total + res > sv->budget)
-        return set_error(GS_ERR_BUSY, "scene does not fit the HBM budget");
+    uint64_t res = scene_bytes(s);
+    if (used_total(sv) + res > sv->budget) return set_error(GS_ERR_BUSY, "scene does not fit the HBM budget");
     SceneEntry e;
     e.s = s;
     e.resident = res;
@@ -345,7 +369,7 @@ gs_status gs_server_stats(gs_server* sv, uint64_t* host_stats) {
     if (!sv || !host_stats) return set_error(GS_ERR_ARG, "bad gs_server_stats arguments");
     std::lock_guard<std::mutex> lk(sv->mu);
     host_stats[0] = sv->budget;
-    host_stats[1] = resident_total(sv);
+    host_stats[1] = used_total(sv) - sv->scratch_total;
     host_stats[2] = sv->scratch_total;
     host_stats[3] = sv->queue.size();
     host_stats[4] = sv->completed;

@@ -154,3 +154,60 @@ def test_boxes_after_a_failed_upload(fake):
         G.gs_inject_and_render(h, ADDR, 8, 1, G.GS_GUARD_PRIM, 1, ADDR, stream=0)
     clean(h)
     """)
+
+
+SMALL = 1 << 20   # counters, cameras and the like, that the account leaves out
+
+
+@pytest.mark.parametrize("sizes", [((1600, 1040),), ((2592, 1944), (640, 480))])
+def test_server_account(fake, sizes):
+    """The server's resident bytes are the memory that its scenes hold, campaigns'
+    batch buffers included; a tight budget holds, and what a campaign grew by is given
+    back to a render that waits."""
+    run(fake, f"""
+    small = {SMALL}
+    L.fake_counts(100_000, 30)   # five tiles a primitive: within what a render is admitted for
+    h = scene()
+    G.gs_set_views(h, cams(*{sizes}), stream=0)
+    scene_live = L.fake_live()
+
+    def check(srv, slack=small):
+        s = G.gs_server_stats(srv)
+        assert abs(s["resident"] + s["scratch"] - L.fake_live()) < slack, (s, L.fake_live())
+        return s
+
+    def ask(srv, **kw):
+        G.gs_server_wait(srv, G.gs_server_submit(srv, G.make_request(**kw)))
+
+    campaign = dict(kind=G.GS_REQ_CAMPAIGN, scene=0, dev_flips=ADDR, nflips=20_000, dev_results=ADDR)
+    render = dict(kind=G.GS_REQ_RENDER, scene=0, cam=cams((1600, 1040))[0], dev_rgb=ADDR)
+    srv = G.gs_server_create(1 << 40, 1)
+    G.gs_server_add_scene(srv, h)
+    check(srv)
+    ask(srv, **campaign)
+    big = check(srv)["resident"]
+    assert big > scene_live + (100 << 20)
+    before = L.fake_live()
+    ask(srv, **render)
+    s = G.gs_server_stats(srv)
+    assert s["scratch"] >= L.fake_live() - before > 0   # reserved by its estimate
+    scratch = s["scratch"]
+    G.gs_server_destroy(srv)
+    G.gs_free_scene(h)
+    assert L.fake_live() < small
+
+    h = scene()
+    G.gs_set_views(h, cams(*{sizes}), stream=0)
+    budget = L.fake_live() + scratch + (40 << 20)
+    srv = G.gs_server_create(budget, 1)
+    G.gs_server_add_scene(srv, h)
+    for _ in range(3):
+        ask(srv, **campaign)
+        s = check(srv, small + scratch)
+        assert s["resident"] + s["scratch"] <= budget and L.fake_live() <= budget + small
+        ask(srv, **render)
+        s = G.gs_server_stats(srv)
+        assert s["resident"] + s["scratch"] <= budget and L.fake_live() <= budget + small
+    G.gs_server_destroy(srv)
+    clean(h)
+    """)
