@@ -326,15 +326,21 @@ int batch_cap(int B, int chunk) {
 }
 
 // Buffers for a call of B variants (at most `chunk` a batch): a smaller batch where they
-// would take more than batch_room, or than there is memory.  Returns the variants a batch
-// can have in *chunk.
+// would take more than batch_room, or than there is memory.  Memory is looked at before
+// anything is given up, so the next call of this size settles for the same batch and
+// keeps its buffers.  Returns the variants a batch can have in *chunk.
 gs_status size_batch(gs_scene* s, int B, int* chunk) {
+    constexpr size_t kSlack = 16ull << 20;   // the allocator's granules
     while (true) {
         const int cap = batch_cap(B, *chunk);
         const BatchSize need = batch_size(s, std::max(cap, s->cap_B), std::max(cap, s->cap_flips)), held = batch_held(s);
-        if (cap > 64 && !batch_fits(need, held) && need.bytes() > s->batch_room) {
-            *chunk = cap / 2;
-            continue;
+        if (cap > 64 && !batch_fits(need, held)) {
+            size_t avail = 0, all = 0;
+            GS_CUDA(cudaMemGetInfo(&avail, &all));
+            if (need.bytes() > s->batch_room || need.bytes() + kSlack > avail + held.bytes()) {
+                *chunk = cap / 2;
+                continue;
+            }
         }
         const gs_status rs = ensure_batch_buffers(s, cap, 1);
         if (rs != GS_ERR_OOM || cap <= 64) return rs;

@@ -211,3 +211,33 @@ def test_server_account(fake, sizes):
     G.gs_server_destroy(srv)
     clean(h)
     """)
+
+
+def test_batch_size_settles(fake):
+    """Where memory is short for the whole batch, a campaign settles for a smaller one:
+    the next calls of its size allocate nothing, and the whole batch is back once there
+    is memory."""
+    run(fake, """
+    L.fake_counts(100_000, 30, 100)
+    h = scene()
+    G.gs_set_views(h, cams((1600, 1040)), stream=0)
+    held = L.fake_live()
+
+    def campaign(B=20_000):
+        a = L.fake_allocations()
+        G.gs_inject_and_render(h, ADDR, B, 1, -1, 0, ADDR, stream=0)
+        return L.fake_allocations() - a
+
+    for room in (40 << 20, 300 << 20, 1 << 30):
+        G.gs_set_views(h, cams((1600, 1040)), stream=0)
+        L.fake_limit(held + room)
+        campaign()
+        assert held + room // 4 < L.fake_live() <= held + room   # about as much as there is room for
+        assert campaign() == 0 and campaign() == 0
+        L.fake_limit((1 << 64) - 1)
+        assert campaign() > 0 and L.fake_live() > held + (2 << 30)
+        assert campaign() == 0
+        G.gs_free_scene(h)
+        h = scene()
+    clean(h)
+    """)
