@@ -291,8 +291,8 @@ GS_API gs_status gs_read_kernel_ms(gs_scene* scene, float* ms);
  * binning + tile lists + tile ranges, ms[2] = blend (3 floats), and counts[0] =
  * primitives, counts[1] = (tile, primitive) pairs of that view, counts[2] = 8-bit
  * digits of the depth keys (4), counts[3] = 8-bit digits of the tile ids: the
- * passes a radix sort of the keys takes (4 uint64; grids of up to 13,900 tiles are
- * listed by counting instead).  GS_ERR_STATE while timing is off or before the
+ * passes a radix sort of the keys takes (4 uint64; most grids of up to 13,900
+ * tiles are listed by counting instead).  GS_ERR_STATE while timing is off or before the
  * first gs_render after it was switched on. */
 GS_API gs_status gs_read_render_ms(gs_scene* scene, float* ms, uint64_t* counts);
 /* Most variants per dirty-tile batch (0 = largest allowed: 65536 / K, as far as

@@ -5,8 +5,8 @@
 // by depth once (32-bit depth bits, 4 stable passes of 8 bits, values = primitive
 // index, ties kept in index order; small scenes in one block), and their (tile,
 // primitive) pairs, in that order, are dealt to the tiles' lists: by counting, for
-// grids of up to kDirectTiles tiles, else by writing the pairs out and sorting them
-// stably by tile id (ceil(log2 tiles / 8) passes).  The result equals a stable sort
+// most grids of up to kDirectTiles tiles (listed_by_counting), else by writing the pairs
+// out and sorting them stably by tile id (ceil(log2 tiles / 8) passes).  The result equals a stable sort
 // of (tile << 32 | depth bits) keys emitted in primitive order, with depth ties
 // broken by primitive index.
 //
@@ -346,8 +346,9 @@ __global__ __launch_bounds__(kScanBlockT) void k_scan_apply(const uint32_t* in, 
 //   k_tile_place: each warp walks its run again and writes every pair's primitive
 //     at its place: tile start + earlier segments + earlier warps + rank in the run.
 // A list is then in (segment, warp, pair) order, the depth order.  The counters of
-// a warp take 2 bytes a tile, so this runs for grids of up to kDirectTiles tiles;
-// larger ones keep the radix sort of (tile, primitive) pairs below.  Per pair it
+// a warp take 2 bytes a tile, so this runs for grids of up to kDirectTiles tiles; larger
+// ones, and large scenes on large ones, keep the radix sort of (tile, primitive) pairs
+// below.  Per pair it
 // moves 4 B (the primitive, written once) where the sort of 12-bit to 16-bit tile
 // ids moved 60 (emission, two passes, ranges).  Bound by the placing walk's chain per
 // 64 pairs and its stores, a sector per pair: 12.25M pairs of a 2M-primitive,
@@ -356,6 +357,13 @@ __global__ __launch_bounds__(kScanBlockT) void k_scan_apply(const uint32_t* in, 
 // ---------------------------------------------------------------------------
 constexpr int kDirectTiles = 13900;
 constexpr int kWalkGroups = 4;   // see walk_pairs
+
+// Is a grid of nt tiles listed by counting for a scene of n primitives?  Up to about 7,000
+// tiles two blocks fit an SM; with one, the walks of long pair streams fall behind the
+// sort: 2M primitives on 7,684 tiles (12.4M pairs) 440 us against 478, on 10,000 tiles
+// (12.2M) 498 against 474, on 13,000 (17.4M) 620 against 554; 600,000 primitives on 13,000
+// tiles (5.7M) 241 against 271.
+bool listed_by_counting(uint64_t n, int nt) { return nt <= 9000 || (nt <= kDirectTiles && n <= (1ull << 20)); }
 
 // Blocks, warps and shared memory of the two walks for a grid of nt tiles.
 struct DirectShape {
@@ -960,7 +968,7 @@ gs_status alloc_render_work(RenderWork& w, uint64_t n, uint64_t cap_pairs, int n
         w.cap_pairs = cap_pairs;
     }
     // the pair sort's other buffers: only for grids that are not listed by counting
-    const bool radix = ntiles > kDirectTiles;
+    const bool radix = !listed_by_counting(n, ntiles);
     if (radix && w.cap_pairs > w.radix_pairs) {
         w.radix_pairs = 0;
         GS_TRY(A(w.pkey[0], w.cap_pairs));
@@ -1007,7 +1015,7 @@ static size_t work_bytes(uint64_t n, uint64_t pairs, uint64_t radix_pairs, uint6
     return prims + 4 * pairs + radix + 4 * tab_words + sizeof(uint2) * (size_t)ntiles + 64;
 }
 size_t render_work_bytes(uint64_t n, uint64_t pairs, int ntiles) {
-    const bool radix = ntiles > kDirectTiles;
+    const bool radix = !listed_by_counting(n, ntiles);
     return work_bytes(n, pairs, radix ? pairs : 0, std::max<uint64_t>(radix ? pairs : 0, n),
                       radix ? 0 : direct_tab_words(std::max(ntiles, 1), pairs), ntiles);
 }
@@ -1043,7 +1051,8 @@ void free_render_work(RenderWork& w) {
 gs_status build_tile_lists(RenderWork& w, uint64_t n, int tiles_x, int tiles_y, uint32_t** ids_out, cudaStream_t st) {
     int ntiles = tiles_x * tiles_y;
     // every segment's rows are written, so the tables have to hold them all
-    if (ntiles <= kDirectTiles && direct_words(direct_shape(ntiles, w.cap_pairs), ntiles) > w.tab_words)
+    const bool counting = listed_by_counting(n, ntiles);
+    if (counting && direct_words(direct_shape(ntiles, w.cap_pairs), ntiles) > w.tab_words)
         return set_error(GS_ERR_CAPACITY, "the counting tables were not sized for this tile grid");
     int cur = 0;
     unsigned blocks = (unsigned)div_up(std::max<uint64_t>(n, 1), 256);
@@ -1071,7 +1080,7 @@ gs_status build_tile_lists(RenderWork& w, uint64_t n, int tiles_x, int tiles_y, 
     int tbits = 1;
     while ((1 << tbits) < ntiles) tbits++;
     w.passes[1] = (tbits + 7) / 8;
-    if (ntiles <= kDirectTiles) {
+    if (counting) {
         const DirectShape d = direct_shape(ntiles, w.cap_pairs);
         const int thr = d.warps * 32;
         const int tpad = (ntiles + 7) & ~7;   // table rows: whole 16-byte pieces

@@ -1,0 +1,32 @@
+"""gs_bin_tiles on both sides of the choice between counting and the pair sort by the
+number of primitives, one tile or two each.  The reference is numpy's stable sort."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n", [(1 << 20), (1 << 20) + 1])
+@pytest.mark.parametrize("tx,ty", [(100, 90), (91, 99), (139, 100)])
+def test_lists_of_large_scenes(n, tx, ty):
+    import torch
+
+    import paper_2606_21791_gb300 as P
+    P.build()
+    from paper_2606_21791_gb300 import gs as G
+    G.load_library()
+    rng = np.random.default_rng(n + tx)
+    depth = np.round(rng.uniform(0.5, 40.0, n), 2).astype(np.float32)   # many ties
+    x, y = rng.integers(0, tx, n), rng.integers(0, ty, n)
+    w = rng.integers(0, 3, n)   # nothing, one tile, two
+    rects = np.stack([x, y, np.minimum(x + w, tx), y + 1], axis=1).astype(np.int32)
+    wide = np.minimum(x + w, tx) - x
+    prim = np.repeat(np.arange(n), wide)
+    tile = (y * tx + x)[prim] + np.concatenate([[0], (prim[1:] == prim[:-1]).astype(int)])
+    order = np.lexsort((prim, depth[prim], tile))
+    off = torch.zeros(tx * ty + 1, dtype=torch.int32, device="cuda")
+    ids = torch.zeros(len(prim), dtype=torch.int32, device="cuda")
+    assert G.gs_bin_tiles(torch.from_numpy(depth).cuda(), torch.from_numpy(rects).cuda(), n, tx, ty, off, ids,
+                          len(prim)) == len(prim)
+    assert np.array_equal(ids.cpu().numpy(), prim[order])
+    assert np.array_equal(off.cpu().numpy(), np.concatenate([[0], np.cumsum(np.bincount(tile, minlength=tx * ty))]))

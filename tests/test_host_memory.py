@@ -93,11 +93,12 @@ def test_counting_tables_hold_every_grid(fake):
                                  [1, 1000, 1536, 2049, 300_000, 5_000_000, 40_000_000, 2_000_000_000]):
         L.fake_counts(min(cap, 1000), 0)
         G.gs_bin_tiles(ADDR, ADDR, 1, tx, ty, ADDR, ADDR, cap, stream=0)
-    h = scene(n=400_000)
-    L.fake_counts(9_000_000, 0)
-    for W, H in ((2200, 1600), (640, 480), (16, 16), (1600, 1040), (100, 1600), (2592, 1944), (800, 800)):
-        G.gs_render(h, cams((W, H)), ADDR, stream=0)
-    clean(h)
+    for n in (400_000, 1_200_000):
+        h = scene(n=n)
+        L.fake_counts(9_000_000, 0)
+        for W, H in ((2200, 1600), (640, 480), (16, 16), (1600, 1040), (100, 1600), (2592, 1944), (1900, 1250), (800, 800)):
+            G.gs_render(h, cams((W, H)), ADDR, stream=0)
+        clean(h)
     """)
 
 
