@@ -30,8 +30,10 @@ constexpr int kScanT = 1024;
 // Items per thread of a radix pass over up to cap items (kRI below; kRT * kRI per
 // block).  More items make longer runs in the write-out, fewer make more blocks: 4
 // up to 2^19 items (134,826 keys: 22 us a pass of three kernels at 16 items, 17 at
-// 4), 8 up to 2^24 (2M keys: 31 against 28 us; 4 items: 32), 16 beyond.
-int radix_items(uint64_t cap) { return cap <= (1ull << 19) ? 4 : (cap <= (1ull << 24) ? 8 : 16); }
+// 4), 8 up to 2^22 (2M keys: 31 against 28 us; 4 items: 32), 16 beyond (6.6M pairs of
+// 600,000 primitives: depth sort and lists 271 us at 16 items, 287 at 8; 9.4M: 327, 353).
+constexpr uint64_t kItems4 = 1ull << 19, kItems8 = 1ull << 22;
+int radix_items(uint64_t cap) { return cap <= kItems4 ? 4 : (cap <= kItems8 ? 8 : 16); }
 
 __device__ __forceinline__ uint64_t item_count(const unsigned long long* dcount, uint64_t scount) {
     if (!dcount) return scount;
@@ -893,8 +895,7 @@ __global__ __launch_bounds__(kSmallT) void k_order_small(uint32_t* __restrict__ 
 int radix_blocks(uint64_t cap) { return (int)std::max<uint64_t>(1, div_up(cap, (uint64_t)kRT * radix_items(cap))); }
 // the most blocks of any pass over up to cap items
 int radix_blocks_upto(uint64_t cap) {
-    return std::max({radix_blocks(cap), radix_blocks(std::min<uint64_t>(cap, 1ull << 19)),
-                     radix_blocks(std::min<uint64_t>(cap, 1ull << 24))});
+    return std::max({radix_blocks(cap), radix_blocks(std::min(cap, kItems4)), radix_blocks(std::min(cap, kItems8))});
 }
 
 int hist_parts(int nblocks) { return (int)div_up((uint64_t)256 * nblocks, kScanTile); }
