@@ -35,14 +35,15 @@ void fill_view_ptrs(void* host_dst, const ViewState& vs, uint32_t bin0);
 gs_status launch_exclusive_scan(const uint32_t* in, uint64_t n, uint32_t* out, unsigned long long* scratch,
                                 unsigned long long* total, cudaStream_t st);
 uint64_t scan_scratch_len(uint64_t n);
-gs_status launch_blend_clean(const ViewState& v, uint32_t* counts, unsigned int* clean_nonfin, cudaStream_t st);
+gs_status launch_blend_clean(const ViewState& v, uint32_t* counts, uint32_t* blk_cnt, unsigned int* clean_nonfin,
+                             cudaStream_t st);
 gs_status launch_ranks(const uint32_t* key, const uint32_t* id, uint64_t n, const ViewState& v, cudaStream_t st);
 gs_status launch_row_counts(const ViewState& v, uint32_t* rows, cudaStream_t st);
-gs_status launch_list_lens(const uint32_t* counts, uint64_t n, uint32_t cap, uint32_t* lens, cudaStream_t st);
-gs_status launch_fill_lists(const ViewState& v, const uint32_t* off, uint32_t cap, cudaStream_t st);
+gs_status launch_list_lens(const uint32_t* counts, uint64_t n, uint32_t* lens, cudaStream_t st);
+gs_status launch_fill_lists(const ViewState& v, const uint32_t* off, cudaStream_t st);
 gs_status launch_offsets_to_ranges(const uint32_t* offsets, int ntiles, uint2* ranges, cudaStream_t st);
 uint32_t key_to_bits(uint32_t key, int fmt);
-int dirty_grid();
+void dirty_grids();
 
 static thread_local std::string g_last_error;
 
@@ -380,7 +381,7 @@ gs_status run_dirty_batch(gs_scene* s, int B, int guard_mode, uint64_t mask, boo
     for (auto& g : s->graphs)
         if (g.B == B && g.guard == guard_mode && g.mask == mask && g.ssim == ssim && g.regions == regions) ge = &g;
     if (!ge) {
-        dirty_grid();   // occupancy query outside the capture
+        dirty_grids();
         cudaStream_t cs;
         GS_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
         GraphEntry g;
@@ -697,48 +698,80 @@ static gs_status place(Buf& buf, std::initializer_list<Part> parts) {
     return GS_OK;
 }
 
-// Entries of a view's blend lists (22 B each) that are kept: views with more
-// (hundreds of barely visible primitives over every pixel) keep the front of
-// each pixel's list and read the rest from the tile's list.
-constexpr uint64_t kMaxListEntries = 1ull << 29;
+// Is a view with E blend-list entries, whose 8x8 blocks keep S entries for 64 pixels
+// each, dense: better re-blended from its block lists?  The walk of a pixel's
+// own list costs 20 B an entry, an evaluation of a block's entry serves 64 pixels.  Lists
+// win where a pixel takes few of its block's entries or has few to walk.  Campaigns of
+// 4,000 upsets at 1600x1040, lists against blocks: 0.88 of the entries taken, 89 a pixel:
+// 1.85 and 1.28 ms; 0.78, 58: 0.79 and 0.68; 0.66, 55: 0.48 and 0.43; 0.62, 60: 0.82 and
+// 0.90; 0.45, 50: 0.42 and 0.60; 1.0, 32 a pixel: 356 and 911.
+constexpr uint64_t kDenseLength = 48;   // entries of a pixel's list (on average) from which a view may be dense
+static bool dense_view(uint64_t E, uint64_t S) { return (double)E >= 0.65 * 64.0 * (double)S; }
 
-// The blend lists and rows of view v (its first pass is done): sizes on
-// the device, one read-back of the totals, then the second pass.
-static gs_status build_lists(gs_scene* s, ViewState& v, Buf& buf, uint32_t* counts, cudaStream_t st) {
+// The lists of view v (its first pass is done): sizes on the device, a read-back of the
+// totals, then the second pass.  Blend lists (24 B an entry) take at most this view's
+// share of the memory that is free -- one for each view still to come, one for what
+// comes behind them -- else, as in a dense view, the block lists take their place.
+static gs_status build_lists(gs_scene* s, ViewState& v, Buf& buf, uint32_t* counts, int views_left, cudaStream_t st) {
     const uint64_t ntiles = (uint64_t)v.cam.tiles_x * v.cam.tiles_y;
-    const uint64_t P = (uint64_t)v.cam.tile_w * v.cam.tile_h, npix = ntiles * P;
-    uint32_t *rows = nullptr, *lens = nullptr, *off = nullptr;
+    const uint64_t P = (uint64_t)v.cam.tile_w * v.cam.tile_h, npix = ntiles * P, nblk = npix / 64;
+    uint32_t *rows = nullptr, *lens = nullptr, *off = nullptr, *boff = nullptr;
     unsigned long long *scratch = nullptr, *total = nullptr;
     GS_TRY(place(s->list_tmp, {{(void**)&rows, 4 * ntiles},
                                {(void**)&lens, 4 * npix},
                                {(void**)&off, 4 * npix},
+                               {(void**)&boff, 4 * nblk},
                                {(void**)&scratch, 8 * scan_scratch_len(npix)},
                                {(void**)&total, 8 * 6}}));
-    GS_TRY(launch_row_counts(v, rows, st));
-    GS_TRY(launch_exclusive_scan(rows, ntiles, v.row_off, scratch, total, st));
-    uint32_t cap = 0xfffffffdu;
     unsigned long long tot[6];
-    while (true) {
-        GS_TRY(launch_list_lens(counts, npix, cap, lens, st));
-        GS_TRY(launch_exclusive_scan(lens, npix, off, scratch, total + 3, st));
+    auto read_totals = [&]() -> gs_status {
         GS_CUDA(cudaMemcpyAsync(tot, total, sizeof(tot), cudaMemcpyDeviceToHost, st));
         GS_CUDA(cudaStreamSynchronize(st));
-        if (tot[2] >= 0xffffffffull) return set_error(GS_ERR_CAPACITY, "too many blend-list rows");
-        if (tot[5] > std::max<uint64_t>(kMaxListEntries, kWalk * npix)) {
-            cap = (uint32_t)std::min<uint64_t>(cap / 2, std::max<uint64_t>(kMaxListEntries / npix, kWalk) - kWalk);
-            continue;
-        }
-        const gs_status rs = place(buf, {{(void**)&v.row_idx, 4 * P * tot[2]},
-                                         {(void**)&v.ent, sizeof(float4) * tot[5]},
-                                         {(void**)&v.rk, 4 * tot[5]},
-                                         {(void**)&v.state, sizeof(float4) * (tot[5] / kWalk)}});
-        if (rs == GS_OK) break;
-        if (rs != GS_ERR_OOM || cap == 0) return rs;
-        // keep less of the lists (a quarter of the mean length at a time)
-        cap = (uint32_t)std::min<uint64_t>(cap / 4, tot[5] / npix / 4);
+        return GS_OK;
+    };
+    GS_TRY(launch_row_counts(v, rows, st));
+    GS_TRY(launch_exclusive_scan(rows, ntiles, v.row_off, scratch, total, st));
+    GS_TRY(launch_list_lens(counts, npix, lens, st));
+    GS_TRY(launch_exclusive_scan(lens, npix, off, scratch, total + 3, st));
+    GS_TRY(read_totals());
+    const uint64_t nrows = tot[2], E = tot[5];
+    const uint64_t bytes = 4 * P * nrows + (16 + 4) * E + 16 * (E / kWalk);   // and at most 1 KB to align the parts
+    bool lists = nrows < 0xffffffffull && E < 0xffffffffull;
+    if (lists && (!buf.p || bytes > buf.cap)) {
+        size_t avail = 0, all = 0;
+        GS_CUDA(cudaMemGetInfo(&avail, &all));
+        lists = bytes <= (avail + buf.cap) / (uint64_t)(views_left + 1);
     }
-    v.ck_total = tot[2] - ntiles;
-    return launch_fill_lists(v, off, cap, st);
+    bool counted = false;   // tot[2]: entries of the block lists
+    auto count_blocks = [&]() -> gs_status {
+        if (counted) return GS_OK;
+        counted = true;
+        GS_TRY(launch_exclusive_scan(v.sub_cnt, nblk, boff, scratch, total, st));
+        return read_totals();
+    };
+    if (lists && E >= kDenseLength * npix) {
+        GS_TRY(count_blocks());
+        lists = !dense_view(E, tot[2]);
+    }
+    if (lists) {
+        const gs_status rs = place(buf, {{(void**)&v.row_idx, 4 * P * nrows},
+                                         {(void**)&v.ent, sizeof(float4) * E},
+                                         {(void**)&v.rk, 4 * E},
+                                         {(void**)&v.state, sizeof(float4) * (E / kWalk)}});
+        if (rs != GS_OK && rs != GS_ERR_OOM) return rs;
+        lists = rs == GS_OK;
+    }
+    if (!lists) {
+        v.row_idx = v.rk = nullptr;
+        v.ent = v.state = nullptr;
+        GS_TRY(count_blocks());
+        if (tot[2] >= 0xffffffffull) return set_error(GS_ERR_CAPACITY, "too many block-list entries");
+        GS_TRY(place(buf, {{(void**)&v.sub, sizeof(uint2) * tot[2]},
+                           {(void**)&v.sub_off, 4 * nblk},
+                           {(void**)&v.row_state, sizeof(float4) * 64 * (tot[2] / kRowStride + nblk)}}));
+        GS_CUDA(cudaMemcpyAsync(v.sub_off, boff, 4 * nblk, cudaMemcpyDeviceToDevice, st));
+    }
+    return launch_fill_lists(v, off, st);
 }
 
 // The clean per-view state of gs_set_views, for validated arguments.
@@ -779,15 +812,16 @@ static gs_status build_views(gs_scene* s, const gs_camera* host_cams, int K, cud
                                            {(void**)&v.row_key, (size_t)4 * ntiles * kRowsPerTile},
                                            {(void**)&v.row_off, (size_t)4 * ntiles},
                                            {(void**)&v.row_cnt, (size_t)4 * ntiles},
+                                           {(void**)&v.sub_cnt, 4 * tpix / 64},
                                            {(void**)&counts, 4 * tpix}}));
         GS_CUDA(cudaMemcpyAsync(v.recs, s->work.recs, sizeof(BlendRec) * s->n, cudaMemcpyDeviceToDevice, st));
         GS_CUDA(cudaMemcpyAsync(v.rects, s->work.rects, sizeof(uint2) * s->n, cudaMemcpyDeviceToDevice, st));
         GS_CUDA(cudaMemcpyAsync(v.ids, ids, sizeof(uint32_t) * np, cudaMemcpyDeviceToDevice, st));
         GS_CUDA(cudaMemcpyAsync(v.ranges, s->work.ranges, sizeof(uint2) * ntiles, cudaMemcpyDeviceToDevice, st));
         GS_TRY(launch_ranks(s->work.dkey[s->work.cur], s->work.dval[s->work.cur], s->n, v, st));
-        GS_TRY(launch_blend_clean(v, counts, s->clean_nonfin + k, st));
-        GS_TRY(build_lists(s, v, s->view_bufs[2 * k + 1], counts, st));
+        GS_TRY(launch_blend_clean(v, counts, v.sub_cnt, s->clean_nonfin + k, st));
         v.npairs = np;
+        GS_TRY(build_lists(s, v, s->view_bufs[2 * k + 1], counts, K - k, st));
         fill_view_ptrs(vptrs.data() + view_ptrs_size() * k, v, all_tiles);
         all_tiles += (uint32_t)ntiles;
         max_pairs = std::max(max_pairs, np);

@@ -33,6 +33,7 @@ constexpr int kMaxWords = 59;
 constexpr int kMaxPairs = 65536;      // (variant, view) pairs per dirty-tile batch
 constexpr uint64_t kMaxCands = 1ull << 28;   // candidate tiles a batch has room for, unless it is small (20 B each)
 constexpr int kSmallPairs = 8192, kSmallBatch = 2048;   // such a batch; also the largest with SSIM on
+constexpr int kRowStride = 64;        // list entries from one row to the next (see ViewPtrs)
 constexpr int kRowsPerTile = 64;      // rows of a tile after row 0
 constexpr int kWalk = 4;              // blend-list entries taken at a time: 64 bytes
 // first bit of the sign and exponent bits a sign+exponent code protects
@@ -138,7 +139,13 @@ struct ViewPtrs {
     const float4* state;         // clean blend (T, C) in front of every kWalk-th entry of the lists
     int W, H, tiles_x, tile_w, tile_h;
     uint32_t bin0;               // tiles of the views before this one
-    uint32_t pad[2];
+    // a dense view (no blend lists): per 8x8 block the entries of its tile's list that
+    // its cull leaves, as (primitive, rank), and the clean blend (T, C) of its pixels in
+    // front of every kRowStride-th of them
+    const uint2* sub;
+    const uint32_t* sub_off;
+    const uint32_t* sub_cnt;
+    const float4* row_state;
 };
 
 constexpr uint32_t kNoRank = 0xfffffffeu;   // above every primitive's rank, below a list's end (0xffffffff)
@@ -238,7 +245,10 @@ struct ViewState {
     float4* ent = nullptr;           // pixel blend lists (alpha, r, g, b)
     uint32_t* rk = nullptr;          // their ranks
     float4* state = nullptr;         // clean blend in front of every kWalk-th entry of the lists
-    uint64_t ck_total = 0;           // rows after the tiles' row 0
+    uint2* sub = nullptr;            // dense views, in place of the five above: block lists (see ViewPtrs)
+    uint32_t* sub_off = nullptr;
+    uint32_t* sub_cnt = nullptr;     // [8x8 blocks] entries that a block's cull leaves
+    float4* row_state = nullptr;
     uint64_t npairs = 0;
     uint64_t cap_pairs = 0;
 };

@@ -21,6 +21,7 @@
 // per pixel, re-blends the pixels that can change from their own blend lists
 // (kept with the clean view), with the clean entry left out and the corrupted
 // record at its (depth, index) place, and compares them on the fly.
+#include <algorithm>
 #include <mutex>
 
 #include "gs_internal.h"
@@ -86,38 +87,10 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
-// Exponent of the Gaussian at offset (dx, dy): -(ca dx^2 + cc dy^2)/2 - cb dx dy,
-// evaluated as s = fma(cc dy, dy, ca dx dx), power = fma(-cb dx, dy, -s/2): each
-// product rounded on its own, each sum fused with its product (one rounding).
-// Every evaluation here (and the oracle's) takes this order, so it is
-// reproducible bit for bit -- which matters for near-degenerate conics, where
-// cancellation makes the rounding error large compared with the value.  No
-// product feeds a separate addition, so the packed two-pixel form in the walk
-// (fp32x2 operations) computes the same bits as this scalar one.
-__device__ __forceinline__ float gauss_power(float ca, float cb, float cc, float dx, float dy) {
-    const float t1 = __fmul_rn(__fmul_rn(ca, dx), dx);
-    const float s = __fmaf_rn(__fmul_rn(cc, dy), dy, t1);
-    return __fmaf_rn(__fmul_rn(-cb, dx), dy, __fmul_rn(-0.5f, s));
-}
-
-// alpha of a record at a pixel centre as the blend computes it, before the cap;
-// returns false where the blend skips the record (power > 0 or alpha < 1/255).
-__device__ __forceinline__ bool blend_alpha(float mx, float my, float ca, float cb, float cc, float opac, float pxc,
-                                            float pyc, float& alpha) {
-    const float power = gauss_power(ca, cb, cc, __fsub_rn(mx, pxc), __fsub_rn(my, pyc));
-    if (power > 0.0f) return false;
-    alpha = opac * ex2_approx(__fmul_rn(power, kLog2e));
-    return !(alpha < 1.0f / 255.0f);
-}
-
 // Each warp tests 32 staged entries at a time against its pixel block (one box
 // load per lane, a ballot), then walks only the survivors in list order.  An
 // entry culled here cannot reach alpha >= 1/255 at any of the warp's pixels, so
 // skipping it changes no pixel; a NaN box never culls.
-// List entries per row of a tile: where each pixel's blend list stands is kept for
-// every kRowStride-th entry of the tile's list, up to its last stop.
-constexpr int kRowStride = 64;
-
 // Survivors a warp takes at a time: their alphas do not depend on the pixel
 // state, so they are computed as independent chains, then applied in list order.
 // The front-to-back step of one entry at one pixel (alpha capped at 0.99, NaN
@@ -156,10 +129,16 @@ __device__ __forceinline__ bool apply_entry(Pix& p, bool live, bool ok, float a,
 }
 
 // alpha of an entry at this lane's two pixels, which share a column (centres
-// (pxc, pyA) and (pxc, pyB), npy = (-pyA, -pyB)): the x offset and the exponent's
-// terms that depend on it alone (ca dx dx, -cb dx) are computed once for both,
-// the rest of gauss_power's order as packed fp32x2 operations over the two
-// pixels, so every pixel gets the bits of a one-pixel evaluation (blend_alpha).
+// (pxc, pyA) and (pxc, pyB), npy = (-pyA, -pyB)); ok: the blend takes the entry there
+// (power <= 0 or NaN, alpha not below 1/255).  The exponent of the Gaussian at offset
+// (dx, dy), power = -(ca dx^2 + cc dy^2)/2 - cb dx dy, is evaluated as s = fma(cc dy, dy,
+// ca dx dx), power = fma(-cb dx, dy, -s/2): each product rounded on its own, each sum
+// fused with its product (one rounding).  Every evaluation here (and the oracle's) takes
+// this order, so it is reproducible bit for bit -- which matters for near-degenerate
+// conics, where cancellation makes the rounding error large compared with the value.
+// The x offset and the terms that depend on it alone are computed once for both pixels,
+// the rest as packed fp32x2 operations: no product feeds a separate addition, so they
+// compute the bits of the scalar order.
 __device__ __forceinline__ float2 alpha_pair(const EntryQ& q, float pxc, float2 npy, bool& okA, bool& okB) {
     const float dx = __fsub_rn(q.q0.x, pxc);
     const float t1 = __fmul_rn(__fmul_rn(q.q0.z, dx), dx);
@@ -207,8 +186,8 @@ __device__ __forceinline__ void walk_survivors2(unsigned m, int c, const Fetch& 
     }
 }
 
-// The two pixels of a lane in a full-frame tile: 8x8 block b = warp of the
-// tile, pixel A at (lane % 8, lane / 8) of the block, B four rows below; u0 and
+// The two pixels of a lane in 8x8 block b of a tile (the full-frame kernels: b =
+// warp): pixel A at (lane % 8, lane / 8) of the block, B four rows below; u0 and
 // u1 are their indices in the tile's natural (8x4 block) order.
 struct Pix2Geo {
     int px, pyA, pyB, u0, u1;
@@ -217,8 +196,8 @@ struct Pix2Geo {
     bool inA, inB;
 };
 
-__device__ __forceinline__ Pix2Geo pix2_geo(int tile_x, int tile_y, int tw, int th, int W, int H) {
-    const int lane = threadIdx.x & 31, b = threadIdx.x >> 5, lg = tile_lgx(tw);
+__device__ __forceinline__ Pix2Geo pix2_geo(int tile_x, int tile_y, int tw, int th, int W, int H, int b) {
+    const int lane = threadIdx.x & 31, lg = tile_lgx(tw);
     Pix2Geo g;
     const int bx = tile_x * tw + block_x0(b, lg), by = tile_y * th + block_y0(b, lg);
     g.px = bx + (lane & 7);
@@ -278,11 +257,13 @@ __device__ __forceinline__ bool rect_reachable(float mx, float my, float ca, flo
 
 // The clean views' stages: records as they are, one entry per thread and batch.
 constexpr int kStageMax = kBT / 2;
-struct RawStage {
-    float4 q0[kStageMax];   // mx, my, ca, cb
-    float4 q1[kStageMax];   // cc, opacity, ex, ey
-    float4 q2[kStageMax];   // r, g, b, depth
+template <int N>
+struct RawStageN {
+    float4 q0[N];   // mx, my, ca, cb
+    float4 q1[N];   // cc, opacity, ex, ey
+    float4 q2[N];   // r, g, b, depth
 };
+using RawStage = RawStageN<kStageMax>;
 
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
     const unsigned saddr = (unsigned)__cvta_generic_to_shared(smem);
@@ -368,9 +349,9 @@ __device__ __forceinline__ void blend_chunk2(const Stage& s, int c, int cnt, con
     walk_survivors2(m, c, fetch, g.pxc, g.pycA, g.pycB, apply, after);
 }
 
-template <bool CONIC, class Apply, class After>
-__device__ __forceinline__ void blend_chunk2(const RawStage& s, int c, int cnt, const Pix2Geo& g, const Apply& apply,
-                                             const After& after) {
+// survivors of entries [c, c + 32) of a raw stage
+template <bool CONIC, int N>
+__device__ __forceinline__ unsigned chunk_survivors(const RawStageN<N>& s, int c, int cnt, const Pix2Geo& g) {
     const int j = c + (threadIdx.x & 31);
     bool pass = false;
     float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
@@ -384,6 +365,12 @@ __device__ __forceinline__ void blend_chunk2(const RawStage& s, int c, int cnt, 
         pass = pass && rect_reachable(a.x, a.y, a.z, a.w, b.x, b.y, g.wx0, g.wx1, g.wy0, g.wy1);
         m = __ballot_sync(0xffffffffu, pass);
     }
+    return m;
+}
+
+template <int N, class Apply, class After>
+__device__ __forceinline__ void walk_raw2(unsigned m, const RawStageN<N>& s, int c, const Pix2Geo& g,
+                                          const Apply& apply, const After& after) {
     auto fetch = [&](int e) {
         const float4 q1 = s.q1[e], q2 = s.q2[e];
         return EntryQ{s.q0[e], q1.x, q1.y, q2.x, q2.y, q2.z};
@@ -480,7 +467,7 @@ __global__ __launch_bounds__(kBT / 2) void k_blend_full(const BlendRec* __restri
     __shared__ Stage s;
     const int tile = blockIdx.x;
     const uint32_t P = (uint32_t)(tw * th);   // pixels of a tile = records staged per batch
-    const Pix2Geo g = pix2_geo(tile % tiles_x, tile / tiles_x, tw, th, W, H);
+    const Pix2Geo g = pix2_geo(tile % tiles_x, tile / tiles_x, tw, th, W, H, threadIdx.x >> 5);
     Pix pA{1.0f, 0.0f, 0.0f, 0.0f, !g.inA}, pB{1.0f, 0.0f, 0.0f, 0.0f, !g.inB};
     const uint2 rg = ranges[tile];
     unsigned int nev = 0, staged = 0;
@@ -523,13 +510,15 @@ __global__ __launch_bounds__(kBT / 2) void k_blend_full(const BlendRec* __restri
 
 // ---------------------------------------------------------------------------
 // Clean views: the blend of k_blend_full, and what the dirty-tile engine keeps
-// of it.  Two passes of the same blend:
-//   FILL = false: the image, the rank of the entry that stopped each pixel
-//     (0xffffffff if none), each tile's largest stop and the length of each
-//     pixel's blend list;
-//   FILL = true: the pixels' blend lists, the blend's state in front of every
-//     kWalk-th of their entries, and the rows that say where each list stands at
-//     every kRowStride-th entry of the tile's list.
+// of it.  Two passes of the same blend, the second in one of two forms:
+//   kImage: the image, the rank of the entry that stopped each pixel (0xffffffff if
+//     none), each tile's largest stop and the length of each pixel's blend list;
+//   kLists: the pixels' blend lists, the blend's state in front of every kWalk-th of
+//     their entries, and the rows that say where each list stands at every
+//     kRowStride-th entry of the tile's list;
+//   kBlocks: of a view without blend lists (a dense one, see dense_view in gs_api.cu),
+//     each 8x8 block's list -- the entries of the tile's list that its cull leaves --
+//     and the pixels' states in front of every kRowStride-th of its entries.
 //
 // A pixel's blend list holds the entries its blend takes (power <= 0 and alpha >=
 // 1/255), front to back, as (capped alpha, colour) and rank in the view's order.
@@ -543,12 +532,11 @@ __global__ __launch_bounds__(kBT / 2) void k_blend_full(const BlendRec* __restri
 // rounding) < 1e-4: it has stopped.  (A NaN alpha makes the product NaN, which
 // ends no list; a NaN corrupted alpha makes every channel NaN for good, wherever
 // the walk ends.)  The end is marked by an alpha so large that T (1 - alpha) <
-// 1e-4 for any T, kListEnd at rank 0xffffffff; a list cut at `cap` entries (views
-// whose lists would not fit) is marked by kListCut at the rank from which the
-// tile's list has to be read.
+// 1e-4 for any T, kListEnd at rank 0xffffffff.
 // ---------------------------------------------------------------------------
 constexpr float kListEndT = 0.9e-6f;
-constexpr float kListEnd = 1e30f, kListCut = 2e30f;
+constexpr float kListEnd = 1e30f;
+enum CleanPass { kImage, kLists, kBlocks };
 
 struct CleanPix {
     float T, c0, c1, c2;   // the clean blend (frozen where it stopped)
@@ -556,19 +544,25 @@ struct CleanPix {
     bool stopped, done;    // done: the list ends here
     uint32_t stop, last;   // rank and list position of the entry that stopped it
     uint32_t n;            // entries taken
-    uint32_t off, flushed; // FILL: start of the list, entries written out
+    uint32_t off, flushed; // kLists: start of the list, entries written out
 };
 
 struct ListOut {
     float4* ent;
     uint32_t* rk;
     const uint32_t* off;   // [tiles * pixels of a tile] start of each pixel's list
-    uint32_t cap;          // most entries kept per pixel
     float4* state;
     uint32_t* row_idx;
     const uint32_t* row_off;
     const uint32_t* row_cnt;
+    uint2* sub;            // kBlocks: (primitive, rank) of the blocks' entries
+    const uint32_t* sub_off;
+    float4* row_state;
 };
+
+// First row of the states of a block whose list starts at `off` (tb: the block's number
+// in its view): a block of n entries has n / kRowStride + 1.
+__device__ __forceinline__ size_t block_rows(uint32_t off, uint32_t tb) { return (size_t)(off / (uint32_t)kRowStride) + tb; }
 
 // Entries of a pixel on their way to its list: a lane takes an entry here and
 // there, so writing each by itself would cost two partial stores per entry (0.72
@@ -588,6 +582,7 @@ __device__ __forceinline__ void store_pair(float4* p, const float4& a, const flo
 }
 
 // four entries [p.flushed, p.flushed + 4) of ring column `col` to the list
+static_assert(kWalk == 4, "lists start and end on the pieces written here and read by the dirty walk");
 __device__ __forceinline__ void flush4(CleanPix& p, const ListRing& ring, int col, const ListOut& lo) {
     const int k = (int)(p.flushed & 4u);
     const size_t at = (size_t)p.off + p.flushed;
@@ -598,7 +593,7 @@ __device__ __forceinline__ void flush4(CleanPix& p, const ListRing& ring, int co
     p.flushed += 4u;
 }
 
-template <bool FILL>
+template <CleanPass PASS>
 __device__ __forceinline__ void clean_entry(CleanPix& p, bool live, bool ok, float a, float cr, float cg, float cb,
                                             uint32_t rank, uint32_t li, const ListOut& lo, ListRing* ring, int col) {
     const bool act = live && ok;
@@ -612,24 +607,22 @@ __device__ __forceinline__ void clean_entry(CleanPix& p, bool live, bool ok, flo
     p.c1 = upd ? __fmaf_rn(cg, w, p.c1) : p.c1;
     p.c2 = upd ? __fmaf_rn(cb, w, p.c2) : p.c2;
     p.T = upd ? Tn : p.T;
-    if (!FILL) {
+    if (PASS == kImage) {
         p.stop = (run && !upd) ? rank : p.stop;
         p.last = (run && !upd) ? li : p.last;
     }
     p.stopped = p.stopped || (run && !upd);
     p.Tv = act ? Tn : p.Tv;
-    if (FILL && act && p.n <= lo.cap) {
-        const bool cut = p.n == lo.cap;
-        ring->e[p.n & 7u][col] = cut ? make_float4(kListCut, 0.0f, 0.0f, 0.0f) : make_float4(al, cr, cg, cb);
+    if (PASS == kLists && act) {
+        ring->e[p.n & 7u][col] = make_float4(al, cr, cg, cb);
         ring->r[p.n & 7u][col] = rank;
+        if ((p.n & (kWalk - 1u)) == 0u) lo.state[(p.off + p.n) / kWalk] = before;   // the state in front of this entry
     }
-    if (FILL && act && p.n <= lo.cap && (p.n & (kWalk - 1u)) == 0u)   // the state in front of this entry
-        lo.state[(p.off + p.n) / kWalk] = before;
     p.n += act ? 1u : 0u;
     p.done = p.done || (act && Tn < kListEndT);
 }
 
-template <bool FILL>
+template <CleanPass PASS>
 __global__ __launch_bounds__(kBT / 2) void k_blend_clean(const BlendRec* __restrict__ recs,
                                                         const uint32_t* __restrict__ ids,
                                                         const uint32_t* __restrict__ rank,
@@ -637,38 +630,47 @@ __global__ __launch_bounds__(kBT / 2) void k_blend_clean(const BlendRec* __restr
                                                         int tw, int th, float* __restrict__ img,
                                                         uint32_t* __restrict__ stop, uint32_t* __restrict__ tile_stop,
                                                         uint32_t* __restrict__ tile_last, uint32_t* __restrict__ counts,
+                                                        uint32_t* __restrict__ blk_cnt,
                                                         unsigned int* __restrict__ clean_nonfin, ListOut lo) {
-    extern __shared__ __align__(16) unsigned char ring_mem[];   // FILL: one ListRing per warp
+    extern __shared__ __align__(16) unsigned char ring_mem[];   // kLists: one ListRing per warp
     __shared__ RawStage st[2];
     __shared__ uint32_t rks[2][kStageMax];   // ranks of the staged entries
     const int tile = blockIdx.x, lane = threadIdx.x & 31;
-    ListRing* ring = FILL ? reinterpret_cast<ListRing*>(ring_mem) + (threadIdx.x >> 5) : nullptr;
+    ListRing* ring = PASS == kLists ? reinterpret_cast<ListRing*>(ring_mem) + (threadIdx.x >> 5) : nullptr;
     const uint32_t P = (uint32_t)(tw * th);
-    const Pix2Geo g = pix2_geo(tile % tiles_x, tile / tiles_x, tw, th, W, H);
+    const Pix2Geo g = pix2_geo(tile % tiles_x, tile / tiles_x, tw, th, W, H, threadIdx.x >> 5);
     CleanPix pA{1.0f, 0.0f, 0.0f, 0.0f, 1.0f, !g.inA, !g.inA, 0xffffffffu, 0xffffffffu, 0u, 0u, 0u};
     CleanPix pB{1.0f, 0.0f, 0.0f, 0.0f, 1.0f, !g.inB, !g.inB, 0xffffffffu, 0xffffffffu, 0u, 0u, 0u};
     const uint2 rg = ranges[tile];
-    const uint32_t row0 = FILL ? lo.row_off[tile] : 0u, rows = FILL ? lo.row_cnt[tile] : 0u;
-    if (FILL) {
+    const uint32_t row0 = PASS == kLists ? lo.row_off[tile] : 0u, rows = PASS == kLists ? lo.row_cnt[tile] : 0u;
+    const uint32_t tb = (uint32_t)tile * (blockDim.x >> 5) + (threadIdx.x >> 5);   // this warp's block
+    const uint32_t sub0 = PASS == kBlocks ? lo.sub_off[tb] : 0u;
+    uint32_t nsub = 0;   // entries that the cull has left
+    if (PASS == kLists) {
         pA.off = lo.off[(size_t)tile * P + g.u0];
         pB.off = lo.off[(size_t)tile * P + g.u1];
     }
-    auto put_row = [&](uint32_t j) {   // after the first j kRowStride entries of the tile's list
-        const size_t r = (size_t)(row0 + j) * P;
-        lo.row_idx[r + g.u0] = pA.off + min(pA.n, lo.cap);
-        lo.row_idx[r + g.u1] = pB.off + min(pB.n, lo.cap);
+    auto put_row = [&](uint32_t j) {
+        if (PASS == kLists) {   // after the first j kRowStride entries of the tile's list
+            const size_t r = (size_t)(row0 + j) * P;
+            lo.row_idx[r + g.u0] = pA.off + pA.n;
+            lo.row_idx[r + g.u1] = pB.off + pB.n;
+        } else {                // ... of the block's list
+            float4* r = lo.row_state + (block_rows(sub0, tb) + j) * 64 + lane;
+            r[0] = make_float4(pA.T, pA.c0, pA.c1, pA.c2);
+            r[32] = make_float4(pB.T, pB.c0, pB.c1, pB.c2);
+        }
     };
-    if (FILL) put_row(0u);
+    if (PASS != kImage) put_row(0u);
     uint32_t at = 0;   // list index of entry 0 of the staged batch
     const uint32_t* rk = rks[0];
     auto apply = [&](int e, bool v, bool okA, bool okB, float2 a, float cr, float cg, float cb) {
-        clean_entry<FILL>(pA, v && !pA.done, okA, a.x, cr, cg, cb, rk[e], at + (uint32_t)e, lo, ring, lane);
-        clean_entry<FILL>(pB, v && !pB.done, okB, a.y, cr, cg, cb, rk[e], at + (uint32_t)e, lo, ring, lane + 32);
+        clean_entry<PASS>(pA, v && !pA.done, okA, a.x, cr, cg, cb, rk[e], at + (uint32_t)e, lo, ring, lane);
+        clean_entry<PASS>(pB, v && !pB.done, okB, a.y, cr, cg, cb, rk[e], at + (uint32_t)e, lo, ring, lane + 32);
     };
-    // entries of the ring not yet written out (a cut list takes one past cap: its mark)
-    auto pending = [&](const CleanPix& p) { return (int)(min(p.n, lo.cap + 1u) - p.flushed); };
+    auto pending = [&](const CleanPix& p) { return (int)(p.n - p.flushed); };   // entries of the ring not yet written out
     auto drain = [&]() {   // after each walk group: make room for the next
-        if (!FILL) return;
+        if (PASS != kLists) return;
         if (!__any_sync(0xffffffffu, max(pending(pA), pending(pB)) > 8 - kAlphaGroup)) return;
         if (pending(pA) >= 4) flush4(pA, *ring, lane, lo);
         if (pending(pB) >= 4) flush4(pB, *ring, lane + 32, lo);
@@ -680,21 +682,37 @@ __global__ __launch_bounds__(kBT / 2) void k_blend_clean(const BlendRec* __restr
             rk = rks[k];
             for (int c = 0; c < cnt && !__all_sync(0xffffffffu, pA.done && pB.done); c += 32) {
                 const uint32_t li = at + (uint32_t)c;
-                if (FILL && li > 0 && li % kRowStride == 0 && li / kRowStride <= rows) put_row(li / kRowStride);
-                blend_chunk2<true>(s, c, cnt, g, apply, drain);
+                if (PASS == kLists && li > 0 && li % kRowStride == 0 && li / kRowStride <= rows) put_row(li / kRowStride);
+                unsigned m = chunk_survivors<true>(s, c, cnt, g);
+                if (PASS != kBlocks) {
+                    nsub += (unsigned)__popc(m);
+                    walk_raw2(m, s, c, g, apply, drain);
+                    continue;
+                }
+                if ((m >> lane) & 1u)
+                    lo.sub[(size_t)sub0 + nsub + (uint32_t)__popc(m & ((1u << lane) - 1u))] =
+                        make_uint2(ids[rg.x + li + (uint32_t)lane], rk[c + lane]);
+                while (m) {   // up to the next row, then the rest
+                    const unsigned room = (unsigned)kRowStride - nsub % (unsigned)kRowStride;
+                    const unsigned part = (unsigned)__popc(m) <= room ? m : m & (0xffffffffu >> (31u - __fns(m, 0, (int)room)));
+                    walk_raw2(part, s, c, g, apply, drain);
+                    nsub += (unsigned)__popc(part);
+                    m &= ~part;
+                    if (nsub % (unsigned)kRowStride == 0u) put_row(nsub / (unsigned)kRowStride);
+                }
             }
         },
         [&] { return pA.done && pB.done; });
-    if (FILL) {
+    if (PASS == kBlocks) return;
+    if (PASS == kImage && lane == 0) blk_cnt[tb] = nsub;
+    if (PASS == kLists) {
         auto finish = [&](CleanPix& p, int col) {
-            if (p.n <= lo.cap) {
-                ring->e[p.n & 7u][col] = make_float4(kListEnd, 0.0f, 0.0f, 0.0f);
-                ring->r[p.n & 7u][col] = 0xffffffffu;
-                if ((p.n & (kWalk - 1u)) == 0u)   // a walk may resume at the mark itself
-                    lo.state[(p.off + p.n) / kWalk] = make_float4(p.T, p.c0, p.c1, p.c2);
-            }
-            // the list's space is a multiple of eight entries: whole pieces, up to the mark
-            while (p.flushed <= min(p.n, lo.cap)) flush4(p, *ring, col, lo);
+            ring->e[p.n & 7u][col] = make_float4(kListEnd, 0.0f, 0.0f, 0.0f);
+            ring->r[p.n & 7u][col] = 0xffffffffu;
+            if ((p.n & (kWalk - 1u)) == 0u)   // a walk may resume at the mark itself
+                lo.state[(p.off + p.n) / kWalk] = make_float4(p.T, p.c0, p.c1, p.c2);
+            // the list's space is a multiple of kWalk entries: whole pieces, up to the mark
+            while (p.flushed <= p.n) flush4(p, *ring, col, lo);
         };
         finish(pA, lane);
         finish(pB, lane + 32);
@@ -778,11 +796,11 @@ __global__ void k_row_keys(const uint2* __restrict__ ranges, const uint32_t* __r
     row_key[i] = (uint32_t)r <= row_cnt[t] ? rank[ids[ranges[t].x + (uint32_t)(r * kRowStride) - 1u]] : 0xffffffffu;
 }
 
-// Space of each pixel's blend list: its entries (at most cap) and the end mark,
-// in whole groups of kWalk.
-__global__ void k_list_lens(const uint32_t* __restrict__ counts, uint64_t n, uint32_t cap, uint32_t* __restrict__ lens) {
+// Space of each pixel's blend list: its entries and the end mark, in whole groups of
+// kWalk.
+__global__ void k_list_lens(const uint32_t* __restrict__ counts, uint64_t n, uint32_t* __restrict__ lens) {
     const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) lens[i] = (min(counts[i], cap) + (uint32_t)kWalk) & ~(uint32_t)(kWalk - 1);
+    if (i < n) lens[i] = (counts[i] + (uint32_t)kWalk) & ~(uint32_t)(kWalk - 1);
 }
 
 // Image pairs (blockIdx.y): a stream over both images, four pixels (three 16-byte
@@ -1253,17 +1271,21 @@ struct __align__(16) DirtyVar {   // one candidate
     unsigned long long mask[kDirtyBlocks];    // active pixels of each 8x8 block
 };
 
-template <bool COUNT>
-__global__ __launch_bounds__(kDirtyThreads, 5) void k_dirty(const ViewPtrs* __restrict__ views,
-                                                           const DirtyDesc* __restrict__ desc,
-                                                           const uint2* __restrict__ cand, int tw, int th,
-                                                           unsigned int* __restrict__ counts,
-                                                           uint32_t* __restrict__ bins, uint32_t nbins,
-                                                           CmpAcc* __restrict__ acc, bool regions,
-                                                           unsigned long long* work, SsimBufs sb) {
+// DENSE: the candidates of dense views, which keep block lists: step (2) takes a
+// candidate's 8x8 block per warp, two pixels per lane, and evaluates the block's list
+// from the last row in front of the change, as the full-frame blend does, records
+// streamed through two stages per warp.  Where nearly every entry of a block is taken
+// at every pixel, 64 pixels then share a record of 48 B instead of reading 20 B of list
+// each.  mixed: the views are of both kinds, each kernel skips the other's candidates.
+template <bool COUNT, bool DENSE>
+__global__ __launch_bounds__(kDirtyThreads, DENSE ? 4 : 5) void k_dirty(
+    const ViewPtrs* __restrict__ views, const DirtyDesc* __restrict__ desc, const uint2* __restrict__ cand, int tw,
+    int th, unsigned int* __restrict__ counts, uint32_t* __restrict__ bins, uint32_t nbins, CmpAcc* __restrict__ acc,
+    bool regions, bool mixed, unsigned long long* work, SsimBufs sb) {
     __shared__ DirtyVar var[kUnitVars];
     __shared__ float alpha[kUnitVars][kTilePix];   // the corrupted entry's capped alpha at each pixel, -1: not taken
-    __shared__ uint16_t pairs[kUnitVars * kTilePix];   // candidate << 8 | 8x8 block << 6 | pixel of the block
+    __shared__ uint16_t pairs[DENSE ? 1 : kUnitVars * kTilePix];   // candidate << 8 | 8x8 block << 6 | pixel of the block
+    __shared__ RawStageN<DENSE ? 32 : 1> stage[DENSE ? kDirtyWarps : 1][2];
     __shared__ uint32_t wsum[kDirtyWarps];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int lg = tile_lgx(tw), nb = (tw * th) >> 6;
@@ -1289,7 +1311,7 @@ __global__ __launch_bounds__(kDirtyThreads, 5) void k_dirty(const ViewPtrs* __re
     for (uint32_t unit = blockIdx.x, drawn = 0u;; unit = next_unit) {
         const uint32_t c0 = unit * per;
         if (c0 >= ncand) break;   // the same for the whole block
-        if (tid == 0) drawn = gridDim.x + atomicAdd(&counts[0], 1u);
+        if (tid == 0) drawn = gridDim.x + atomicAdd(&counts[DENSE ? 8 : 0], 1u);
         const long long t0 = COUNT ? clock64() : 0;
         const int nv = (int)min(per, ncand - c0);
         __syncthreads();   // the previous candidates are done with the shared arrays
@@ -1310,7 +1332,7 @@ __global__ __launch_bounds__(kDirtyThreads, 5) void k_dirty(const ViewPtrs* __re
             const uint32_t ins = has_new ? d.new_rank : kNoRank, pp = has_old ? d.old_rank : kNoRank;
             const uint32_t cut = min(ins, pp);
             unsigned mA = 0u, mB = 0u;
-            if ((c.x >> (20 + b)) & 1u) {
+            if (((c.x >> (20 + b)) & 1u) && (!mixed || (v.sub != nullptr) == DENSE)) {
                 const int wA = block_upper(b, lg), wB = wA + (1 << lg);
                 // this lane's two pixels of the block: (lane % 8, lane / 8) and four rows below
                 const uint32_t* stop = v.stop + (size_t)tile * P + lane;
@@ -1352,11 +1374,13 @@ __global__ __launch_bounds__(kDirtyThreads, 5) void k_dirty(const ViewPtrs* __re
             }
             if (lane == 0) var[vi].mask[b] = (unsigned long long)mA | ((unsigned long long)mB << 32);
             if (b == 0) {
-                // the rows in front of the first change (the keys ascend)
-                const uint32_t* key = v.row_key + (size_t)tile * kRowsPerTile + lane;
-                const uint32_t key0 = key[0], key1 = key[32];
-                const uint32_t row = v.row_off[tile] + (uint32_t)(__popc(__ballot_sync(0xffffffffu, key0 < cut)) +
-                                                                  __popc(__ballot_sync(0xffffffffu, key1 < cut)));
+                uint32_t row = 0u;
+                if (!DENSE && (!mixed || v.sub == nullptr)) {   // the rows in front of the first change (the keys ascend)
+                    const uint32_t* key = v.row_key + (size_t)tile * kRowsPerTile + lane;
+                    const uint32_t key0 = key[0], key1 = key[32];
+                    row = v.row_off[tile] + (uint32_t)(__popc(__ballot_sync(0xffffffffu, key0 < cut)) +
+                                                       __popc(__ballot_sync(0xffffffffu, key1 < cut)));
+                }
                 if (lane == 0) {
                     DirtyVar& q = var[vi];
                     q.row_idx = v.row_idx + (size_t)row * P;
@@ -1403,184 +1427,276 @@ __global__ __launch_bounds__(kDirtyThreads, 5) void k_dirty(const ViewPtrs* __re
                 }
             }
         }
-        // the pairs by pixel: thread t lists the candidates of pixel t
-        uint32_t m = 0u;
-        if (tid < nb * 64)
-            for (int vi = 0; vi < nv; vi++) m |= ((unsigned)(var[vi].mask[tid >> 6] >> (tid & 63)) & 1u) << vi;
-        const uint32_t cnt = (uint32_t)__popc(m);
-        uint32_t incl = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        if (lane == 31) wsum[warp] = incl;
-        __syncthreads();
-        uint32_t at = incl - cnt, npairs = 0;
-#pragma unroll
-        for (int w = 0; w < kDirtyWarps; w++) {
-            at += w < warp ? wsum[w] : 0u;
-            npairs += wsum[w];
-        }
-        for (; m; m &= m - 1u) pairs[at++] = (uint16_t)((__ffs(m) - 1) << 8 | tid);
-        __syncthreads();
-        if (COUNT) t_pro += clock64() - t0;
         unsigned int nev = 0, nst = 0;
-        for (uint32_t r0 = (uint32_t)warp * 32u; r0 < npairs; r0 += kDirtyThreads) {
-            const long long t1 = COUNT ? clock64() : 0;
-            const bool act = r0 + (uint32_t)lane < npairs;
-            const int code = pairs[act ? r0 + (uint32_t)lane : r0];
-            const int vi = code >> 8, u8 = code & 255, b = u8 >> 6, u6 = u8 & 63;
-            DirtyVar& q = var[vi];
-            const int lx = block_x0(b, lg) + (u6 & 7), ly = block_y0(b, lg) + (u6 >> 3);   // in the tile
-            const int u = (block_upper(b, lg) + ((u6 >> 5) << lg)) * 32 + (u6 & 31);
-            DirtyPix p{1.0f, 0.0f, 0.0f, 0.0f};
-            float k0 = 0.0f, k1 = 0.0f, k2 = 0.0f;   // the clean pixel
-            if (act) {
-                const float4* ent = q.ent;
-                uint32_t i = q.row_idx[u] & ~(uint32_t)(kWalk - 1);
-                const float* kp = q.clean + (ly * q.W3 + lx * 3);
-                k0 = kp[0];
-                k1 = kp[1];
-                k2 = kp[2];
-                const float4 st = q.state[i / kWalk];
-                p.T = st.x;
-                p.c0 = st.y;
-                p.c1 = st.z;
-                p.c2 = st.w;
-                const uint32_t ins = q.ins, pp = q.pp;
-                const float na = alpha[vi][u8];   // the corrupted entry at this pixel, when its blend takes it
-                bool pend = !(na < 0.0f);         // still to be inserted (a NaN alpha too)
-                bool old = pp != kNoRank;         // the removed entry may still lie ahead
-                float4 e[kWalk];
-                float last = 0.0f;                // the alpha that ended the walk
-                bool end = false;
-                do {
-#pragma unroll
-                    for (int k = 0; k < kWalk; k += 2) load_pair(ent + i + k, e[k], e[k + 1]);
+        if (DENSE) {
+            __syncthreads();   // the delta units, where there are any
+            if (COUNT) t_pro += clock64() - t0;
+            for (int task = warp; task < nv * nb; task += kDirtyWarps) {
+                const int vi = task / nb, b = task % nb;
+                DirtyVar& q = var[vi];
+                const unsigned long long mask = q.mask[b];
+                if (!mask) continue;
+                const long long t1 = COUNT ? clock64() : 0;
+                const ViewPtrs& v = views[q.cx >> 24];
+                const Pix2Geo g = pix2_geo((int)(q.cy & 0xffffu), (int)(q.cy >> 16), tw, th, v.W, v.H, b);
+                const bool actA = (mask >> lane) & 1ull, actB = (mask >> (32 + lane)) & 1ull;
+                const uint32_t ins = q.ins, pp = q.pp, cut = min(ins, pp);
+                // the block's list, and how many of its entries lie in front of the first change
+                const uint32_t tb = q.tile * (uint32_t)nb + (uint32_t)b, n = v.sub_cnt[tb], off = v.sub_off[tb];
+                const uint2* __restrict__ sub = v.sub + off;
+                uint32_t lo = 0, hi = n;
+                while (lo < hi) {
+                    const uint32_t step = (hi - lo + 31u) / 32u, i = lo + (uint32_t)lane * step;
+                    const int k = __popc(__ballot_sync(0xffffffffu, i < hi && sub[i].y < cut));   // they come first
+                    hi = k == 0 ? lo : min(hi, lo + (uint32_t)k * step);
+                    lo = k == 0 ? lo : lo + (uint32_t)(k - 1) * step + 1u;
+                }
+                const uint32_t row = lo / (uint32_t)kRowStride;   // resume from this row
+                const float4* rs = v.row_state + (block_rows(off, tb) + row) * 64 + lane;
+                const float4 sA = rs[0], sB = rs[32];
+                Pix pA{sA.x, sA.y, sA.z, sA.w, !actA}, pB{sB.x, sB.y, sB.z, sB.w, !actB};
+                const float naA = alpha[vi][b * 64 + lane], naB = alpha[vi][b * 64 + 32 + lane];
+                bool pend = ins != kNoRank;   // the corrupted entry is still to be inserted
+                auto insert = [&] {
+                    pend = false;
+                    apply_entry(pA, !pA.done, !(naA < 0.0f), naA, q.r, q.g, q.b);
+                    apply_entry(pB, !pB.done, !(naB < 0.0f), naB, q.r, q.g, q.b);
+                };
+                auto apply = [&](int, bool has, bool okA, bool okB, float2 a, float cr, float cg, float cb) {
+                    const bool liveA = has && !pA.done, liveB = has && !pB.done;
+                    if (COUNT) nev += (liveA && okA ? 1u : 0u) + (liveB && okB ? 1u : 0u);
+                    apply_entry(pA, liveA, okA, a.x, cr, cg, cb);
+                    apply_entry(pB, liveB, okB, a.y, cr, cg, cb);
+                };
+                auto fetch = [&](int k, uint32_t id) {
+                    const float4* src = reinterpret_cast<const float4*>(v.recs + id);
+                    cp_async16(&stage[warp][k].q0[lane], src);
+                    cp_async16(&stage[warp][k].q1[lane], src + 1);
+                    cp_async16(&stage[warp][k].q2[lane], src + 2);
+                };
+                const uint2 none = make_uint2(0u, 0xffffffffu);   // behind the list's end: of the last rank
+                uint32_t i = row * (uint32_t)kRowStride + (uint32_t)lane;   // this lane's entries: i, i + 32, ...
+                uint2 cur = i < n ? sub[i] : none;
+                if (i < n) fetch(0, cur.x);
+                uint2 next = i + 32u < n ? sub[i + 32u] : none;
+                for (uint32_t base = row * (uint32_t)kRowStride, k = 0; base < n; base += 32u, k ^= 1u) {
+                    cp_async_wait_all();
+                    __syncwarp();   // the entries are there for every lane, and every lane is done with the other stage
+                    const uint32_t rank = cur.y;
+                    if (i + 32u < n) fetch((int)k ^ 1, next.x);
+                    cur = next;
+                    next = i + 64u < n ? sub[i + 64u] : none;
+                    i += 32u;
                     if (COUNT) nst++;
-                    if (pend || old) {   // ranks matter until both changes are behind
-                        // the first entry of this group behind the corrupted one (the end's rank is
-                        // above every other) and the removed entry
-                        int at_new = 0, at_old = kWalk;
-                        uint32_t q_last = 0u;
-#pragma unroll
-                        for (int k = 0; k < kWalk; k += 4) {
-                            const uint4 x = __ldg(reinterpret_cast<const uint4*>(q.rk + i + k));
-                            const int first = x.x >= ins ? 0 : (x.y >= ins ? 1 : (x.z >= ins ? 2 : (x.w >= ins ? 3 : 4)));
-                            at_new = at_new == k ? k + first : at_new;
-                            at_old = x.x == pp ? k : (x.y == pp ? k + 1 : (x.z == pp ? k + 2 : (x.w == pp ? k + 3 : at_old)));
-                            q_last = x.w;
+                    const uint32_t left = n - base;
+                    unsigned m = (left >= 32u ? 0xffffffffu : (1u << left) - 1u) & ~__ballot_sync(0xffffffffu, rank == pp);
+                    if (pend) {
+                        const unsigned behind = __ballot_sync(0xffffffffu, rank >= ins);   // (past the list's end too)
+                        if (behind) {
+                            walk_raw2(m & ~behind, stage[warp][k], 0, g, apply, [] {});
+                            insert();
+                            m &= behind;
                         }
-                        at_new = pend ? at_new : kWalk;
+                    }
+                    walk_raw2(m, stage[warp][k], 0, g, apply, [] {});
+                    if (__all_sync(0xffffffffu, pA.done && pB.done)) break;
+                }
+                cp_async_wait_all();   // leave no copy in flight
+                __syncwarp();
+                if (pend) insert();   // (pixels that have stopped take no more)
+                const long long t2 = COUNT ? clock64() : 0;
+                DirtySum s{};
+                uint32_t maxb = 0u;
+                auto finish = [&](const Pix& p, bool act, int py, int half) {
+                    if (!act) return;
+                    const int lx = g.px - (int)(q.cy & 0xffffu) * tw, ly = py - (int)(q.cy >> 16) * th;   // in the tile
+                    const float* kp = q.clean + (ly * q.W3 + lx * 3);
+                    const float k0 = kp[0], k1 = kp[1], k2 = kp[2];
+                    const float a0 = __fadd_rn(p.c0, p.T), a1 = __fadd_rn(p.c1, p.T), a2 = __fadd_rn(p.c2, p.T);
+                    const DirtySum d = dirty_sum(a0, a1, a2, k0, k1, k2);
+                    s.fx_lo += d.fx_lo;
+                    s.fx_hi += d.fx_hi;
+                    s.counts += d.counts;
+                    maxb = max(maxb, d.maxbits);
+                    if (regions && d.foot) {
+                        const unsigned long long cell = cell_bit(g.px, py, v.W, v.H);
+                        if ((unsigned)cell) atomicOr(&q.cells_lo, (unsigned)cell);
+                        if ((unsigned)(cell >> 32)) atomicOr(&q.cells_hi, (unsigned)(cell >> 32));
+                    }
+                    if (sb.plan && q.unit[b] != 0xffffffffu) {
+                        sb.deltas[(size_t)(2u * q.unit[b] + (uint32_t)half) * 32 + lane] = make_float4(a0, a1, a2, 0.0f);
+                        const bool ch = __float_as_uint(a0) != __float_as_uint(k0) ||
+                                        __float_as_uint(a1) != __float_as_uint(k1) || __float_as_uint(a2) != __float_as_uint(k2);
+                        if (ch)
+                            atomicOr(&q.edge, 16u | (lx < 5 ? 1u : 0u) | (lx > tw - 6 ? 2u : 0u) | (ly < 5 ? 4u : 0u) |
+                                                  (ly > th - 6 ? 8u : 0u));
+                    }
+                };
+                finish(pA, actA, g.pyA, 0);
+                finish(pB, actB, g.pyB, 1);
+                s.fx_lo = __reduce_add_sync(0xffffffffu, s.fx_lo);   // 64 pixels: below 2^26 and 2^27, counts below 2^7 a field
+                s.fx_hi = __reduce_add_sync(0xffffffffu, s.fx_hi);
+                s.counts = __reduce_add_sync(0xffffffffu, s.counts);
+                maxb = __reduce_max_sync(0xffffffffu, maxb);
+                if (lane == 0) {
+                    if (s.fx_lo) atomicAdd(&q.fx_lo, s.fx_lo);
+                    if (s.fx_hi) atomicAdd(&q.fx_hi, s.fx_hi);
+                    if (s.counts) atomicAdd(&q.counts, s.counts);
+                    if (maxb) atomicMax(&q.maxbits, maxb);
+                }
+                if (COUNT) {
+                    t_walk += t2 - t1;
+                    t_epi += clock64() - t2;
+                    if (lane == 0) {
+                        const unsigned npix = (unsigned)__popcll(mask);
+                        atomicAdd(&work[8], (unsigned long long)nst * 32ull);
+                        atomicAdd(&work[9], (unsigned long long)nst * 32ull);
+                        atomicAdd(&work[14], (unsigned long long)npix);
+                        atomicAdd(&work[15], (unsigned long long)nst * 32ull * npix);
+                    }
+                    nst = 0;
+                }
+            }
+        }
+        if (!DENSE) {
+            // the pairs by pixel: thread t lists the candidates of pixel t
+            uint32_t m = 0u;
+            if (tid < nb * 64)
+                for (int vi = 0; vi < nv; vi++) m |= ((unsigned)(var[vi].mask[tid >> 6] >> (tid & 63)) & 1u) << vi;
+            const uint32_t cnt = (uint32_t)__popc(m);
+            uint32_t incl = cnt;
 #pragma unroll
-                        for (int k = 0; k < kWalk; k++) {
-                            // a cut list's rest, and an entry that belongs there, come from the tile's list
-                            if (k == at_new && !end && e[k].x != kListCut) {
-                                pend = false;
-                                if (COUNT) nev++;
-                                last = na;
-                                end = p.take(na, q.r, q.g, q.b);
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            if (lane == 31) wsum[warp] = incl;
+            __syncthreads();
+            uint32_t at = incl - cnt, npairs = 0;
+#pragma unroll
+            for (int w = 0; w < kDirtyWarps; w++) {
+                at += w < warp ? wsum[w] : 0u;
+                npairs += wsum[w];
+            }
+            for (; m; m &= m - 1u) pairs[at++] = (uint16_t)((__ffs(m) - 1) << 8 | tid);
+            __syncthreads();
+            if (COUNT) t_pro += clock64() - t0;
+            for (uint32_t r0 = (uint32_t)warp * 32u; r0 < npairs; r0 += kDirtyThreads) {
+                const long long t1 = COUNT ? clock64() : 0;
+                const bool act = r0 + (uint32_t)lane < npairs;
+                const int code = pairs[act ? r0 + (uint32_t)lane : r0];
+                const int vi = code >> 8, u8 = code & 255, b = u8 >> 6, u6 = u8 & 63;
+                DirtyVar& q = var[vi];
+                const int lx = block_x0(b, lg) + (u6 & 7), ly = block_y0(b, lg) + (u6 >> 3);   // in the tile
+                const int u = (block_upper(b, lg) + ((u6 >> 5) << lg)) * 32 + (u6 & 31);
+                DirtyPix p{1.0f, 0.0f, 0.0f, 0.0f};
+                float k0 = 0.0f, k1 = 0.0f, k2 = 0.0f;   // the clean pixel
+                if (act) {
+                    const float4* ent = q.ent;
+                    uint32_t i = q.row_idx[u] & ~(uint32_t)(kWalk - 1);
+                    const float* kp = q.clean + (ly * q.W3 + lx * 3);
+                    k0 = kp[0];
+                    k1 = kp[1];
+                    k2 = kp[2];
+                    const float4 st = q.state[i / kWalk];
+                    p.T = st.x;
+                    p.c0 = st.y;
+                    p.c1 = st.z;
+                    p.c2 = st.w;
+                    const uint32_t ins = q.ins, pp = q.pp;
+                    const float na = alpha[vi][u8];   // the corrupted entry at this pixel, when its blend takes it
+                    bool pend = !(na < 0.0f);         // still to be inserted (a NaN alpha too)
+                    bool old = pp != kNoRank;         // the removed entry may still lie ahead
+                    float4 e[kWalk];
+                    float last = 0.0f;                // the alpha that ended the walk
+                    bool end = false;
+                    do {
+#pragma unroll
+                        for (int k = 0; k < kWalk; k += 2) load_pair(ent + i + k, e[k], e[k + 1]);
+                        if (COUNT) nst++;
+                        if (pend || old) {   // ranks matter until both changes are behind
+                            // the first entry of this group behind the corrupted one (the end's rank is
+                            // above every other) and the removed entry
+                            const uint4 x = __ldg(reinterpret_cast<const uint4*>(q.rk + i));
+                            const int first = x.x >= ins ? 0 : (x.y >= ins ? 1 : (x.z >= ins ? 2 : (x.w >= ins ? 3 : 4)));
+                            const int at_new = pend ? first : kWalk;
+                            const int at_old = x.x == pp ? 0 : (x.y == pp ? 1 : (x.z == pp ? 2 : (x.w == pp ? 3 : kWalk)));
+#pragma unroll
+                            for (int k = 0; k < kWalk; k++) {
+                                if (k == at_new && !end) {
+                                    pend = false;
+                                    if (COUNT) nev++;
+                                    last = na;
+                                    end = p.take(na, q.r, q.g, q.b);
+                                }
+                                if (!end && k != at_old) {
+                                    if (COUNT) nev++;
+                                    last = e[k].x;
+                                    end = p.take(e[k].x, e[k].y, e[k].z, e[k].w);
+                                }
                             }
-                            if (!end && (k != at_old || e[k].x == kListCut)) {
+                            old = old && x.w < pp;
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < kWalk; k++) {
+                                if (end) continue;
                                 if (COUNT) nev++;
                                 last = e[k].x;
                                 end = p.take(e[k].x, e[k].y, e[k].z, e[k].w);
                             }
                         }
-                        old = old && q_last < pp;
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < kWalk; k++) {
-                            if (end) continue;
-                            if (COUNT) nev++;
-                            last = e[k].x;
-                            end = p.take(e[k].x, e[k].y, e[k].z, e[k].w);
-                        }
-                    }
-                    i += kWalk;
-                } while (!end);
-                p.poison(last);
-                if (last == kListCut) {
-                    // a list cut short: the rest comes from the tile's list, from the mark's rank on
-                    const ViewPtrs& v = views[q.cx >> 24];
-                    const float x = (float)((int)(q.cy & 0xffffu) * tw + lx) + 0.5f;
-                    const float y = (float)((int)(q.cy >> 16) * th + ly) + 0.5f;
-                    uint32_t from = 0xffffffffu;
-                    for (int k = 0; k < kWalk; k++) {
-                        const uint32_t j = i - kWalk + (uint32_t)k;
-                        if (ent[j].x == kListCut && from == 0xffffffffu) from = q.rk[j];
-                    }
-                    const uint2 rg = v.ranges[q.tile];
-                    const uint32_t L = rg.y - rg.x;
-                    bool stopped = false;
-                    for (uint32_t j = 0; j <= L && !stopped; j++) {   // j == L: the list's end
-                        const uint32_t id = j < L ? v.ids[rg.x + j] : 0u, rank = j < L ? v.rank[id] : 0xffffffffu;
-                        if (rank < from) continue;
-                        if (pend && rank >= ins) {
-                            pend = false;
-                            stopped = p.take(na, q.r, q.g, q.b);
-                            p.poison(na);
-                        }
-                        if (rank == pp || j == L || stopped) continue;
-                        const BlendRec z = load_rec(v.recs, id);
-                        float al;
-                        if (COUNT) nev++;
-                        if (blend_alpha(z.mx, z.my, z.ca, z.cb, z.cc, z.opac, x, y, al)) {
-                            al = al > 0.99f ? 0.99f : al;
-                            stopped = p.take(al, z.r, z.g, z.b);
-                            p.poison(al);
-                        }
-                    }
+                        i += kWalk;
+                    } while (!end);
+                    p.poison(last);
                 }
-            }
-            __syncwarp();
-            const long long t2 = COUNT ? clock64() : 0;
-            // compare with the clean image; every inactive pixel keeps its clean value
-            // (Delta = 0), and the clean image's non-finite pixels are counted once per
-            // view at finalize
-            const float a0 = __fadd_rn(p.c0, p.T), a1 = __fadd_rn(p.c1, p.T), a2 = __fadd_rn(p.c2, p.T);
-            DirtySum s{};
-            if (act) s = dirty_sum(a0, a1, a2, k0, k1, k2);
-            const bool one = nv == 1;   // block-uniform
-            if (one) {
-                s.fx_lo = __reduce_add_sync(0xffffffffu, s.fx_lo);
-                s.fx_hi = __reduce_add_sync(0xffffffffu, s.fx_hi);
-                s.counts = __reduce_add_sync(0xffffffffu, s.counts);
-                s.maxbits = __reduce_max_sync(0xffffffffu, s.maxbits);
-            }
-            if (one ? lane == 0 : act) {
-                if (s.fx_lo) atomicAdd(&q.fx_lo, s.fx_lo);
-                if (s.fx_hi) atomicAdd(&q.fx_hi, s.fx_hi);
-                if (s.counts) atomicAdd(&q.counts, s.counts);
-                if (s.maxbits) atomicMax(&q.maxbits, s.maxbits);
-            }
-            if (regions && act && s.foot) {   // screen cells holding a footprint pixel
-                const ViewPtrs& v = views[q.cx >> 24];
-                const unsigned long long cell = cell_bit((int)(q.cy & 0xffffu) * tw + lx, (int)(q.cy >> 16) * th + ly, v.W, v.H);
-                if ((unsigned)cell) atomicOr(&q.cells_lo, (unsigned)cell);
-                if ((unsigned)(cell >> 32)) atomicOr(&q.cells_hi, (unsigned)(cell >> 32));
-            }
-            if (sb.plan && act && q.unit[b] != 0xffffffffu) {   // dirty-tile SSIM: the new values
-                sb.deltas[(size_t)(2u * q.unit[b] + (uint32_t)(u6 >> 5)) * 32 + (u6 & 31)] = make_float4(a0, a1, a2, 0.0f);
-                // where the changed pixels are: which neighbouring tiles their SSIM windows reach
-                const bool ch = __float_as_uint(a0) != __float_as_uint(k0) || __float_as_uint(a1) != __float_as_uint(k1) ||
-                                __float_as_uint(a2) != __float_as_uint(k2);
-                if (ch)
-                    atomicOr(&q.edge, 16u | (lx < 5 ? 1u : 0u) | (lx > tw - 6 ? 2u : 0u) | (ly < 5 ? 4u : 0u) |
-                                          (ly > th - 6 ? 8u : 0u));
-            }
-            if (COUNT) {
-                const unsigned steps = __reduce_max_sync(0xffffffffu, nst);
-                nst = 0;
-                t_walk += t2 - t1;
-                t_epi += clock64() - t2;
-                if (lane == 0) {
-                    const unsigned npix = min(32u, npairs - r0);
-                    atomicAdd(&work[8], (unsigned long long)(steps * kWalk));
-                    atomicAdd(&work[9], (unsigned long long)(steps * kWalk));
-                    atomicAdd(&work[14], (unsigned long long)npix);
-                    atomicAdd(&work[15], (unsigned long long)steps * kWalk * npix);
+                __syncwarp();
+                const long long t2 = COUNT ? clock64() : 0;
+                // compare with the clean image; every inactive pixel keeps its clean value
+                // (Delta = 0), and the clean image's non-finite pixels are counted once per
+                // view at finalize
+                const float a0 = __fadd_rn(p.c0, p.T), a1 = __fadd_rn(p.c1, p.T), a2 = __fadd_rn(p.c2, p.T);
+                DirtySum s{};
+                if (act) s = dirty_sum(a0, a1, a2, k0, k1, k2);
+                const bool one = nv == 1;   // block-uniform
+                if (one) {
+                    s.fx_lo = __reduce_add_sync(0xffffffffu, s.fx_lo);
+                    s.fx_hi = __reduce_add_sync(0xffffffffu, s.fx_hi);
+                    s.counts = __reduce_add_sync(0xffffffffu, s.counts);
+                    s.maxbits = __reduce_max_sync(0xffffffffu, s.maxbits);
+                }
+                if (one ? lane == 0 : act) {
+                    if (s.fx_lo) atomicAdd(&q.fx_lo, s.fx_lo);
+                    if (s.fx_hi) atomicAdd(&q.fx_hi, s.fx_hi);
+                    if (s.counts) atomicAdd(&q.counts, s.counts);
+                    if (s.maxbits) atomicMax(&q.maxbits, s.maxbits);
+                }
+                if (regions && act && s.foot) {   // screen cells holding a footprint pixel
+                    const ViewPtrs& v = views[q.cx >> 24];
+                    const unsigned long long cell = cell_bit((int)(q.cy & 0xffffu) * tw + lx, (int)(q.cy >> 16) * th + ly, v.W, v.H);
+                    if ((unsigned)cell) atomicOr(&q.cells_lo, (unsigned)cell);
+                    if ((unsigned)(cell >> 32)) atomicOr(&q.cells_hi, (unsigned)(cell >> 32));
+                }
+                if (sb.plan && act && q.unit[b] != 0xffffffffu) {   // dirty-tile SSIM: the new values
+                    sb.deltas[(size_t)(2u * q.unit[b] + (uint32_t)(u6 >> 5)) * 32 + (u6 & 31)] = make_float4(a0, a1, a2, 0.0f);
+                    // where the changed pixels are: which neighbouring tiles their SSIM windows reach
+                    const bool ch = __float_as_uint(a0) != __float_as_uint(k0) || __float_as_uint(a1) != __float_as_uint(k1) ||
+                                    __float_as_uint(a2) != __float_as_uint(k2);
+                    if (ch)
+                        atomicOr(&q.edge, 16u | (lx < 5 ? 1u : 0u) | (lx > tw - 6 ? 2u : 0u) | (ly < 5 ? 4u : 0u) |
+                                              (ly > th - 6 ? 8u : 0u));
+                }
+                if (COUNT) {
+                    const unsigned steps = __reduce_max_sync(0xffffffffu, nst);
+                    nst = 0;
+                    t_walk += t2 - t1;
+                    t_epi += clock64() - t2;
+                    if (lane == 0) {
+                        const unsigned npix = min(32u, npairs - r0);
+                        atomicAdd(&work[8], (unsigned long long)(steps * kWalk));
+                        atomicAdd(&work[9], (unsigned long long)(steps * kWalk));
+                        atomicAdd(&work[14], (unsigned long long)npix);
+                        atomicAdd(&work[15], (unsigned long long)steps * kWalk * npix);
+                    }
                 }
             }
         }
@@ -1669,32 +1785,37 @@ gs_status launch_blend_compare(const BlendRec* recs, const uint32_t* ids, const 
 }
 
 // First pass over a clean view: image, stops, list lengths.
-gs_status launch_blend_clean(const ViewState& v, uint32_t* counts, unsigned int* clean_nonfin, cudaStream_t st) {
+gs_status launch_blend_clean(const ViewState& v, uint32_t* counts, uint32_t* blk_cnt, unsigned int* clean_nonfin,
+                             cudaStream_t st) {
     const DevCamera& cam = v.cam;
     const int tx = cam.tiles_x, ty = cam.tiles_y, P = cam.tile_w * cam.tile_h / 2;
     if (tx * ty == 0) return GS_OK;
-    k_blend_clean<false><<<tx * ty, P, 0, st>>>(v.recs, v.ids, v.rank, v.ranges, cam.W, cam.H, tx, cam.tile_w,
-                                                cam.tile_h, v.clean, v.stop, v.tile_stop, v.tile_last, counts,
-                                                clean_nonfin, ListOut{});
+    k_blend_clean<kImage><<<tx * ty, P, 0, st>>>(v.recs, v.ids, v.rank, v.ranges, cam.W, cam.H, tx, cam.tile_w,
+                                                 cam.tile_h, v.clean, v.stop, v.tile_stop, v.tile_last, counts,
+                                                 blk_cnt, clean_nonfin, ListOut{});
     GS_CUDA(cudaGetLastError());
     return GS_OK;
 }
 
-// Second pass: blend lists (off: their starts, at most cap entries each) and checkpoint rows.
-gs_status launch_fill_lists(const ViewState& v, const uint32_t* off, uint32_t cap, cudaStream_t st) {
+// Second pass: blend lists (off: their starts), or, of a dense view, block lists.
+gs_status launch_fill_lists(const ViewState& v, const uint32_t* off, cudaStream_t st) {
     const DevCamera& cam = v.cam;
     const int tx = cam.tiles_x, ty = cam.tiles_y, P = cam.tile_w * cam.tile_h / 2;
     if (tx * ty == 0) return GS_OK;
-    const int smem = (int)sizeof(ListRing) * (P / 32);
+    const bool dense = v.sub != nullptr;
+    const int smem = dense ? 0 : (int)sizeof(ListRing) * (P / 32);
     // the largest tile's, not this one's: the attribute is the process's, and another
     // thread may fill lists of another tile shape between these lines
     constexpr int most = (int)sizeof(ListRing) * (kBT / 2 / 32);
-    GS_CUDA(cudaFuncSetAttribute(k_blend_clean<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-    k_blend_clean<true><<<tx * ty, P, smem, st>>>(v.recs, v.ids, v.rank, v.ranges, cam.W, cam.H, tx, cam.tile_w,
-                                                  cam.tile_h, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
-                                                  ListOut{v.ent, v.rk, off, cap, v.state, v.row_idx, v.row_off, v.row_cnt});
-    k_row_keys<<<(tx * ty * kRowsPerTile + 255) / 256, 256, 0, st>>>(v.ranges, v.ids, v.rank, v.row_cnt, tx * ty,
-                                                                       v.row_key);
+    GS_CUDA(cudaFuncSetAttribute(k_blend_clean<kLists>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    auto fill = dense ? k_blend_clean<kBlocks> : k_blend_clean<kLists>;
+    fill<<<tx * ty, P, smem, st>>>(v.recs, v.ids, v.rank, v.ranges, cam.W, cam.H, tx, cam.tile_w, cam.tile_h, nullptr,
+                                   nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
+                                   ListOut{v.ent, v.rk, off, v.state, v.row_idx, v.row_off, v.row_cnt, v.sub, v.sub_off,
+                                           v.row_state});
+    if (!dense)
+        k_row_keys<<<(tx * ty * kRowsPerTile + 255) / 256, 256, 0, st>>>(v.ranges, v.ids, v.rank, v.row_cnt, tx * ty,
+                                                                           v.row_key);
     GS_CUDA(cudaGetLastError());
     return GS_OK;
 }
@@ -1712,8 +1833,8 @@ gs_status launch_row_counts(const ViewState& v, uint32_t* rows, cudaStream_t st)
     return GS_OK;
 }
 
-gs_status launch_list_lens(const uint32_t* counts, uint64_t n, uint32_t cap, uint32_t* lens, cudaStream_t st) {
-    if (n > 0) k_list_lens<<<(unsigned)div_up(n, 256), 256, 0, st>>>(counts, n, cap, lens);
+gs_status launch_list_lens(const uint32_t* counts, uint64_t n, uint32_t* lens, cudaStream_t st) {
+    if (n > 0) k_list_lens<<<(unsigned)div_up(n, 256), 256, 0, st>>>(counts, n, lens);
     GS_CUDA(cudaGetLastError());
     return GS_OK;
 }
@@ -1764,15 +1885,19 @@ gs_status launch_finalize_dirty(const CmpAcc* acc, int count, gs_result* out, co
     return GS_OK;
 }
 
-int dirty_grid() {
-    static int blocks = 0;
-    if (!blocks) {
+template <bool DENSE>
+static int resident_blocks() {
+    static const int blocks = [] {
         int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dirty<false>, kDirtyThreads, 0);
-        if (per_sm < 1) per_sm = 1;
-        blocks = per_sm * num_sms();
-    }
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dirty<false, DENSE>, kDirtyThreads, 0);
+        return std::max(per_sm, 1) * num_sms();
+    }();
     return blocks;
+}
+// the occupancy queries, outside any stream capture
+void dirty_grids() {
+    resident_blocks<false>();
+    resident_blocks<true>();
 }
 
 gs_status launch_dirty_ssim(const void* dev_views, int K, unsigned int* queue, const SsimBufs& sb, CmpAcc* acc,
@@ -1785,9 +1910,10 @@ gs_status launch_dirty_ssim(const void* dev_views, int K, unsigned int* queue, c
 constexpr int kSortPairs = 512;
 
 // One batch after the injector.  ev_mid (optional): recorded between the plan and
-// the blend kernel.  s->queue, cleared by the finaliser but for [6]: [0] units drawn,
-// [1] tile rows, [2] candidates and [3] their blocks to look at, [4] bin places, [5] SSIM
-// delta units, [6] batch generation, [7] tiles the SSIM visits, [9] SSIM plan slots.
+// the blend kernel.  s->queue, cleared by the finaliser but for [6]: [0] units drawn (of
+// dense views: [8]), [1] tile rows, [2] candidates and [3] their blocks to look at, [4]
+// bin places, [5] SSIM delta units, [6] batch generation, [7] tiles the SSIM visits, [9]
+// SSIM plan slots.
 gs_status launch_dirty_blend(gs_scene* s, int BK, bool regions, const SsimBufs& sb, cudaStream_t st) {
     const ViewPtrs* views = (const ViewPtrs*)s->dev_views;
     const int plan_blocks = num_sms() * 8;
@@ -1804,10 +1930,14 @@ gs_status launch_dirty_blend(gs_scene* s, int BK, bool regions, const SsimBufs& 
         cudaError_t e = cudaEventRecordWithFlags(s->ev_kp, st, cudaEventRecordExternal);
         if (e != cudaSuccess) return set_error(GS_ERR_CUDA, cudaGetErrorString(e));
     }
-    auto dirty = work ? k_dirty<true> : k_dirty<false>;
-    dirty<<<dirty_grid(), kDirtyThreads, 0, st>>>(views, s->desc, bin ? s->cand_sorted : s->cand,
-                                                  s->tile_w, s->tile_h, s->queue, s->bins, bin ? nbins : 0u, s->acc,
-                                                  regions, work, sb);
+    const int dense_views = (int)std::count_if(s->views.begin(), s->views.end(), [](const ViewState& v) { return v.sub != nullptr; });
+    const bool mixed = dense_views > 0 && dense_views < s->K;
+    auto dirty = [&](auto kernel, int blocks) {
+        kernel<<<blocks, kDirtyThreads, 0, st>>>(views, s->desc, bin ? s->cand_sorted : s->cand, s->tile_w, s->tile_h,
+                                                 s->queue, s->bins, bin ? nbins : 0u, s->acc, regions, mixed, work, sb);
+    };
+    if (dense_views < s->K) dirty(work ? k_dirty<true, false> : k_dirty<false, false>, resident_blocks<false>());
+    if (dense_views > 0) dirty(work ? k_dirty<true, true> : k_dirty<false, true>, resident_blocks<true>());
     if (sb.plan) GS_TRY(launch_dirty_ssim(s->dev_views, s->K, s->queue, sb, s->acc, st));
     GS_CUDA(cudaGetLastError());
     return GS_OK;
@@ -1833,6 +1963,10 @@ void fill_view_ptrs(void* host_dst, const ViewState& vs, uint32_t bin0) {
     v.ent = vs.ent;
     v.rk = vs.rk;
     v.state = vs.state;
+    v.sub = vs.sub;
+    v.sub_off = vs.sub_off;
+    v.sub_cnt = vs.sub_cnt;
+    v.row_state = vs.row_state;
     v.W = vs.cam.W;
     v.H = vs.cam.H;
     v.tiles_x = vs.cam.tiles_x;

@@ -20,8 +20,9 @@ std::map<uintptr_t, size_t> live;                 // device allocations
 std::map<const void*, std::string> names;         // kernels by their host address
 std::string report;                               // what went wrong, one line each
 size_t limit = ~(size_t)0, total_live = 0;
-uint64_t n_alloc = 0, pairs = 0, list_mean = 0, big_alloc = 0;
-uint64_t scan_n = 0, scan_each = 0;               // what the next scan of a view's build adds up to
+uint64_t n_alloc = 0, pairs = 0;
+uint64_t list_mean = 0, block_mean = 0;           // entries of a pixel's blend list, of a block's list
+uint64_t npix = 0, scan_n = 0;                    // pixels of the view that is built, length of the scan under way
 
 struct Cfg {
     dim3 g, b;
@@ -109,15 +110,13 @@ void hook(const std::string& name, void** a) {
         t[2] = sum;
     };
     if (is("k_order_small")) put(arg<unsigned long long*>(a, 7), pairs, arg<uint64_t>(a, 8));
-    if (is("k_row_counts")) scan_n = (uint64_t)arg<int>(a, 2), scan_each = 1;
-    if (is("k_list_lens")) {
-        const uint64_t cap = arg<uint32_t>(a, 2);
-        scan_n = arg<uint64_t>(a, 1);
-        scan_each = ((list_mean < cap ? list_mean : cap) + 4) & ~(uint64_t)3;
-    }
+    if (is("k_list_lens")) npix = arg<uint64_t>(a, 1);
+    if (is("15k_scan_partialsP")) scan_n = arg<uint64_t>(a, 1);
     if (is("k_scan_partials_top")) {
         const uint64_t cap = arg<uint64_t>(a, 3);
-        put(arg<unsigned long long*>(a, 2), cap == ~0ull ? scan_n * scan_each : pairs, cap);
+        // a view's build: list lengths, its blocks' entries, or rows (one a tile)
+        const uint64_t each = scan_n == npix ? (list_mean + 4) & ~(uint64_t)3 : (scan_n == npix / 64 ? block_mean : 1);
+        put(arg<unsigned long long*>(a, 2), cap == ~0ull ? scan_n * each : pairs, cap);
     }
 }
 
@@ -129,7 +128,11 @@ extern "C" {
 
 // what the tests set and read
 __attribute__((visibility("default"))) void fake_limit(uint64_t bytes) { limit = bytes; }
-__attribute__((visibility("default"))) void fake_counts(uint64_t p, uint64_t mean) { pairs = p, list_mean = mean; }
+__attribute__((visibility("default"))) void fake_counts(uint64_t p, uint64_t list, uint64_t block) {
+    pairs = p;
+    list_mean = list;
+    block_mean = block;
+}
 __attribute__((visibility("default"))) uint64_t fake_live() { return total_live; }
 __attribute__((visibility("default"))) uint64_t fake_allocations() { return n_alloc; }
 __attribute__((visibility("default"))) const char* fake_report() { return report.c_str(); }

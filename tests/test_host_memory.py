@@ -41,7 +41,7 @@ for f in ("fake_live", "fake_allocations"):
     getattr(L, f).restype = C.c_uint64
 L.fake_report.restype = C.c_char_p
 L.fake_limit.argtypes = [C.c_uint64]
-L.fake_counts.argtypes = [C.c_uint64, C.c_uint64]
+L.fake_counts.argtypes = [C.c_uint64] * 3
 ADDR = 1 << 20   # stands for a device buffer: no kernel runs
 
 def scene(n=20_000, degree=0, fmt=S.FP32):
@@ -75,7 +75,7 @@ def test_full_rerender_over_views_of_different_sizes(fake, first, second, tile):
     run(fake, f"""
     h = scene()
     G.gs_set_tile(h, *{tile}, stream=0)
-    L.fake_counts(2_000_000, 20)
+    L.fake_counts(2_000_000, 20, 100)
     G.gs_set_views(h, cams({first}, {second}), stream=0)
     for flips in (1, 1000, 5000):
         G.gs_inject_and_render_full(h, ADDR, 2, flips, -1, 0, ADDR, stream=0)
@@ -91,11 +91,11 @@ def test_counting_tables_hold_every_grid(fake):
     total = np.zeros(1, np.uint64)
     for (tx, ty), cap in product([(1, 1), (7, 1), (9, 9), (50, 50), (100, 65), (69, 100), (83, 83), (139, 100), (140, 100)],
                                  [1, 1000, 1536, 2049, 300_000, 5_000_000, 40_000_000, 2_000_000_000]):
-        L.fake_counts(min(cap, 1000), 0)
+        L.fake_counts(min(cap, 1000), 0, 100)
         G.gs_bin_tiles(ADDR, ADDR, 1, tx, ty, ADDR, ADDR, cap, stream=0)
     for n in (400_000, 1_200_000):
         h = scene(n=n)
-        L.fake_counts(9_000_000, 0)
+        L.fake_counts(9_000_000, 0, 100)
         for W, H in ((2200, 1600), (640, 480), (16, 16), (1600, 1040), (100, 1600), (2592, 1944), (1900, 1250), (800, 800)):
             G.gs_render(h, cams((W, H)), ADDR, stream=0)
         clean(h)
@@ -113,7 +113,7 @@ def test_scratch_after_a_failed_growth(fake):
             ids = [G.gs_server_add_scene(srv, h) for h in (small, big)]
 
             def render(i, size, pairs):
-                L.fake_counts(pairs, 0)
+                L.fake_counts(pairs, 0, 100)
                 t = G.gs_server_submit(srv, G.make_request(G.GS_REQ_RENDER, ids[i], cams(size)[0], dev_rgb=ADDR))
                 G.gs_server_wait(srv, t)
 
@@ -167,7 +167,7 @@ def test_server_account(fake, sizes):
     back to a render that waits."""
     run(fake, f"""
     small = {SMALL}
-    L.fake_counts(100_000, 30)   # five tiles a primitive: within what a render is admitted for
+    L.fake_counts(100_000, 30, 100)   # five tiles a primitive: within what a render is admitted for
     h = scene()
     G.gs_set_views(h, cams(*{sizes}), stream=0)
     scene_live = L.fake_live()
@@ -240,5 +240,22 @@ def test_batch_size_settles(fake):
         assert campaign() == 0
         G.gs_free_scene(h)
         h = scene()
+    clean(h)
+    """)
+
+
+@pytest.mark.parametrize("room", [60, 100, 105, 150, 400])
+def test_lists_leave_room(fake, room):
+    """Blend lists take a view's share of what is free: several views of long lists are
+    set where memory holds a part of them only (room: percent of one view's lists)."""
+    run(fake, f"""
+    n_lists = 200
+    L.fake_counts(100_000, n_lists, 1000)
+    npix = 1600 * 1040
+    h = scene()
+    L.fake_limit(L.fake_live() + (400 << 20) + npix * 24 * n_lists * {room} // 100)
+    G.gs_set_views(h, cams(*[(1600, 1040)] * 3), stream=0)
+    G.gs_inject_and_render(h, ADDR, 20_000, 1, -1, 0, ADDR, stream=0)
+    G.gs_render(h, cams((1600, 1040)), ADDR, stream=0)
     clean(h)
     """)
