@@ -215,6 +215,21 @@ struct Union1 {
     }
 };
 
+// The tile lists' pair stream: run w of `runs` equal ones over pairs [0, total), and the
+// step from 64 pairs to the next of [.., end).  Totals go up to 2^32 - 2: no sum here
+// passes 32 bits.
+__host__ __device__ inline void pair_run(uint32_t total, uint32_t runs, uint32_t w, uint32_t& p0, uint32_t& p1) {
+    const uint32_t len = total / runs + (total % runs != 0u ? 1u : 0u);
+    const uint64_t at = (uint64_t)w * len;
+    p0 = at < total ? (uint32_t)at : total;
+    p1 = total - p0 > len ? p0 + len : total;
+}
+__host__ __device__ inline bool pair_next(uint32_t& b, uint32_t end) {
+    if (end - b <= 64u) return false;
+    b += 64u;
+    return true;
+}
+
 // ----------------------------------------------------------------------------
 // per-view clean state and scratch
 // ----------------------------------------------------------------------------

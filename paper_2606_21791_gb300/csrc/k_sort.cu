@@ -468,11 +468,15 @@ __device__ __forceinline__ void walk_pairs(const uint32_t* __restrict__ sid, con
                 tile = ((xy >> 16) + ty) * (uint32_t)tiles_x + (xy & 0xffffu) + (t - ty * sw);
             };
             // two groups of 32 pairs at a time: their chains overlap
-            for (uint32_t b = first; b < end; b += 64u) {
-                uint32_t t0, i0, t1, i1;
-                pair_of(b, t0, i0);
-                pair_of(b + 32u, t1, i1);
-                f(t0, i0, b + (uint32_t)lane < end, t1, i1, b + 32u + (uint32_t)lane < end);
+            if (first < end) {
+                uint32_t b = first;
+                do {
+                    const uint32_t left = end - b;
+                    uint32_t t0, i0, t1, i1;
+                    pair_of(b, t0, i0);
+                    pair_of(b + 32u, t1, i1);
+                    f(t0, i0, (uint32_t)lane < left, t1, i1, 32u + (uint32_t)lane < left);
+                } while (pair_next(b, end));
             }
         }
         if (gend >= p1) return;
@@ -486,11 +490,8 @@ __device__ __forceinline__ void walk_pairs(const uint32_t* __restrict__ sid, con
 }
 
 // run of this warp
-__device__ __forceinline__ void pair_run(uint32_t total, uint32_t& p0, uint32_t& p1) {
-    const uint32_t runs = gridDim.x * (blockDim.x >> 5), len = (total + runs - 1u) / runs;
-    const uint32_t w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    p0 = (uint32_t)min((uint64_t)w * len, (uint64_t)total);
-    p1 = (uint32_t)min((uint64_t)p0 + len, (uint64_t)total);
+__device__ __forceinline__ void warp_run(uint32_t total, uint32_t& p0, uint32_t& p1) {
+    pair_run(total, gridDim.x * (blockDim.x >> 5), blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), p0, p1);
 }
 
 __global__ void k_tile_hist(const uint32_t* __restrict__ sid, const uint2* __restrict__ srect,
@@ -503,7 +504,7 @@ __global__ void k_tile_hist(const uint32_t* __restrict__ sid, const uint2* __res
     for (int i = threadIdx.x; i < row * warps / 4; i += blockDim.x) reinterpret_cast<uint4*>(hsm)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
     uint32_t p0, p1;
-    pair_run((uint32_t)total[0], p0, p1);
+    warp_run((uint32_t)total[0], p0, p1);
     uint32_t* h = hsm + (threadIdx.x >> 5) * row;
     walk_pairs(sid, srect, off, n, p0, p1, tiles_x,
                [&](uint32_t t0, uint32_t, bool a0, uint32_t t1, uint32_t, bool a1) {
@@ -608,7 +609,7 @@ __global__ void k_tile_place(const uint32_t* __restrict__ sid, const uint2* __re
             reinterpret_cast<const uint4*>(wtab + (size_t)blockIdx.x * warps * tpad)[i];
     __syncthreads();
     uint32_t p0, p1;
-    pair_run((uint32_t)total[0], p0, p1);
+    warp_run((uint32_t)total[0], p0, p1);
     const unsigned lt = (1u << lane) - 1u;
     walk_pairs(sid, srect, off, n, p0, p1, tiles_x,
                [&](uint32_t t0, uint32_t i0, bool a0, uint32_t t1, uint32_t i1, bool a1) {

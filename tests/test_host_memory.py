@@ -259,3 +259,40 @@ def test_lists_leave_room(fake, room):
     G.gs_render(h, cams((1600, 1040)), ADDR, stream=0)
     clean(h)
     """)
+
+
+PAIR_STREAM = """
+#include <cstdio>
+#include "gs_internal.h"
+int main() {
+    const uint32_t totals[] = {0u, 1u, 63u, 12250000u, 4294000000u, 4294967200u, 4294967231u, 4294967294u};
+    for (uint32_t total : totals)
+        for (uint32_t runs : {1u, 7u, 1824u, 2432u, 572664u}) {
+            uint32_t at = 0;
+            for (uint32_t w = 0; w < runs; w++) {   // the runs follow one another and end at the total
+                uint32_t p0, p1;
+                gs::pair_run(total, runs, w, p0, p1);
+                if (p0 != at || p1 < p0) return printf("run %u of %u over %u: %u %u\\n", w, runs, total, p0, p1), 1;
+                at = p1;
+            }
+            if (at != total) return printf("%u of %u pairs in %u runs\\n", at, total, runs), 1;
+        }
+    for (uint32_t end : {1u, 64u, 65u, 1000u, 4294967231u, 4294967232u, 4294967233u, 4294967294u})
+        for (uint32_t first = end > 200u ? end - 200u : 0u; first < end; first++) {
+            uint32_t b = first, n = 1;
+            while (gs::pair_next(b, end) && n < 10u) n++;
+            if (n != (end - first + 63u) / 64u || end - b > 64u) return printf("%u ... %u: %u steps\\n", first, end, n), 1;
+        }
+    return 0;
+}
+"""
+
+
+def test_pair_stream_up_to_32_bits(tmp_path):
+    src, exe = tmp_path / "pairs.cu", tmp_path / "pairs"
+    src.write_text(PAIR_STREAM)
+    cmd = [buildlib.nvcc(), *buildlib.ARCH, "-std=c++17", "-I", buildlib.CSRC, str(src), "-o", str(exe)]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stdout
