@@ -40,10 +40,18 @@ WORKLOAD = ("2M Gaussians (4 clusters, SH degree 3, fp32), 4 ring views 1600x104
 ENGINE = "batched dirty-tile engine (inject, plan, re-blend + compare, finalise), replayed as a CUDA graph"
 FLOP_PER_EVAL = 9           # FP32 ops per blend-list entry of a pixel (FMA = 2)
 BYTES_PER_EVAL = 20         # a blend-list entry: capped alpha, colour, rank
-DIRECT_TILES = 13900        # grids up to this size are listed by counting, larger ones by a radix sort
+DIRECT_TILES = 9000         # grids up to this size are listed by counting, the benchmark's larger ones by a radix sort
+SORT_PAIRS = 512            # (variant, view) pairs of a batch from which its candidates are put in tile order
 L2_FLUSH_BYTES = 256 << 20  # > 129 MB L2
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic_k_dirty_2M_4views.txt")
+TRAFFIC_BATCH = 8192        # the batch of that capture
+
+
+def launches_per_step(variants, views):
+    """Kernels of one batch: injector, plan, dirty-pixel blend, finalise; from SORT_PAIRS
+    (variant, view) pairs on also the candidates' tile order (two kernels)."""
+    return 6 if variants * views >= SORT_PAIRS else 4
 
 
 def log(*a):
@@ -470,7 +478,8 @@ def main():
     stages = render_stages(G, S, h, cams, flush, dev, pk, pk_kind)
 
     # roofline of the dominant kernel (dirty-pixel blend): the blend lists of the dirty
-    # pixels are read once per variant, gathered from L2 and HBM
+    # pixels are read once per variant, gathered from L1, L2 and HBM: achieved and frac
+    # count the bytes the walks ask for, dram_frac those that HBM moved (the capture's)
     clocks = clk.summary()
     kavg = sum(k[1] for k in kern_ms) / len(kern_ms) / 1000.0
     plan_avg = sum(k[0] for k in kern_ms) / len(kern_ms) / 1000.0
@@ -481,6 +490,7 @@ def main():
     hbm_peak = pk.get("hbm_gbs", 6800.0)
     roofline = {"kernel": "k_dirty (dirty-pixel blend + compare)", "bound": "memory", "achieved": achieved,
                 "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak, "traffic": traffic,
+                "dram_frac": traffic / kavg / 1e9 / hbm_peak if traffic and B == TRAFFIC_BATCH else None,
                 "peak_source": f"copy bandwidth, {pk_kind}",
                 "work_per_launch": {"evaluations": evals_per_launch, "bytes_per_eval": BYTES_PER_EVAL,
                                     "flop_per_eval": FLOP_PER_EVAL,
@@ -490,8 +500,8 @@ def main():
                                     "warp_steps": work["warp_steps"] / args.steps,
                                     "warp_steps_blending": work["warp_steps_blending"] / args.steps,
                                     "warp_cycle_share": phase_shares(work),
-                                    # of a walk step's 64 pixel slots: those the plan left active, and
-                                    # those still blending (active and not yet stopped)
+                                    # of a walk step's 32 lanes: those with a pixel, and those whose
+                                    # pixel takes the entry
                                     "slots_active_per_step": work["active_pixel_steps"] / max(work["warp_steps"], 1),
                                     "slots_live_per_step": work["evaluations"] / max(work["warp_steps"], 1),
                                     "plan_drops": {k: work[k] / args.steps for k in
@@ -510,9 +520,7 @@ def main():
                                            "tile set, batch autotuned" if args.tile else
                                            "autotuner (tiles 16x16, 8x8, 32x8; batches of powers of two up to 8192)")},
         "e2e": e2e,
-        # per step: injector, plan, dirty-pixel blend, finalise; in large batches also the
-        # candidates' tile order (two kernels)
-        "gpu_launches": (4 if B <= min(2048, 8192 // K_views) else 6) * args.steps,
+        "gpu_launches": launches_per_step(B, K_views) * args.steps,
         "records_gathered_on_rank0": None if gathered is None else int(gathered.shape[0]),
         "mpix_s_effective": value * K_views * Wd * Hd / 1e6,
         "mpix_s_blended": work["blocks_blended"] * 64 * world / t_total / 1e6,   # 8x8 blocks

@@ -191,7 +191,7 @@ struct __align__(16) DirtyDesc {
     uint16_t ox0, oy0, ox1, oy1;   // clean rect
     uint32_t new_rank;     // clean entries of lower rank lie in front of the corrupted one (kNoRank: not there)
     uint32_t old_rank;     // the clean entry's rank (kNoRank: not there)
-    uint32_t prim, pad;
+    uint32_t pad[2];
 };
 
 // The union of the half-open intervals [n0, n1) and [o0, o1) as a list: first

@@ -671,8 +671,7 @@ __global__ __launch_bounds__(kPrepWarps * 32) void k_inject_prep(
             d.new_rank = binned && __float_as_uint(d.old.depth) == __float_as_uint(d.rec.depth)
                              ? orank
                              : order_lower_bound(v.sdk, v.sid, (uint32_t)n, __float_as_uint(d.rec.depth), p);
-        d.prim = p;
-        d.pad = 0u;
+        d.pad[0] = d.pad[1] = 0u;
         desc[bk] = d;
         CmpAcc z;
         z.sse_fx = 0ull;
