@@ -315,6 +315,9 @@ int max_batch(const gs_scene* s) {
     return (int)std::max<uint64_t>(1, std::max(small, std::min<uint64_t>(kMaxPairs / K, kMaxCands / (K * tiles))));
 }
 
+// Allocations from this size on look at the free memory first (cudaMemGetInfo: 100 us).
+constexpr size_t kLookBytes = 256ull << 20;
+
 // Variants per batch of a campaign: the caller's choice, or the most.
 int campaign_batch(const gs_scene* s) { return s->batch > 0 ? std::min(s->batch, max_batch(s)) : max_batch(s); }
 
@@ -327,24 +330,28 @@ int batch_cap(int B, int chunk) {
 }
 
 // Buffers for a call of B variants (at most `chunk` a batch): a smaller batch where they
-// would take more than batch_room, or than there is memory.  Memory is looked at before
-// anything is given up, so the next call of this size settles for the same batch and
-// keeps its buffers.  Returns the variants a batch can have in *chunk.
+// would take more than batch_room, or than there is memory.  Free memory is looked at
+// before large buffers are given up for larger ones, and before any once memory has run
+// out: the next call of this size then settles for the same batch and keeps its buffers.  Returns the variants a batch can have in *chunk.
 gs_status size_batch(gs_scene* s, int B, int* chunk) {
     constexpr size_t kSlack = 16ull << 20;   // the allocator's granules
     while (true) {
         const int cap = batch_cap(B, *chunk);
         const BatchSize need = batch_size(s, std::max(cap, s->cap_B), std::max(cap, s->cap_flips)), held = batch_held(s);
+        const size_t bytes = need.bytes();
+        bool room = true;
         if (cap > 64 && !batch_fits(need, held)) {
-            size_t avail = 0, all = 0;
-            GS_CUDA(cudaMemGetInfo(&avail, &all));
-            if (need.bytes() > s->batch_room || need.bytes() + kSlack > avail + held.bytes()) {
-                *chunk = cap / 2;
-                continue;
+            room = bytes <= s->batch_room;
+            if (room && (bytes >= kLookBytes || s->batch_short)) {
+                size_t avail = 0, all = 0;
+                GS_CUDA(cudaMemGetInfo(&avail, &all));
+                room = bytes + kSlack <= avail + held.bytes();
             }
         }
-        const gs_status rs = ensure_batch_buffers(s, cap, 1);
+        const gs_status rs = room ? ensure_batch_buffers(s, cap, 1) : GS_ERR_OOM;
+        if (rs == GS_OK) s->batch_short = s->batch_short && cap < batch_cap(B, campaign_batch(s));
         if (rs != GS_ERR_OOM || cap <= 64) return rs;
+        s->batch_short = true;
         *chunk = cap / 2;
     }
 }
@@ -737,7 +744,7 @@ static gs_status build_lists(gs_scene* s, ViewState& v, Buf& buf, uint32_t* coun
     const uint64_t nrows = tot[2], E = tot[5];
     const uint64_t bytes = 4 * P * nrows + (16 + 4) * E + 16 * (E / kWalk);   // and at most 1 KB to align the parts
     bool lists = nrows < 0xffffffffull && E < 0xffffffffull;
-    if (lists && (!buf.p || bytes > buf.cap)) {
+    if (lists && bytes >= kLookBytes && (!buf.p || bytes > buf.cap)) {
         size_t avail = 0, all = 0;
         GS_CUDA(cudaMemGetInfo(&avail, &all));
         lists = bytes <= (avail + buf.cap) / (uint64_t)(views_left + 1);

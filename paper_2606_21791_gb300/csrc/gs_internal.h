@@ -340,6 +340,7 @@ struct gs_scene {
 
     // batch buffers (dirty engine and plain loop)
     size_t batch_room = ~(size_t)0;         // most bytes the batch buffers may take (see allow_batch_growth)
+    bool batch_short = false;               // the last campaign ran in smaller batches for lack of memory
     int cap_B = 0;
     int cap_flips = 0;
     uint64_t cap_flip_mem = 0, cap_pairs = 0, cap_cands = 0, cap_rows = 0, cap_bins = 0;   // elements the buffers below hold
