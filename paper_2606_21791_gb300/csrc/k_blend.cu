@@ -1307,11 +1307,13 @@ __global__ __launch_bounds__(kDirtyThreads, DENSE ? 4 : 5) void k_dirty(
     // measurement builds: SM cycles each warp spends per phase (the activity of the
     // candidates' pixels, the walk, the comparison and reductions)
     long long t_pro = 0, t_walk = 0, t_epi = 0;
-    // units are drawn: the first by place, the next ones while this one is at work
-    for (uint32_t unit = blockIdx.x, drawn = 0u;; unit = next_unit) {
+    // units are drawn: the first by place, the next ones while this one is at work (none
+    // where every unit has its block: the blocks' additions to one word take 2 us)
+    const bool more = ncand > gridDim.x * per;
+    for (uint32_t unit = blockIdx.x, drawn = ncand;; unit = next_unit) {
         const uint32_t c0 = unit * per;
-        if (c0 >= ncand) break;   // the same for the whole block
-        if (tid == 0) drawn = gridDim.x + atomicAdd(&counts[DENSE ? 8 : 0], 1u);
+        if (unit >= ncand || c0 >= ncand) break;   // the same for the whole block
+        if (tid == 0 && more) drawn = gridDim.x + atomicAdd(&counts[DENSE ? 8 : 0], 1u);
         const long long t0 = COUNT ? clock64() : 0;
         const int nv = (int)min(per, ncand - c0);
         __syncthreads();   // the previous candidates are done with the shared arrays
