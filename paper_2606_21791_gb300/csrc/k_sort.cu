@@ -397,14 +397,15 @@ size_t direct_words(const DirectShape& d, int nt) {
 
 // Words that serve every grid of up to nt tiles at a pair capacity of cap.  A block's
 // shared memory bounds tiles x warps per SM, so one wave of blocks takes the same at
-// any grid.  In small scenes the segments go with the capacity: room for the largest
-// grid then, so that a render of another size finds its tables there.  Beyond one wave
-// they go with the capacity too, for the grid at hand.
+// any grid (34 MB); beyond it the segments go with the capacity.  Small scenes have few
+// segments: 1 MB serves them, and a render of another size mostly finds its tables there
+// (a first render of 6,741 primitives at 800x800: 350 us with 1 or 34 MB, 460 with 3).
 size_t direct_tab_words(int nt, uint64_t cap) {
-    const auto per_seg = [](int n) { return (size_t)(n + 8) * (4 + 1); };
-    const size_t wave = (size_t)num_sms() * (220 * 1024 / 4);   // tiles x (warps + 2) x blocks, two bytes each
-    const size_t few = (size_t)div_up(std::max<uint64_t>(cap, 1), 6 * 256) * per_seg(kDirectTiles);
-    return std::max(std::min(wave, few), (size_t)div_up(cap, 60000) * per_seg(nt)) + (size_t)kDirectTiles + 64;
+    const auto tables = [nt](uint64_t segs) { return (size_t)segs * (size_t)(nt + 8) * (4 + 1) + (size_t)nt + 64; };
+    constexpr size_t kSmall = 1ull << 18;
+    const size_t wave = (size_t)num_sms() * (220 * 1024 / 4) + kDirectTiles + 64;   // tiles x (warps + 2) x blocks, two bytes each
+    const size_t few = tables(div_up(std::max<uint64_t>(cap, 1), 6 * 256));
+    return std::max(few <= kSmall ? kSmall : wave, tables(div_up(cap, 60000)));
 }
 
 // The pairs [p0, p1) in order, 2 x 32 at a time: f(tile, primitive, active of the
