@@ -266,7 +266,8 @@ GS_API gs_status gs_set_graphs(gs_scene* scene, int enable);
  * (every pixel keeps its clean value), of which [4] tiles by the stop test, [5]
  * tiles by the reach tests, [6] blocks because no pixel is reached, [7] blocks
  * because every reached pixel stopped before the change, [8] list entries
- * stepped over by the dirty-tile blend's warps (the longest of 32 pixels counts),
+ * stepped over by the dirty-tile blend's warps (the longest of 32 pixels counts; in
+ * views that keep block lists, 32 a step),
  * [9] as [8], [10] 8x8 pixel blocks re-blended, and the SM cycles its warps spend
  * per phase: [11] finding the active pixels, [12] the walk over their lists, [13]
  * the comparison with the clean image and the sums, then [14] the pixels

@@ -332,7 +332,8 @@ int batch_cap(int B, int chunk) {
 // Buffers for a call of B variants (at most `chunk` a batch): a smaller batch where they
 // would take more than batch_room, or than there is memory.  Free memory is looked at
 // before large buffers are given up for larger ones, and before any once memory has run
-// out: the next call of this size then settles for the same batch and keeps its buffers.  Returns the variants a batch can have in *chunk.
+// out: the next call of this size then settles for the same batch and keeps its buffers.
+// Returns the variants a batch can have in *chunk.
 gs_status size_batch(gs_scene* s, int B, int* chunk) {
     constexpr size_t kSlack = 16ull << 20;   // the allocator's granules
     while (true) {

@@ -1,26 +1,26 @@
 // (d) front-to-back alpha blending and (e) comparison against the clean frame.
 //
 // Blend (3DGS forward pass, composited over white as in Sec. 3 "Metrics and
-// severity"): one 256-thread block per 16x16 tile, one thread per pixel.  The
-// tile's sorted list is staged through shared memory 256 records at a time.
-// Each warp owns an 8x4 pixel block and skips, warp-uniformly, every staged
-// primitive whose alpha >= 1/255 box (BlendRec::ex/ey, conservative) misses the
-// block.  Per pixel: power = -(a dx^2 + c dy^2)/2 - b dx dy; skip power > 0;
+// severity"): one block of tw th / 2 threads per tw x th tile, a warp per 8x8 block of
+// pixels, two pixels per lane.  The tile's sorted list is staged through shared memory a
+// tile's pixels' worth of records at a time.  Each warp skips every staged primitive
+// whose alpha >= 1/255 box (BlendRec::ex/ey, conservative) misses its block, 32 at a
+// time.  Per pixel: power = -(a dx^2 + c dy^2)/2 - b dx dy; skip power > 0;
 // alpha = opacity exp(power); skip alpha < 1/255; alpha capped at 0.99; stop
 // before the primitive that would take T below 1e-4; C += colour alpha T.
 // The block leaves as soon as all of its pixels have stopped.
 //
-// Compare (Definitions 1-2): per tile, squared differences of [0,1]-clamped
-// images (NaN counts as 0) are summed in a fixed reduction tree, turned into a
-// fixed-point integer and added atomically, so a (variant, view) record does not
-// depend on which tiles ran or in what order: a dirty-tile re-blend and a full
-// re-render give identical records.
+// Compare (Definitions 1-2): squared differences of [0,1]-clamped images (NaN counts
+// as 0), each pixel's rounded to a fixed-point integer, are summed and added
+// atomically, so a (variant, view) record does not depend on which tiles ran or in
+// what order: a dirty-tile re-blend and a full re-render give identical records.
 //
 // Dirty-tile engine: the plan lists the (variant, view, tile) candidates that the
 // flipped primitive's clean or corrupted record can reach; the dirty blend decides
-// per pixel, re-blends the pixels that can change from their own blend lists
-// (kept with the clean view), with the clean entry left out and the corrupted
-// record at its (depth, index) place, and compares them on the fly.
+// per pixel, re-blends the pixels that can change from their own blend lists (in dense
+// views from their block's list; both kept with the clean view), with the clean entry
+// left out and the corrupted record at its (depth, index) place, and compares them on
+// the fly.
 #include <algorithm>
 #include <mutex>
 
@@ -562,7 +562,9 @@ struct ListOut {
 
 // First row of the states of a block whose list starts at `off` (tb: the block's number
 // in its view): a block of n entries has n / kRowStride + 1.
-__device__ __forceinline__ size_t block_rows(uint32_t off, uint32_t tb) { return (size_t)(off / (uint32_t)kRowStride) + tb; }
+__device__ __forceinline__ size_t block_rows(uint32_t off, uint32_t tb) {
+    return (size_t)(off / (uint32_t)kRowStride) + tb;
+}
 
 // Entries of a pixel on their way to its list: a lane takes an entry here and
 // there, so writing each by itself would cost two partial stores per entry (0.72
@@ -1247,11 +1249,12 @@ struct DirtyPix {
 // pixels over the lanes (32 lists per warp) the walk took 150 SM cycles per group of
 // 8 entries whatever the occupancy.  Why 16 candidates: a tile of a 2M-primitive
 // view holds three of a batch's, which would leave most of a block's warps idle.
-// Bound by issue and the gathers' latency together (43% of issue slots, 18% of the
-// DRAM rate at 24 warps per SM; 40 warps of 48 registers and 4 entries at a time
-// took it from 4.6 to 3.6 ms).  20,000 upsets of a 2M-primitive scene in four
-// 1600x1040 views: 3.55 ms, where the walk over block sublists with every alpha
-// evaluated took 6.0 ms.
+// Bound by the gathers' latency and the longest walk of a unit: 42% of issue slots, 49%
+// of the DRAM rate, 17 of a walk step's 32 lanes blending (1,024 upsets of 500,000
+// primitives, four views).  20,000 upsets of a 2M-primitive scene in four 1600x1040 views:
+// 40 warps of 48 registers per SM and 4 entries at a time 4.6 to 3.6 ms (the walk over
+// block lists with every alpha evaluated took 6.0); drawn units took 8,192 of them from
+// 1.56 to 1.38 ms.
 constexpr int kDirtyWarps = 8;   // warps per block
 constexpr int kDirtyThreads = kDirtyWarps * 32;
 static_assert(kDirtyThreads >= kTilePix, "a thread per pixel of the tile");
